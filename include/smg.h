@@ -120,7 +120,13 @@ enum {
                                  most 512) are split over two warps of 8 rows per lane (the
                                  wide-line kernel, with its clusters and tables) instead of one
                                  warp of 16 (the general plane cycle); lines longer than 512 rows
-                                 always take the wide-line kernel.  The two differ by rounding */
+                                 always take the wide-line kernel.  The two differ by rounding */,
+    SMG_OPT_MODAL = 14        /* 1 (default): the cycle runs in the sine eigenvectors of the x-lines
+                                 where that is the faster form (every FP32 and BF16 cycle, FP64 ones
+                                 with x-lines of at most 160 rows): the same relaxations, with an
+                                 exact line solve a division per mode; 0: the plane kernels, to which
+                                 the options above on threads, clusters, step orders, tables and
+                                 restriction apply.  The two differ by rounding */
 };
 
 /*

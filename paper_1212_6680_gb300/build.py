@@ -20,8 +20,12 @@ LIB = os.path.join(HERE, "libsmg.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 KS = (1, 2, 3, 4, 6, 8, 16)
 SOURCES = ["api.cpp", "hierarchy.cpp", "cycle.cu", "krylov_kernels.cu", "lobpcg.cu", "noalloc.cu", "batched.cu", "net.cu",
-           "net_api.cpp", "conv_tc.cu", "gram_tc.cu"]
+           "net_api.cpp", "conv_tc.cu", "gram_tc.cu", "modal.cu"]
 WKS = (8, 16)  # rows per lane of the wide-line kernel's segments (plane_wide.cu, one unit each)
+
+
+# mode-space configurations (modal_inst.cu): 0 float / 1 double, lanes a plane, lines a lane
+MODAL = ((0, 8, 4), (0, 8, 8), (0, 8, 16), (0, 16, 16), (0, 32, 16), (1, 8, 4), (1, 8, 8), (1, 16, 8), (1, 32, 8), (1, 32, 16))
 
 
 def nvcc() -> str:
@@ -46,6 +50,9 @@ def _units():
     for w in WKS:
         units.append((os.path.join(CSRC, "plane_wide.cu"), os.path.join(BUILD, f"plane_wide_w{w}.o"), ["-x", "cu"],
                       [f"-DSMG_WK={w}"]))
+    for t, g, k in MODAL:
+        units.append((os.path.join(CSRC, "modal_inst.cu"), os.path.join(BUILD, f"modal_{t}_{g}_{k}.o"), ["-x", "cu"],
+                      [f"-DSMG_MT={t}", f"-DSMG_MG={g}", f"-DSMG_MK={k}"]))
     for k in (1, 2, 3, 4):
         src = os.path.join(CSRC, "batched_inst.cu")
         units.append((src, os.path.join(BUILD, f"batched_k{k}.o"), ["-x", "cu"], [f"-DSMG_K={k}"]))

@@ -13,6 +13,7 @@
 #include "../../include/smg.h"
 #include "krylov.h"
 #include "lobpcg.h"
+#include "modal.h"
 #include "net.h"
 #include "smg_internal.h"
 
@@ -111,6 +112,9 @@ struct smg_ctx {
     int cluster_max32 = 0;          // largest cluster for FP32-compute plane relaxations; 0 = chosen
                                     // per size (see relax)
     int num_sms = 0;
+    int modal = 1;                  // 1: the cycle in the x-lines' sine eigenvectors where use_modal holds
+    bool modal_now = false;         // the level vectors in place are that cycle's
+    ModalPlan mp;
     // Krylov vectors (one right-hand side)
     double *d_r = nullptr, *d_p = nullptr, *d_q = nullptr, *d_dr = nullptr;
     double *d_bh = nullptr, *d_xh = nullptr;  // device copies for host-pointer calls
@@ -174,6 +178,8 @@ void free_levels(smg_ctx *h) {
     h->d_ws = nullptr;
     h->ws_bytes = 0;
     h->nb_alloc = 0;
+    modal_free(h->mp);
+    h->modal_now = false;
 }
 
 size_t compute_bytes(Prec p) { return p == Prec::F64 ? 8 : 4; }
@@ -212,6 +218,11 @@ PlaneLayout with_solo_levels(const HostHierarchy &H, size_t elem_bytes, int R, i
     return base;
 }
 
+// Whether the cycle runs in the x-lines' sine eigenvectors (modal.cuh): every FP32 and BF16 cycle; an
+// FP64 cycle up to kModalMaxNx64 points a line (its transforms are FP64 products of order nx / 2).
+constexpr int kModalMaxNx64 = 160;
+bool use_modal(const smg_ctx *h) { return h->modal && (h->prec != Prec::F64 || h->nx <= kModalMaxNx64); }
+
 // Allocate level vectors for nb right-hand sides in the current precision, and the plane
 // workspace; configure the kernels' dynamic shared memory.
 int ensure_levels(smg_ctx *h, int nb) {
@@ -219,6 +230,22 @@ int ensure_levels(smg_ctx *h, int nb) {
     free_levels(h);
     const HostHierarchy &H = h->H;
     const size_t sb = storage_bytes(h->prec);
+    if (use_modal(h)) {
+        const int e = modal_build(h->mp, H, h->prec == Prec::F64, nb, h->npre, h->npost, h->coarse_iters);
+        if (e == 0) {
+            // the Krylov kernels read T r of one right-hand side in the storage precision
+            h->d_f.assign(1, nullptr);
+            h->d_u.assign(1, nullptr);
+            SMG_CUDA(cudaMalloc(&h->d_u[0], static_cast<size_t>(h->N()) * sb));
+            h->modal_now = true;
+            h->nb_alloc = nb;
+            h->alloc_prec = h->prec;
+            return SMG_OK;
+        }
+        modal_free(h->mp);
+        if (e != static_cast<int>(cudaErrorNotSupported))
+            return fail(SMG_ERR_CUDA, std::string("mode-space cycle: ") + cudaGetErrorString(static_cast<cudaError_t>(e)));
+    }
     h->d_f.assign(H.L, nullptr);
     h->d_u.assign(H.L, nullptr);
     for (int l = 0; l < H.L; ++l) {
@@ -443,8 +470,8 @@ struct RegionTimer {
     double bytes;
     cudaEvent_t e0 = nullptr;
     RegionTimer(smg_ctx *h_, cudaStream_t st_, int cls_, double bytes_) : h(h_), st(st_), cls(cls_), bytes(bytes_) {
-        // the learned correction (class 5) is also timed in profile mode 1, beside level 0
-        if (h->profile == 2 || (h->profile == 1 && cls == 5)) {
+        // the learned correction (class 5) and the mode-space cycle (class 0) are also timed in mode 1
+        if (h->profile == 2 || (h->profile == 1 && (cls == 5 || cls == 0))) {
             e0 = take_event(h);
             cudaEventRecord(e0, st);
         }
@@ -599,8 +626,31 @@ int relax(smg_ctx *h, int l, int colour, int mode, int iters, bool coarsest, con
     return SMG_OK;
 }
 
-// u0 = T f0 for nb right-hand sides; f0, u0 in storage precision, level-0 layout.
+// u0 = T f0 for nb right-hand sides in mode space: f0 in FP64, u0 of type `type`.
+int run_modal(smg_ctx *h, int nb, const double *f0, Prec type, void *u0, cudaStream_t st) {
+    const double n = static_cast<double>(h->N()) * nb, cb = h->mp.f64 ? 8.0 : 4.0;
+    {
+        RegionTimer rt(h, st, 3, n * (8.0 + cb));
+        const cudaError_t e = modal_transform_in(h->mp, nb, f0, st, h->launches);
+        if (e != cudaSuccess) return fail(SMG_ERR_CUDA, std::string("transform launch: ") + cudaGetErrorString(e));
+    }
+    {
+        RegionTimer rt(h, st, 0, n * 2.0 * cb);
+        const cudaError_t e = modal_cycle(h->mp, nb, st, h->launches);
+        if (e != cudaSuccess) return fail(SMG_ERR_CUDA, std::string("mode-space cycle launch: ") + cudaGetErrorString(e));
+    }
+    {
+        RegionTimer rt(h, st, 3, n * (cb + static_cast<double>(storage_bytes(type))));
+        const cudaError_t e = modal_transform_out(h->mp, nb, type, u0, st, h->launches);
+        if (e != cudaSuccess) return fail(SMG_ERR_CUDA, std::string("transform launch: ") + cudaGetErrorString(e));
+    }
+    return SMG_OK;
+}
+
+// u0 = T f0 for nb right-hand sides; f0, u0 in storage precision, level-0 layout (in mode space f0
+// in FP64).
 int run_cycle(smg_ctx *h, int nb, const void *f0, void *u0, cudaStream_t st) {
+    if (h->modal_now) return run_modal(h, nb, static_cast<const double *>(f0), h->prec, u0, st);
     const HostHierarchy &H = h->H;
     const int L = H.L;
     int rc;
@@ -747,10 +797,12 @@ int krylov_device(smg_ctx *h, int variant, const double *b, double *x, double to
     }
     const bool f64 = (h->prec == Prec::F64);
     const bool ident = (h->precond == 0);                           // T = I: s is r itself
-    void *f0 = f64 ? static_cast<void *>(h->d_r) : h->d_f[0];     // cycle input  = (S) r
+    // cycle input: (S) r, written by the Krylov kernels, or r itself (FP64 cycles and mode space)
+    const bool own_f0 = !f64 && !h->modal_now;
+    void *f0 = own_f0 ? h->d_f[0] : static_cast<void *>(h->d_r);
     void *u0 = ident ? static_cast<void *>(h->d_r) : h->d_u[0];   // s = T r
     const Prec kp = ident ? Prec::F64 : h->prec;                    // storage type of s
-    void *f0k = (f64 || ident) ? nullptr : f0;                      // what the Krylov kernels write
+    void *f0k = (own_f0 && !ident) ? f0 : nullptr;                  // what the Krylov kernels write
     const double tol2 = tol * tol;
     // the device-side loop: not with the learned correction, training-pair capture or per-launch
     // profiling (their host-side steps and events sit between the kernels of an iteration)
@@ -932,6 +984,7 @@ int smg_set_option(smg_handle h, int option, int value) {
         return SMG_OK;
     case SMG_OPT_COARSE_ITERS:
         if (value < 1 || value > 64) return fail(SMG_ERR_ARG, "coarse_iters must be in [1, 64]");
+        if (value != h->coarse_iters && h->modal_now) free_levels(h);  // part of its kernels' arguments
         h->coarse_iters = value;
         return SMG_OK;
     case SMG_OPT_THREADS:
@@ -980,6 +1033,11 @@ int smg_set_option(smg_handle h, int option, int value) {
         if (value != 0 && value != 1) return fail(SMG_ERR_ARG, "lean must be 0 or 1");
         h->lean = value;
         return SMG_OK;
+    case SMG_OPT_MODAL:
+        if (value != 0 && value != 1) return fail(SMG_ERR_ARG, "modal must be 0 or 1");
+        if (value != h->modal) free_levels(h);
+        h->modal = value;
+        return SMG_OK;
     case SMG_OPT_PROFILE:
         if (value < 0 || value > 2) return fail(SMG_ERR_ARG, "profile must be 0, 1 or 2");
         h->profile = value;
@@ -996,7 +1054,9 @@ int smg_apply_batched(smg_handle h, int nb, const double *R, double *S, void *st
     int rc;
     if ((rc = ensure_levels(h, nb)) != SMG_OK) return rc;
     const long long n = h->N() * nb;
-    if (h->prec == Prec::F64) {
+    if (h->modal_now) {
+        if ((rc = run_modal(h, nb, R, Prec::F64, S, st)) != SMG_OK) return rc;
+    } else if (h->prec == Prec::F64) {
         if ((rc = run_cycle(h, nb, R, S, st)) != SMG_OK) return rc;
     } else {
         SMG_CUDA(launch_convert_to(h->prec, n, R, h->d_f[0], st));
