@@ -25,7 +25,7 @@ WKS = (8, 16)  # rows per lane of the wide-line kernel's segments (plane_wide.cu
 
 
 # mode-space configurations (modal_inst.cu): 0 float / 1 double, lanes a plane, lines a lane
-MODAL = ((0, 8, 4), (0, 8, 8), (0, 8, 16), (0, 16, 16), (0, 32, 16), (1, 8, 4), (1, 8, 8), (1, 16, 8), (1, 32, 8), (1, 32, 16))
+MODAL = ((0, 8, 4), (0, 8, 8), (0, 16, 8), (0, 16, 16), (0, 32, 16), (1, 8, 4), (1, 8, 8), (1, 16, 8), (1, 32, 8), (1, 32, 16))
 
 
 def nvcc() -> str:

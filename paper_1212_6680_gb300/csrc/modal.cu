@@ -13,6 +13,9 @@
 // of both parities.  FP32: bound by FFMA issue (64 FMAs to 12 shared-memory reads a step).
 #include <cmath>
 #include <cstring>
+#include <map>
+#include <string>
+#include <vector>
 
 #include "modal.cuh"
 
@@ -33,13 +36,6 @@ template <> __device__ __forceinline__ float out_val<float, float>(float v) { re
 template <> __device__ __forceinline__ double out_val<double, float>(float v) { return widen_f32(v); }
 template <> __device__ __forceinline__ __nv_bfloat16 out_val<__nv_bfloat16, float>(float v) { return __float2bfloat16_rn(v); }
 template <> __device__ __forceinline__ double out_val<double, double>(double v) { return v; }
-
-struct SineArgs {
-    int nx, ny, nz, pitch;   // pitch: lines per plane of the mode vectors (lines ny .. pitch-1 are zero)
-    int nh;                  // odd modes, and pairs of points: ceil(nx / 2)
-    int hp;                  // order of the stored matrices (nh rounded up to 32)
-    const void *mat;         // [4][hp][hp]: by point odd, even; by mode odd, even
-};
 
 // One stage: acc[p][i][j] += sum_k A_p[k][line i] B_p[k][mode j] for both parities p.  In FP32 the stage's
 // sum is formed apart and added once, which keeps the rounding error of a long line that of a short
@@ -120,16 +116,14 @@ __device__ __forceinline__ void stage_matrix(T *b0, T *b1, const T *m0, const T 
 
 // fhat[rhs][mode][line] = sum_x s_mode(x) f[rhs][line][x]; modes in the order odd, even.
 template <class T>
-__global__ void __launch_bounds__(128) sine_in_kernel(const __grid_constant__ SineArgs g, const double *__restrict__ f, T *__restrict__ out) {
+__device__ __forceinline__ void sine_in_body(const SineArgs &g, const double *__restrict__ fr, T *__restrict__ o, int line_tile, int mode_tile,
+                                             unsigned char *smem_raw) {
     constexpr int TM = tm_lines<T>(), BM = 16 * TM, LD = BM + 4, NL = BM * kBK / 128;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
     SineSmem<T, TM> &s = *reinterpret_cast<SineSmem<T, TM> *>(smem_raw);
-    pdl_trigger();
     const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
-    const long long lines = static_cast<long long>(g.nz) * g.pitch, p0 = static_cast<long long>(blockIdx.x) * BM;
-    const int c0 = blockIdx.y * kBN, ne = g.nx / 2;
+    const long long lines = static_cast<long long>(g.nz) * g.pitch, p0 = static_cast<long long>(line_tile) * BM;
+    const int c0 = mode_tile * kBN, ne = g.nx / 2;
     const T *m0 = static_cast<const T *>(g.mat), *m1 = m0 + static_cast<long long>(g.hp) * g.hp;
-    const double *fr = f + static_cast<long long>(blockIdx.z) * g.nx * g.ny * g.nz;
     line_offsets(s, g, p0);
     stage_matrix(s.b[0][0], s.b[0][1], m0, m1, g.hp, 0, c0);
     pdl_wait();
@@ -177,7 +171,6 @@ __global__ void __launch_bounds__(128) sine_in_kernel(const __grid_constant__ Si
         if (more) fold(cur ^ 1, (kt + 1) * kBK);
         __syncthreads();
     }
-    T *o = out + static_cast<long long>(blockIdx.z) * g.nx * lines;
 #pragma unroll
     for (int p = 0; p < 2; ++p)
 #pragma unroll
@@ -193,21 +186,35 @@ __global__ void __launch_bounds__(128) sine_in_kernel(const __grid_constant__ Si
         }
 }
 
+template <class T>
+__global__ void __launch_bounds__(128) sine_in_kernel(const __grid_constant__ SineArgs g, const double *__restrict__ f, T *__restrict__ out) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    pdl_trigger();
+    const long long rhs = blockIdx.z;
+    sine_in_body<T>(g, f + rhs * g.nx * g.ny * g.nz, out + rhs * g.nx * g.nz * g.pitch, blockIdx.x, blockIdx.y, smem_raw);
+}
+__global__ void __launch_bounds__(128) sine_in_batch_kernel(const SineJob *__restrict__ jobs, const SineTile *__restrict__ tiles,
+                                                        const int *active) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const SineTile t = tiles[blockIdx.x];
+    if (active[t.sys] != 1) return;
+    const SineJob j = jobs[t.sys];
+    sine_in_body<float>(j.g, j.in, j.fh, t.line_tile, t.mode_tile, smem_raw);
+}
+
 // u[rhs][line][x] = sum_mode s_mode(x) uhat[rhs][mode][line]: both parities' sums for 32 points and their
 // mirror images, sum and difference staged in shared memory so that lines are written whole words in x order.
 template <class T, class S>
-__global__ void __launch_bounds__(128) sine_out_kernel(const __grid_constant__ SineArgs g, const T *__restrict__ uh, S *__restrict__ u) {
+__device__ __forceinline__ void sine_out_body(const SineArgs &g, const T *__restrict__ in, S *__restrict__ ur, int line_tile, int mode_tile,
+                                              unsigned char *smem_raw) {
     constexpr int TM = tm_lines<T>(), BM = 16 * TM, LD = BM + 4;
     constexpr int PER = 16 / sizeof(T), NA = kBK * BM / PER / 128;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
     SineSmem<T, TM> &s = *reinterpret_cast<SineSmem<T, TM> *>(smem_raw);
-    pdl_trigger();
     const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
-    const long long lines = static_cast<long long>(g.nz) * g.pitch, p0 = static_cast<long long>(blockIdx.x) * BM;
-    const int c0 = blockIdx.y * kBN, ne = g.nx / 2;
+    const long long lines = static_cast<long long>(g.nz) * g.pitch, p0 = static_cast<long long>(line_tile) * BM;
+    const int c0 = mode_tile * kBN, ne = g.nx / 2;
     const long long hh = static_cast<long long>(g.hp) * g.hp;
     const T *m0 = static_cast<const T *>(g.mat) + 2 * hh, *m1 = m0 + hh;
-    const T *in = uh + static_cast<long long>(blockIdx.z) * g.nx * lines;
     line_offsets(s, g, p0);
     stage_matrix(s.b[0][0], s.b[0][1], m0, m1, g.hp, 0, c0);
     pdl_wait();
@@ -264,7 +271,6 @@ __global__ void __launch_bounds__(128) sine_out_kernel(const __grid_constant__ S
             w[(ty * TM + i) * LS + kBN + tx * 4 + j] = acc[0][i][j] - acc[1][i][j];
         }
     __syncthreads();
-    S *ur = u + static_cast<long long>(blockIdx.z) * g.nx * g.ny * g.nz;
     const int lane = tid & 31, x = c0 + lane;
     for (int i = tid >> 5; i < BM; i += 4) {
         const long long o = s.off[i];
@@ -272,6 +278,22 @@ __global__ void __launch_bounds__(128) sine_out_kernel(const __grid_constant__ S
         if (x < g.nh) ur[o + x] = out_val<S, T>(w[i * LS + lane]);
         if (x < ne) ur[o + g.nx - 1 - x] = out_val<S, T>(w[i * LS + kBN + lane]);
     }
+}
+
+template <class T, class S>
+__global__ void __launch_bounds__(128) sine_out_kernel(const __grid_constant__ SineArgs g, const T *__restrict__ uh, S *__restrict__ u) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    pdl_trigger();
+    const long long rhs = blockIdx.z;
+    sine_out_body<T, S>(g, uh + rhs * g.nx * g.nz * g.pitch, u + rhs * g.nx * g.ny * g.nz, blockIdx.x, blockIdx.y, smem_raw);
+}
+__global__ void __launch_bounds__(128) sine_out_batch_kernel(const SineJob *__restrict__ jobs, const SineTile *__restrict__ tiles,
+                                                         const int *active) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const SineTile t = tiles[blockIdx.x];
+    if (active[t.sys] != 1) return;
+    const SineJob j = jobs[t.sys];
+    sine_out_body<float, float>(j.g, j.uh, j.out, t.line_tile, t.mode_tile, smem_raw);
 }
 
 // ---- prolongation and correction on a level above the tail -------------------------------------------
@@ -299,7 +321,7 @@ __global__ void __launch_bounds__(256) modal_prolong_kernel(const __grid_constan
     if (z & 1) {
         add(z >> 1, T(1));
     } else {
-        const T *zc = A.zc + (A.plane_base[l] + z) * kCoefPerPlane;
+        const T *zc = A.zt + A.ptype[A.plane_base[l] + z] * kCoefPerPlane;
         if (z > 0) add(z / 2 - 1, zc[6]);
         if (z / 2 < nzc) add(z / 2, zc[7]);
     }
@@ -311,7 +333,7 @@ __global__ void __launch_bounds__(256) modal_prolong_kernel(const __grid_constan
 #define SMG_MODAL_CFG(MT, GG, KK) extern const ModalKernels<std::conditional_t<MT == 0, float, double>> modal_kernels_##MT##_##GG##_##KK
 SMG_MODAL_CFG(0, 8, 4);
 SMG_MODAL_CFG(0, 8, 8);
-SMG_MODAL_CFG(0, 8, 16);
+SMG_MODAL_CFG(0, 16, 8);
 SMG_MODAL_CFG(0, 16, 16);
 SMG_MODAL_CFG(0, 32, 16);
 SMG_MODAL_CFG(1, 8, 4);
@@ -323,7 +345,7 @@ SMG_MODAL_CFG(1, 32, 16);
 ModalConfig modal_config(int ny, bool f64) {
     if (ny <= 32) return {8, 4};
     if (ny <= 64) return {8, 8};
-    if (ny <= 128) return f64 ? ModalConfig{16, 8} : ModalConfig{8, 16};
+    if (ny <= 128) return {16, 8};
     if (ny <= 256) return f64 ? ModalConfig{32, 8} : ModalConfig{16, 16};
     return {32, 16};
 }
@@ -331,8 +353,7 @@ ModalConfig modal_config(int ny, bool f64) {
 template <>
 const ModalKernels<float> &modal_kernels<float>(ModalConfig c) {
     if (c.K == 4) return modal_kernels_0_8_4;
-    if (c.K == 8) return modal_kernels_0_8_8;
-    if (c.G == 8) return modal_kernels_0_8_16;
+    if (c.K == 8) return c.G == 8 ? modal_kernels_0_8_8 : modal_kernels_0_16_8;
     return c.G == 16 ? modal_kernels_0_16_16 : modal_kernels_0_32_16;
 }
 template <>
@@ -343,8 +364,8 @@ const ModalKernels<double> &modal_kernels<double>(ModalConfig c) {
     return c.G == 16 ? modal_kernels_1_16_8 : modal_kernels_1_32_8;
 }
 
-// The 16 coefficients of line y of 2D level m of the plane with coefficient table pc (pairs (s, t) stand
-// for s lambda + t): the diagonal, the couplings to lines y-1 and y+1, then for an even line its
+// The coefficients of line y of 2D level m of the plane with coefficient table pc (pairs (s, t) stand for
+// s lambda + t): the diagonal, the couplings to lines y-1 and y+1, then for an even line its
 // interpolation weights, for an odd line 2j+1 the restriction's multipliers of lines 2j-1, 2j+1, 2j+3 and
 // the diagonal of coarse line j.
 static void raw_line(const HostHierarchy &H, const double *pc, int m, int y, double *r) {
@@ -390,7 +411,7 @@ size_t up(size_t v, size_t to) { return (v + to - 1) / to * to; }
 
 // Shared memory of the tail from level lt on (offsets into a), 0 when it does not fit.
 template <class T>
-size_t plan_tail(ModalArgs<T> &a, int lt, const ModalKernels<T> &k) {
+size_t plan_tail(ModalArgs<T> &a, int lt, ModalConfig cfg, const ModalKernels<T> &k) {
     const size_t row = a.sm_pitch;
     size_t o = 0;
     int cls = 1;
@@ -403,95 +424,150 @@ size_t plan_tail(ModalArgs<T> &a, int lt, const ModalKernels<T> &k) {
         if (l + 1 < a.L) cls = std::max(cls, a.ncls[l]);
         if (o * sizeof(T) > kModalSmem) return 0;
     }
-    a.sm_tab = static_cast<int>(up(o, 4));
-    o = a.sm_tab + static_cast<size_t>(cls) * k.table_elems;
-    const size_t planes = a.plane_base[a.L - 1] + 1 - a.plane_base[lt];
-    a.sm_zc = static_cast<int>(o);
-    o += planes * kCoefPerPlane;
-    size_t b = up(o * sizeof(T), 16);
-    a.sm_tab64 = static_cast<int>(b);
-    b += static_cast<size_t>(k.table64_elems) * 8;
-    a.sm_cls = static_cast<int>(b);
-    b += up(planes, 16);
+    auto elems = [&](int &at, size_t n) {
+        at = static_cast<int>(o = up(o, 4));
+        o += n;
+    };
+    elems(a.sm_tab, static_cast<size_t>(cls) * k.table_elems);
+    elems(a.sm_stage, static_cast<size_t>(cls) * a.blk);
+    elems(a.sm_zt, static_cast<size_t>(a.nptype) * kCoefPerPlane);
+    size_t b = o * sizeof(T);
+    auto bytes = [&](int &at, size_t n) {
+        at = static_cast<int>(b = up(b, 16));
+        b += n;
+    };
+    const int k6 = cfg.G * cfg.K / 32;  // Tab<32, k6>::kElems, and the level-0 couplings with one line a lane
+    bytes(a.sm_tab64, sizeof(double) * (9 * 32 * (k6 - 1) + 1024 + 32 * k6 + (k6 == 1 ? 64 : 0)));
+    bytes(a.sm_ltype, 2 * static_cast<size_t>(a.sum_ny));
+    bytes(a.sm_ptype, 2 * static_cast<size_t>(a.plane_base[a.L - 1] + 1 - a.plane_base[lt]));
+    bytes(a.sm_pcls, 2 * static_cast<size_t>(a.nptype));
     return b <= kModalSmem ? b : 0;
 }
 
+}  // namespace
+
 template <class T>
-int build(ModalPlan &p, ModalArgs<T> &a, const HostHierarchy &H) {
-    const int nx = H.nx, L = H.L, nb = p.nb;
-    const ModalKernels<T> &k = modal_kernels<T>(p.cfg);
+int modal_plan(ModalHost<T> &h, const HostHierarchy &H, ModalConfig cfg, int nb, int npre, int npost, int coarse_iters) {
+    const int nx = H.nx, L = H.L, nh = (nx + 1) / 2;
+    h.cfg = cfg;
+    ModalArgs<T> &a = h.a;
     std::memset(&a, 0, sizeof(a));
     a.nmode = nx;
     a.ny = H.ny;
-    a.pitch = p.pitch;
+    a.pitch = static_cast<int>(up(H.ny, 4));
     a.L = L;
     a.P = H.P;
     a.sum_ny = H.sum_ny;
-    a.npre = p.npre;
-    a.npost = p.npost;
-    a.coarse_iters = p.coarse_iters;
+    a.npre = npre;
+    a.npost = npost;
+    a.coarse_iters = coarse_iters;
     for (int m = 0; m < H.P; ++m) a.ny_m[m] = H.ny_m[m], a.line_base[m] = H.line_base[m];
-    a.sm_pitch = static_cast<int>(up(H.ny, p.cfg.K));
-    // plane classes and their line coefficients
-    std::vector<unsigned char> cls(H.nplanes_total);
-    std::vector<T> raw, zc(H.zcoef.begin(), H.zcoef.end());
-    std::vector<double> raw64(static_cast<size_t>(H.sum_ny) * kRawPerLine), lam(nx);
-    int base = 0;
+    a.sm_pitch = static_cast<int>(up(H.ny, cfg.K));
+    // plane classes; plane types: planes with equal coefficients and class
+    std::vector<unsigned short> ptype(H.nplanes_total), pcls, ltype(H.sum_ny);
+    std::vector<T> zt;
+    std::vector<const double *> reps;  // each class's plane table
+    std::map<std::string, int> seen;
     for (int l = 0; l < L; ++l) {
         std::vector<int> slot, rep;
         a.nz[l] = H.nz_l[l];
         a.plane_base[l] = H.plane_base[l];
-        a.cls_base[l] = base;
+        a.cls_base[l] = static_cast<int>(reps.size());
         a.ncls[l] = plane_classes(H, l, slot, rep);
-        if (a.ncls[l] > 255) return static_cast<int>(cudaErrorNotSupported);
-        base += a.ncls[l];
-        for (int z = 0; z < a.nz[l]; ++z) cls[H.plane_base[l] + z] = static_cast<unsigned char>(slot[z]);
-        for (int z : rep) {
-            const double *pc = &H.pcoef[static_cast<size_t>(H.plane_base[l] + z) * H.sum_ny * kCoefPerLine];
-            for (int m = 0; m < H.P; ++m)
-                for (int y = 0; y < H.ny_m[m]; ++y) {
-                    double r[kRawPerLine];
-                    raw_line(H, pc, m, y, r);
-                    for (double v : r) raw.push_back(static_cast<T>(v));
-                    if (l == L - 1)
-                        std::memcpy(&raw64[static_cast<size_t>(H.line_base[m] + y) * kRawPerLine], r, sizeof(r));
-                }
+        for (int z = 0; z < a.nz[l]; ++z) {
+            const double *zc = &H.zcoef[static_cast<size_t>(H.plane_base[l] + z) * kCoefPerPlane];
+            std::string key(reinterpret_cast<const char *>(zc), sizeof(double) * kCoefPerPlane);
+            key.append(reinterpret_cast<const char *>(&slot[z]), sizeof(int));
+            const auto it = seen.emplace(key, static_cast<int>(seen.size()));
+            if (it.second) {
+                for (int i = 0; i < kCoefPerPlane; ++i) zt.push_back(static_cast<T>(zc[i]));
+                pcls.push_back(static_cast<unsigned short>(slot[z]));
+            }
+            ptype[H.plane_base[l] + z] = static_cast<unsigned short>(it.first->second);
         }
+        for (int z : rep) reps.push_back(&H.pcoef[static_cast<size_t>(H.plane_base[l] + z) * H.sum_ny * kCoefPerLine]);
     }
+    a.ncls_all = static_cast<int>(reps.size());
+    a.nptype = static_cast<int>(pcls.size());
+    // line types: lines with equal coefficients in every class
+    std::vector<std::vector<double>> rows;  // [type][class][kRawPerLine]
+    seen.clear();
+    for (int m = 0; m < H.P; ++m)
+        for (int y = 0; y < H.ny_m[m]; ++y) {
+            std::vector<double> r(reps.size() * kRawPerLine);
+            for (size_t c = 0; c < reps.size(); ++c) raw_line(H, reps[c], m, y, &r[c * kRawPerLine]);
+            const auto it = seen.emplace(std::string(reinterpret_cast<const char *>(r.data()), r.size() * sizeof(double)),
+                                         static_cast<int>(rows.size()));
+            if (it.second) rows.push_back(std::move(r));
+            ltype[H.line_base[m] + y] = static_cast<unsigned short>(it.first->second);
+        }
+    a.ntype = static_cast<int>(rows.size());
+    a.blk = a.ntype * kRow + cfg.G * cfg.G;
+    std::vector<double> raw(static_cast<size_t>(a.ncls_all) * a.ntype * kRawPerLine), lam(nx);
+    for (int t = 0; t < a.ntype; ++t)
+        for (int c = 0; c < a.ncls_all; ++c)
+            std::memcpy(&raw[(static_cast<size_t>(c) * a.ntype + t) * kRawPerLine], &rows[t][static_cast<size_t>(c) * kRawPerLine],
+                        kRawPerLine * sizeof(double));
     const double pi = 3.14159265358979323846;
     for (int q = 0; q < nx; ++q) {
-        const int kk = q < p.nh ? 2 * q + 1 : 2 * (q - p.nh) + 2;
+        const int kk = q < nh ? 2 * q + 1 : 2 * (q - nh) + 2;
         const double s = std::sin(pi * kk / (2.0 * (nx + 1)));
         lam[q] = 4.0 * s * s;
     }
-    // coefficients on the device
-    const size_t b_zc = up(zc.size() * sizeof(T), 256), b_raw = up(raw.size() * sizeof(T), 256),
-                 b_r64 = up(raw64.size() * 8, 256), b_lam = up(lam.size() * 8, 256), b_cls = up(cls.size(), 256);
-    MCHK(cudaMalloc(&p.d_tab, b_zc + b_raw + b_r64 + b_lam + b_cls));
-    unsigned char *d = static_cast<unsigned char *>(p.d_tab);
-    auto put = [&](const void *src, size_t bytes, size_t room) {
-        const cudaError_t e = cudaMemcpy(d, src, bytes, cudaMemcpyHostToDevice);
-        d += room;
-        return e;
-    };
-    a.zc = reinterpret_cast<const T *>(d);
-    MCHK(put(zc.data(), zc.size() * sizeof(T), b_zc));
-    a.raw = reinterpret_cast<const T *>(d);
-    MCHK(put(raw.data(), raw.size() * sizeof(T), b_raw));
-    a.raw64 = reinterpret_cast<const double *>(d);
-    MCHK(put(raw64.data(), raw64.size() * 8, b_r64));
-    a.lam = reinterpret_cast<const double *>(d);
-    MCHK(put(lam.data(), lam.size() * 8, b_lam));
-    a.cls = d;
-    MCHK(put(cls.data(), cls.size(), b_cls));
-    // transform matrices: by point (odd, even modes), then by mode
-    const size_t hp = p.hp;
+    const size_t sizes[] = {raw.size() * 8, lam.size() * 8, zt.size() * sizeof(T), ptype.size() * 2, pcls.size() * 2, ltype.size() * 2};
+    const void *const src[] = {raw.data(), lam.data(), zt.data(), ptype.data(), pcls.data(), ltype.data()};
+    size_t o = 0;
+    for (int i = 0; i < 6; ++i) {
+        h.at[i] = o;
+        o += up(sizes[i], 256);
+    }
+    h.shared.assign(o, 0);
+    for (int i = 0; i < 6; ++i) std::memcpy(h.shared.data() + h.at[i], src[i], sizes[i]);
+    h.coef_values = static_cast<size_t>(nx) * a.ncls_all * a.blk;
+    h.coef64_values = static_cast<size_t>(nx) * (a.ntype * kRow + 1024);
+    // the first level whose coarser levels all fit in one CTA's shared memory
+    const ModalKernels<T> &k = modal_kernels<T>(cfg);
+    h.smem = 0;
+    for (int lt = 0; lt < L && h.smem == 0; ++lt) h.smem = plan_tail(a, lt, cfg, k);
+    if (h.smem == 0) return static_cast<int>(cudaErrorNotSupported);
+    h.vec_bytes = 0;
+    h.vec_off.clear();
+    for (int l = 0; l <= a.lt; ++l)
+        for (int t = 0; t < 2; ++t) {
+            h.vec_off.push_back(h.vec_bytes);
+            h.vec_bytes += up(static_cast<size_t>(nb) * nx * a.nz[l] * a.pitch * sizeof(T), 256);
+        }
+    return 0;
+}
+
+template <class T>
+void modal_place(ModalHost<T> &h, unsigned char *shared, T *coef, double *coef64, unsigned char *vec) {
+    ModalArgs<T> &a = h.a;
+    a.raw = reinterpret_cast<const double *>(shared + h.at[0]);
+    a.lam = reinterpret_cast<const double *>(shared + h.at[1]);
+    a.zt = reinterpret_cast<const T *>(shared + h.at[2]);
+    a.ptype = reinterpret_cast<const unsigned short *>(shared + h.at[3]);
+    a.pcls = reinterpret_cast<const unsigned short *>(shared + h.at[4]);
+    a.ltype = reinterpret_cast<const unsigned short *>(shared + h.at[5]);
+    a.coef64 = coef64;
+    a.coef = coef;
+    for (int l = 0; l <= a.lt; ++l) {
+        a.fw[l] = reinterpret_cast<T *>(vec + h.vec_off[2 * l]);
+        a.f[l] = a.fw[l];
+        a.u[l] = reinterpret_cast<T *>(vec + h.vec_off[2 * l + 1]);
+    }
+}
+
+template <class T>
+std::vector<T> sine_matrices(int nx) {
+    const int nh = (nx + 1) / 2;
+    const size_t hp = up(nh, 32);
+    const double pi = 3.14159265358979323846, sc = std::sqrt(2.0 / (nx + 1));
     std::vector<T> mat(4 * hp * hp, T(0));
-    const double sc = std::sqrt(2.0 / (nx + 1));
     std::vector<double> sines(2 * (nx + 1));
     for (int i = 0; i < 2 * (nx + 1); ++i) sines[i] = sc * std::sin(pi * i / (nx + 1));
-    for (int x = 0; x < p.nh; ++x)
-        for (int q = 0; q < p.nh; ++q)
+    for (int x = 0; x < nh; ++x)
+        for (int q = 0; q < nh; ++q)
             for (int par = 0; par < 2; ++par) {
                 if (par == 1 && (q >= nx / 2 || x >= nx / 2)) continue;
                 const long long ph = static_cast<long long>(x + 1) * (2 * q + 1 + par) % (2 * (nx + 1));
@@ -499,40 +575,63 @@ int build(ModalPlan &p, ModalArgs<T> &a, const HostHierarchy &H) {
                 mat[par * hp * hp + x * hp + q] = v;
                 mat[(2 + par) * hp * hp + q * hp + x] = v;
             }
+    return mat;
+}
+
+int modal_tail_threads(size_t smem, long long ctas, int num_sms, int most, int planes, int G) {
+    if (ctas > num_sms) {
+        if (4 * (smem + 2048) <= kModalSmem) most = std::min(most, 128);
+        else if (2 * (smem + 2048) <= kModalSmem) most = std::min(most, 256);
+    }
+    const int want = (planes + 1) / 2 * G;
+    return std::min(most, std::max(128, (want + 31) / 32 * 32));
+}
+
+template int modal_plan<float>(ModalHost<float> &, const HostHierarchy &, ModalConfig, int, int, int, int);
+template void modal_place<float>(ModalHost<float> &, unsigned char *, float *, double *, unsigned char *);
+template std::vector<float> sine_matrices<float>(int);
+
+namespace {
+
+template <class T>
+int build(ModalPlan &p, ModalHost<T> &h, const HostHierarchy &H, int npre, int npost, int coarse_iters) {
+    const ModalConfig cfg = modal_config(H.ny, sizeof(T) == 8);
+    if (int e = modal_plan<T>(h, H, cfg, p.nb, npre, npost, coarse_iters)) return e;
+    const ModalKernels<T> &k = modal_kernels<T>(cfg);
+    const size_t b_coef = up(h.coef_values * sizeof(T), 256), b_64 = up(h.coef64_values * 8, 256);
+    MCHK(cudaMalloc(&p.d_tab, h.shared.size() + b_64 + b_coef));
+    MCHK(cudaMalloc(&p.d_buf, h.vec_bytes));
+    unsigned char *d = static_cast<unsigned char *>(p.d_tab);
+    MCHK(cudaMemcpy(d, h.shared.data(), h.shared.size(), cudaMemcpyHostToDevice));
+    double *c64 = reinterpret_cast<double *>(d + h.shared.size());
+    T *coef = reinterpret_cast<T *>(d + h.shared.size() + b_64);
+    modal_place<T>(h, d, coef, c64, static_cast<unsigned char *>(p.d_buf));
+    MCHK(k.setup(h.a, coef, c64, 0));
+    const std::vector<T> mat = sine_matrices<T>(H.nx);
     MCHK(cudaMalloc(&p.d_sin, mat.size() * sizeof(T)));
     MCHK(cudaMemcpy(p.d_sin, mat.data(), mat.size() * sizeof(T), cudaMemcpyHostToDevice));
-    // the first level whose coarser levels all fit in one CTA's shared memory
-    p.smem = 0;
-    for (p.lt = 0; p.lt < L; ++p.lt)
-        if ((p.smem = plan_tail(a, p.lt, k)) != 0) break;
-    if (p.smem == 0) return static_cast<int>(cudaErrorNotSupported);
-    const int groups = (a.nz[p.lt] + 1) / 2, want = groups * p.cfg.G;
-    p.threads = std::min(k.max_threads, std::max(128, (want + 31) / 32 * 32));
-    // mode vectors: f and u of levels 0 .. lt
-    size_t total = 0;
-    std::vector<size_t> off;
-    for (int l = 0; l <= p.lt; ++l)
-        for (int t = 0; t < 2; ++t) {
-            off.push_back(total);
-            total += up(static_cast<size_t>(nb) * nx * a.nz[l] * a.pitch * sizeof(T), 256);
-        }
-    MCHK(cudaMalloc(&p.d_buf, total));
-    unsigned char *bb = static_cast<unsigned char *>(p.d_buf);
-    for (int l = 0; l <= p.lt; ++l) {
-        a.fw[l] = reinterpret_cast<T *>(bb + off[2 * l]);
-        a.f[l] = a.fw[l];
-        a.u[l] = reinterpret_cast<T *>(bb + off[2 * l + 1]);
-    }
-    MCHK(cudaMalloc(&p.d_args, sizeof(a)));
-    MCHK(cudaMemcpy(p.d_args, &a, sizeof(a), cudaMemcpyHostToDevice));
+    p.sine = SineArgs{H.nx, H.ny, H.nz, h.a.pitch, (H.nx + 1) / 2, static_cast<int>(up((H.nx + 1) / 2, 32)), p.d_sin};
+    MCHK(cudaMalloc(&p.d_args, sizeof(h.a)));
+    MCHK(cudaMemcpy(p.d_args, &h.a, sizeof(h.a), cudaMemcpyHostToDevice));
+    int dev = 0;
+    MCHK(cudaGetDevice(&dev));
+    MCHK(cudaDeviceGetAttribute(&p.num_sms, cudaDevAttrMultiProcessorCount, dev));
+    MCHK(cudaStreamSynchronize(0));  // the set-up kernel: callers' streams need not wait for the default one
     return 0;
 }
 
 template <class T>
-cudaError_t cycle(const ModalPlan &p, const ModalArgs<T> &a, int nb, cudaStream_t st, long long &launches) {
-    const ModalKernels<T> &k = modal_kernels<T>(p.cfg);
+cudaError_t prolong(const ModalArgs<T> &a, int l, int nb, cudaStream_t st) {
+    const long long n = static_cast<long long>(a.nz[l]) * (a.pitch / 4);
+    return launch_pdl(modal_prolong_kernel<T>, dim3(static_cast<unsigned>((n + 255) / 256), a.nmode, nb), dim3(256), 0, st, a, l);
+}
+
+template <class T>
+cudaError_t cycle(const ModalPlan &p, const ModalHost<T> &h, int nb, cudaStream_t st, long long &launches) {
+    const ModalArgs<T> &a = h.a;
+    const ModalKernels<T> &k = modal_kernels<T>(h.cfg);
     cudaError_t e;
-    for (int l = 0; l < p.lt; ++l) {
+    for (int l = 0; l < a.lt; ++l) {
         if (a.npre == 1 && k.slab_fits(a, l)) {
             if ((e = k.slab(a, l, nb, st)) != cudaSuccess) return e;
             launches += 1;
@@ -546,12 +645,11 @@ cudaError_t cycle(const ModalPlan &p, const ModalArgs<T> &a, int nb, cudaStream_
         if ((e = k.restrict_(a, l, nb, st)) != cudaSuccess) return e;
         launches += 1;
     }
-    if ((e = k.tail(static_cast<const ModalArgs<T> *>(p.d_args), a.nmode, nb, p.threads, p.smem, st)) != cudaSuccess) return e;
+    const int threads = modal_tail_threads(h.smem, static_cast<long long>(a.nmode) * nb, p.num_sms, k.max_threads, a.nz[a.lt], h.cfg.G);
+    if ((e = k.tail(static_cast<const ModalArgs<T> *>(p.d_args), a.nmode, nb, threads, h.smem, st)) != cudaSuccess) return e;
     launches += 1;
-    for (int l = p.lt - 1; l >= 0; --l) {
-        const long long n = static_cast<long long>(a.nz[l]) * (a.pitch / 4);
-        e = launch_pdl(modal_prolong_kernel<T>, dim3(static_cast<unsigned>((n + 255) / 256), a.nmode, nb), dim3(256), 0, st, a, l);
-        if (e != cudaSuccess) return e;
+    for (int l = a.lt - 1; l >= 0; --l) {
+        if ((e = prolong(a, l, nb, st)) != cudaSuccess) return e;
         launches += 1;
         for (int s = 0; s < a.npost; ++s)
             for (int c = 1; c >= 0; --c) {
@@ -562,13 +660,11 @@ cudaError_t cycle(const ModalPlan &p, const ModalArgs<T> &a, int nb, cudaStream_
     return cudaSuccess;
 }
 
-SineArgs sine_args(const ModalPlan &p) { return SineArgs{p.nx, p.ny, p.nz, p.pitch, p.nh, p.hp, p.d_sin}; }
-
 template <class T>
 dim3 sine_grid(const ModalPlan &p, int nb) {
-    const long long lines = static_cast<long long>(p.nz) * p.pitch;
+    const long long lines = static_cast<long long>(p.sine.nz) * p.sine.pitch;
     constexpr int BM = 16 * tm_lines<T>();
-    return dim3(static_cast<unsigned>((lines + BM - 1) / BM), (p.nh + kBN - 1) / kBN, nb);
+    return dim3(static_cast<unsigned>((lines + BM - 1) / BM), (p.sine.nh + kBN - 1) / kBN, nb);
 }
 
 template <class T>
@@ -576,14 +672,14 @@ cudaError_t sine_in(const ModalPlan &p, int nb, const double *f, T *out, cudaStr
     constexpr size_t smem = sizeof(SineSmem<T, tm_lines<T>()>);
     cudaError_t e = raise_smem_attr(reinterpret_cast<const void *>(&sine_in_kernel<T>), smem);
     if (e != cudaSuccess) return e;
-    return launch_pdl(sine_in_kernel<T>, sine_grid<T>(p, nb), dim3(128), smem, st, sine_args(p), f, out);
+    return launch_pdl(sine_in_kernel<T>, sine_grid<T>(p, nb), dim3(128), smem, st, p.sine, f, out);
 }
 template <class T, class S>
 cudaError_t sine_out(const ModalPlan &p, int nb, const T *uh, void *u, cudaStream_t st) {
     constexpr size_t smem = sizeof(SineSmem<T, tm_lines<T>()>);
     cudaError_t e = raise_smem_attr(reinterpret_cast<const void *>(&sine_out_kernel<T, S>), smem);
     if (e != cudaSuccess) return e;
-    return launch_pdl(sine_out_kernel<T, S>, sine_grid<T>(p, nb), dim3(128), smem, st, sine_args(p), uh, static_cast<S *>(u));
+    return launch_pdl(sine_out_kernel<T, S>, sine_grid<T>(p, nb), dim3(128), smem, st, p.sine, uh, static_cast<S *>(u));
 }
 
 }  // namespace
@@ -591,30 +687,48 @@ cudaError_t sine_out(const ModalPlan &p, int nb, const T *uh, void *u, cudaStrea
 int modal_build(ModalPlan &p, const HostHierarchy &H, bool f64, int nb, int npre, int npost, int coarse_iters) {
     modal_free(p);
     p.f64 = f64;
-    p.nx = H.nx, p.ny = H.ny, p.nz = H.nz, p.nb = nb, p.L = H.L;
-    p.nh = (H.nx + 1) / 2;
-    p.hp = static_cast<int>(up(p.nh, 32));
-    p.npre = npre, p.npost = npost, p.coarse_iters = coarse_iters;
-    p.pitch = static_cast<int>(up(H.ny, 4));
-    p.cfg = modal_config(H.ny, f64);
-    return f64 ? build<double>(p, p.a64, H) : build<float>(p, p.a32, H);
+    p.nb = nb;
+    return f64 ? build<double>(p, p.h64, H, npre, npost, coarse_iters) : build<float>(p, p.h32, H, npre, npost, coarse_iters);
 }
 
 cudaError_t modal_transform_in(const ModalPlan &p, int nb, const double *f0, cudaStream_t st, long long &launches) {
     launches += 1;
-    return p.f64 ? sine_in<double>(p, nb, f0, p.a64.fw[0], st) : sine_in<float>(p, nb, f0, p.a32.fw[0], st);
+    return p.f64 ? sine_in<double>(p, nb, f0, p.h64.a.fw[0], st) : sine_in<float>(p, nb, f0, p.h32.a.fw[0], st);
 }
 
 cudaError_t modal_cycle(const ModalPlan &p, int nb, cudaStream_t st, long long &launches) {
-    return p.f64 ? cycle<double>(p, p.a64, nb, st, launches) : cycle<float>(p, p.a32, nb, st, launches);
+    return p.f64 ? cycle<double>(p, p.h64, nb, st, launches) : cycle<float>(p, p.h32, nb, st, launches);
 }
 
 cudaError_t modal_transform_out(const ModalPlan &p, int nb, Prec type, void *u0, cudaStream_t st, long long &launches) {
     launches += 1;
-    if (p.f64) return sine_out<double, double>(p, nb, p.a64.u[0], u0, st);
-    if (type == Prec::F64) return sine_out<float, double>(p, nb, p.a32.u[0], u0, st);
-    if (type == Prec::BF16) return sine_out<float, __nv_bfloat16>(p, nb, p.a32.u[0], u0, st);
-    return sine_out<float, float>(p, nb, p.a32.u[0], u0, st);
+    if (p.f64) return sine_out<double, double>(p, nb, p.h64.a.u[0], u0, st);
+    if (type == Prec::F64) return sine_out<float, double>(p, nb, p.h32.a.u[0], u0, st);
+    if (type == Prec::BF16) return sine_out<float, __nv_bfloat16>(p, nb, p.h32.a.u[0], u0, st);
+    return sine_out<float, float>(p, nb, p.h32.a.u[0], u0, st);
 }
+
+int sine_line_tiles(const SineArgs &g) {
+    constexpr int BM = 16 * tm_lines<float>();
+    return static_cast<int>((static_cast<long long>(g.nz) * g.pitch + BM - 1) / BM);
+}
+int sine_mode_tiles(const SineArgs &g) { return (g.nh + kBN - 1) / kBN; }
+
+cudaError_t launch_sine_in_batch(const SineJob *jobs, const SineTile *tiles, int ntiles, const int *active, cudaStream_t st) {
+    constexpr size_t smem = sizeof(SineSmem<float, tm_lines<float>()>);
+    cudaError_t e = raise_smem_attr(reinterpret_cast<const void *>(&sine_in_batch_kernel), smem);
+    if (e != cudaSuccess) return e;
+    sine_in_batch_kernel<<<ntiles, 128, smem, st>>>(jobs, tiles, active);
+    return cudaGetLastError();
+}
+cudaError_t launch_sine_out_batch(const SineJob *jobs, const SineTile *tiles, int ntiles, const int *active, cudaStream_t st) {
+    constexpr size_t smem = sizeof(SineSmem<float, tm_lines<float>()>);
+    cudaError_t e = raise_smem_attr(reinterpret_cast<const void *>(&sine_out_batch_kernel), smem);
+    if (e != cudaSuccess) return e;
+    sine_out_batch_kernel<<<ntiles, 128, smem, st>>>(jobs, tiles, active);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_modal_prolong(const ModalArgs<float> &a, int l, int nb, cudaStream_t st) { return prolong(a, l, nb, st); }
 
 }  // namespace smg

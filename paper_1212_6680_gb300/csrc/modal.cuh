@@ -18,12 +18,16 @@
 // One plane of one mode is a vector of ny values.  G lanes hold K consecutive lines each
 // (G K >= ny, both powers of two), and the plane's y-cycle runs in registers:
 //   * coarse line i of level m+1 is line 2i+1 of level m, so a lane's K lines hold K/2 lines of the
-//     next level, and so on: the first log2 K levels need a shuffle only at the lane borders, the
-//     rest has one line per lane (level log2 K + t at lanes 2^t - 1 (mod 2^t));
+//     next level, and so on: the first log2 K levels need shuffles only at the lane borders;
+//   * from level log2 K on (one line per lane) the rest of the y-cycle is a linear map of G values
+//     that depends on the mode and the plane's class only: one G x G product with a matrix formed at
+//     set-up (log2 G levels of dependent shuffles before: 510 of 1190 cycles of a plane's latency);
 //   * right-hand sides are kept divided by the line's diagonal (gi = g / (S lambda + T)), which
 //     turns each relaxation into two FMAs a line and makes the first even sweep the identity;
 //   * the lines' multipliers come from a table in shared memory, laid out so that a group's lanes
-//     read consecutive words; planes with equal coefficients (plane_classes) share one.
+//     read consecutive words.  It is spread there at each z-level from the few line types that
+//     differ (ModalArgs), fetched by cp.async while the level before is relaxed: formed in the
+//     kernel with its divisions it took 5300 of about 14000 cycles a level.
 // Lines past the end have zero multipliers, so no step tests for them.
 #pragma once
 
@@ -52,80 +56,66 @@ __device__ __forceinline__ void st4(double *p, double x, double y, double z, dou
 constexpr int ilog2(int n) { return n <= 1 ? 0 : 1 + ilog2(n / 2); }
 
 // Layout of one plane class's line table (elements of T).  In-register level m (K >> m lines a lane):
-// per even line {a-, a+, wm, wp}, per odd line {a-, a+, ca, cc} and cb; level log2 K + t: the same per
-// lane.  a-, a+: couplings over the diagonal; wm, wp: interpolation weights; ca, cb, cc: the
-// restriction from lines 2j-1, 2j+1, 2j+3 to coarse line j, over the coarse line's diagonal.
+// per even line {a-, a+, wm, wp}, per odd line {a-, a+, ca, cc} and cb.  a-, a+: couplings over the
+// diagonal; wm, wp: interpolation weights; ca, cb, cc: the restriction from lines 2j-1, 2j+1, 2j+3 to
+// coarse line j, over the coarse line's diagonal.  Then the G x G matrix D of the levels from log2 K
+// on (D[k][lane], four k together) and the reciprocal diagonals of level 0.
 template <int G, int K>
 struct Tab {
-    static constexpr int M0 = ilog2(K), TM = ilog2(G);
-    static constexpr int quad(int m) { return m == 0 ? 0 : quad(m - 1) + (K >> (m - 1)) * G; }
+    static constexpr int M0 = ilog2(K);
+    static constexpr int quad(int m) { return 2 * G * (K - (K >> m)); }
     static constexpr int even(int m) { return 4 * quad(m); }
     static constexpr int odd(int m) { return 4 * (quad(m) + (K >> m) / 2 * G); }
-    static constexpr int cross(int t) { return 4 * (quad(M0) + t * G); }
-    static constexpr int kScal = 4 * (quad(M0) + (TM + 1) * G);
-    static constexpr int scal(int m) { return m == 0 ? kScal : scal(m - 1) + (K >> (m - 1)) / 2 * G; }
-    static constexpr int xscal(int t) { return scal(M0) + t * G; }
-    static constexpr int kInv = kScal + (scal(M0) - kScal) + (TM + 1) * G;
-    static constexpr int kElems = (kInv + K * G + 3) / 4 * 4;
-    static constexpr int kEntries = quad(M0) + (TM + 1) * G;
-    // reciprocal diagonal of line lane K + j of level 0: four lines of a lane together
-    __host__ __device__ static constexpr int inv(int lane, int j) {
+    static constexpr int kScal = 4 * quad(M0);
+    static constexpr int scal(int m) { return kScal + G * (K - (K >> m)); }
+    static constexpr int kDense = scal(M0) + (G * (K - 1)) % 4;  // a multiple of 4
+    static constexpr int kInv = kDense + G * G;
+    static constexpr int kElems = kInv + K * G;
+    static constexpr int kEntries = quad(M0);  // lines of the in-register levels
+    __host__ __device__ static constexpr int dense(int k, int lane) { return kDense + ((k / 4) * G + lane) * 4 + (k & 3); }
+    __host__ __device__ static constexpr int inv(int lane, int j) {  // four lines of a lane together
         return kInv + (K >= 4 ? ((j / 4) * G + lane) * 4 + (j & 3) : j * G + lane);
     }
 };
+// values of one class in global memory: the line types' rows, then D row by row of four k (Tab::dense)
+template <int G> constexpr int class_values(int ntype) { return ntype * kRow + G * G; }
 
-// Entry e of the table of one plane class for the mode with eigenvalue lam.
+// Spread the rows of ncls classes (class c's values at src + c blk, in shared or global memory) over their
+// tables.  Entry e of a class: level m, lane, and the lane's line j of that level (line y of the level).
 template <class T, int G, int K>
-__device__ __forceinline__ void table_entry(T *tab, const T *__restrict__ raw, const T lam, const int *ny_m,
-                                            const int *line_base, const int P, int e) {
+__device__ __forceinline__ void spread_tables(T *tab, const T *src, int ncls, int blk, const unsigned short *ltype, const int *ny_m,
+                                              const int *line_base, int P, int ntype, int tid, int nt) {
     using L = Tab<G, K>;
-    int m = 0, n = K, lane, j = 0, y, t = -1;
-    while (n > 1 && e >= n * G) {
-        e -= n * G;
-        ++m;
-        n >>= 1;
-    }
-    bool line = true;
-    if (n > 1) {
-        y = e;
-        lane = e / n;
-        j = e - lane * n;
-    } else {
-        t = e / G;
-        lane = e - t * G;
-        m += t;
-        line = ((lane + 1) & ((1 << t) - 1)) == 0;
-        y = ((lane + 1) >> t) - 1;
-    }
-    T inv = T(0), am = T(0), ap = T(0), p = T(0), q = T(0), cb = T(0);
-    const bool is_odd = (y & 1) != 0;
-    if (line && m < P && y < ny_m[m]) {
-        const T *r = raw + static_cast<long long>(line_base[m] + y) * kRawPerLine;
-        const V4<T> r0 = ld4(r), r1 = ld4(r + 4);
-        inv = T(1) / fma(r0.x, lam, r0.y);
-        am = fma(r0.z, lam, r0.w) * inv;
-        ap = fma(r1.x, lam, r1.y) * inv;
-        if (is_odd) {
-            const V4<T> r2 = ld4(r + 8), r3 = ld4(r + 12);
-            const T ic = T(1) / fma(r3.x, lam, r3.y);
-            p = fma(r1.z, lam, r1.w) * ic;
-            cb = fma(r2.x, lam, r2.y) * ic;
-            q = fma(r2.z, lam, r2.w) * ic;
-        } else {
-            p = r1.z;
-            q = r1.w;
+    constexpr int kLines = K == 1 ? G : L::kEntries, kItems = kLines + G * G / 4;
+    for (int it = tid; it < ncls * kItems; it += nt) {
+        const int c = it / kItems, e = it - c * kItems;
+        T *t = tab + c * L::kElems;
+        const T *s = src + c * blk;
+        if (e >= kLines) {
+            const int i = 4 * (e - kLines);
+            const V4<T> v = ld4(s + ntype * kRow + i);
+            st4(t + L::kDense + i, v.x, v.y, v.z, v.w);
+            continue;
         }
+        int m = 0, y = e;
+#pragma unroll
+        for (int q = 0; q + 1 < L::M0; ++q)
+            if (m == q && y >= (K >> q) * G) y -= (K >> q) * G, m = q + 1;
+        const int lg = L::M0 - m, lane = y >> lg, j = y & ((1 << lg) - 1), i = j >> 1;
+        V4<T> v{T(0), T(0), T(0), T(0)};
+        T inv = T(0), cb = T(0);
+        if (m < P && y < ny_m[m]) {
+            const T *r = s + ltype[line_base[m] + y] * kRow;
+            v = ld4(r);
+            inv = r[4];
+            cb = r[5];
+        }
+        if constexpr (K > 1) {
+            st4(t + 4 * (2 * G * (K - (1 << lg)) + ((j & 1) ? (G << lg) / 2 : 0) + i * G + lane), v.x, v.y, v.z, v.w);
+            if (j & 1) t[L::kScal + G * (K - (1 << lg)) + i * G + lane] = cb;
+        }
+        if (m == 0) t[L::inv(lane, j)] = inv;
     }
-    if (t < 0) {
-        const int i = j >> 1;
-        const int base4 = 4 * ((m == 0 ? 0 : 2 * G * (K - (K >> m))) + ((j & 1) ? n / 2 * G : 0) + i * G + lane);
-        st4(tab + base4, am, ap, p, q);
-        if (j & 1) tab[L::kScal + G * (K - (K >> m)) + i * G + lane] = cb;
-    } else {
-        st4(tab + L::cross(0) + 4 * (t * G + lane), am, ap, p, q);
-        tab[L::xscal(0) + t * G + lane] = cb;
-    }
-    if (m == 0) tab[L::inv(lane, j)] = inv;
 }
 
 // Shuffles within a group of G lanes; at the group's ends they return the lane's own value, which the
@@ -135,31 +125,19 @@ __device__ __forceinline__ T up(T v, int s) { return __shfl_up_sync(0xffffffffu,
 template <class T, int G>
 __device__ __forceinline__ T dn(T v, int s) { return __shfl_down_sync(0xffffffffu, v, s, G); }
 
-// The y-cycle from level log2 K on (one line per lane): gi in, the correction out.
+// The y-cycle from level log2 K on: gi in, the correction out.
 template <class T, int G, int K>
-__device__ __forceinline__ T ycycle_cross(T gi0, const T *tab, int ln) {
-    using L = Tab<G, K>;
-    T gi[L::TM + 1];
-    gi[0] = gi0;
+__device__ __forceinline__ T ycycle_dense(T gi, const T *tab, int ln) {
+    T a = T(0), b = T(0);
 #pragma unroll
-    for (int t = 0; t < L::TM; ++t) {
-        const int s = 1 << t;
-        const V4<T> c = ld4(tab + L::cross(t) + 4 * ln);
-        const T cb = tab[L::xscal(t) + ln];
-        const T o = gi[t] - c.x * up<T, G>(gi[t], s) - c.y * dn<T, G>(gi[t], s);
-        gi[t + 1] = c.z * up<T, G>(o, 2 * s) + cb * o + c.w * dn<T, G>(o, 2 * s);
+    for (int k = 0; k < G; k += 4) {
+        const V4<T> d = ld4(tab + Tab<G, K>::dense(k, ln));
+        a = fma(d.x, __shfl_sync(0xffffffffu, gi, k, G), a);
+        b = fma(d.y, __shfl_sync(0xffffffffu, gi, k + 1, G), b);
+        a = fma(d.z, __shfl_sync(0xffffffffu, gi, k + 2, G), a);
+        b = fma(d.w, __shfl_sync(0xffffffffu, gi, k + 3, G), b);
     }
-    T c = gi[L::TM];
-#pragma unroll
-    for (int t = L::TM - 1; t >= 0; --t) {
-        const int s = 1 << t;
-        const V4<T> k = ld4(tab + L::cross(t) + 4 * ln);
-        const T v = gi[t] + k.z * up<T, G>(c, s) + k.w * dn<T, G>(c, s);       // even lines + P c
-        const T o = gi[t] - k.x * up<T, G>(v, s) - k.y * dn<T, G>(v, s);       // odd lines
-        const T e = gi[t] - k.x * up<T, G>(o, s) - k.y * dn<T, G>(o, s);       // even lines again
-        c = (((ln + 1) >> t) & 1) ? e : o;
-    }
-    return c;
+    return a + b;
 }
 
 // The y-cycle from in-register level M on: g (right-hand sides over the diagonals) in, the
@@ -170,7 +148,7 @@ __device__ __forceinline__ void ycycle(T (&g)[(K >> M)], const T *tab, int ln) {
     using L = Tab<G, K>;
     constexpr int N = K >> M;
     if constexpr (N == 1) {
-        g[0] = ycycle_cross<T, G, K>(g[0], tab, ln);
+        g[0] = ycycle_dense<T, G, K>(g[0], tab, ln);
     } else {
         constexpr int H = N / 2;
         T c[H];
@@ -241,6 +219,12 @@ __device__ __forceinline__ void load_row(T (&v)[K], const T *row, int ln, int pi
         for (int j = 0; j < R::CH; ++j) v[q * R::CH + j] = u.t[j];
     }
 }
+// The same from either place: shared rows are swizzled, global ones are not.
+template <class T, int K>
+__device__ __forceinline__ void load_row_at(T (&v)[K], const T *row, bool shared, int ln, int pitch) {
+    if (shared) load_row<T, K, true>(v, row, ln, pitch);
+    else load_row<T, K, false>(v, row, ln, pitch);
+}
 template <class T, int K, bool SM>
 __device__ __forceinline__ void store_row(T *row, const T (&v)[K], int ln, int pitch) {
     using R = RowMap<T, K>;
@@ -260,10 +244,11 @@ template <class T>
 struct Rows {
     T *p;
     int pitch, z0;   // lines per row; the plane the first row holds
+    bool shared;
     __device__ __forceinline__ T *at(int z) const { return p + static_cast<long long>(z - z0) * pitch; }
 };
 
-// One plane's part of f - sum (M (lambda + Ly) + Kc) u, on a row u (zero where the plane is absent).
+// One plane's part of f - sum (M (lambda + Ly) + Kc) u, on a row u (M = Kc = 0 where the plane is absent).
 // Ly u is formed from first differences, which are exact where u is smooth, before it meets M: on
 // coarse z-levels M / Kc grows like 4^l while u is dominated by smooth lines, and M (4 u) - M (u + u) - ...
 // would leave a rounding error of eps M u, white over the lines of this one mode, in a residual of
@@ -283,27 +268,19 @@ __device__ __forceinline__ void couple(T (&g)[K], const T (&u)[K], T M, T Kc, T 
         g[j] = fma(-M, fma(lam, u[j], d), g[j]);
     }
 }
-template <class T, int K>
-__device__ __forceinline__ void zero_row(T (&v)[K]) {
-#pragma unroll
-    for (int j = 0; j < K; ++j) v[j] = T(0);
-}
-
 // Relaxation of plane z: u_z = C_z (f - A u)_z (modes 0 and 1: the own plane is zero, mode 0: all
 // planes are) or u_z += (mode 2).  cross: the couplings between planes have an in-plane part (all
-// levels but the finest).  The result stays in g.
-template <class T, int G, int K, bool SMU, bool SMF>
-__device__ __forceinline__ void relax_plane(T (&g)[K], const Rows<T> &u, const Rows<T> &f, int z, int nz, const T *zc,
-                                            const T *tab, T lam, int mode, bool cross, int ln) {
-    load_row<T, K, SMF>(g, f.at(z), ln, f.pitch);
+// levels but the finest).  f's row comes in g; the result stays there.
+template <class T, int G, int K, bool SMU>
+__device__ __forceinline__ void relax_plane(T (&g)[K], const Rows<T> &u, int z, int nz, const T *zc, const T *tab, T lam, int mode,
+                                            bool cross, int ln) {
     if (mode > 0) {
-        T v[K];
-        if (z > 0) load_row<T, K, SMU>(v, u.at(z - 1), ln, u.pitch);
-        else zero_row<T, K>(v);
+        // a plane at the end couples to its one neighbour; the other's coefficients are zero
+        T v[K], w[K];
+        load_row<T, K, SMU>(v, u.at(z > 0 ? z - 1 : z + 1), ln, u.pitch);
+        load_row<T, K, SMU>(w, u.at(z + 1 < nz ? z + 1 : z - 1), ln, u.pitch);
         couple<T, G, K>(g, v, zc[0], zc[3], lam, cross, ln);
-        if (z + 1 < nz) load_row<T, K, SMU>(v, u.at(z + 1), ln, u.pitch);
-        else zero_row<T, K>(v);
-        couple<T, G, K>(g, v, zc[2], zc[5], lam, cross, ln);
+        couple<T, G, K>(g, w, zc[2], zc[5], lam, cross, ln);
         if (mode == 2) {
             load_row<T, K, SMU>(v, u.at(z), ln, u.pitch);
             couple<T, G, K>(g, v, zc[1], zc[4], lam, true, ln);
@@ -327,40 +304,121 @@ __device__ __forceinline__ void relax_plane(T (&g)[K], const Rows<T> &u, const R
     }
 }
 
-// Coarse plane Z's right-hand side P^T (f - A u): the residuals of planes 2Z, 2Z+1 and 2Z+2 with the
-// weights of P, as one combination of five planes of u and three of f.  zc_level: plane 0's row.
-template <class T, int G, int K, bool SMU, bool SMF>
-__device__ __forceinline__ void restrict_plane(T (&g)[K], const Rows<T> &u, const Rows<T> &f, int Z, int nz,
-                                               const T *zc_level, T lam, bool cross, int ln) {
-    const int o = 2 * Z + 1;
-    const T *zo = zc_level + o * kCoefPerPlane, *z0 = zo - kCoefPerPlane, *z1 = zo + kCoefPerPlane;
-    const bool h1 = o + 1 < nz;
-    const T w0 = z0[7], w1 = h1 ? z1[6] : T(0);
-    T v[K];
-    load_row<T, K, SMF>(g, f.at(o), ln, f.pitch);
-    load_row<T, K, SMF>(v, f.at(o - 1), ln, f.pitch);
-#pragma unroll
-    for (int j = 0; j < K; ++j) g[j] = fma(w0, v[j], g[j]);
-    if (h1) {
-        load_row<T, K, SMF>(v, f.at(o + 1), ln, f.pitch);
-#pragma unroll
-        for (int j = 0; j < K; ++j) g[j] = fma(w1, v[j], g[j]);
+// Sixteen bytes of a row at chunk c (shared rows are swizzled, global ones are not), and one value.
+template <class T, int K>
+struct Chunk {
+    static constexpr int CH = RowMap<T, K>::CH;
+    union {
+        T t[CH];
+        uint4 q;
+    };
+    __device__ __forceinline__ void load(const Rows<T> &r, int z, int c) {
+        q = reinterpret_cast<const uint4 *>(r.at(z))[r.shared ? RowMap<T, K>::chunk(c) : c];
     }
-    if (Z > 0) load_row<T, K, SMU>(v, u.at(o - 2), ln, u.pitch);
-    else zero_row<T, K>(v);
-    couple<T, G, K>(g, v, w0 * z0[0], w0 * z0[3], lam, cross, ln);
-    load_row<T, K, SMU>(v, u.at(o - 1), ln, u.pitch);
-    couple<T, G, K>(g, v, fma(w0, z0[1], zo[0]), fma(w0, z0[4], zo[3]), lam, true, ln);
-    load_row<T, K, SMU>(v, u.at(o), ln, u.pitch);
-    couple<T, G, K>(g, v, zo[1] + w0 * z0[2] + (h1 ? w1 * z1[0] : T(0)), zo[4] + w0 * z0[5] + (h1 ? w1 * z1[3] : T(0)),
-                    lam, true, ln);
-    if (h1) load_row<T, K, SMU>(v, u.at(o + 1), ln, u.pitch);
-    else zero_row<T, K>(v);
-    couple<T, G, K>(g, v, h1 ? fma(w1, z1[1], zo[2]) : T(0), h1 ? fma(w1, z1[4], zo[5]) : T(0), lam, true, ln);
-    const bool h2 = o + 2 < nz;
-    if (h2) load_row<T, K, SMU>(v, u.at(o + 2), ln, u.pitch);
-    else zero_row<T, K>(v);
-    couple<T, G, K>(g, v, h2 ? w1 * z1[2] : T(0), h2 ? w1 * z1[5] : T(0), lam, cross, ln);
+    __device__ __forceinline__ void store(const Rows<T> &r, int z, int c) const {
+        reinterpret_cast<uint4 *>(r.at(z))[r.shared ? RowMap<T, K>::chunk(c) : c] = q;
+    }
+};
+
+// Runs body(plane, chunk) for planes 0 .. count-1 and chunks 0 .. nch-1 of each, the chunks of a plane on
+// neighbouring lanes.
+template <class F>
+__device__ __forceinline__ void for_chunks(int count, int nch, F body) {
+    const int lg = nch >= 17 ? 5 : nch >= 9 ? 4 : nch >= 5 ? 3 : 2;  // lanes of a plane: 2^lg
+    for (int c = threadIdx.x & ((1 << lg) - 1); c < nch; c += 1 << lg)
+        for (int z = threadIdx.x >> lg; z < count; z += blockDim.x >> lg) body(z, c);
+}
+
+// A row's chunk with the lines before and after it.
+template <class T, int K>
+struct Window {
+    Chunk<T, K> v;
+    T l, r;
+    __device__ __forceinline__ void load(const Rows<T> &u, int z, int c, int nch, bool ends) {
+        constexpr int CH = Chunk<T, K>::CH;
+        v.load(u, z, c);
+        l = r = T(0);
+        if (!ends) return;
+        const T *row = u.at(z);
+        const int yl = max(c * CH - 1, 0), yr = min(c + 1, nch - 1) * CH;
+        l = row[u.shared ? RowMap<T, K>::elem(yl) : yl];
+        r = row[u.shared ? RowMap<T, K>::elem(yr) : yr];
+        if (c == 0) l = T(0);
+        if (c + 1 == nch) r = T(0);
+    }
+    // couple() for this chunk
+    __device__ __forceinline__ void couple(Chunk<T, K> &g, T M, T Kc, T lam, bool in_plane) const {
+        constexpr int CH = Chunk<T, K>::CH;
+#pragma unroll
+        for (int j = 0; j < CH; ++j) g.t[j] = fma(-Kc, v.t[j], g.t[j]);
+        if (!in_plane) return;
+#pragma unroll
+        for (int j = 0; j < CH; ++j) {
+            const T d = (v.t[j] - (j > 0 ? v.t[(j + CH - 1) % CH] : l)) + (v.t[j] - (j + 1 < CH ? v.t[(j + 1) % CH] : r));
+            g.t[j] = fma(-M, fma(lam, v.t[j], d), g.t[j]);
+        }
+    }
+};
+
+// Coarse plane Z's right-hand side P^T (f - A u) at chunk c: the residuals of planes 2Z, 2Z+1 and 2Z+2 with
+// the weights of P, as one combination of five planes of u and three of f.  row(z): plane z's coefficients.
+// Planes past the ends are replaced by the last one: their weights and couplings are zero (an odd
+// plane's weights are).  All loads are issued before the arithmetic.
+template <class T, int K>
+struct RestrictF {
+    Chunk<T, K> f0, g, f1;   // planes 2Z, 2Z+1, 2Z+2 of f
+    __device__ __forceinline__ void load(const Rows<T> &f, int Z, int nz, int c) {
+        f0.load(f, 2 * Z, c);
+        g.load(f, 2 * Z + 1, c);
+        f1.load(f, min(2 * Z + 2, nz - 1), c);
+    }
+};
+template <class T, int K, class F>
+__device__ __forceinline__ void restrict_chunk(RestrictF<T, K> &r, const Rows<T> &u, int Z, int nz, F row, T lam, bool cross, int c,
+                                               int nch) {
+    constexpr int CH = Chunk<T, K>::CH;
+    Chunk<T, K> &g = r.g;
+    const int o = 2 * Z + 1, e1 = min(o + 1, nz - 1);
+    const T *zo = row(o), *z0 = row(o - 1), *z1 = row(e1);
+    Window<T, K> v0, v1, v2, v3, v4;
+    v0.load(u, max(o - 2, 0), c, nch, cross);
+    v1.load(u, o - 1, c, nch, true);
+    v2.load(u, o, c, nch, true);
+    v3.load(u, e1, c, nch, true);
+    v4.load(u, min(o + 2, nz - 1), c, nch, cross);
+    const T w0 = z0[7], w1 = z1[6];
+#pragma unroll
+    for (int j = 0; j < CH; ++j) g.t[j] = fma(w1, r.f1.t[j], fma(w0, r.f0.t[j], g.t[j]));
+    v0.couple(g, w0 * z0[0], w0 * z0[3], lam, cross);
+    v1.couple(g, fma(w0, z0[1], zo[0]), fma(w0, z0[4], zo[3]), lam, true);
+    v2.couple(g, fma(w1, z1[0], fma(w0, z0[2], zo[1])), fma(w1, z1[3], fma(w0, z0[5], zo[4])), lam, true);
+    v3.couple(g, fma(w1, z1[1], zo[2]), fma(w1, z1[4], zo[5]), lam, true);
+    v4.couple(g, w1 * z1[2], w1 * z1[5], lam, cross);
+}
+
+// The restriction of coarse planes Z0 .. Z0 + count - 1, chunks 0 .. nchw - 1 (those from nch on are past
+// the rows: zero), f's chunks one plane ahead; store(Z, chunk, value).
+template <class T, int K, class F, class S>
+__device__ __forceinline__ void restrict_planes(int Z0, int count, int nch, int nchw, const Rows<T> &u, const Rows<T> &f, int nz, F row,
+                                                T lam, bool cross, S store) {
+    const int lg = nchw >= 17 ? 5 : nchw >= 9 ? 4 : nchw >= 5 ? 3 : 2, dz = blockDim.x >> lg, z0 = threadIdx.x >> lg;
+    if (z0 >= count) return;
+    for (int c = threadIdx.x & ((1 << lg) - 1); c < nchw; c += 1 << lg) {
+        if (c >= nch) {
+            Chunk<T, K> zero;
+            zero.q = make_uint4(0u, 0u, 0u, 0u);
+            for (int z = z0; z < count; z += dz) store(Z0 + z, c, zero);
+            continue;
+        }
+        RestrictF<T, K> next;
+        next.load(f, Z0 + z0, nz, c);
+        for (int z = z0; z < count; z += dz) {
+            RestrictF<T, K> r = next;
+            if (z + dz < count) next.load(f, Z0 + z + dz, nz, c);
+            restrict_chunk<T, K>(r, u, Z0 + z, nz, row, lam, cross, c, nch);
+            store(Z0 + z, c, r.g);
+        }
+    }
 }
 
 // The coarsest level: its one plane in FP64 by one warp (C steps of u += C (f - A u)).
@@ -384,8 +442,8 @@ __device__ __forceinline__ void coarsest(const T *frow, T *urow, int ny, int ite
             const double ul = up<double, 32>(u[K6 - 1], 1), ur = dn<double, 32>(u[0], 1);
 #pragma unroll
             for (int j = 0; j < K6; ++j) {
-                const double *k = K6 == 1 ? tab + L::cross(0) + 4 * lane
-                                          : tab + ((j & 1) ? L::odd(0) : L::even(0)) + 4 * ((j >> 1) * 32 + lane);
+                const double *k = tab + (K6 == 1 ? L::kElems + 2 * lane
+                                                 : ((j & 1) ? L::odd(0) : L::even(0)) + 4 * ((j >> 1) * 32 + lane));
                 g[j] = fi[j] - u[j] - k[0] * (j > 0 ? u[(j + K6 - 1) % K6] : ul) - k[1] * (j + 1 < K6 ? u[(j + 1) % K6] : ur);
             }
         }
@@ -399,150 +457,295 @@ __device__ __forceinline__ void coarsest(const T *frow, T *urow, int ny, int ite
         if (y < ny) stv<T, double>(urow + (SM ? RowMap<T, K>::elem(y) : y), u[j]);
     }
 }
+// its table: with one line a lane the couplings of level 0 (needed beyond the first step) follow it
+template <int G, int K> constexpr int tab64_elems() { return Tab<32, G * K / 32>::kElems + (G * K == 32 ? 64 : 0); }
 
-// Runs body(plane, active) for the planes first, first + step, ... (count of them), one per group of G
-// lanes; every lane of a warp takes the same number of trips (groups past the end repeat the last
-// plane with active = false).
-template <int G, class F>
-__device__ __forceinline__ void for_planes(int count, int first, int step, F body) {
-    const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5, sub = (threadIdx.x & 31) / G;
+// Runs body(plane, active, f row) for the planes first, first + step, ... (count of them), one per group
+// of G lanes; every lane of a warp takes the same number of trips (groups past the end repeat the last
+// plane with active = false).  The next plane's f row is on its way while one is relaxed: from global
+// memory its latency is as long as the relaxation.
+template <class T, int G, int K, class F>
+__device__ __forceinline__ void for_planes(int count, int first, int step, const Rows<T> &f, F body) {
     constexpr int GPW = 32 / G;
-    for (int p0 = warp * GPW; p0 < count; p0 += nw * GPW) {
-        const int p = p0 + sub;
-        body(first + step * min(p, count - 1), p < count);
+    const int p0 = (threadIdx.x >> 5) * GPW, dp = (blockDim.x >> 5) * GPW, sub = (threadIdx.x & 31) / G, ln = (threadIdx.x & 31) % G;
+    if (p0 >= count) return;
+    auto plane = [&](int p) { return first + step * min(p, count - 1); };
+    T next[K];
+    load_row_at<T, K>(next, f.at(plane(p0 + sub)), f.shared, ln, f.pitch);
+    for (int p = p0; p < count; p += dp) {
+        T g[K];
+#pragma unroll
+        for (int j = 0; j < K; ++j) g[j] = next[j];
+        if (p + dp < count) load_row_at<T, K>(next, f.at(plane(p + dp + sub)), f.shared, ln, f.pitch);
+        body(plane(p + sub), p + sub < count, g);
     }
 }
 
-template <class T, int G, int K>
-__device__ __forceinline__ void build_tables(T *tab, const ModalArgs<T> &A, int l, T lam, int tid, int nt) {
-    const T *raw = A.raw + static_cast<long long>(A.cls_base[l]) * A.sum_ny * kRawPerLine;
-    const int per = Tab<G, K>::kEntries;
-    for (int e = tid; e < per * A.ncls[l]; e += nt) {
-        const int c = e / per;
-        table_entry<T, G, K>(tab + c * Tab<G, K>::kElems, raw + static_cast<long long>(c) * A.sum_ny * kRawPerLine, lam,
-                             A.ny_m, A.line_base, A.P, e - c * per);
+// ---- set-up: the multipliers and matrices of every mode and class ------------------------------------
+
+// The y-cycle below the in-register levels on the unit vectors: thread k of a warp runs level m0 with
+// right-hand side (over the diagonals) e_k.  rows: this class's line types in FP64.
+template <int G>
+__device__ void dense_column(double *col, int k, const double *rows, const unsigned short *ltype, const int *ny_m,
+                             const int *line_base, int P, int m0) {
+    double gi[2 * G], c[G];
+    const int n0 = m0 < P ? ny_m[m0] : 0;
+    for (int i = 0; i < G; ++i) gi[i] = 0.0, col[i] = 0.0;
+    if (k >= n0) return;
+    gi[k] = 1.0;
+    int m = m0, base = 0;  // level m's right-hand sides start at base
+    auto row = [&](int mm, int y) { return rows + ltype[line_base[mm] + y] * kRow; };
+    for (; m + 1 < P; ++m) {
+        const int n = ny_m[m];
+        double *g = gi + base, *gc = g + n;
+        double prev = 0.0, here = 0.0;
+        auto odd = [&](int y) {
+            const double *r = row(m, y);
+            return g[y] - r[0] * g[y - 1] - (y + 1 < n ? r[1] * g[y + 1] : 0.0);
+        };
+        here = n > 1 ? odd(1) : 0.0;
+        for (int j = 0; j < n / 2; ++j) {
+            const double next = 2 * j + 3 < n ? odd(2 * j + 3) : 0.0;
+            const double *r = row(m, 2 * j + 1);
+            gc[j] = r[2] * prev + r[5] * here + r[3] * next;
+            prev = here;
+            here = next;
+        }
+        base += n;
+    }
+    c[0] = gi[base];
+    for (--m; m >= m0; --m) {
+        const int n = ny_m[m], nc = n / 2;
+        base -= n;
+        double *g = gi + base, v[G];
+        for (int y = 0; y < n; y += 2) {
+            const double *r = row(m, y);
+            v[y] = g[y] + (y > 0 ? r[2] * c[y / 2 - 1] : 0.0) + (y / 2 < nc ? r[3] * c[y / 2] : 0.0);
+        }
+        for (int y = 1; y < n; y += 2) {
+            const double *r = row(m, y);
+            v[y] = g[y] - r[0] * v[y - 1] - (y + 1 < n ? r[1] * v[y + 1] : 0.0);
+        }
+        for (int y = 0; y < n; y += 2) {
+            const double *r = row(m, y);
+            c[y] = g[y] - (y > 0 ? r[0] * v[y - 1] : 0.0) - (y + 1 < n ? r[1] * v[y + 1] : 0.0);
+        }
+        for (int y = 1; y < n; y += 2) c[y] = v[y];
+    }
+    for (int i = 0; i < n0; ++i) col[i] = c[i];
+}
+
+// rows of one class from its raw coefficients (s, t): s lambda + t
+__device__ __forceinline__ void type_row(double *r, const double *__restrict__ raw, double lam) {
+    auto at = [&](int i) { return fma(raw[i], lam, raw[i + 1]); };
+    const double inv = 1.0 / at(0);
+    r[0] = at(2) * inv;
+    r[1] = at(4) * inv;
+    r[4] = inv;
+    r[5] = r[6] = r[7] = 0.0;
+    if (raw[12] == 0.0) {  // an even line: its weights
+        r[2] = raw[6];
+        r[3] = raw[7];
+    } else {
+        const double ic = 1.0 / at(12);
+        r[2] = at(6) * ic;
+        r[3] = at(10) * ic;
+        r[5] = at(8) * ic;
     }
 }
+
+// One warp per (mode, class): rows and matrix in FP64, rounded to T; the last class's (the coarsest
+// level's) also in FP64 for the 32 lanes of coarsest().  FP64-pipe bound; once per set-up.
+template <class T, int G, int K>
+__global__ void __launch_bounds__(128) modal_setup_kernel(const __grid_constant__ ModalArgs<T> A, T *coef, double *coef64) {
+    extern __shared__ double rows_all[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    double *rows = rows_all + warp * A.ntype * kRow;
+    const long long job = static_cast<long long>(blockIdx.x) * nw + warp;
+    if (job >= static_cast<long long>(A.nmode) * A.ncls_all) return;
+    const int mode_idx = static_cast<int>(job / A.ncls_all), c = static_cast<int>(job - static_cast<long long>(mode_idx) * A.ncls_all);
+    const double lam = A.lam[mode_idx];
+    T *out = coef + job * A.blk;
+    for (int t = lane; t < A.ntype; t += 32) {
+        double r[kRow];
+        type_row(r, A.raw + (static_cast<long long>(c) * A.ntype + t) * kRawPerLine, lam);
+        for (int i = 0; i < kRow; ++i) {
+            rows[t * kRow + i] = r[i];
+            out[t * kRow + i] = static_cast<T>(r[i]);
+        }
+    }
+    __syncwarp();
+    double col[32];
+    if (lane < G) {
+        dense_column<G>(col, lane, rows, A.ltype, A.ny_m, A.line_base, A.P, ilog2(K));
+        for (int i = 0; i < G; ++i) out[A.ntype * kRow + ((lane / 4) * G + i) * 4 + (lane & 3)] = static_cast<T>(col[i]);
+    }
+    if (c == A.ncls_all - 1) {
+        constexpr int K6 = G * K / 32;
+        double *o = coef64 + static_cast<long long>(mode_idx) * class_values<32>(A.ntype);
+        for (int t = lane; t < A.ntype * kRow; t += 32) o[t] = rows[t];
+        dense_column<32>(col, lane, rows, A.ltype, A.ny_m, A.line_base, A.P, ilog2(K6));
+        for (int i = 0; i < 32; ++i) o[A.ntype * kRow + ((lane / 4) * 32 + i) * 4 + (lane & 3)] = col[i];
+    }
+}
+
+// ---- the tail ---------------------------------------------------------------------------------------
+
+__device__ __forceinline__ void cp_async16(void *dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(static_cast<unsigned>(__cvta_generic_to_shared(dst))), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 template <class T>
 constexpr int modal_threads() { return sizeof(T) == 8 ? 256 : 512; }
 
-// The cycle of one mode (blockIdx.x) and right-hand side (blockIdx.y) on the tail levels.
+// Phase-trace hook for latency studies: compiled out unless SMG_MODAL_TRACE names a device function
+// `void f(int op, int level)` called after each step.
+#ifdef SMG_MODAL_TRACE
+#define SMG_MTRACE(op, l) SMG_MODAL_TRACE((op), (l))
+#else
+#define SMG_MTRACE(op, l) ((void)0)
+#endif
+
+enum : int { OP_START = 0, OP_RELAX = 1, OP_RESTRICT = 2, OP_COARSEST = 3, OP_PROLONG = 4, OP_STORE = 5, OP_TABLES = 6, OP_END = 7 };
+
+// The cycle of one mode and right-hand side on the tail levels, as one loop over its steps, a CTA
+// barrier after each: every kind of step is compiled once (inlined at each place of the cycle it
+// appears, the kernel would not fit the instruction cache).
 template <class T, int G, int K>
 __device__ __forceinline__ void tail_body(const ModalArgs<T> &A, int mode_idx, int rhs, unsigned char *smem) {
     T *sm = reinterpret_cast<T *>(smem);
     const int tid = threadIdx.x, nt = blockDim.x, ln = (tid & 31) % G;
-    const int L = A.L, lt = A.lt, sp = A.sm_pitch;
-    T *tab = sm + A.sm_tab, *zcs = sm + A.sm_zc;
+    const int L = A.L, lt = A.lt, sp = A.sm_pitch, npre = A.npre, npost = A.npost;
+    T *tab = sm + A.sm_tab, *stage = sm + A.sm_stage, *zt = sm + A.sm_zt;
     double *tab64 = reinterpret_cast<double *>(smem + A.sm_tab64);
-    unsigned char *cls = smem + A.sm_cls;
-    const double lam64 = A.lam[mode_idx];
-    const T lam = static_cast<T>(lam64);
+    unsigned short *ltype = reinterpret_cast<unsigned short *>(smem + A.sm_ltype), *ptype = reinterpret_cast<unsigned short *>(smem + A.sm_ptype),
+                   *pcls = reinterpret_cast<unsigned short *>(smem + A.sm_pcls);
+    const T lam = static_cast<T>(A.lam[mode_idx]);
     const int pb = A.plane_base[lt], np = A.plane_base[L - 1] + 1 - pb;
-    for (int i = tid; i < np * kCoefPerPlane; i += nt) zcs[i] = A.zc[pb * kCoefPerPlane + i];
-    for (int i = tid; i < np; i += nt) cls[i] = A.cls[pb + i];
-    constexpr int K6 = G * K / 32;
-    auto build64 = [&](int t0, int n) {
-        for (int e = t0; e < Tab<32, K6>::kEntries; e += n)
-            table_entry<double, 32, K6>(tab64, A.raw64, lam64, A.ny_m, A.line_base, A.P, e);
-    };
-    if (lt < L - 1) build_tables<T, G, K>(tab, A, lt, lam, tid, nt);
-    build64(tid, nt);
-    pdl_wait();
-    __syncthreads();
+    constexpr int K6 = G * K / 32, CH = Chunk<T, K>::CH;
     const long long vec = static_cast<long long>(rhs) * A.nmode + mode_idx;
-    const Rows<T> fg{const_cast<T *>(A.f[lt]) + vec * A.nz[lt] * A.pitch, A.pitch, 0};
-    T *ug = A.u[lt] + vec * A.nz[lt] * A.pitch;
-    auto U = [&](int l) { return Rows<T>{sm + A.sm_u[l], sp, 0}; };
-    auto F = [&](int l) { return Rows<T>{sm + A.sm_f[l], sp, 0}; };
-    auto relax = [&](int l, int colour, int mode) {
-        const int nz = A.nz[l], n = colour ? nz / 2 : (nz + 1) / 2;
-        const T *zl = zcs + (A.plane_base[l] - pb) * kCoefPerPlane;
-        const unsigned char *cl = cls + A.plane_base[l] - pb;
-        const Rows<T> u = U(l);
-        for_planes<G>(n, colour, 2, [&](int z, bool act) {
-            T g[K];
-            const T *tb = tab + cl[z] * Tab<G, K>::kElems;
-            if (l == lt) relax_plane<T, G, K, true, false>(g, u, fg, z, nz, zl + z * kCoefPerPlane, tb, lam, mode, l > 0, ln);
-            else relax_plane<T, G, K, true, true>(g, u, F(l), z, nz, zl + z * kCoefPerPlane, tb, lam, mode, true, ln);
-            if (act) store_row<T, K, true>(u.at(z), g, ln, sp);
-        });
-        __syncthreads();
-    };
-    for (int l = lt; l + 1 < L; ++l) {
-        for (int s = 0; s < A.npre; ++s) {
-            relax(l, 0, s == 0 ? 0 : 2);
-            relax(l, 1, s == 0 ? 1 : 2);
+    const Rows<T> fg{const_cast<T *>(A.f[lt]) + vec * A.nz[lt] * A.pitch, A.pitch, 0, false};
+    const Rows<T> ug{A.u[lt] + vec * A.nz[lt] * A.pitch, A.pitch, 0, false};
+    auto U = [&](int l) { return Rows<T>{sm + A.sm_u[l], sp, 0, true}; };
+    auto F = [&](int l) { return l == lt ? fg : Rows<T>{sm + A.sm_f[l], sp, 0, true}; };
+    int op = OP_START, l = lt, colour = 0, sweep = 0;
+    bool down = true;
+    while (op != OP_END) {
+        const unsigned short *pt = ptype + A.plane_base[l] - pb;
+        auto row = [&](int z) -> const T * { return zt + pt[z] * kCoefPerPlane; };
+        // fetch the classes of the level relaxed after this one
+        int fetch = -1;
+        if (op == OP_START) fetch = lt;
+        else if (op == OP_RELAX && sweep == 0 && colour == (down ? 0 : 1)) fetch = down ? l + 1 : l - 1;
+        else if (op == OP_COARSEST && npost > 0) fetch = L - 2;
+        if (fetch >= lt && fetch < L - 1) {
+            const T *src = A.coef + (static_cast<long long>(mode_idx) * A.ncls_all + A.cls_base[fetch]) * A.blk;
+            for (int i = tid; i < A.ncls[fetch] * A.blk / CH; i += nt) cp_async16(stage + i * CH, src + i * CH);
         }
-        const T *zl = zcs + (A.plane_base[l] - pb) * kCoefPerPlane;
-        const Rows<T> fc = F(l + 1);
-        if (l + 2 < L) build_tables<T, G, K>(tab, A, l + 1, lam, tid, nt);
-        for_planes<G>(A.nz[l + 1], 0, 1, [&](int Z, bool act) {
-            T g[K];
-            if (l == lt) restrict_plane<T, G, K, true, false>(g, U(l), fg, Z, A.nz[l], zl, lam, l > 0, ln);
-            else restrict_plane<T, G, K, true, true>(g, U(l), F(l), Z, A.nz[l], zl, lam, true, ln);
-            if (act) store_row<T, K, true>(fc.at(Z), g, ln, sp);
-        });
-        __syncthreads();
-    }
-    if (tid < 32) {
-        if (lt == L - 1) coarsest<T, G, K, false>(fg.p, ug, A.ny, A.coarse_iters, tab64, tid);
-        else coarsest<T, G, K, true>(sm + A.sm_f[L - 1], sm + A.sm_u[L - 1], A.ny, A.coarse_iters, tab64, tid);
-    }
-    if (lt == L - 1) {
-        // the lines past ny of a one-plane cycle: zero, as the transform expects
-        for (int y = A.ny + tid; y < A.pitch; y += nt) ug[y] = T(0);
-        return;
-    }
-    if (K6 * 32 > A.ny) {  // rows keep zeros past ny
-        T *ul = sm + A.sm_u[L - 1];
-        for (int y = A.ny + tid; y < sp; y += nt) ul[RowMap<T, K>::elem(y)] = T(0);
-    }
-    __syncthreads();
-    for (int l = L - 2; l >= lt; --l) {
-        const bool last = l == lt && A.npost == 0;
-        const T *zl = zcs + (A.plane_base[l] - pb) * kCoefPerPlane;
-        const int nzc = A.nz[l + 1];
-        const Rows<T> u = U(l), uc = U(l + 1);
-        if (A.npost > 0) build_tables<T, G, K>(tab, A, l, lam, tid, nt);
-        for_planes<G>(A.nz[l], 0, 1, [&](int z, bool act) {
-            T g[K], v[K];
-            load_row<T, K, true>(g, u.at(z), ln, sp);
-            if (z & 1) {
-                load_row<T, K, true>(v, uc.at(z >> 1), ln, sp);
-#pragma unroll
-                for (int j = 0; j < K; ++j) g[j] += v[j];
+        // spread the line tables of the next level to be relaxed (nothing reads the present ones now)
+        int tl = -1;
+        if (op == OP_TABLES) tl = lt;
+        else if (op == OP_RESTRICT) tl = l + 1;
+        else if (op == OP_PROLONG && npost > 0) tl = l;
+        if (tl >= 0 && tl < L - 1)
+            spread_tables<T, G, K>(tab, stage, A.ncls[tl], A.blk, ltype, A.ny_m, A.line_base, A.P, A.ntype, tid, nt);
+        if (op == OP_RELAX) {
+            const int nz = A.nz[l], n = colour ? nz / 2 : (nz + 1) / 2;
+            const int mode = (down && sweep == 0) ? colour : 2;
+            const Rows<T> u = U(l), f = F(l);
+            for_planes<T, G, K>(n, colour, 2, f, [&](int z, bool act, T (&g)[K]) {
+                relax_plane<T, G, K, true>(g, u, z, nz, row(z), tab + pcls[pt[z]] * Tab<G, K>::kElems, lam, mode, l > 0, ln);
+                if (act) store_row<T, K, true>(u.at(z), g, ln, sp);
+            });
+            cp_async_wait();
+        } else if (op == OP_RESTRICT) {
+            const Rows<T> fc = F(l + 1), u = U(l), f = F(l);
+            const int nz = A.nz[l], nch = A.pitch / CH;
+            restrict_planes<T, K>(0, A.nz[l + 1], nch, sp / CH, u, f, nz, row, lam, l > 0,
+                                  [&](int Z, int c, const Chunk<T, K> &g) { g.store(fc, Z, c); });
+        } else if (op == OP_COARSEST) {
+            if (lt == L - 1) {  // the only level: straight to global memory
+                if (tid < 32) coarsest<T, G, K, false>(fg.p, ug.p, A.ny, A.coarse_iters, tab64, tid);
+                for (int y = A.ny + tid; y < A.pitch; y += nt) ug.p[y] = T(0);
             } else {
-                const T wm = zl[z * kCoefPerPlane + 6], wp = zl[z * kCoefPerPlane + 7];
-                if (z > 0) {
-                    load_row<T, K, true>(v, uc.at(z / 2 - 1), ln, sp);
-#pragma unroll
-                    for (int j = 0; j < K; ++j) g[j] = fma(wm, v[j], g[j]);
-                }
-                if (z / 2 < nzc) {
-                    load_row<T, K, true>(v, uc.at(z / 2), ln, sp);
-#pragma unroll
-                    for (int j = 0; j < K; ++j) g[j] = fma(wp, v[j], g[j]);
-                }
+                T *ul = sm + A.sm_u[L - 1];
+                if (tid < 32) coarsest<T, G, K, true>(sm + A.sm_f[L - 1], ul, A.ny, A.coarse_iters, tab64, tid);
+                for (int y = A.ny + tid; y < sp; y += nt) ul[RowMap<T, K>::elem(y)] = T(0);
             }
-            if (act) {
-                if (last) store_row<T, K, false>(ug + static_cast<long long>(z) * A.pitch, g, ln, A.pitch);
-                else store_row<T, K, true>(u.at(z), g, ln, sp);
-            }
-        });
-        if (!last) __syncthreads();
-        for (int s = 0; s < A.npost; ++s) {
-            relax(l, 1, 2);
-            relax(l, 0, 2);
+            cp_async_wait();
+        } else if (op == OP_PROLONG || op == OP_STORE) {
+            // u_l += P u_{l+1}; on the last level, with no sweep to follow, straight to global memory
+            const bool add = op == OP_PROLONG, out = l == lt && (!add || npost == 0);
+            const int nzc = add ? A.nz[l + 1] : 1;
+            const Rows<T> u = U(l), uc = U(min(l + 1, L - 1));
+            for_chunks(A.nz[l], (out ? A.pitch : sp) / CH, [&](int z, int c) {
+                Chunk<T, K> g, v, w;
+                g.load(u, z, c);
+                if (add) {
+                    // coarse planes z/2 - 1 and z/2 of an even z (weights zero past the ends); z/2 alone of an odd z
+                    const T *zr = row(z);
+                    v.load(uc, max(z / 2 - 1, 0), c);
+                    w.load(uc, min(z / 2, nzc - 1), c);
+                    const T wm = zr[6], wp = (z & 1) ? T(1) : zr[7];
+#pragma unroll
+                    for (int j = 0; j < CH; ++j) g.t[j] = fma(wp, w.t[j], fma(wm, v.t[j], g.t[j]));
+                }
+                g.store(out ? ug : u, z, c);
+            });
+        } else if (op == OP_TABLES) {
+            // the coarsest plane's table is spread over 32 lanes, from global memory
+            const double *src = A.coef64 + static_cast<long long>(mode_idx) * class_values<32>(A.ntype);
+            spread_tables<double, 32, K6>(tab64, src, 1, 0, ltype, A.ny_m, A.line_base, A.P, A.ntype, tid, nt);
+            if (K6 == 1)
+                for (int i = tid; i < 32; i += nt) {
+                    tab64[Tab<32, K6>::kElems + 2 * i] = i < A.ny ? src[ltype[i] * kRow] : 0.0;
+                    tab64[Tab<32, K6>::kElems + 2 * i + 1] = i < A.ny ? src[ltype[i] * kRow + 1] : 0.0;
+                }
+            pdl_wait();
+        } else {  // OP_START: what does not depend on the right-hand side
+            for (int i = tid; i < A.nptype * kCoefPerPlane; i += nt) zt[i] = A.zt[i];
+            for (int i = tid; i < A.nptype; i += nt) pcls[i] = A.pcls[i];
+            for (int i = tid; i < np; i += nt) ptype[i] = A.ptype[pb + i];
+            for (int i = tid; i < A.sum_ny; i += nt) ltype[i] = A.ltype[i];
+            cp_async_wait();
         }
-    }
-    if (A.npost > 0) {
-        const Rows<T> u = U(lt);
-        for_planes<G>(A.nz[lt], 0, 1, [&](int z, bool act) {
-            T g[K];
-            load_row<T, K, true>(g, u.at(z), ln, sp);
-            if (act) store_row<T, K, false>(ug + static_cast<long long>(z) * A.pitch, g, ln, A.pitch);
-        });
+        __syncthreads();
+        SMG_MTRACE(op, l);
+        // the next step
+        if (op == OP_START) {
+            op = OP_TABLES;
+        } else if (op == OP_TABLES) {
+            op = lt == L - 1 ? OP_COARSEST : OP_RELAX;
+        } else if (op == OP_RELAX) {
+            const int last = down ? 1 : 0;
+            if (colour != last) {
+                colour = last;
+            } else {
+                colour = 1 - last;
+                if (++sweep == (down ? npre : npost)) {
+                    sweep = 0;
+                    if (down) op = OP_RESTRICT;
+                    else if (l == lt) op = OP_STORE;
+                    else op = OP_PROLONG, --l;
+                }
+            }
+        } else if (op == OP_RESTRICT) {
+            ++l;
+            op = l == L - 1 ? OP_COARSEST : OP_RELAX;
+        } else if (op == OP_COARSEST) {
+            down = false;
+            colour = 1;
+            op = l == lt ? OP_END : OP_PROLONG;
+            --l;
+        } else if (op == OP_PROLONG) {
+            if (npost > 0) op = OP_RELAX;
+            else if (l == lt) op = OP_END;
+            else --l;
+        } else {
+            op = OP_END;
+        }
     }
 }
 
@@ -557,7 +760,28 @@ __global__ void __launch_bounds__(modal_threads<T>(), 1) modal_tail_kernel(const
     tail_body<T, G, K>(A, blockIdx.x, blockIdx.y, smem);
 }
 
+// One (system, mode) of a list per CTA; systems that are not being iterated are skipped.
+template <class T, int G, int K>
+__global__ void __launch_bounds__(modal_threads<T>(), 1) modal_tail_batch_kernel(const ModalArgs<T> *__restrict__ args,
+                                                                              const ModalTask *__restrict__ tasks, const int *active) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ ModalArgs<T> A;
+    const ModalTask t = tasks[blockIdx.x];
+    if (active[t.sys] != 1) return;
+    for (unsigned i = threadIdx.x; i < sizeof(ModalArgs<T>) / 4; i += blockDim.x)
+        reinterpret_cast<unsigned *>(&A)[i] = reinterpret_cast<const unsigned *>(args + t.sys)[i];
+    __syncthreads();
+    tail_body<T, G, K>(A, t.mode, 0, smem);
+}
+
 // ---- levels above the tail, over global memory ------------------------------------------------------
+
+// The line tables of level l for one mode, from global memory.
+template <class T, int G, int K>
+__device__ __forceinline__ void level_tables(T *tab, const ModalArgs<T> &A, int l, int mode_idx) {
+    spread_tables<T, G, K>(tab, A.coef + (static_cast<long long>(mode_idx) * A.ncls_all + A.cls_base[l]) * A.blk, A.ncls[l], A.blk,
+                           A.ltype, A.ny_m, A.line_base, A.P, A.ntype, threadIdx.x, blockDim.x);
+}
 
 // The down-sweep of level l with one pre-relaxation (red, black, residual and restriction) for coarse
 // planes Z0 .. Z1-1 of one mode in one CTA: the fine planes 2 Z0 - 2 .. 2 Z1 + 2 the result depends on
@@ -567,32 +791,29 @@ template <class T, int G, int K>
 __global__ void __launch_bounds__(modal_threads<T>(), 1) modal_slab_kernel(const __grid_constant__ ModalArgs<T> A, int l, int nslab) {
     extern __shared__ __align__(16) unsigned char smem[];
     pdl_trigger();
-    T *sm = reinterpret_cast<T *>(smem);
-    const int tid = threadIdx.x, nt = blockDim.x, ln = (tid & 31) % G;
+    constexpr int CH = Chunk<T, K>::CH;
+    const int ln = (threadIdx.x & 31) % G;
     const int sp = A.sm_pitch, nz = A.nz[l], nzc = A.nz[l + 1], mode_idx = blockIdx.y;
     const int Z0 = static_cast<int>(static_cast<long long>(nzc) * blockIdx.x / nslab);
     const int Z1 = static_cast<int>(static_cast<long long>(nzc) * (blockIdx.x + 1) / nslab);
     const int za = max(0, 2 * Z0 - 2), zb = min(nz, 2 * Z1 + 3);
     const int own0 = 2 * Z0, own1 = (Z1 == nzc) ? nz : 2 * Z1;
-    T *tab = sm;
-    T *ur = sm + A.ncls[l] * Tab<G, K>::kElems;
-    const double lam64 = A.lam[mode_idx];
-    const T lam = static_cast<T>(lam64);
-    build_tables<T, G, K>(tab, A, l, lam, tid, nt);
+    T *tab = reinterpret_cast<T *>(smem);
+    T *ur = tab + A.ncls[l] * Tab<G, K>::kElems;
+    const T lam = static_cast<T>(A.lam[mode_idx]);
+    level_tables<T, G, K>(tab, A, l, mode_idx);
     pdl_wait();
     __syncthreads();
     const long long vec = static_cast<long long>(blockIdx.z) * A.nmode + mode_idx;
-    const T *zl = A.zc + A.plane_base[l] * kCoefPerPlane;
-    const unsigned char *cl = A.cls + A.plane_base[l];
-    const Rows<T> f{const_cast<T *>(A.f[l]) + vec * nz * A.pitch, A.pitch, 0}, u{ur, sp, za};
-    const Rows<T> ug{A.u[l] + vec * nz * A.pitch, A.pitch, 0};
+    const unsigned short *pt = A.ptype + A.plane_base[l];
+    auto row = [&](int z) -> const T * { return A.zt + pt[z] * kCoefPerPlane; };
+    const Rows<T> f{const_cast<T *>(A.f[l]) + vec * nz * A.pitch, A.pitch, 0, false}, u{ur, sp, za, true};
+    const Rows<T> ug{A.u[l] + vec * nz * A.pitch, A.pitch, 0, false};
     for (int colour = 0; colour < 2; ++colour) {
         const int first = za + ((za & 1) != colour), end = colour ? min(nz, 2 * Z1 + 2) : zb;
         const int n = end > first ? (end - first + 1) / 2 : 0;
-        for_planes<G>(n, first, 2, [&](int z, bool act) {
-            T g[K];
-            relax_plane<T, G, K, true, false>(g, u, f, z, nz, zl + z * kCoefPerPlane, tab + cl[z] * Tab<G, K>::kElems, lam,
-                                              colour, l > 0, ln);
+        for_planes<T, G, K>(n, first, 2, f, [&](int z, bool act, T (&g)[K]) {
+            relax_plane<T, G, K, true>(g, u, z, nz, row(z), tab + A.pcls[pt[z]] * Tab<G, K>::kElems, lam, colour, l > 0, ln);
             if (act) {
                 store_row<T, K, true>(u.at(z), g, ln, sp);
                 if (z >= own0 && z < own1) store_row<T, K, false>(ug.at(z), g, ln, A.pitch);
@@ -600,12 +821,10 @@ __global__ void __launch_bounds__(modal_threads<T>(), 1) modal_slab_kernel(const
         });
         __syncthreads();
     }
-    const Rows<T> fc{A.fw[l + 1] + vec * nzc * A.pitch, A.pitch, 0};
-    for_planes<G>(Z1 - Z0, Z0, 1, [&](int Z, bool act) {
-        T g[K];
-        restrict_plane<T, G, K, true, false>(g, u, f, Z, nz, zl, lam, l > 0, ln);
-        if (act) store_row<T, K, false>(fc.at(Z), g, ln, A.pitch);
-    });
+    const Rows<T> fc{A.fw[l + 1] + vec * nzc * A.pitch, A.pitch, 0, false};
+    const int nch = A.pitch / CH;
+    restrict_planes<T, K>(Z0, Z1 - Z0, nch, nch, u, f, nz, row, lam, l > 0,
+                          [&](int Z, int c, const Chunk<T, K> &g) { g.store(fc, Z, c); });
 }
 
 // One colour of level l (blockIdx.x: a share of its planes; y: mode; z: right-hand side).
@@ -614,23 +833,21 @@ __global__ void __launch_bounds__(256, 1) modal_relax_kernel(const __grid_consta
     extern __shared__ __align__(16) unsigned char smem[];
     pdl_trigger();
     T *tab = reinterpret_cast<T *>(smem);
-    const int tid = threadIdx.x, ln = (tid & 31) % G, nz = A.nz[l], mode_idx = blockIdx.y;
-    const double lam64 = A.lam[mode_idx];
-    const T lam = static_cast<T>(lam64);
-    build_tables<T, G, K>(tab, A, l, lam, tid, blockDim.x);
+    const int ln = (threadIdx.x & 31) % G, nz = A.nz[l], mode_idx = blockIdx.y;
+    const T lam = static_cast<T>(A.lam[mode_idx]);
+    level_tables<T, G, K>(tab, A, l, mode_idx);
     pdl_wait();
     __syncthreads();
     const long long vec = static_cast<long long>(blockIdx.z) * A.nmode + mode_idx;
-    const T *zl = A.zc + A.plane_base[l] * kCoefPerPlane;
-    const unsigned char *cl = A.cls + A.plane_base[l];
-    const Rows<T> f{const_cast<T *>(A.f[l]) + vec * nz * A.pitch, A.pitch, 0}, u{A.u[l] + vec * nz * A.pitch, A.pitch, 0};
+    const unsigned short *pt = A.ptype + A.plane_base[l];
+    const Rows<T> f{const_cast<T *>(A.f[l]) + vec * nz * A.pitch, A.pitch, 0, false};
+    const Rows<T> u{A.u[l] + vec * nz * A.pitch, A.pitch, 0, false};
     const int n = colour ? nz / 2 : (nz + 1) / 2;
     const int p0 = static_cast<int>(static_cast<long long>(n) * blockIdx.x / gridDim.x);
     const int p1 = static_cast<int>(static_cast<long long>(n) * (blockIdx.x + 1) / gridDim.x);
-    for_planes<G>(p1 - p0, colour + 2 * p0, 2, [&](int z, bool act) {
-        T g[K];
-        relax_plane<T, G, K, false, false>(g, u, f, z, nz, zl + z * kCoefPerPlane, tab + cl[z] * Tab<G, K>::kElems, lam, mode,
-                                           l > 0, ln);
+    for_planes<T, G, K>(p1 - p0, colour + 2 * p0, 2, f, [&](int z, bool act, T (&g)[K]) {
+        relax_plane<T, G, K, false>(g, u, z, nz, A.zt + pt[z] * kCoefPerPlane, tab + A.pcls[pt[z]] * Tab<G, K>::kElems, lam, mode,
+                                    l > 0, ln);
         if (act) store_row<T, K, false>(u.at(z), g, ln, A.pitch);
     });
 }
@@ -639,19 +856,19 @@ template <class T, int G, int K>
 __global__ void __launch_bounds__(256, 1) modal_restrict_kernel(const __grid_constant__ ModalArgs<T> A, int l) {
     pdl_trigger();
     pdl_wait();
-    const int ln = (threadIdx.x & 31) % G, nz = A.nz[l], nzc = A.nz[l + 1], mode_idx = blockIdx.y;
+    const int nz = A.nz[l], nzc = A.nz[l + 1], mode_idx = blockIdx.y;
     const T lam = static_cast<T>(A.lam[mode_idx]);
     const long long vec = static_cast<long long>(blockIdx.z) * A.nmode + mode_idx;
-    const T *zl = A.zc + A.plane_base[l] * kCoefPerPlane;
-    const Rows<T> f{const_cast<T *>(A.f[l]) + vec * nz * A.pitch, A.pitch, 0}, u{A.u[l] + vec * nz * A.pitch, A.pitch, 0};
-    const Rows<T> fc{A.fw[l + 1] + vec * nzc * A.pitch, A.pitch, 0};
+    const unsigned short *pt = A.ptype + A.plane_base[l];
+    auto row = [&](int z) -> const T * { return A.zt + pt[z] * kCoefPerPlane; };
+    const Rows<T> f{const_cast<T *>(A.f[l]) + vec * nz * A.pitch, A.pitch, 0, false};
+    const Rows<T> u{A.u[l] + vec * nz * A.pitch, A.pitch, 0, false};
+    const Rows<T> fc{A.fw[l + 1] + vec * nzc * A.pitch, A.pitch, 0, false};
     const int p0 = static_cast<int>(static_cast<long long>(nzc) * blockIdx.x / gridDim.x);
     const int p1 = static_cast<int>(static_cast<long long>(nzc) * (blockIdx.x + 1) / gridDim.x);
-    for_planes<G>(p1 - p0, p0, 1, [&](int Z, bool act) {
-        T g[K];
-        restrict_plane<T, G, K, false, false>(g, u, f, Z, nz, zl, lam, l > 0, ln);
-        if (act) store_row<T, K, false>(fc.at(Z), g, ln, A.pitch);
-    });
+    const int nch = A.pitch / Chunk<T, K>::CH;
+    restrict_planes<T, K>(p0, p1 - p0, nch, nch, u, f, nz, row, lam, l > 0,
+                          [&](int Z, int c, const Chunk<T, K> &g) { g.store(fc, Z, c); });
 }
 
 }  // namespace smg

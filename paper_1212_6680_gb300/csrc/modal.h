@@ -3,6 +3,8 @@
 
 #include <cuda_runtime.h>
 
+#include <vector>
+
 #include "smg_internal.h"
 
 namespace smg {
@@ -11,33 +13,44 @@ constexpr int kMaxZLevels = 13;   // nz <= 4096
 
 // The V-cycle of one system on its mode grids, as the kernels read it (T: float or double).
 // "Tail" levels are the z-levels lt .. L-1, which one CTA per mode runs in shared memory.
+//
+// Coefficients.  Planes of a level with equal 2D hierarchies form a class (plane_classes; two a level
+// here: the planes away from the end, and the last).  Lines whose coefficients agree in every class
+// form a line type (about five per 2D level: next to the ends, and even and odd between).  For each
+// mode and class, modal_setup_kernel forms once the kRow multipliers of every line type and the G x G
+// matrix of the y-cycle below the levels a lane holds: `blk` values, which the kernels spread over
+// their lines.
 template <class T>
 struct ModalArgs {
     int nmode, ny, pitch;      // x-modes, lines, and lines per plane in global memory (ny rounded up to 4)
     int L, lt;                 // z-levels; first tail level
     int P, sum_ny;             // 2D levels and their lines in all
     int npre, npost, coarse_iters;
+    int ntype, nptype, ncls_all, blk;  // line types, plane types, classes of all levels, values per class
     int ny_m[kMaxPlaneLevels], line_base[kMaxPlaneLevels];
     int nz[kMaxZLevels];       // planes of each z-level
     int plane_base[kMaxZLevels];
-    int cls_base[kMaxZLevels]; // first table of the level in `raw` (tables of one level are contiguous)
+    int cls_base[kMaxZLevels]; // first class of the level
     int ncls[kMaxZLevels];     // plane classes of the level
     int sm_u[kMaxZLevels], sm_f[kMaxZLevels];  // shared-memory offsets (elements of T) of the tail levels
     int sm_pitch;              // lines per plane in shared memory
-    int sm_tab, sm_zc;         // offsets (elements of T) of the line tables and the plane coefficients
-    int sm_tab64, sm_cls;      // offsets (bytes) of the coarsest plane's FP64 table and the class indices
+    int sm_tab, sm_stage, sm_zt;         // offsets (elements of T): line tables, staged classes, plane types
+    int sm_tab64, sm_ltype, sm_ptype, sm_pcls;  // offsets (bytes)
     const T *f[kMaxZLevels];   // right-hand sides and iterates in global memory: [rhs][mode][plane][pitch],
     T *u[kMaxZLevels];         // levels 0 .. lt
     T *fw[kMaxZLevels];        // f, writable (levels 1 .. lt)
-    const T *zc;               // [planes of all levels][8]
-    const T *raw;              // [tables][sum_ny][16] line coefficients (raw_line_table)
-    const double *raw64;       // the coarsest level's table in FP64
-    const unsigned char *cls;  // [planes of all levels] plane class within the level
+    const T *zt;               // [plane types][8] plane coefficients
+    const unsigned short *ptype;  // [planes of all levels] plane type
+    const unsigned short *pcls;   // [plane types] class within the level
+    const unsigned short *ltype;  // [sum_ny] line type
+    const T *coef;             // [mode][class][blk]
+    const double *coef64;      // [mode][blk64]: the coarsest level's class in FP64, 32 lanes
     const double *lam;         // [nmode] eigenvalues of the x-line Laplacian
+    const double *raw;         // [class][ntype][kRawPerLine]: what the multipliers are formed from
 };
 
-// Line tables of one plane class: 16 values a line (raw_line_table in modal_host.cpp).
-constexpr int kRawPerLine = 16;
+constexpr int kRawPerLine = 14;  // raw_line in modal.cu
+constexpr int kRow = 8;          // multipliers of a line type
 
 // Lanes per plane and lines per lane for planes of ny lines.
 struct ModalConfig {
@@ -45,24 +58,50 @@ struct ModalConfig {
 };
 ModalConfig modal_config(int ny, bool f64);
 
-// Shared memory the tail kernel may use, and its threads.
+// Shared memory the tail kernel may use.
 constexpr size_t kModalSmem = 227 * 1024 - 2048;
+
+// The transforms of one system's x-lines into mode space and back (modal.cu).
+struct SineArgs {
+    int nx, ny, nz, pitch;   // pitch: lines per plane of the mode vectors (lines ny .. pitch-1 are zero)
+    int nh;                  // odd modes, and pairs of points: ceil(nx / 2)
+    int hp;                  // order of the stored matrices (nh rounded up to 32)
+    const void *mat;         // [4][hp][hp]: by point odd, even; by mode odd, even
+};
+
+// One system's mode-space cycle as planned on the host: its kernel arguments, the bytes its modes share
+// and what else it needs on the device (set by modal_place).
+template <class T>
+struct ModalHost {
+    ModalArgs<T> a;
+    ModalConfig cfg{16, 8};
+    size_t smem = 0;                   // tail kernel
+    std::vector<unsigned char> shared; // raw, lam, zt, ptype, pcls, ltype
+    size_t at[6] = {0};
+    size_t coef_values = 0, coef64_values = 0, vec_bytes = 0;
+    std::vector<size_t> vec_off;       // f and u of levels 0 .. lt
+};
+template <class T>
+int modal_plan(ModalHost<T> &h, const HostHierarchy &H, ModalConfig cfg, int nb, int npre, int npost, int coarse_iters);
+template <class T>
+void modal_place(ModalHost<T> &h, unsigned char *shared, T *coef, double *coef64, unsigned char *vec);
+template <class T>
+std::vector<T> sine_matrices(int nx);
+// Threads of the tail kernel for systems that need smem bytes when ctas of them are to run: the kernel
+// takes 128 registers a thread, so 512 threads fill an SM; with more CTAs than SMs the SM is shared by as
+// many as the shared memory allows, else one CTA takes it whole (as far as its planes fill it).
+int modal_tail_threads(size_t smem, long long ctas, int num_sms, int most, int planes, int G);
 
 struct ModalPlan {
     bool f64 = false;
-    int nx = 0, ny = 0, nz = 0, nb = 0, nh = 0;  // nh: odd modes (ceil(nx / 2))
-    int npre = 1, npost = 0, coarse_iters = 1;
-    ModalConfig cfg{8, 16};
-    size_t smem = 0;              // tail kernel
-    int threads = 0;
-    int lt = 0, L = 0, pitch = 0;
-    ModalArgs<float> a32;         // host copies of the kernel arguments
-    ModalArgs<double> a64;
+    int nb = 0, threads = 0, num_sms = 0;
+    ModalHost<float> h32;
+    ModalHost<double> h64;
+    SineArgs sine{};
     void *d_args = nullptr;
     void *d_buf = nullptr;        // mode-space vectors
     void *d_tab = nullptr;        // coefficients
     void *d_sin = nullptr;        // transform matrices
-    int hp = 0;                   // their padded order
 };
 
 // Tables and buffers for nb right-hand sides; 0, or a cudaError_t.
@@ -76,17 +115,40 @@ cudaError_t modal_transform_in(const ModalPlan &p, int nb, const double *f0, cud
 cudaError_t modal_cycle(const ModalPlan &p, int nb, cudaStream_t st, long long &launches);
 cudaError_t modal_transform_out(const ModalPlan &p, int nb, Prec type, void *u0, cudaStream_t st, long long &launches);
 
+// Many systems at once (batched.cu), FP32: their transforms and tails as one launch each, the CTAs taken
+// from lists of (system, tile) and (system, mode); systems whose active flag is not 1 are skipped.
+struct SineJob {
+    SineArgs g;
+    const double *in;      // physical right-hand side
+    float *fh;             // mode-space right-hand side and result
+    const float *uh;
+    float *out;            // physical result
+};
+struct SineTile {
+    int sys, line_tile, mode_tile;
+};
+int sine_line_tiles(const SineArgs &g);
+int sine_mode_tiles(const SineArgs &g);
+cudaError_t launch_sine_in_batch(const SineJob *jobs, const SineTile *tiles, int ntiles, const int *active, cudaStream_t st);
+cudaError_t launch_sine_out_batch(const SineJob *jobs, const SineTile *tiles, int ntiles, const int *active, cudaStream_t st);
+struct ModalTask {
+    int sys, mode;
+};
+cudaError_t launch_modal_prolong(const ModalArgs<float> &a, int l, int nb, cudaStream_t st);
+
 // Kernels of one configuration (modal_inst.cu).
 template <class T>
 struct ModalKernels {
+    cudaError_t (*setup)(const ModalArgs<T> &a, T *coef, double *coef64, cudaStream_t st);
     cudaError_t (*tail)(const ModalArgs<T> *d_args, int nmode, int nb, int threads, size_t smem, cudaStream_t st);
+    cudaError_t (*tail_batch)(const ModalArgs<T> *d_args, const ModalTask *tasks, int ntasks, const int *active, int threads,
+                              size_t smem, cudaStream_t st);
     cudaError_t (*slab)(const ModalArgs<T> &a, int l, int nb, cudaStream_t st);
     cudaError_t (*relax)(const ModalArgs<T> &a, int l, int colour, int mode, int nb, cudaStream_t st);
     cudaError_t (*restrict_)(const ModalArgs<T> &a, int l, int nb, cudaStream_t st);
-    int table_elems;     // of one plane class (elements of T)
-    int table64_elems;   // of the coarsest plane (doubles)
-    int max_threads;
     bool (*slab_fits)(const ModalArgs<T> &a, int l);
+    int table_elems;     // a class's line table in shared memory (elements of T)
+    int max_threads;
 };
 template <class T>
 const ModalKernels<T> &modal_kernels(ModalConfig c);

@@ -12,10 +12,31 @@ using T = float;
 using T = double;
 #endif
 
+cudaError_t setup(const ModalArgs<T> &a, T *coef, double *coef64, cudaStream_t st) {
+    const long long jobs = static_cast<long long>(a.nmode) * a.ncls_all;
+    const size_t smem = sizeof(double) * 4 * a.ntype * kRow;
+    cudaError_t e = raise_smem_attr(reinterpret_cast<const void *>(&modal_setup_kernel<T, G, K>), smem);
+    if (e != cudaSuccess) return e;
+    modal_setup_kernel<T, G, K><<<static_cast<unsigned>((jobs + 3) / 4), 128, smem, st>>>(a, coef, coef64);
+    return cudaGetLastError();
+}
+
 cudaError_t tail(const ModalArgs<T> *d_args, int nmode, int nb, int threads, size_t smem, cudaStream_t st) {
     cudaError_t e = raise_smem_attr(reinterpret_cast<const void *>(&modal_tail_kernel<T, G, K>), smem);
     if (e != cudaSuccess) return e;
     return launch_pdl(modal_tail_kernel<T, G, K>, dim3(nmode, nb), dim3(threads), smem, st, d_args);
+}
+
+cudaError_t tail_batch(const ModalArgs<T> *d_args, const ModalTask *tasks, int ntasks, const int *active, int threads, size_t smem,
+                       cudaStream_t st) {
+#if SMG_MT == 0
+    cudaError_t e = raise_smem_attr(reinterpret_cast<const void *>(&modal_tail_batch_kernel<T, G, K>), smem);
+    if (e != cudaSuccess) return e;
+    modal_tail_batch_kernel<T, G, K><<<ntasks, threads, smem, st>>>(d_args, tasks, active);
+    return cudaGetLastError();
+#else
+    return cudaErrorNotSupported;  // the batched solver runs FP32 cycles
+#endif
 }
 
 // The slab's coarse planes: as many as its red planes (the slab's share + 3) fit in one pass over the
@@ -64,6 +85,6 @@ cudaError_t restrict_(const ModalArgs<T> &a, int l, int nb, cudaStream_t st) {
 #define SMG_CAT(a, b, c, d) SMG_CAT_(a, b, c, d)
 extern const ModalKernels<T> SMG_CAT(modal_kernels_, SMG_MT, SMG_MG, SMG_MK);
 const ModalKernels<T> SMG_CAT(modal_kernels_, SMG_MT, SMG_MG, SMG_MK) = {
-    tail, slab, relax, restrict_, Tab<G, K>::kElems, Tab<32, G * K / 32>::kElems, modal_threads<T>(), slab_fits};
+    setup, tail, tail_batch, slab, relax, restrict_, slab_fits, Tab<G, K>::kElems, modal_threads<T>()};
 
 }  // namespace smg
