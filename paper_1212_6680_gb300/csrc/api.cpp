@@ -116,7 +116,7 @@ struct smg_ctx {
     bool modal_now = false;         // the level vectors in place are that cycle's
     ModalPlan mp;
     // Krylov vectors (one right-hand side)
-    double *d_r = nullptr, *d_p = nullptr, *d_q = nullptr, *d_dr = nullptr;
+    double *d_r = nullptr, *d_p = nullptr, *d_q = nullptr;
     double *d_bh = nullptr, *d_xh = nullptr;  // device copies for host-pointer calls
     KrylovWork kw;
     KrylovScalars *h_sc = nullptr;  // pinned host mirror
@@ -706,7 +706,6 @@ int ensure_krylov(smg_ctx *h) {
     SMG_CUDA(cudaMalloc(&h->d_r, b));
     SMG_CUDA(cudaMalloc(&h->d_p, b));
     SMG_CUDA(cudaMalloc(&h->d_q, b));
-    SMG_CUDA(cudaMalloc(&h->d_dr, b));
     SMG_CUDA(cudaMalloc(&h->kw.sc, sizeof(KrylovScalars)));
     SMG_CUDA(cudaMalloc(&h->kw.part, sizeof(double) * 2 * 2 * kMaxReduceBlocks));
     SMG_CUDA(cudaMalloc(&h->kw.counter, sizeof(unsigned)));
@@ -758,7 +757,7 @@ bool ensure_solve_graph(smg_ctx *h, void *f0, void *u0, Prec kp, void *f0k, bool
         ok = cudaStreamBeginCaptureToGraph(h->gs, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed) == cudaSuccess;
         if (ok) {
             bool launched = ident || run_cycle(h, 1, f0, u0, h->gs) == SMG_OK;
-            launched = launched && kry_iteration_tail(kp, h->nx, h->ny, h->nz, u0, x, h->d_r, h->d_p, h->d_q, h->d_dr,
+            launched = launched && kry_iteration_tail(kp, h->nx, h->ny, h->nz, u0, x, h->d_r, h->d_p, h->d_q,
                                                       f0k, h->kw, h->gs, cond, 1) == cudaSuccess;
             h->launches += 4;
             cudaGraph_t out = nullptr;
@@ -881,7 +880,7 @@ int krylov_device(smg_ctx *h, int variant, const double *b, double *x, double to
         }
         {
             RegionTimer rt(h, ls, 4, 0.0);
-            SMG_CUDA(kry_iteration_tail(kp, h->nx, h->ny, h->nz, u0, x, h->d_r, h->d_p, h->d_q, h->d_dr, f0k, h->kw, ls));
+            SMG_CUDA(kry_iteration_tail(kp, h->nx, h->ny, h->nz, u0, x, h->d_r, h->d_p, h->d_q, f0k, h->kw, ls));
         }
         h->launches += 4;
         k += 1;
@@ -1380,7 +1379,6 @@ int smg_destroy(smg_handle h) {
     cudaFree(h->d_r);
     cudaFree(h->d_p);
     cudaFree(h->d_q);
-    cudaFree(h->d_dr);
     cudaFree(h->d_bh);
     cudaFree(h->d_xh);
     cudaFree(h->kw.sc);

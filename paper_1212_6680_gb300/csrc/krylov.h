@@ -7,14 +7,13 @@
 
 namespace smg {
 
-constexpr int kMaxReduceBlocks = 1216;  // CTAs of a reduction kernel on HBM-resident vectors (8 x 152 SMs)
-constexpr int kReduceBlocks = 304;      // CTAs of a reduction kernel on L2-resident vectors (2 x 152 SMs)
+constexpr int kMaxReduceBlocks = 152;  // CTAs of a reduction kernel (one per SM)
 
 // Scalars of Algorithm 1 kept on the device between kernels.
 struct KrylovScalars {
     double rho;       // (s_k, r_k)
     double rho_prev;  // (s_{k-1}, r_{k-1})
-    double sdr;       // (s_k, r_k - r_{k-1})
+    double sdr;       // (s_k, r_k - r_{k-1}) = -alpha_{k-1} (s_k, A p_{k-1})
     double beta, pq, alpha;
     double rr;        // ||r_k||^2 (recurrence)
     double bb;        // ||b||^2
@@ -39,7 +38,6 @@ struct KrylovWork {
     bool fused = false;            // the iteration tail as one cooperative kernel where it fits
 };
 
-int reduction_blocks(long long n);
 cudaError_t kry_init_residual(Prec st_prec, int nx, int ny, int nz, const double *b, const double *x, double *r,
                               void *f0, KrylovWork &w, cudaStream_t st);
 cudaError_t kry_true_residual(int nx, int ny, int nz, const double *b, const double *x, KrylovWork &w,
@@ -49,7 +47,7 @@ cudaError_t kry_true_residual(int nx, int ny, int nz, const double *b, const dou
 // graph that repeats the iteration: 1 (run another) while status == 0, rr > tol2 bb and
 // it < maxit, else 0.
 cudaError_t kry_iteration_tail(Prec st_prec, int nx, int ny, int nz, const void *s, double *x, double *r, double *p,
-                               double *q, double *dr, void *f0, KrylovWork &w, cudaStream_t st,
+                               double *q, void *f0, KrylovWork &w, cudaStream_t st,
                                cudaGraphConditionalHandle cond = 0, int use_cond = 0);
 
 }  // namespace smg

@@ -38,39 +38,56 @@ __device__ __forceinline__ DSum shfl_down_dsum(const DSum &v, int o) {
 }
 
 // Inner products: every thread accumulates its (about 2N / (threads in the grid)) products with
-// FMA, the block adds the thread partials pairwise (warp shuffles, then one warp over the warp
-// sums), and the last block to finish combines the block partials with error-free TwoSum
-// (compensated summation).  FP64 work per element stays at one FMA, which matters on GB300
-// where an FP64 operation costs as much SM time as dozens of FP32 ones.
+// FMA, the block adds the thread partials through shared memory, and the last block to finish
+// combines the block partials with error-free TwoSum (compensated summation).  FP64 work per
+// element stays at one FMA, which matters on GB300 where a warp's FP64 instruction holds its
+// sub-partition's unit for about 64 cycles however few lanes it serves.  That prices the reductions
+// themselves: a shuffle tree in every warp is 5 instructions a warp and value, and compensated sums
+// 6 a term.  So the grid is one CTA of up to 1024 threads per SM (152 partials instead of 608), a
+// block folds its partials four to one on full warps (36 instructions a value instead of 165), and
+// one warp per value does the compensated pass.  128^3, of the 122 us of an iteration's four kernels:
+// see reduction_grid().
+constexpr int kMaxThreads = 1024;
+
 template <int NV>
 __device__ __forceinline__ void block_reduce_plain(double (&v)[NV]) {
-    __shared__ double sh[NV][32];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    __shared__ double sh[NV][kMaxThreads];
+    const int t = threadIdx.x;
+    int n = blockDim.x;
+    while (n > 32) {
+        const int f = (n % 4 == 0 && n / 4 >= 32) ? 4 : 2, m = n / f;  // blockDim.x is a multiple of 64, or 32
+        if (t < n)
 #pragma unroll
-    for (int k = 0; k < NV; ++k)
-        for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
-    if (lane == 0)
-        for (int k = 0; k < NV; ++k) sh[k][w] = v[k];
-    __syncthreads();
-    if (w == 0) {
+            for (int k = 0; k < NV; ++k) sh[k][t] = v[k];
+        __syncthreads();
+        if (t < m)
 #pragma unroll
-        for (int k = 0; k < NV; ++k) {
-            v[k] = (lane < nw) ? sh[k][lane] : 0.0;
-            for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
-        }
+            for (int k = 0; k < NV; ++k) {
+                double a = v[k] + sh[k][t + m];
+                if (f == 4) a += sh[k][t + 2 * m] + sh[k][t + 3 * m];
+                v[k] = a;
+            }
+        n = m;
+        __syncthreads();
     }
-    __syncthreads();
+    if (t < 32)
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int k = 0; k < NV; ++k) {
+                const double w = __shfl_down_sync(0xffffffffu, v[k], o);
+                v[k] += (t + o < n) ? w : 0.0;
+            }
 }
 
 // Write this block's partials; the last block to finish sums all of them (compensated) into
-// tot[].  Returns true in every thread of the last block.
+// tot[] (thread 0's is the sum).  Returns true in every thread of the last block.
 template <int NV>
 __device__ __forceinline__ bool grid_reduce(double (&v)[NV], DSum *part, unsigned *counter, double (&tot)[NV]) {
     __shared__ bool last;
     __shared__ double res[NV];
     block_reduce_plain<NV>(v);
     if (threadIdx.x == 0) {
-        for (int k = 0; k < NV; ++k) part[static_cast<size_t>(blockIdx.x) * NV + k] = DSum{v[k], 0.0};
+        for (int k = 0; k < NV; ++k) part[static_cast<size_t>(blockIdx.x) * NV + k].s = v[k];
         __threadfence();
         const unsigned t = atomicAdd(counter, 1u);
         last = (t == gridDim.x - 1);
@@ -78,28 +95,39 @@ __device__ __forceinline__ bool grid_reduce(double (&v)[NV], DSum *part, unsigne
     __syncthreads();
     if (!last) return false;
     __threadfence();
-    if (threadIdx.x < 32) {
-        const int lane = threadIdx.x;
-        for (int k = 0; k < NV; ++k) {
-            DSum w{0.0, 0.0};
-            for (unsigned b = lane; b < gridDim.x; b += 32) {
-                const volatile DSum *vp = &part[static_cast<size_t>(b) * NV + k];
-                two_sum_acc(w, vp->s);
-            }
-            for (int o = 16; o > 0; o >>= 1) w = dsum_combine(w, shfl_down_dsum(w, o));
-            if (lane == 0) res[k] = w.s + w.c;
-        }
-        if (lane == 0) *counter = 0u;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    for (int k = w; k < NV; k += nw) {
+        DSum a{0.0, 0.0};
+        for (unsigned b = lane; b < gridDim.x; b += 32) two_sum_acc(a, __ldcg(&part[static_cast<size_t>(b) * NV + k].s));
+        for (int o = 16; o > 0; o >>= 1) a = dsum_combine(a, shfl_down_dsum(a, o));
+        if (lane == 0) res[k] = a.s + a.c;
     }
     __syncthreads();
+#pragma unroll
     for (int k = 0; k < NV; ++k) tot[k] = res[k];
+    if (threadIdx.x == 0) *counter = 0u;
     return true;
 }
 
+// n / d for 0 <= n < 2^31 by a multiplication (Granlund and Montgomery's invariant division).
+struct FastDiv {
+    unsigned mul, shift, d;
+};
+inline FastDiv fast_div(int d) {
+    unsigned s = 0;
+    while ((1ull << s) < static_cast<unsigned long long>(d)) ++s;
+    return FastDiv{static_cast<unsigned>(((1ull << 32) * ((1ull << s) - d)) / d + 1), s, static_cast<unsigned>(d)};
+}
+__device__ __forceinline__ int div_by(int n, const FastDiv &f) {
+    return static_cast<int>((__umulhi(static_cast<unsigned>(n), f.mul) + static_cast<unsigned>(n)) >> f.shift);
+}
+struct GridDiv {  // rows of nx values (or nx / 4 chunks), ny rows a plane
+    FastDiv row, plane;
+};
+
 __device__ __forceinline__ double stencil7(const double *__restrict__ u, long long i, int x, int y, int z, int nx,
                                            int ny, int nz, long long np) {
-    double nb = 0.0;
-    if (x > 0) nb += u[i - 1];
+    double nb = (x > 0) ? u[i - 1] : 0.0;
     if (x < nx - 1) nb += u[i + 1];
     if (y > 0) nb += u[i - nx];
     if (y < ny - 1) nb += u[i + nx];
@@ -128,14 +156,14 @@ __device__ __forceinline__ void finish_update(KrylovScalars *sc, double rr, cuda
 
 // r = b - A x ; f0 = (S) r ; rr = ||r||^2 ; bb = ||b||^2 ; restart = 1.
 template <class S>
-__global__ void k_init_residual(int nx, int ny, int nz, const double *__restrict__ b, const double *__restrict__ x,
+__global__ void __launch_bounds__(kMaxThreads) k_init_residual(int nx, int ny, int nz, const double *__restrict__ b, const double *__restrict__ x,
                                 double *__restrict__ r, S *__restrict__ f0, KrylovScalars *sc, DSum *part,
-                                unsigned *counter) {
+                                unsigned *counter, GridDiv gd) {
     const long long np = static_cast<long long>(nx) * ny;
     double a0 = 0.0, a1 = 0.0;
-    const int npi = nx * ny, n32 = npi * nz;
+    const int n32 = nx * ny * nz;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n32; i += gridDim.x * blockDim.x) {
-        const int zz = i / npi, ip = i - zz * npi, yy = ip / nx, xx = ip - yy * nx;
+        const int row = div_by(i, gd.row), xx = i - row * nx, zz = div_by(row, gd.plane), yy = row - zz * ny;
         const double bi = b[i];
         const double ri = bi - stencil7(x, i, xx, yy, zz, nx, ny, nz, np);
         r[i] = ri;
@@ -154,13 +182,13 @@ __global__ void k_init_residual(int nx, int ny, int nz, const double *__restrict
 }
 
 // tt = ||b - A x||^2 (true residual).
-__global__ void k_true_residual(int nx, int ny, int nz, const double *__restrict__ b, const double *__restrict__ x,
-                                KrylovScalars *sc, DSum *part, unsigned *counter) {
+__global__ void __launch_bounds__(kMaxThreads) k_true_residual(int nx, int ny, int nz, const double *__restrict__ b, const double *__restrict__ x,
+                                KrylovScalars *sc, DSum *part, unsigned *counter, GridDiv gd) {
     const long long np = static_cast<long long>(nx) * ny;
     double a0 = 0.0;
-    const int npi = nx * ny, n32 = npi * nz;
+    const int n32 = nx * ny * nz;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n32; i += gridDim.x * blockDim.x) {
-        const int zz = i / npi, ip = i - zz * npi, yy = ip / nx, xx = ip - yy * nx;
+        const int row = div_by(i, gd.row), xx = i - row * nx, zz = div_by(row, gd.plane), yy = row - zz * ny;
         const double ri = b[i] - stencil7(x, i, xx, yy, zz, nx, ny, nz, np);
         a0 = fma(ri, ri, a0);
     }
@@ -169,10 +197,11 @@ __global__ void k_true_residual(int nx, int ny, int nz, const double *__restrict
     if (grid_reduce<1>(v, part, counter, tot) && threadIdx.x == 0) sc->tt = tot[0];
 }
 
-// rho = (s, r), sdr = (s, r_k - r_{k-1}); beta by eq. (1), eq. (2) or 0.
+// rho = (s, r), sdr = (s, r_k - r_{k-1}); beta by eq. (1), eq. (2) or 0.  r_k - r_{k-1} = -alpha A p of the
+// step before, still in q: eq. (2)'s extra vector needs no storage of its own.
 template <class S>
-__global__ void k_dots_beta(long long n, const S *__restrict__ s, const double *__restrict__ r,
-                            const double *__restrict__ dr, KrylovScalars *sc, DSum *part, unsigned *counter) {
+__global__ void __launch_bounds__(kMaxThreads) k_dots_beta(long long n, const S *__restrict__ s, const double *__restrict__ r,
+                            const double *__restrict__ q, KrylovScalars *sc, DSum *part, unsigned *counter) {
     pdl_trigger();
     pdl_wait();
     const int variant = sc->variant;
@@ -182,30 +211,30 @@ __global__ void k_dots_beta(long long n, const S *__restrict__ s, const double *
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n32; i += gridDim.x * blockDim.x) {
         const double si = ldv<double>(s + i);
         a0 = fma(si, r[i], a0);
-        if (need_sdr) a1 = fma(si, dr[i], a1);
+        if (need_sdr) a1 = fma(si, q[i], a1);
     }
     double v[2] = {a0, a1};
     double tot[2];
     if (grid_reduce<2>(v, part, counter, tot) && threadIdx.x == 0) {
-        const double rho = tot[0];
+        const double rho = tot[0], sdr = -sc->alpha * tot[1];
         double beta = 0.0;
         if (sc->restart == 0 && variant != 2) {
             if (sc->rho_prev == 0.0) {
                 sc->status = -4;
             } else {
-                beta = (variant == 0) ? rho / sc->rho_prev : tot[1] / sc->rho_prev;
+                beta = (variant == 0) ? rho / sc->rho_prev : sdr / sc->rho_prev;
             }
         }
         if (!isfinite(rho) || !isfinite(beta)) sc->status = -6;
         sc->rho = rho;
-        sc->sdr = tot[1];
+        sc->sdr = sdr;
         sc->beta = beta;
     }
 }
 
 // p = s + beta p
 template <class S>
-__global__ void k_update_p(long long n, const S *__restrict__ s, double *__restrict__ p, const KrylovScalars *sc) {
+__global__ void __launch_bounds__(kMaxThreads) k_update_p(long long n, const S *__restrict__ s, double *__restrict__ p, const KrylovScalars *sc) {
     pdl_trigger();
     pdl_wait();
     const double beta = sc->beta;
@@ -217,15 +246,15 @@ __global__ void k_update_p(long long n, const S *__restrict__ s, double *__restr
 }
 
 // q = A p ; pq = (p, q) ; alpha = rho / pq
-__global__ void k_spmv_alpha(int nx, int ny, int nz, const double *__restrict__ p, double *__restrict__ q,
-                             KrylovScalars *sc, DSum *part, unsigned *counter) {
+__global__ void __launch_bounds__(kMaxThreads) k_spmv_alpha(int nx, int ny, int nz, const double *__restrict__ p, double *__restrict__ q,
+                             KrylovScalars *sc, DSum *part, unsigned *counter, GridDiv gd) {
     pdl_trigger();
     pdl_wait();
     const long long np = static_cast<long long>(nx) * ny;
     double a0 = 0.0;
-    const int npi = nx * ny, n32 = npi * nz;
+    const int n32 = nx * ny * nz;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n32; i += gridDim.x * blockDim.x) {
-        const int zz = i / npi, ip = i - zz * npi, yy = ip / nx, xx = ip - yy * nx;
+        const int row = div_by(i, gd.row), xx = i - row * nx, zz = div_by(row, gd.plane), yy = row - zz * ny;
         const double qi = stencil7(p, i, xx, yy, zz, nx, ny, nz, np);
         q[i] = qi;
         a0 = fma(p[i], qi, a0);
@@ -244,23 +273,20 @@ __global__ void k_spmv_alpha(int nx, int ny, int nz, const double *__restrict__ 
     }
 }
 
-// x += alpha p ; r_new = r - alpha q ; dr = r_new - r ; r = r_new ; f0 = (S) r_new ; rr = ||r_new||^2
+// x += alpha p ; r_new = r - alpha q ; r = r_new ; f0 = (S) r_new ; rr = ||r_new||^2
 template <class S>
-__global__ void k_update_xr(long long n, double *__restrict__ x, const double *__restrict__ p, double *__restrict__ r,
-                            const double *__restrict__ q, double *__restrict__ dr, S *__restrict__ f0,
+__global__ void __launch_bounds__(kMaxThreads) k_update_xr(long long n, double *__restrict__ x, const double *__restrict__ p, double *__restrict__ r,
+                            const double *__restrict__ q, S *__restrict__ f0,
                             KrylovScalars *sc, DSum *part, unsigned *counter, cudaGraphConditionalHandle cond,
                             int use_cond) {
     pdl_trigger();
     pdl_wait();
     const double alpha = sc->alpha;
-    const bool want_dr = (sc->variant == 1);
     double a0 = 0.0;
     const int n32 = static_cast<int>(n);
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n32; i += gridDim.x * blockDim.x) {
         x[i] = fma(alpha, p[i], x[i]);
-        const double ro = r[i];
-        const double rn = fma(-alpha, q[i], ro);
-        if (want_dr) dr[i] = rn - ro;
+        const double rn = fma(-alpha, q[i], r[i]);
         r[i] = rn;
         if (f0 != nullptr) stv<S, double>(f0 + i, rn);
         a0 = fma(rn, rn, a0);
@@ -311,8 +337,8 @@ template <> __device__ __forceinline__ void sts4<__nv_bfloat16>(__nv_bfloat16 *p
 }
 
 template <class S>
-__global__ void k_dots_beta4(int nc, const S *__restrict__ s, const double *__restrict__ r,
-                             const double *__restrict__ dr, KrylovScalars *sc, DSum *part, unsigned *counter) {
+__global__ void __launch_bounds__(kMaxThreads) k_dots_beta4(int nc, const S *__restrict__ s, const double *__restrict__ r,
+                             const double *__restrict__ q, KrylovScalars *sc, DSum *part, unsigned *counter) {
     pdl_trigger();
     pdl_wait();
     const int variant = sc->variant;
@@ -327,7 +353,7 @@ __global__ void k_dots_beta4(int nc, const S *__restrict__ s, const double *__re
         for (int k = 0; k < 4; ++k) a0 = fma(sv[k], rv[k], a0);
         if (need_sdr) {
             double dv[4];
-            ld4(dv, dr + 4 * c);
+            ld4(dv, q + 4 * c);
 #pragma unroll
             for (int k = 0; k < 4; ++k) a1 = fma(sv[k], dv[k], a1);
         }
@@ -335,24 +361,24 @@ __global__ void k_dots_beta4(int nc, const S *__restrict__ s, const double *__re
     double v[2] = {a0, a1};
     double tot[2];
     if (grid_reduce<2>(v, part, counter, tot) && threadIdx.x == 0) {
-        const double rho = tot[0];
+        const double rho = tot[0], sdr = -sc->alpha * tot[1];
         double beta = 0.0;
         if (sc->restart == 0 && variant != 2) {
             if (sc->rho_prev == 0.0) {
                 sc->status = -4;
             } else {
-                beta = (variant == 0) ? rho / sc->rho_prev : tot[1] / sc->rho_prev;
+                beta = (variant == 0) ? rho / sc->rho_prev : sdr / sc->rho_prev;
             }
         }
         if (!isfinite(rho) || !isfinite(beta)) sc->status = -6;
         sc->rho = rho;
-        sc->sdr = tot[1];
+        sc->sdr = sdr;
         sc->beta = beta;
     }
 }
 
 template <class S>
-__global__ void k_update_p4(int nc, const S *__restrict__ s, double *__restrict__ p, const KrylovScalars *sc) {
+__global__ void __launch_bounds__(kMaxThreads) k_update_p4(int nc, const S *__restrict__ s, double *__restrict__ p, const KrylovScalars *sc) {
     pdl_trigger();
     pdl_wait();
     const double beta = sc->beta;
@@ -373,29 +399,21 @@ __global__ void k_update_p4(int nc, const S *__restrict__ s, double *__restrict_
 
 // q = A p on four consecutive points of an x-row (nx % 4 == 0), the neighbour terms summed in the
 // order of stencil7.
-__global__ void k_spmv_alpha4(int nx, int ny, int nz, const double *__restrict__ p, double *__restrict__ q,
-                              KrylovScalars *sc, DSum *part, unsigned *counter) {
+__global__ void __launch_bounds__(kMaxThreads) k_spmv_alpha4(int nx, int ny, int nz, const double *__restrict__ p, double *__restrict__ q,
+                              KrylovScalars *sc, DSum *part, unsigned *counter, GridDiv gd) {
     pdl_trigger();
     pdl_wait();
     const int nq = nx >> 2, npi = nx * ny, nc = (npi >> 2) * nz;
     double a0 = 0.0;
 #pragma unroll 2
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < nc; c += gridDim.x * blockDim.x) {
-        const int row = c / nq, xq = c - row * nq;
-        const int zz = row / ny, yy = row - zz * ny, xx = 4 * xq;
+        const int row = div_by(c, gd.row), xq = c - row * nq;
+        const int zz = div_by(row, gd.plane), yy = row - zz * ny, xx = 4 * xq;
         const int i = 4 * c;
-        double pc[4], nb[4] = {0.0, 0.0, 0.0, 0.0};
+        double pc[4];
         ld4(pc, p + i);
         const double pl = (xx > 0) ? p[i - 1] : 0.0, pr = (xx + 4 < nx) ? p[i + 4] : 0.0;
-        // x-1, x+1
-        if (xx > 0) nb[0] += pl;
-        nb[1] += pc[0];
-        nb[2] += pc[1];
-        nb[3] += pc[2];
-        nb[0] += pc[1];
-        nb[1] += pc[2];
-        nb[2] += pc[3];
-        if (xx + 4 < nx) nb[3] += pr;
+        double nb[4] = {pl + pc[1], pc[0] + pc[2], pc[1] + pc[3], pc[2] + pr};
         double t[4];
         if (yy > 0) {
             ld4(t, p + i - nx);
@@ -440,14 +458,13 @@ __global__ void k_spmv_alpha4(int nx, int ny, int nz, const double *__restrict__
 }
 
 template <class S>
-__global__ void k_update_xr4(int nc, double *__restrict__ x, const double *__restrict__ p, double *__restrict__ r,
-                             const double *__restrict__ q, double *__restrict__ dr, S *__restrict__ f0,
+__global__ void __launch_bounds__(kMaxThreads) k_update_xr4(int nc, double *__restrict__ x, const double *__restrict__ p, double *__restrict__ r,
+                             const double *__restrict__ q, S *__restrict__ f0,
                              KrylovScalars *sc, DSum *part, unsigned *counter, cudaGraphConditionalHandle cond,
                              int use_cond) {
     pdl_trigger();
     pdl_wait();
     const double alpha = sc->alpha;
-    const bool want_dr = (sc->variant == 1);
     double a0 = 0.0;
 #pragma unroll 2
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < nc; c += gridDim.x * blockDim.x) {
@@ -465,12 +482,6 @@ __global__ void k_update_xr4(int nc, double *__restrict__ x, const double *__res
         }
         st4(x + i, xv);
         st4(r + i, rn);
-        if (want_dr) {
-            double dv[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) dv[k] = rn[k] - ro[k];
-            st4(dr + i, dv);
-        }
         if (f0 != nullptr) sts4<S>(f0 + i, rn);
     }
     double v[1] = {a0};
@@ -490,11 +501,11 @@ __device__ __forceinline__ void ld4cg(double (&v)[4], const double *p) {
 }
 
 template <class S>
-__global__ void __launch_bounds__(256) k_tail_fused(int nx, int ny, int nz, const S *__restrict__ s, double *x,
-                                                    double *r, double *p, double *q, double *dr, S *f0,
+__global__ void __launch_bounds__(kMaxThreads) k_tail_fused(int nx, int ny, int nz, const S *__restrict__ s, double *x,
+                                                    double *r, double *p, double *q, S *f0,
                                                     KrylovScalars *sc, DSum *part, unsigned *counter, unsigned *bar,
                                                     long long spin_limit, cudaGraphConditionalHandle cond,
-                                                    int use_cond) {
+                                                    int use_cond, GridDiv gd) {
     const int nq = nx >> 2, npi = nx * ny, nc = (npi >> 2) * nz;
     const int stride = gridDim.x * blockDim.x, c0 = blockIdx.x * blockDim.x + threadIdx.x;
     unsigned *bcount = bar, *bgen = bar + 1;
@@ -527,7 +538,7 @@ __global__ void __launch_bounds__(256) k_tail_fused(int nx, int ny, int nz, cons
             for (int k = 0; k < 4; ++k) a0 = fma(sv[k], rv[k], a0);
             if (need_sdr) {
                 double dv[4];
-                ld4(dv, dr + 4 * c);
+                ld4(dv, q + 4 * c);
 #pragma unroll
                 for (int k = 0; k < 4; ++k) a1 = fma(sv[k], dv[k], a1);
             }
@@ -535,18 +546,18 @@ __global__ void __launch_bounds__(256) k_tail_fused(int nx, int ny, int nz, cons
         double v[2] = {a0, a1};
         double tot[2];
         if (grid_reduce<2>(v, part, counter, tot) && threadIdx.x == 0) {
-            const double rho = tot[0];
+            const double rho = tot[0], sdr = -sc->alpha * tot[1];
             double beta = 0.0;
             if (sc->restart == 0 && variant != 2) {
                 if (sc->rho_prev == 0.0) {
                     sc->status = -4;
                 } else {
-                    beta = (variant == 0) ? rho / sc->rho_prev : tot[1] / sc->rho_prev;
+                    beta = (variant == 0) ? rho / sc->rho_prev : sdr / sc->rho_prev;
                 }
             }
             if (!isfinite(rho) || !isfinite(beta)) sc->status = -6;
             sc->rho = rho;
-            sc->sdr = tot[1];
+            sc->sdr = sdr;
             sc->beta = beta;
         }
     }
@@ -580,20 +591,13 @@ __global__ void __launch_bounds__(256) k_tail_fused(int nx, int ny, int nz, cons
         double a0 = 0.0;
 #pragma unroll 2
         for (int c = c0; c < nc; c += stride) {
-            const int row = c / nq, xq = c - row * nq;
-            const int zz = row / ny, yy = row - zz * ny, xx = 4 * xq;
+            const int row = div_by(c, gd.row), xq = c - row * nq;
+            const int zz = div_by(row, gd.plane), yy = row - zz * ny, xx = 4 * xq;
             const int i = 4 * c;
-            double pc[4], nb[4] = {0.0, 0.0, 0.0, 0.0};
+            double pc[4];
             ld4cg(pc, p + i);
             const double pl = (xx > 0) ? __ldcg(p + i - 1) : 0.0, pr = (xx + 4 < nx) ? __ldcg(p + i + 4) : 0.0;
-            if (xx > 0) nb[0] += pl;
-            nb[1] += pc[0];
-            nb[2] += pc[1];
-            nb[3] += pc[2];
-            nb[0] += pc[1];
-            nb[1] += pc[2];
-            nb[2] += pc[3];
-            if (xx + 4 < nx) nb[3] += pr;
+            double nb[4] = {pl + pc[1], pc[0] + pc[2], pc[1] + pc[3], pc[2] + pr};
             double t[4];
             if (yy > 0) {
                 ld4cg(t, p + i - nx);
@@ -640,11 +644,10 @@ __global__ void __launch_bounds__(256) k_tail_fused(int nx, int ny, int nz, cons
         give_up();
         return;
     }
-    // ---- x += alpha p, r_new = r - alpha q, dr, f0 = (S) r_new, rr ----
+    // ---- x += alpha p, r_new = r - alpha q, f0 = (S) r_new, rr ----
     {
         const double alpha = __ldcg(&sc->alpha);
-        const bool want_dr = (sc->variant == 1);
-        double a0 = 0.0;
+            double a0 = 0.0;
 #pragma unroll 2
         for (int c = c0; c < nc; c += stride) {
             const int i = 4 * c;
@@ -661,12 +664,6 @@ __global__ void __launch_bounds__(256) k_tail_fused(int nx, int ny, int nz, cons
             }
             st4(x + i, xv);
             st4(r + i, rn);
-            if (want_dr) {
-                double dv[4];
-#pragma unroll
-                for (int k = 0; k < 4; ++k) dv[k] = rn[k] - ro[k];
-                st4(dr + i, dv);
-            }
             if (f0 != nullptr) sts4<S>(f0 + i, rn);
         }
         double v[1] = {a0};
@@ -676,27 +673,17 @@ __global__ void __launch_bounds__(256) k_tail_fused(int nx, int ny, int nz, cons
 }
 
 // ---- launchers --------------------------------------------------------------------------------
-// Grid of the reduction kernels, measured on GB300: while the Krylov vectors (about six of N
-// doubles) stay in the 129 MB L2, two 256-thread CTAs per SM (each thread sums tens of
-// products; the last CTA's compensated pass over the partials stays short); past that the
-// kernels stream from HBM and need every SM full of warps (8 CTAs per SM) to keep enough loads
-// in flight.
-int reduction_blocks(long long n) {
-    long long b = (n + 256LL * 16 - 1) / (256LL * 16);
-    const long long cap = (n <= (4LL << 20)) ? kReduceBlocks : kMaxReduceBlocks;
-    if (b < 1) b = 1;
-    if (b > cap) b = cap;
-    return static_cast<int>(b);
-}
-
-// Grid of the 4-element-chunk kernels: four 256-thread CTAs per SM (a thread handles a few chunks
-// at 128^3; the partials stay within the reduction buffer).
-int reduction_blocks4(long long n) {
-    long long b = (n / 4 + 255) / 256;
-    const long long cap = (n <= (4LL << 20)) ? 4 * 152 : kMaxReduceBlocks;
-    if (b < 1) b = 1;
-    if (b > cap) b = cap;
-    return static_cast<int>(b);
+// Grid of the Krylov kernels over `items` elements or chunks: one CTA per SM, of as many threads as
+// give every SM work (an FP64 unit serves its SM alone, so small grids are spread thin), 64 to 1024.
+struct RedGrid {
+    int blocks, threads;
+};
+RedGrid reduction_grid(long long items) {
+    constexpr int kSMs = 152;
+    long long t = (items + kSMs - 1) / kSMs;
+    t = std::min<long long>(kMaxThreads, std::max<long long>(64, (t + 63) / 64 * 64));
+    const long long b = std::max<long long>(1, std::min<long long>(kSMs, (items + t - 1) / t));
+    return RedGrid{static_cast<int>(b), static_cast<int>(t)};
 }
 
 // Polls of a grid-barrier wait in the fused tail before it gives up (about a second).
@@ -711,7 +698,7 @@ bool fused_tail_fits(int nb) {
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
     if (per_sm[dev] == 0) {
         int b = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_tail_fused<S>, 256, 0) != cudaSuccess ||
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_tail_fused<S>, kMaxThreads, 0) != cudaSuccess ||
             cudaDeviceGetAttribute(&sms[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
             cudaGetLastError();
             return false;
@@ -731,66 +718,70 @@ bool fused_tail_fits(int nb) {
 cudaError_t kry_init_residual(Prec st_prec, int nx, int ny, int nz, const double *b, const double *x, double *r,
                               void *f0, KrylovWork &w, cudaStream_t st) {
     const long long n = static_cast<long long>(nx) * ny * nz;
-    const int nb = reduction_blocks(n);
-    SMG_PREC_SWITCH(st_prec, k_init_residual<S><<<nb, 256, 0, st>>>(nx, ny, nz, b, x, r, static_cast<S *>(f0),
-                                                                      w.sc, w.part, w.counter));
+    const RedGrid g = reduction_grid(n);
+    SMG_PREC_SWITCH(st_prec, k_init_residual<S><<<g.blocks, g.threads, 0, st>>>(nx, ny, nz, b, x, r, static_cast<S *>(f0),
+                                                                      w.sc, w.part, w.counter, GridDiv{fast_div(nx), fast_div(ny)}));
     return cudaGetLastError();
 }
 
 cudaError_t kry_true_residual(int nx, int ny, int nz, const double *b, const double *x, KrylovWork &w,
                               cudaStream_t st) {
     const long long n = static_cast<long long>(nx) * ny * nz;
-    k_true_residual<<<reduction_blocks(n), 256, 0, st>>>(nx, ny, nz, b, x, w.sc, w.part, w.counter);
+    const RedGrid g = reduction_grid(n);
+    k_true_residual<<<g.blocks, g.threads, 0, st>>>(nx, ny, nz, b, x, w.sc, w.part, w.counter,
+                                                        GridDiv{fast_div(nx), fast_div(ny)});
     return cudaGetLastError();
 }
 
 cudaError_t kry_iteration_tail(Prec st_prec, int nx, int ny, int nz, const void *s, double *x, double *r, double *p,
-                               double *q, double *dr, void *f0, KrylovWork &w, cudaStream_t st,
+                               double *q, void *f0, KrylovWork &w, cudaStream_t st,
                                cudaGraphConditionalHandle cond, int use_cond) {
     const long long n = static_cast<long long>(nx) * ny * nz;
-    const int nb = reduction_blocks(n);
+    const RedGrid g1 = reduction_grid(n);
     cudaError_t e = cudaSuccess;
     auto al16 = [](const void *v) { return v == nullptr || (reinterpret_cast<uintptr_t>(v) & 15u) == 0; };
-    if (nx % 4 == 0 && al16(s) && al16(x) && al16(r) && al16(p) && al16(q) && al16(dr) && al16(f0)) {
+    if (nx % 4 == 0 && al16(s) && al16(x) && al16(r) && al16(p) && al16(q) && al16(f0)) {
         const int nc = static_cast<int>(n / 4);
-        const int nb4 = reduction_blocks4(n);
+        const RedGrid g4 = reduction_grid(nc);
+        const GridDiv gd4{fast_div(nx / 4), fast_div(ny)};
         SMG_PREC_SWITCH(st_prec, {
             const S *sp = static_cast<const S *>(s);
             S *f0p = static_cast<S *>(f0);
-            if (w.fused && w.bar != nullptr && fused_tail_fits<S>(nb4)) {
+            if (w.fused && w.bar != nullptr && fused_tail_fits<S>(g4.blocks)) {
                 // one cooperative launch: the runtime refuses it unless every CTA is resident
                 cudaLaunchConfig_t cfg = {};
-                cfg.gridDim = dim3(nb4);
-                cfg.blockDim = dim3(256);
+                cfg.gridDim = dim3(g4.blocks);
+                cfg.blockDim = dim3(g4.threads);
                 cfg.stream = st;
                 cudaLaunchAttribute attr[1];
                 attr[0].id = cudaLaunchAttributeCooperative;
                 attr[0].val.cooperative = 1;
                 cfg.attrs = attr;
                 cfg.numAttrs = 1;
-                e = cudaLaunchKernelEx(&cfg, k_tail_fused<S>, nx, ny, nz, sp, x, r, p, q, dr, f0p, w.sc, w.part, w.counter,
-                                       w.bar, static_cast<long long>(kTailSpinLimit), cond, use_cond);
+                e = cudaLaunchKernelEx(&cfg, k_tail_fused<S>, nx, ny, nz, sp, x, r, p, q, f0p, w.sc, w.part, w.counter,
+                                       w.bar, static_cast<long long>(kTailSpinLimit), cond, use_cond, gd4);
                 return e != cudaSuccess ? e : cudaGetLastError();
             }
-            if (e == cudaSuccess) e = launch_pdl(k_dots_beta4<S>, dim3(nb4), dim3(256), 0, st, nc, sp, r, dr, w.sc, w.part, w.counter);
-            if (e == cudaSuccess) e = launch_pdl(k_update_p4<S>, dim3(nb4), dim3(256), 0, st, nc, sp, p, w.sc);
+            if (e == cudaSuccess) e = launch_pdl(k_dots_beta4<S>, dim3(g4.blocks), dim3(g4.threads), 0, st, nc, sp, r, q, w.sc, w.part, w.counter);
+            if (e == cudaSuccess) e = launch_pdl(k_update_p4<S>, dim3(g4.blocks), dim3(g4.threads), 0, st, nc, sp, p, w.sc);
             if (e == cudaSuccess)
-                e = launch_pdl(k_spmv_alpha4, dim3(nb4), dim3(256), 0, st, nx, ny, nz, p, q, w.sc, w.part, w.counter);
+                e = launch_pdl(k_spmv_alpha4, dim3(g4.blocks), dim3(g4.threads), 0, st, nx, ny, nz, p, q, w.sc, w.part, w.counter, gd4);
             if (e == cudaSuccess)
-                e = launch_pdl(k_update_xr4<S>, dim3(nb4), dim3(256), 0, st, nc, x, p, r, q, dr, f0p, w.sc, w.part, w.counter,
+                e = launch_pdl(k_update_xr4<S>, dim3(g4.blocks), dim3(g4.threads), 0, st, nc, x, p, r, q, f0p, w.sc, w.part, w.counter,
                                cond, use_cond);
         });
         return e != cudaSuccess ? e : cudaGetLastError();
     }
+    const GridDiv gd{fast_div(nx), fast_div(ny)};
     SMG_PREC_SWITCH(st_prec, {
         const S *sp = static_cast<const S *>(s);
         S *f0p = static_cast<S *>(f0);
-        if (e == cudaSuccess) e = launch_pdl(k_dots_beta<S>, dim3(nb), dim3(256), 0, st, n, sp, r, dr, w.sc, w.part, w.counter);
-        if (e == cudaSuccess) e = launch_pdl(k_update_p<S>, dim3(nb), dim3(256), 0, st, n, sp, p, w.sc);
+        if (e == cudaSuccess) e = launch_pdl(k_dots_beta<S>, dim3(g1.blocks), dim3(g1.threads), 0, st, n, sp, r, q, w.sc, w.part, w.counter);
+        if (e == cudaSuccess) e = launch_pdl(k_update_p<S>, dim3(g1.blocks), dim3(g1.threads), 0, st, n, sp, p, w.sc);
         if (e == cudaSuccess)
-            e = launch_pdl(k_spmv_alpha, dim3(nb), dim3(256), 0, st, nx, ny, nz, p, q, w.sc, w.part, w.counter);
+            e = launch_pdl(k_spmv_alpha, dim3(g1.blocks), dim3(g1.threads), 0, st, nx, ny, nz, p, q, w.sc, w.part, w.counter, gd);
         if (e == cudaSuccess)
-            e = launch_pdl(k_update_xr<S>, dim3(nb), dim3(256), 0, st, n, x, p, r, q, dr, f0p, w.sc, w.part, w.counter, cond,
+            e = launch_pdl(k_update_xr<S>, dim3(g1.blocks), dim3(g1.threads), 0, st, n, x, p, r, q, f0p, w.sc, w.part, w.counter, cond,
                            use_cond);
     });
     return e != cudaSuccess ? e : cudaGetLastError();
