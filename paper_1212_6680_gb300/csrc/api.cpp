@@ -128,7 +128,7 @@ struct smg_ctx {
     std::vector<cudaEvent_t> event_pool;
     // relative recurrence residuals ||r_k|| / ||b|| of the last krylov_solve, k = 0 .. iters
     std::vector<double> hist;
-    double *d_hist = nullptr;       // device copy written by the x/r update (hist_cap entries)
+    double *d_hist = nullptr;       // ||r_k||^2, written by the x/r update (hist_cap entries)
     int hist_cap = 0;
     // Device-side solve loop (SMG_OPT_GRAPH): one CUDA graph whose conditional while node repeats
     // V-cycle + Krylov tail until the recurrence residual meets tol, maxit is reached or a
@@ -897,6 +897,8 @@ int krylov_device(smg_ctx *h, int variant, const double *b, double *x, double to
     if (k > 0) {
         SMG_CUDA(cudaMemcpyAsync(h->hist.data() + 1, h->d_hist + 1, sizeof(double) * k, cudaMemcpyDeviceToHost, ls));
         SMG_CUDA(cudaStreamSynchronize(ls));
+        const double bb0 = h->h_sc->bb > 0.0 ? h->h_sc->bb : 1.0;
+        for (int i = 1; i <= k; ++i) h->hist[i] = std::sqrt(h->hist[i] / bb0);
     }
     if (graph) {
         SMG_CUDA(cudaEventRecord(h->gev, ls));

@@ -25,7 +25,7 @@ struct KrylovScalars {
     int maxit;        // the solve's iteration limit
     int pad;
     double tol2;      // tol^2: the device-side loop continues while rr > tol2 * bb
-    double *hist;     // when set: hist[it] = sqrt(rr / bb) after every x/r update
+    double *hist;     // when set: hist[it] = rr after every x/r update
 };
 
 struct DSum;

@@ -39,14 +39,13 @@ __device__ __forceinline__ DSum shfl_down_dsum(const DSum &v, int o) {
 
 // Inner products: every thread accumulates its (about 2N / (threads in the grid)) products with
 // FMA, the block adds the thread partials through shared memory, and the last block to finish
-// combines the block partials with error-free TwoSum (compensated summation).  FP64 work per
+// combines the block partials exactly (warp_sum_exact).  FP64 work per
 // element stays at one FMA, which matters on GB300 where a warp's FP64 instruction holds its
 // sub-partition's unit for about 64 cycles however few lanes it serves.  That prices the reductions
-// themselves: a shuffle tree in every warp is 5 instructions a warp and value, and compensated sums
+// themselves: a shuffle tree in every warp is 5 instructions a warp and value, a compensated sum
 // 6 a term.  So the grid is one CTA of up to 1024 threads per SM (152 partials instead of 608), a
 // block folds its partials four to one on full warps (36 instructions a value instead of 165), and
-// one warp per value does the compensated pass.  128^3, of the 122 us of an iteration's four kernels:
-// see reduction_grid().
+// one warp per value adds the block partials as integers. 
 constexpr int kMaxThreads = 1024;
 
 template <int NV>
@@ -79,7 +78,57 @@ __device__ __forceinline__ void block_reduce_plain(double (&v)[NV]) {
             }
 }
 
-// Write this block's partials; the last block to finish sums all of them (compensated) into
+// The sum of one warp's values (kPer a lane), rounded once: integers in place of error-free FP64
+// additions, of which 70 would follow one another here (a dependent FP64 instruction takes about as long
+// as 15 integer ones).  Every value is aligned to the largest exponent in 128 bits -- 53 bits of mantissa
+// above 56 further bits, 18 bits of headroom for the count -- so only bits below 2^-108 of the largest
+// value are lost.  Sums with infinities, NaNs or exponents near the ends of the range go through
+// compensated FP64 additions.  The result is lane 0's.
+template <int kPer>
+__device__ __forceinline__ double warp_sum_exact(const double (&p)[kPer]) {
+    unsigned emax = 1u;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) emax = max(emax, static_cast<unsigned>(__double2hiint(p[i]) >> 20) & 0x7ffu);
+    emax = __reduce_max_sync(0xffffffffu, emax);
+    if (emax < 128u || emax > 2000u) {
+        DSum a{p[0], 0.0};
+#pragma unroll
+        for (int i = 1; i < kPer; ++i) two_sum_acc(a, p[i]);
+        for (int o = 16; o > 0; o >>= 1) a = dsum_combine(a, shfl_down_dsum(a, o));
+        return isfinite(a.s) ? a.s + a.c : a.s;  // the correction of an infinite sum is NaN
+    }
+    unsigned __int128 t = 0;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+        const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(p[i]));
+        const unsigned e = static_cast<unsigned>(b >> 52) & 0x7ffu, s = emax - max(e, 1u);
+        const unsigned long long m = (b & 0xfffffffffffffull) | (e ? 0x10000000000000ull : 0ull);
+        const unsigned __int128 v = s <= 56u ? static_cast<unsigned __int128>(m) << (56u - s)
+                                             : static_cast<unsigned __int128>(s < 120u ? m >> (s - 56u) : 0ull);
+        t = (b >> 63) ? t - v : t + v;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long lo = __shfl_down_sync(0xffffffffu, static_cast<unsigned long long>(t), o);
+        const unsigned long long hi = __shfl_down_sync(0xffffffffu, static_cast<unsigned long long>(t >> 64), o);
+        t += (static_cast<unsigned __int128>(hi) << 64) | lo;
+    }
+    const unsigned long long sign = static_cast<unsigned long long>(t >> 127) << 63;
+    if (sign) t = -t;
+    unsigned long long hi = static_cast<unsigned long long>(t >> 64), lo = static_cast<unsigned long long>(t);
+    if ((hi | lo) == 0ull) return 0.0;
+    const int z = hi ? __clzll(static_cast<long long>(hi)) : 64 + __clzll(static_cast<long long>(lo));
+    t <<= z;  // the leading bit to bit 127
+    hi = static_cast<unsigned long long>(t >> 64);
+    lo = static_cast<unsigned long long>(t);
+    unsigned long long mant = hi >> 11;  // 53 bits, then round to nearest, ties to even
+    const unsigned long long rest = hi & 0x7ffull;
+    if (rest > 0x400ull || (rest == 0x400ull && (lo != 0ull || (mant & 1ull)))) mant += 1ull;
+    // bit 108 of the sum has the value 2^(emax - 1023); a carry out of the mantissa raises the exponent
+    const unsigned long long e = static_cast<unsigned long long>(static_cast<int>(emax) + 19 - z);
+    return __longlong_as_double(static_cast<long long>(sign | ((e << 52) + (mant - 0x10000000000000ull))));
+}
+
+// Write this block's partials; the last block to finish sums all of them (rounded once) into
 // tot[] (thread 0's is the sum).  Returns true in every thread of the last block.
 template <int NV>
 __device__ __forceinline__ bool grid_reduce(double (&v)[NV], DSum *part, unsigned *counter, double (&tot)[NV]) {
@@ -88,19 +137,23 @@ __device__ __forceinline__ bool grid_reduce(double (&v)[NV], DSum *part, unsigne
     block_reduce_plain<NV>(v);
     if (threadIdx.x == 0) {
         for (int k = 0; k < NV; ++k) part[static_cast<size_t>(blockIdx.x) * NV + k].s = v[k];
-        __threadfence();
-        const unsigned t = atomicAdd(counter, 1u);
+        unsigned t;
+        asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(t) : "l"(counter) : "memory");
         last = (t == gridDim.x - 1);
     }
     __syncthreads();
     if (!last) return false;
-    __threadfence();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
     for (int k = w; k < NV; k += nw) {
-        DSum a{0.0, 0.0};
-        for (unsigned b = lane; b < gridDim.x; b += 32) two_sum_acc(a, __ldcg(&part[static_cast<size_t>(b) * NV + k].s));
-        for (int o = 16; o > 0; o >>= 1) a = dsum_combine(a, shfl_down_dsum(a, o));
-        if (lane == 0) res[k] = a.s + a.c;
+        constexpr int kPer = (kMaxReduceBlocks + 31) / 32;
+        double p[kPer];
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) {
+            const unsigned b = lane + 32 * i;
+            p[i] = b < gridDim.x ? __ldcg(&part[static_cast<size_t>(b) * NV + k].s) : 0.0;
+        }
+        const double t = warp_sum_exact<kPer>(p);
+        if (lane == 0) res[k] = t;
     }
     __syncthreads();
 #pragma unroll
@@ -121,6 +174,15 @@ inline FastDiv fast_div(int d) {
 __device__ __forceinline__ int div_by(int n, const FastDiv &f) {
     return static_cast<int>((__umulhi(static_cast<unsigned>(n), f.mul) + static_cast<unsigned>(n)) >> f.shift);
 }
+// This CTA's share of n items: contiguous (a grid-wide stride leaves some CTAs a whole trip more than
+// others: 4 against 3 at 128^3, and takes a CTA's rows apart), walked with the CTA's threads.
+struct Share {
+    int begin, end;
+};
+__device__ __forceinline__ Share cta_share(int n) {
+    return Share{static_cast<int>(static_cast<long long>(n) * blockIdx.x / gridDim.x) + static_cast<int>(threadIdx.x),
+                 static_cast<int>(static_cast<long long>(n) * (blockIdx.x + 1) / gridDim.x)};
+}
 struct GridDiv {  // rows of nx values (or nx / 4 chunks), ny rows a plane
     FastDiv row, plane;
 };
@@ -140,18 +202,19 @@ __device__ __forceinline__ double stencil7(const double *__restrict__ u, long lo
 // history and, inside the CUDA graph that repeats the iteration, its loop condition.
 __device__ __forceinline__ void finish_update(KrylovScalars *sc, double rr, cudaGraphConditionalHandle cond,
                                               int use_cond) {
+    const int it = sc->it + 1;
+    const double bb = sc->bb > 0.0 ? sc->bb : 1.0;
+    int status = sc->status;
+    if (!isfinite(rr)) sc->status = status = -6;
+    if (use_cond) {
+        const bool go = status == 0 && !(rr <= sc->tol2 * bb) && it < sc->maxit;
+        cudaGraphSetConditional(cond, go ? 1u : 0u);
+    }
     sc->rr = rr;
     sc->rho_prev = sc->rho;
     sc->restart = 0;
-    if (!isfinite(rr)) sc->status = -6;
-    const int it = sc->it + 1;
     sc->it = it;
-    const double bb = sc->bb > 0.0 ? sc->bb : 1.0;
-    if (sc->hist != nullptr) sc->hist[it] = sqrt(rr / bb);
-    if (use_cond) {
-        const bool go = sc->status == 0 && !(rr <= sc->tol2 * bb) && it < sc->maxit;
-        cudaGraphSetConditional(cond, go ? 1u : 0u);
-    }
+    if (sc->hist != nullptr) sc->hist[it] = rr;  // the host takes sqrt(rr / bb)
 }
 
 // r = b - A x ; f0 = (S) r ; rr = ||r||^2 ; bb = ||b||^2 ; restart = 1.
@@ -161,8 +224,8 @@ __global__ void __launch_bounds__(kMaxThreads) k_init_residual(int nx, int ny, i
                                 unsigned *counter, GridDiv gd) {
     const long long np = static_cast<long long>(nx) * ny;
     double a0 = 0.0, a1 = 0.0;
-    const int n32 = nx * ny * nz;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n32; i += gridDim.x * blockDim.x) {
+    const Share sh = cta_share(nx * ny * nz);
+    for (int i = sh.begin; i < sh.end; i += blockDim.x) {
         const int row = div_by(i, gd.row), xx = i - row * nx, zz = div_by(row, gd.plane), yy = row - zz * ny;
         const double bi = b[i];
         const double ri = bi - stencil7(x, i, xx, yy, zz, nx, ny, nz, np);
@@ -186,8 +249,8 @@ __global__ void __launch_bounds__(kMaxThreads) k_true_residual(int nx, int ny, i
                                 KrylovScalars *sc, DSum *part, unsigned *counter, GridDiv gd) {
     const long long np = static_cast<long long>(nx) * ny;
     double a0 = 0.0;
-    const int n32 = nx * ny * nz;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n32; i += gridDim.x * blockDim.x) {
+    const Share sh = cta_share(nx * ny * nz);
+    for (int i = sh.begin; i < sh.end; i += blockDim.x) {
         const int row = div_by(i, gd.row), xx = i - row * nx, zz = div_by(row, gd.plane), yy = row - zz * ny;
         const double ri = b[i] - stencil7(x, i, xx, yy, zz, nx, ny, nz, np);
         a0 = fma(ri, ri, a0);
@@ -207,8 +270,8 @@ __global__ void __launch_bounds__(kMaxThreads) k_dots_beta(long long n, const S 
     const int variant = sc->variant;
     const bool need_sdr = (variant == 1) && (sc->restart == 0);
     double a0 = 0.0, a1 = 0.0;
-    const int n32 = static_cast<int>(n);
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n32; i += gridDim.x * blockDim.x) {
+    const Share sh = cta_share(static_cast<int>(n));
+    for (int i = sh.begin; i < sh.end; i += blockDim.x) {
         const double si = ldv<double>(s + i);
         a0 = fma(si, r[i], a0);
         if (need_sdr) a1 = fma(si, q[i], a1);
@@ -238,8 +301,8 @@ __global__ void __launch_bounds__(kMaxThreads) k_update_p(long long n, const S *
     pdl_trigger();
     pdl_wait();
     const double beta = sc->beta;
-    const int n32 = static_cast<int>(n);
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n32; i += gridDim.x * blockDim.x) {
+    const Share sh = cta_share(static_cast<int>(n));
+    for (int i = sh.begin; i < sh.end; i += blockDim.x) {
         const double si = ldv<double>(s + i);
         p[i] = (beta == 0.0) ? si : fma(beta, p[i], si);
     }
@@ -252,8 +315,8 @@ __global__ void __launch_bounds__(kMaxThreads) k_spmv_alpha(int nx, int ny, int 
     pdl_wait();
     const long long np = static_cast<long long>(nx) * ny;
     double a0 = 0.0;
-    const int n32 = nx * ny * nz;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n32; i += gridDim.x * blockDim.x) {
+    const Share sh = cta_share(nx * ny * nz);
+    for (int i = sh.begin; i < sh.end; i += blockDim.x) {
         const int row = div_by(i, gd.row), xx = i - row * nx, zz = div_by(row, gd.plane), yy = row - zz * ny;
         const double qi = stencil7(p, i, xx, yy, zz, nx, ny, nz, np);
         q[i] = qi;
@@ -283,8 +346,8 @@ __global__ void __launch_bounds__(kMaxThreads) k_update_xr(long long n, double *
     pdl_wait();
     const double alpha = sc->alpha;
     double a0 = 0.0;
-    const int n32 = static_cast<int>(n);
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n32; i += gridDim.x * blockDim.x) {
+    const Share sh = cta_share(static_cast<int>(n));
+    for (int i = sh.begin; i < sh.end; i += blockDim.x) {
         x[i] = fma(alpha, p[i], x[i]);
         const double rn = fma(-alpha, q[i], r[i]);
         r[i] = rn;
@@ -336,28 +399,97 @@ template <> __device__ __forceinline__ void sts4<__nv_bfloat16>(__nv_bfloat16 *p
     reinterpret_cast<uint2 *>(p)[0] = a;
 }
 
+// One chunk as stored: 16-byte words.
+template <class S>
+struct RawChunk {
+    static constexpr int W = static_cast<int>(sizeof(S)) * 4 / 16 > 0 ? static_cast<int>(sizeof(S)) * 4 / 16 : 1;
+    uint4 w[W];
+};
+template <>
+struct RawChunk<__nv_bfloat16> {
+    uint2 w[1];
+};
+template <class S>
+__device__ __forceinline__ RawChunk<S> raw4(const S *p) {
+    RawChunk<S> r;
+    using Q = std::remove_reference_t<decltype(r.w[0])>;
+#pragma unroll
+    for (int i = 0; i < static_cast<int>(sizeof(r) / sizeof(Q)); ++i) r.w[i] = reinterpret_cast<const Q *>(p)[i];
+    return r;
+}
+template <class S>
+__device__ __forceinline__ void widen4(double (&v)[4], const RawChunk<S> &r) {
+    lds4<S>(v, reinterpret_cast<const S *>(&r));
+}
+
+// (s, r) and, when wanted, (s, q) over this CTA's chunks; the next chunk is on its way while one is
+// summed (3.4 chunks a thread at 128^3: a load's latency each otherwise).
+template <class S>
+__device__ __forceinline__ void dots_share(double &a0, double &a1, const Share &sh, const S *s, const double *r, const double *q,
+                                           bool with_q) {
+    if (sh.begin >= sh.end) return;
+    RawChunk<S> ns = raw4<S>(s + 4 * sh.begin);
+    RawChunk<double> nr = raw4<double>(r + 4 * sh.begin), nq;
+    if (with_q) nq = raw4<double>(q + 4 * sh.begin);
+    for (int c = sh.begin; c < sh.end; c += blockDim.x) {
+        const RawChunk<S> cs = ns;
+        const RawChunk<double> cr = nr, cq = nq;
+        const int n = c + static_cast<int>(blockDim.x);
+        if (n < sh.end) {
+            ns = raw4<S>(s + 4 * n);
+            nr = raw4<double>(r + 4 * n);
+            if (with_q) nq = raw4<double>(q + 4 * n);
+        }
+        double sv[4], v[4];
+        widen4<S>(sv, cs);
+        widen4<double>(v, cr);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) a0 = fma(sv[k], v[k], a0);
+        if (with_q) {
+            widen4<double>(v, cq);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) a1 = fma(sv[k], v[k], a1);
+        }
+    }
+}
+
+// p = s + beta p over this CTA's chunks (p = s when beta is 0: p may hold anything then).
+template <class S>
+__device__ __forceinline__ void update_p_share(const Share &sh, const S *s, double *p, double beta) {
+    if (sh.begin >= sh.end) return;
+    const bool keep = beta != 0.0;
+    RawChunk<S> ns = raw4<S>(s + 4 * sh.begin);
+    RawChunk<double> np;
+    if (keep) np = raw4<double>(p + 4 * sh.begin);
+    for (int c = sh.begin; c < sh.end; c += blockDim.x) {
+        const RawChunk<S> cs = ns;
+        const RawChunk<double> cp = np;
+        const int n = c + static_cast<int>(blockDim.x);
+        if (n < sh.end) {
+            ns = raw4<S>(s + 4 * n);
+            if (keep) np = raw4<double>(p + 4 * n);
+        }
+        double sv[4], pv[4];
+        widen4<S>(sv, cs);
+        if (keep) {
+            widen4<double>(pv, cp);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) sv[k] = fma(beta, pv[k], sv[k]);
+        }
+        st4(p + 4 * c, sv);
+    }
+}
+
 template <class S>
 __global__ void __launch_bounds__(kMaxThreads) k_dots_beta4(int nc, const S *__restrict__ s, const double *__restrict__ r,
                              const double *__restrict__ q, KrylovScalars *sc, DSum *part, unsigned *counter) {
     pdl_trigger();
     pdl_wait();
+    const Share sh = cta_share(nc);
     const int variant = sc->variant;
     const bool need_sdr = (variant == 1) && (sc->restart == 0);
     double a0 = 0.0, a1 = 0.0;
-#pragma unroll 2
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < nc; c += gridDim.x * blockDim.x) {
-        double sv[4], rv[4];
-        lds4<S>(sv, s + 4 * c);
-        ld4(rv, r + 4 * c);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) a0 = fma(sv[k], rv[k], a0);
-        if (need_sdr) {
-            double dv[4];
-            ld4(dv, q + 4 * c);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) a1 = fma(sv[k], dv[k], a1);
-        }
-    }
+    dots_share<S>(a0, a1, sh, s, r, q, need_sdr);
     double v[2] = {a0, a1};
     double tot[2];
     if (grid_reduce<2>(v, part, counter, tot) && threadIdx.x == 0) {
@@ -381,20 +513,9 @@ template <class S>
 __global__ void __launch_bounds__(kMaxThreads) k_update_p4(int nc, const S *__restrict__ s, double *__restrict__ p, const KrylovScalars *sc) {
     pdl_trigger();
     pdl_wait();
+    const Share sh = cta_share(nc);
     const double beta = sc->beta;
-#pragma unroll 2
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < nc; c += gridDim.x * blockDim.x) {
-        double sv[4], pv[4];
-        lds4<S>(sv, s + 4 * c);
-        if (beta == 0.0) {
-            st4(p + 4 * c, sv);
-        } else {
-            ld4(pv, p + 4 * c);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) pv[k] = fma(beta, pv[k], sv[k]);
-            st4(p + 4 * c, pv);
-        }
-    }
+    update_p_share<S>(sh, s, p, beta);
 }
 
 // q = A p on four consecutive points of an x-row (nx % 4 == 0), the neighbour terms summed in the
@@ -404,9 +525,10 @@ __global__ void __launch_bounds__(kMaxThreads) k_spmv_alpha4(int nx, int ny, int
     pdl_trigger();
     pdl_wait();
     const int nq = nx >> 2, npi = nx * ny, nc = (npi >> 2) * nz;
+    const Share sh = cta_share(nc);
     double a0 = 0.0;
 #pragma unroll 2
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < nc; c += gridDim.x * blockDim.x) {
+    for (int c = sh.begin; c < sh.end; c += blockDim.x) {
         const int row = div_by(c, gd.row), xq = c - row * nq;
         const int zz = div_by(row, gd.plane), yy = row - zz * ny, xx = 4 * xq;
         const int i = 4 * c;
@@ -464,10 +586,11 @@ __global__ void __launch_bounds__(kMaxThreads) k_update_xr4(int nc, double *__re
                              int use_cond) {
     pdl_trigger();
     pdl_wait();
+    const Share sh = cta_share(nc);
     const double alpha = sc->alpha;
     double a0 = 0.0;
 #pragma unroll 2
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < nc; c += gridDim.x * blockDim.x) {
+    for (int c = sh.begin; c < sh.end; c += blockDim.x) {
         const int i = 4 * c;
         double xv[4], pv[4], ro[4], qv[4], rn[4];
         ld4(xv, x + i);
@@ -507,7 +630,7 @@ __global__ void __launch_bounds__(kMaxThreads) k_tail_fused(int nx, int ny, int 
                                                     long long spin_limit, cudaGraphConditionalHandle cond,
                                                     int use_cond, GridDiv gd) {
     const int nq = nx >> 2, npi = nx * ny, nc = (npi >> 2) * nz;
-    const int stride = gridDim.x * blockDim.x, c0 = blockIdx.x * blockDim.x + threadIdx.x;
+    const Share sh = cta_share(nc);
     unsigned *bcount = bar, *bgen = bar + 1;
     int *berr = reinterpret_cast<int *>(bar + 2);
     const unsigned nblk = gridDim.x;
@@ -529,20 +652,7 @@ __global__ void __launch_bounds__(kMaxThreads) k_tail_fused(int nx, int ny, int 
         const int variant = sc->variant;
         const bool need_sdr = (variant == 1) && (sc->restart == 0);
         double a0 = 0.0, a1 = 0.0;
-#pragma unroll 2
-        for (int c = c0; c < nc; c += stride) {
-            double sv[4], rv[4];
-            lds4<S>(sv, s + 4 * c);
-            ld4(rv, r + 4 * c);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) a0 = fma(sv[k], rv[k], a0);
-            if (need_sdr) {
-                double dv[4];
-                ld4(dv, q + 4 * c);
-#pragma unroll
-                for (int k = 0; k < 4; ++k) a1 = fma(sv[k], dv[k], a1);
-            }
-        }
+        dots_share<S>(a0, a1, sh, s, r, q, need_sdr);
         double v[2] = {a0, a1};
         double tot[2];
         if (grid_reduce<2>(v, part, counter, tot) && threadIdx.x == 0) {
@@ -568,19 +678,7 @@ __global__ void __launch_bounds__(kMaxThreads) k_tail_fused(int nx, int ny, int 
     // ---- p = s + beta p ----
     {
         const double beta = __ldcg(&sc->beta);
-#pragma unroll 2
-        for (int c = c0; c < nc; c += stride) {
-            double sv[4], pv[4];
-            lds4<S>(sv, s + 4 * c);
-            if (beta == 0.0) {
-                st4(p + 4 * c, sv);
-            } else {
-                ld4(pv, p + 4 * c);
-#pragma unroll
-                for (int k = 0; k < 4; ++k) pv[k] = fma(beta, pv[k], sv[k]);
-                st4(p + 4 * c, pv);
-            }
-        }
+        update_p_share<S>(sh, s, p, beta);
     }
     if (!grid_barrier(bcount, bgen, berr, spin_limit, nblk)) {
         give_up();
@@ -590,7 +688,7 @@ __global__ void __launch_bounds__(kMaxThreads) k_tail_fused(int nx, int ny, int 
     {
         double a0 = 0.0;
 #pragma unroll 2
-        for (int c = c0; c < nc; c += stride) {
+        for (int c = sh.begin; c < sh.end; c += blockDim.x) {
             const int row = div_by(c, gd.row), xq = c - row * nq;
             const int zz = div_by(row, gd.plane), yy = row - zz * ny, xx = 4 * xq;
             const int i = 4 * c;
@@ -649,7 +747,7 @@ __global__ void __launch_bounds__(kMaxThreads) k_tail_fused(int nx, int ny, int 
         const double alpha = __ldcg(&sc->alpha);
             double a0 = 0.0;
 #pragma unroll 2
-        for (int c = c0; c < nc; c += stride) {
+        for (int c = sh.begin; c < sh.end; c += blockDim.x) {
             const int i = 4 * c;
             double xv[4], pv[4], ro[4], qv[4], rn[4];
             ld4(xv, x + i);
