@@ -197,13 +197,13 @@ int lobpcg_solve(smg_handle h, int m, double *X, double *lambda, double tol, int
  * Batched solver: nsys independent systems, each the model problem on its own brick
  * (dims[3s], dims[3s+1], dims[3s+2] = nx, ny, nz of system s), solved together by Algorithm 1
  * (PCG eq. (1), flexible PCG eq. (2) or PSD) preconditioned by SMG with -v npre npost.  Per
- * iteration, one CUDA graph runs one persistent kernel that performs every step of every
- * system's V-cycle (levels aligned from the finest, a bounded grid barrier between steps) and
- * the FP64 Krylov kernels of all systems; converged systems are masked out on the device.
+ * iteration, one CUDA graph runs every system's V-cycle in the sine eigenvectors of its x-lines
+ * (SMG_OPT_MODAL's form: one launch transforms all residuals, one CTA per system and mode runs that
+ * mode's cycle, one launch transforms back) and the FP64 Krylov kernels of all systems;
+ * converged systems are masked out on the device.
  *
- * smg_batched_setup -- builds the hierarchies, allocates every buffer, chooses the schedule
- * (threads per CTA, task order within a step) by timing one V-cycle per candidate (cached per
- * set of grids for the life of the process) and captures the per-iteration graph.
+ * smg_batched_setup -- builds the hierarchies and their tables, allocates every buffer and captures
+ * the per-iteration graph.
  *   dims:  host, 3*nsys ints; 1 <= nx <= 128, 1 <= ny <= 512, 1 <= nz <= 4096; 1 <= nsys <= 4096.
  *   npre, npost: 1 <= npre <= 8, 0 <= npost <= 8.
  *   prec:  SMG_FP32 (FP32 cycle, FP64 coarsest plane, FP64 Krylov); others return SMG_ERR_ARG.
@@ -215,19 +215,17 @@ int lobpcg_solve(smg_handle h, int m, double *X, double *lambda, double tol, int
  *   iters:  host, nsys ints, always written (preconditioner applications per system).
  *   relres: host, nsys doubles (NULL allowed): final true relative residual per system.
  * Stops each system at ||b - A x||_2 <= tol ||b||_2 (true residual); returns SMG_ERR_NOCONV
- * when some system did not reach it in maxit iterations, SMG_ERR_TIMEOUT when a grid-barrier
- * wait gave up, SMG_ERR_BREAKDOWN / SMG_ERR_NAN as krylov_solve.  Synchronises `stream` once
- * per iteration.  Calls on one handle must not overlap.
+ * when some system did not reach it in maxit iterations, SMG_ERR_BREAKDOWN / SMG_ERR_NAN as
+ * krylov_solve.  Synchronises `stream` once per iteration.  Calls on one handle must not overlap.
  *
  * smg_batched_apply -- s_s = T_s r_s for every system s: one application of each system's SMG
  *   V-cycle (section 3: the fixed, linear preconditioner of Algorithm 1) with the handle's
- *   npre/npost, storage precision and tuned schedule, all systems together in exactly one launch
- *   of the persistent V-cycle kernel -- the launch each iteration of smg_batched_solve makes.
+ *   npre/npost and storage precision, all systems together in the launches each iteration of
+ *   smg_batched_solve makes.
  *   r, s:   host arrays of nsys device pointers (system s: nx*ny*nz doubles, layout as
  *           smg_apply); r is rounded to the storage precision on entry, s receives the cycle's
  *           output widened exactly to FP64.  Caller-owned.
- *   Returns SMG_ERR_TIMEOUT when a grid-barrier wait gave up.  Synchronises `stream`.  Calls on
- *   one handle must not overlap (the handle's level vectors are shared).
+ *   Synchronises `stream`.  Calls on one handle must not overlap (the handle's vectors are shared).
  *
  * smg_batched_destroy -- frees the handle (NULL accepted).  Synchronises the device.
  */
@@ -240,19 +238,18 @@ int smg_batched_apply(smg_batched_handle h, const double *const *r, double *cons
 int smg_batched_destroy(smg_batched_handle h);
 
 /*
- * smg_batched_info -- the schedule the set-up's autotuner chose by timing every candidate
- * V-cycle: x-line tile (rows_per_lane K: a warp holds 32 K rows of a line, K from the narrowest
- * that holds every system's lines up to 4), threads per CTA (256 or 512), persistent CTAs
- * (`blocks`: a multiple of the SM count, 1 up to the occupancy limit per SM) and task order
- * (0 system order, 1 longest plane first); also the tasks per V-cycle and the kernel launches the
- * handle has issued so far (the persistent V-cycle counts once per launch).  Host outputs.
+ * smg_batched_info -- the schedule of the V-cycles: threads per CTA of the (system, mode) cycles with the
+ * larger planes (512, one CTA per SM, or 256 when two share an SM), the CTAs resident at once
+ * (`blocks`: a multiple of the SM count), their order (1: largest planes first), the cycles per
+ * application (`tasks`: one per system and mode), the kernel launches the handle has issued so far,
+ * and the widest system's x-line in rows per lane of a warp (ceil(nx / 32)).  Host outputs.
  */
 int smg_batched_info(smg_batched_handle h, int *threads, int *order, int *blocks, long long *tasks,
                      long long *launches, int *rows_per_lane);
 
 /*
  * smg_batched_set_profile / smg_batched_profile_read -- with profiling on, each iteration's
- * graph replay is timed by its event nodes: class 0 the persistent V-cycle kernel, class 1 the
+ * graph replay is timed by its event nodes: class 0 the V-cycles' kernels, class 1 the
  * Krylov kernels.  Read returns replays, total device milliseconds and, for class 0, the
  * algorithmic bytes of the V-cycles performed (storage words each active system's cycle must
  * read and write: 2.5 words per point per relaxation sweep, 5 per point for residual +
@@ -272,8 +269,8 @@ int krylov_solve_batched(int nsys, const int *dims, int npre, int npost, int pre
  * smg_barrier_selftest -- runs a small persistent kernel of 4 CTAs whose grid barrier waits for
  * 4 + extra_blocks CTAs, with a wait limit of about limit_seconds (0 < limit_seconds <= 10).
  * *status (host) receives SMG_OK when the barriers complete (extra_blocks = 0) and
- * SMG_ERR_TIMEOUT when a wait gave up (extra_blocks > 0): the failure path of the barrier that
- * krylov_solve_batched relies on, exercised without faulting or hanging the device.
+ * SMG_ERR_TIMEOUT when a wait gave up (extra_blocks > 0): the failure path of a bounded grid barrier,
+ * exercised without faulting or hanging the device.
  */
 int smg_barrier_selftest(int extra_blocks, double limit_seconds, int *status, void *stream);
 

@@ -53,9 +53,6 @@ def _units():
     for t, g, k in MODAL:
         units.append((os.path.join(CSRC, "modal_inst.cu"), os.path.join(BUILD, f"modal_{t}_{g}_{k}.o"), ["-x", "cu"],
                       [f"-DSMG_MT={t}", f"-DSMG_MG={g}", f"-DSMG_MK={k}"]))
-    for k in (1, 2, 3, 4):
-        src = os.path.join(CSRC, "batched_inst.cu")
-        units.append((src, os.path.join(BUILD, f"batched_k{k}.o"), ["-x", "cu"], [f"-DSMG_K={k}"]))
     for k in KS:
         for prec in (0, 1, 2):
             src = os.path.join(CSRC, "plane_relax_inst.cu")

@@ -299,7 +299,7 @@ def smg_batched_solve(h, variant, b_list, x_list, tol=1e-8, maxit=100, stream=No
 
 
 def smg_batched_apply(h, r_list, s_list, stream=None) -> None:
-    """One persistent V-cycle launch: s_list[i] = T_i r_list[i] (per-system device tensors)."""
+    """One V-cycle of every system: s_list[i] = T_i r_list[i] (per-system device tensors)."""
     nsys = len(r_list)
     rp = (ctypes.c_void_p * nsys)(*[_ptr(t) for t in r_list])
     sp = (ctypes.c_void_p * nsys)(*[_ptr(t) for t in s_list])

@@ -84,3 +84,25 @@ def test_modal_nan_reaches_the_solver(smg):
         x.zero_()
         rc, it, rel = smg.krylov_solve(h.h, "fpcg", b, x, 1e-8, 50)
         assert rc == 0 and rel <= 1e-8
+
+
+@pytest.mark.parametrize("npost", [0, 1])
+def test_modal_batch_of_mixed_sizes_matches_oracle(smg, orc, npost):
+    """One batch of a point, a line, planes that share an SM, planes that fill one and planes that need
+    slabs, at one lane configuration."""
+    dims = np.array([(1, 1, 1), (5, 1, 1), (3, 2, 9), (17, 40, 33), (6, 128, 127), (5, 300, 120), (128, 5, 3)])
+    rh = [inputs.rhs(int(a), int(b), int(c), seed=30 + i) for i, (a, b, c) in enumerate(dims)]
+    r = [torch.from_numpy(v.ravel().copy()).cuda() for v in rh]
+    h = smg.smg_batched_setup(dims, npre=1, npost=npost)
+    try:
+        out = [torch.full_like(v, float("nan")) for v in r]
+        smg.smg_batched_apply(h, r, out)
+        x = [torch.zeros_like(v) for v in r]
+        rc, iters, rel = smg.smg_batched_solve(h, "fpcg", r, x)
+        assert rc == 0 and (rel <= 1e-8).all()
+    finally:
+        smg.smg_batched_destroy(h)
+    for i, (a, b, c) in enumerate(dims):
+        ref = orc.SMG(int(a), int(b), int(c), 1, npost).apply(rh[i])
+        err = np.linalg.norm(out[i].cpu().numpy() - ref.ravel()) / np.linalg.norm(ref)
+        assert err <= 1e-6, (tuple(dims[i]), err)
