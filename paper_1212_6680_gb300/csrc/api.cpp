@@ -234,8 +234,10 @@ int ensure_levels(smg_ctx *h, int nb) {
         const int e = modal_build(h->mp, H, h->prec == Prec::F64, nb, h->npre, h->npost, h->coarse_iters);
         if (e == 0) {
             // the Krylov kernels read T r of one right-hand side in the storage precision
+            // and, for an FP32 cycle, write r rounded to it beside r
             h->d_f.assign(1, nullptr);
             h->d_u.assign(1, nullptr);
+            if (h->prec == Prec::F32) SMG_CUDA(cudaMalloc(&h->d_f[0], static_cast<size_t>(h->N()) * sb));
             SMG_CUDA(cudaMalloc(&h->d_u[0], static_cast<size_t>(h->N()) * sb));
             h->modal_now = true;
             h->nb_alloc = nb;
@@ -626,12 +628,12 @@ int relax(smg_ctx *h, int l, int colour, int mode, int iters, bool coarsest, con
     return SMG_OK;
 }
 
-// u0 = T f0 for nb right-hand sides in mode space: f0 in FP64, u0 of type `type`.
-int run_modal(smg_ctx *h, int nb, const double *f0, Prec type, void *u0, cudaStream_t st) {
+// u0 = T f0 for nb right-hand sides in mode space: f0 of type `in`, u0 of type `type`.
+int run_modal(smg_ctx *h, int nb, Prec in, const void *f0, Prec type, void *u0, cudaStream_t st) {
     const double n = static_cast<double>(h->N()) * nb, cb = h->mp.f64 ? 8.0 : 4.0;
     {
-        RegionTimer rt(h, st, 3, n * (8.0 + cb));
-        const cudaError_t e = modal_transform_in(h->mp, nb, f0, st, h->launches);
+        RegionTimer rt(h, st, 3, n * (static_cast<double>(storage_bytes(in)) + cb));
+        const cudaError_t e = modal_transform_in(h->mp, nb, in, f0, st, h->launches);
         if (e != cudaSuccess) return fail(SMG_ERR_CUDA, std::string("transform launch: ") + cudaGetErrorString(e));
     }
     {
@@ -647,10 +649,10 @@ int run_modal(smg_ctx *h, int nb, const double *f0, Prec type, void *u0, cudaStr
     return SMG_OK;
 }
 
-// u0 = T f0 for nb right-hand sides; f0, u0 in storage precision, level-0 layout (in mode space f0
-// in FP64).
+// u0 = T f0 for nb right-hand sides; f0, u0 in storage precision, level-0 layout (in mode space a BF16
+// cycle's f0 is in FP64).
 int run_cycle(smg_ctx *h, int nb, const void *f0, void *u0, cudaStream_t st) {
-    if (h->modal_now) return run_modal(h, nb, static_cast<const double *>(f0), h->prec, u0, st);
+    if (h->modal_now) return run_modal(h, nb, h->prec == Prec::F32 ? Prec::F32 : Prec::F64, f0, h->prec, u0, st);
     const HostHierarchy &H = h->H;
     const int L = H.L;
     int rc;
@@ -796,8 +798,8 @@ int krylov_device(smg_ctx *h, int variant, const double *b, double *x, double to
     }
     const bool f64 = (h->prec == Prec::F64);
     const bool ident = (h->precond == 0);                           // T = I: s is r itself
-    // cycle input: (S) r, written by the Krylov kernels, or r itself (FP64 cycles and mode space)
-    const bool own_f0 = !f64 && !h->modal_now;
+    // cycle input: (S) r, written by the Krylov kernels, or r itself (FP64 cycles, and BF16 in mode space)
+    const bool own_f0 = !f64 && !(h->modal_now && h->prec == Prec::BF16);
     void *f0 = own_f0 ? h->d_f[0] : static_cast<void *>(h->d_r);
     void *u0 = ident ? static_cast<void *>(h->d_r) : h->d_u[0];   // s = T r
     const Prec kp = ident ? Prec::F64 : h->prec;                    // storage type of s
@@ -1056,7 +1058,7 @@ int smg_apply_batched(smg_handle h, int nb, const double *R, double *S, void *st
     if ((rc = ensure_levels(h, nb)) != SMG_OK) return rc;
     const long long n = h->N() * nb;
     if (h->modal_now) {
-        if ((rc = run_modal(h, nb, R, Prec::F64, S, st)) != SMG_OK) return rc;
+        if ((rc = run_modal(h, nb, Prec::F64, R, Prec::F64, S, st)) != SMG_OK) return rc;
     } else if (h->prec == Prec::F64) {
         if ((rc = run_cycle(h, nb, R, S, st)) != SMG_OK) return rc;
     } else {

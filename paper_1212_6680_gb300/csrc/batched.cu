@@ -102,6 +102,7 @@ struct BKrylov {
     const long long *ch_start;  // offset of the chunk in its system
     const int *ch_len;
     double *r, *p, *q;
+    float *rf;                  // r rounded to FP32 (the cycle's input)
     float *s;                   // T r of every system (the cycle's output)
     const double *const *bptr;
     double *const *xptr;
@@ -158,10 +159,12 @@ __global__ void __launch_bounds__(kBThreads) kb_init(BKrylov k, int only_flagged
         const int l0 = static_cast<int>(k.ch_start[c]), len = k.ch_len[c];
         const double *x = k.xptr[s], *b = k.bptr[s];
         double *r = k.r + sy.off;
+        float *rf = k.rf + sy.off;
 #pragma unroll 2
         for (int li = l0 + threadIdx.x; li < l0 + len; li += kBThreads) {
             const double bi = b[li], ri = bi - stencil_of(x, sy, li);
             r[li] = ri;
+            rf[li] = narrow_f64(ri);
             v[0] = fma(ri, ri, v[0]);
             v[1] = fma(bi, bi, v[1]);
         }
@@ -213,12 +216,13 @@ __global__ void __launch_bounds__(kBThreads) kb_dots(BKrylov k) {
     put_partials<2>(k, c, v);
 }
 
-// smg_batched_apply: every system's right-hand side (caller memory) into r, every system active.
+// smg_batched_apply: every system's right-hand side (caller memory) rounded to the cycle's input, every
+// system active.
 __global__ void __launch_bounds__(kBThreads) kb_apply_in(BKrylov k) {
     const int c = blockIdx.x, s = k.ch_sys[c];
     const double *r = k.bptr[s] + k.ch_start[c];
-    double *to = k.r + k.sys[s].off + k.ch_start[c];
-    for (int t = threadIdx.x; t < k.ch_len[c]; t += kBThreads) to[t] = r[t];
+    float *to = k.rf + k.sys[s].off + k.ch_start[c];
+    for (int t = threadIdx.x; t < k.ch_len[c]; t += kBThreads) to[t] = narrow_f64(r[t]);
     if (threadIdx.x == 0 && c == k.sys[s].c0) k.active[s] = 1;
 }
 
@@ -304,6 +308,7 @@ __global__ void __launch_bounds__(kBThreads) kb_upd_xr(BKrylov k) {
     const int len = k.ch_len[c];
     const double alpha = k.sc[s].alpha;
     double *x = k.xptr[s] + k.ch_start[c], *r = k.r + g0;
+    float *rf = k.rf + g0;
     const double *p = k.p + g0, *q = k.q + g0;
     double v[1] = {0.0};
 #pragma unroll 4
@@ -311,6 +316,7 @@ __global__ void __launch_bounds__(kBThreads) kb_upd_xr(BKrylov k) {
         x[t] = fma(alpha, p[t], x[t]);
         const double rn = fma(-alpha, q[t], r[t]);
         r[t] = rn;
+        rf[t] = narrow_f64(rn);
         v[0] = fma(rn, rn, v[0]);
     }
     put_partials<1>(k, c, v);
@@ -612,6 +618,7 @@ int batched_build(smg_batched_ctx &c, const int *dims, cudaStream_t st) {
     BCHK(buf.alloc(&c.kk.r, vtot));
     BCHK(buf.alloc(&c.kk.p, vtot));
     BCHK(buf.alloc(&c.kk.q, vtot));
+    BCHK(buf.alloc(&c.kk.rf, vtot));
     BCHK(buf.alloc(&c.kk.s, vtot));
     BCHK(cudaMemsetAsync(c.kk.p, 0, vtot * sizeof(double), st));
     BCHK(cudaMemsetAsync(c.kk.q, 0, vtot * sizeof(double), st));
@@ -647,8 +654,8 @@ int batched_build(smg_batched_ctx &c, const int *dims, cudaStream_t st) {
     for (int s : by_size) {
         SysPlan &p = sys[s];
         args[s] = p.m.a;
-        SineArgs g{p.nx, p.ny, p.nz, p.m.a.pitch, (p.nx + 1) / 2, ((p.nx + 1) / 2 + 31) / 32 * 32, d_mats + sines[p.nx]};
-        jobs[s] = SineJob{g, c.kk.r + p.off, p.m.a.fw[0], p.m.a.u[0], c.kk.s + p.off};
+        SineArgs g{p.nx, p.ny, p.nz, p.m.a.pitch, (p.nx + 1) / 2, ((p.nx + 1) / 2 + 63) / 64 * 64, d_mats + sines[p.nx]};
+        jobs[s] = SineJob{g, c.kk.rf + p.off, p.m.a.fw[0], p.m.a.u[0], c.kk.s + p.off};
         for (int m = 0; m < sine_mode_tiles(g); ++m)
             for (int t = 0; t < sine_line_tiles(g); ++t) tiles.push_back(SineTile{s, t, m});
         const int gi = 2 * (p.m.smem + 2048) <= kModalSmem ? 1 : 0;

@@ -1,16 +1,8 @@
 // modal.cu -- the transforms of the x-lines into their sine eigenvectors and back, the prolongation in
 // mode space, and the host side of the mode-space V-cycle (modal.cuh).
 //
-// Transform.  The orthonormal eigenvectors of tridiag(-1, 2, -1) of order n are
-// s_k(x) = sqrt(2 / (n + 1)) sin(pi k x / (n + 1)), x, k = 1 .. n.  s_k is symmetric about the middle for
-// odd k and antisymmetric for even k, so the line is folded first (x with n + 1 - x: sum and
-// difference) and each parity is a product of half the order: n / 2 multiply-adds a point and
-// transform, as two dense products over all lines.  No fast sine transform: n + 1 is 129, 257 or 1281
-// for the sizes in use (few small factors), and at n <= 256 the product costs less than the passes
-// over memory of a factored transform.
-//
-// A CTA of 128 threads forms TM x 16 lines by 32 modes of each parity; a thread holds TM lines x 4 modes
-// of both parities.  FP32: bound by FFMA issue (64 FMAs to 12 shared-memory reads a step).
+// The FP32 transforms are in sine.cu; the FP64 ones here hold 4 lines by 4 modes of each parity a thread and are
+// bound by FP64 issue.
 #include <cmath>
 #include <cstring>
 #include <map>
@@ -28,32 +20,11 @@ constexpr int kBN = 32;      // modes (or pairs of points) of a parity per CTA
 
 template <class T> constexpr int tm_lines() { return 4; }
 
-template <class T> __device__ __forceinline__ T in_val(double v);
-template <> __device__ __forceinline__ float in_val<float>(double v) { return narrow_f64(v); }
-template <> __device__ __forceinline__ double in_val<double>(double v) { return v; }
-template <class S, class T> __device__ __forceinline__ S out_val(T v);
-template <> __device__ __forceinline__ float out_val<float, float>(float v) { return v; }
-template <> __device__ __forceinline__ double out_val<double, float>(float v) { return widen_f32(v); }
-template <> __device__ __forceinline__ __nv_bfloat16 out_val<__nv_bfloat16, float>(float v) { return __float2bfloat16_rn(v); }
-template <> __device__ __forceinline__ double out_val<double, double>(double v) { return v; }
 
-// One stage: acc[p][i][j] += sum_k A_p[k][line i] B_p[k][mode j] for both parities p.  In FP32 the stage's
-// sum is formed apart and added once, which keeps the rounding error of a long line that of a short
-// sum (128 points: 0.94e-7 of the result's norm instead of 1.5e-7, 1280: 1.5e-7).
+// One stage: acc[p][i][j] += sum_k A_p[k][line i] B_p[k][mode j] for both parities p.
 template <class T, int TM>
-__device__ __forceinline__ void sine_stage(T (&sum)[2][TM][4], const T *a0, const T *a1, const T *b0, const T *b1) {
+__device__ __forceinline__ void sine_stage(T (&acc)[2][TM][4], const T *a0, const T *a1, const T *b0, const T *b1) {
     constexpr int LD = 16 * TM + 4;
-    constexpr bool kApart = sizeof(T) == 4;
-    T part[2][TM][4];
-    T (&acc)[2][TM][4] = kApart ? part : sum;
-    if constexpr (kApart) {
-#pragma unroll
-        for (int p = 0; p < 2; ++p)
-#pragma unroll
-            for (int i = 0; i < TM; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) part[p][i][j] = T(0);
-    }
 #pragma unroll 4
     for (int k = 0; k < kBK; ++k) {
         T a[2][TM], b[2][4];
@@ -72,14 +43,6 @@ __device__ __forceinline__ void sine_stage(T (&sum)[2][TM][4], const T *a0, cons
             for (int i = 0; i < TM; ++i)
 #pragma unroll
                 for (int j = 0; j < 4; ++j) acc[p][i][j] = fma(a[p][i], b[p][j], acc[p][i][j]);
-    }
-    if constexpr (kApart) {
-#pragma unroll
-        for (int p = 0; p < 2; ++p)
-#pragma unroll
-            for (int i = 0; i < TM; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) sum[p][i][j] += part[p][i][j];
     }
 }
 
@@ -144,7 +107,7 @@ __device__ __forceinline__ void sine_in_body(const SineArgs &g, const double *__
         const bool two = k0 + lx < ne;  // the middle point of an odd line has no partner: odd modes only
 #pragma unroll
         for (int i = 0; i < NL; ++i) {
-            const T u = in_val<T>(ra[i]), v = in_val<T>(rb[i]);
+            const T u = ra[i], v = rb[i];
             s.a[buf][0][lx * LD + ll + i * (128 / kBK)] = u + v;
             s.a[buf][1][lx * LD + ll + i * (128 / kBK)] = two ? u - v : T(0);
         }
@@ -192,14 +155,6 @@ __global__ void __launch_bounds__(128) sine_in_kernel(const __grid_constant__ Si
     pdl_trigger();
     const long long rhs = blockIdx.z;
     sine_in_body<T>(g, f + rhs * g.nx * g.ny * g.nz, out + rhs * g.nx * g.nz * g.pitch, blockIdx.x, blockIdx.y, smem_raw);
-}
-__global__ void __launch_bounds__(128) sine_in_batch_kernel(const SineJob *__restrict__ jobs, const SineTile *__restrict__ tiles,
-                                                        const int *active) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const SineTile t = tiles[blockIdx.x];
-    if (active[t.sys] != 1) return;
-    const SineJob j = jobs[t.sys];
-    sine_in_body<float>(j.g, j.in, j.fh, t.line_tile, t.mode_tile, smem_raw);
 }
 
 // u[rhs][line][x] = sum_mode s_mode(x) uhat[rhs][mode][line]: both parities' sums for 32 points and their
@@ -275,8 +230,8 @@ __device__ __forceinline__ void sine_out_body(const SineArgs &g, const T *__rest
     for (int i = tid >> 5; i < BM; i += 4) {
         const long long o = s.off[i];
         if (o < 0) continue;
-        if (x < g.nh) ur[o + x] = out_val<S, T>(w[i * LS + lane]);
-        if (x < ne) ur[o + g.nx - 1 - x] = out_val<S, T>(w[i * LS + kBN + lane]);
+        if (x < g.nh) ur[o + x] = static_cast<S>(w[i * LS + lane]);
+        if (x < ne) ur[o + g.nx - 1 - x] = static_cast<S>(w[i * LS + kBN + lane]);
     }
 }
 
@@ -286,14 +241,6 @@ __global__ void __launch_bounds__(128) sine_out_kernel(const __grid_constant__ S
     pdl_trigger();
     const long long rhs = blockIdx.z;
     sine_out_body<T, S>(g, uh + rhs * g.nx * g.nz * g.pitch, u + rhs * g.nx * g.ny * g.nz, blockIdx.x, blockIdx.y, smem_raw);
-}
-__global__ void __launch_bounds__(128) sine_out_batch_kernel(const SineJob *__restrict__ jobs, const SineTile *__restrict__ tiles,
-                                                         const int *active) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const SineTile t = tiles[blockIdx.x];
-    if (active[t.sys] != 1) return;
-    const SineJob j = jobs[t.sys];
-    sine_out_body<float, float>(j.g, j.uh, j.out, t.line_tile, t.mode_tile, smem_raw);
 }
 
 // ---- prolongation and correction on a level above the tail -------------------------------------------
@@ -561,7 +508,7 @@ void modal_place(ModalHost<T> &h, unsigned char *shared, T *coef, double *coef64
 template <class T>
 std::vector<T> sine_matrices(int nx) {
     const int nh = (nx + 1) / 2;
-    const size_t hp = up(nh, 32);
+    const size_t hp = up(nh, 64);
     const double pi = 3.14159265358979323846, sc = std::sqrt(2.0 / (nx + 1));
     std::vector<T> mat(4 * hp * hp, T(0));
     std::vector<double> sines(2 * (nx + 1));
@@ -610,7 +557,7 @@ int build(ModalPlan &p, ModalHost<T> &h, const HostHierarchy &H, int npre, int n
     const std::vector<T> mat = sine_matrices<T>(H.nx);
     MCHK(cudaMalloc(&p.d_sin, mat.size() * sizeof(T)));
     MCHK(cudaMemcpy(p.d_sin, mat.data(), mat.size() * sizeof(T), cudaMemcpyHostToDevice));
-    p.sine = SineArgs{H.nx, H.ny, H.nz, h.a.pitch, (H.nx + 1) / 2, static_cast<int>(up((H.nx + 1) / 2, 32)), p.d_sin};
+    p.sine = SineArgs{H.nx, H.ny, H.nz, h.a.pitch, (H.nx + 1) / 2, static_cast<int>(up((H.nx + 1) / 2, 64)), p.d_sin};
     MCHK(cudaMalloc(&p.d_args, sizeof(h.a)));
     MCHK(cudaMemcpy(p.d_args, &h.a, sizeof(h.a), cudaMemcpyHostToDevice));
     int dev = 0;
@@ -691,9 +638,11 @@ int modal_build(ModalPlan &p, const HostHierarchy &H, bool f64, int nb, int npre
     return f64 ? build<double>(p, p.h64, H, npre, npost, coarse_iters) : build<float>(p, p.h32, H, npre, npost, coarse_iters);
 }
 
-cudaError_t modal_transform_in(const ModalPlan &p, int nb, const double *f0, cudaStream_t st, long long &launches) {
+cudaError_t modal_transform_in(const ModalPlan &p, int nb, Prec type, const void *f0, cudaStream_t st, long long &launches) {
+    // long lines are folded into the iterate's place first: nothing of it is needed yet
+    if (!p.f64) return sine_in_f32(p.sine, nb, type, f0, p.h32.a.fw[0], p.h32.a.u[0], st, launches);
     launches += 1;
-    return p.f64 ? sine_in<double>(p, nb, f0, p.h64.a.fw[0], st) : sine_in<float>(p, nb, f0, p.h32.a.fw[0], st);
+    return sine_in<double>(p, nb, static_cast<const double *>(f0), p.h64.a.fw[0], st);
 }
 
 cudaError_t modal_cycle(const ModalPlan &p, int nb, cudaStream_t st, long long &launches) {
@@ -701,32 +650,9 @@ cudaError_t modal_cycle(const ModalPlan &p, int nb, cudaStream_t st, long long &
 }
 
 cudaError_t modal_transform_out(const ModalPlan &p, int nb, Prec type, void *u0, cudaStream_t st, long long &launches) {
+    if (!p.f64) return sine_out_f32(p.sine, nb, p.h32.a.u[0], type, u0, st, launches);
     launches += 1;
-    if (p.f64) return sine_out<double, double>(p, nb, p.h64.a.u[0], u0, st);
-    if (type == Prec::F64) return sine_out<float, double>(p, nb, p.h32.a.u[0], u0, st);
-    if (type == Prec::BF16) return sine_out<float, __nv_bfloat16>(p, nb, p.h32.a.u[0], u0, st);
-    return sine_out<float, float>(p, nb, p.h32.a.u[0], u0, st);
-}
-
-int sine_line_tiles(const SineArgs &g) {
-    constexpr int BM = 16 * tm_lines<float>();
-    return static_cast<int>((static_cast<long long>(g.nz) * g.pitch + BM - 1) / BM);
-}
-int sine_mode_tiles(const SineArgs &g) { return (g.nh + kBN - 1) / kBN; }
-
-cudaError_t launch_sine_in_batch(const SineJob *jobs, const SineTile *tiles, int ntiles, const int *active, cudaStream_t st) {
-    constexpr size_t smem = sizeof(SineSmem<float, tm_lines<float>()>);
-    cudaError_t e = raise_smem_attr(reinterpret_cast<const void *>(&sine_in_batch_kernel), smem);
-    if (e != cudaSuccess) return e;
-    sine_in_batch_kernel<<<ntiles, 128, smem, st>>>(jobs, tiles, active);
-    return cudaGetLastError();
-}
-cudaError_t launch_sine_out_batch(const SineJob *jobs, const SineTile *tiles, int ntiles, const int *active, cudaStream_t st) {
-    constexpr size_t smem = sizeof(SineSmem<float, tm_lines<float>()>);
-    cudaError_t e = raise_smem_attr(reinterpret_cast<const void *>(&sine_out_batch_kernel), smem);
-    if (e != cudaSuccess) return e;
-    sine_out_batch_kernel<<<ntiles, 128, smem, st>>>(jobs, tiles, active);
-    return cudaGetLastError();
+    return sine_out<double, double>(p, nb, p.h64.a.u[0], u0, st);
 }
 
 cudaError_t launch_modal_prolong(const ModalArgs<float> &a, int l, int nb, cudaStream_t st) { return prolong(a, l, nb, st); }

@@ -65,7 +65,7 @@ constexpr size_t kModalSmem = 227 * 1024 - 2048;
 struct SineArgs {
     int nx, ny, nz, pitch;   // pitch: lines per plane of the mode vectors (lines ny .. pitch-1 are zero)
     int nh;                  // odd modes, and pairs of points: ceil(nx / 2)
-    int hp;                  // order of the stored matrices (nh rounded up to 32)
+    int hp;                  // order of the stored matrices (nh rounded up to 64)
     const void *mat;         // [4][hp][hp]: by point odd, even; by mode odd, even
 };
 
@@ -108,10 +108,10 @@ struct ModalPlan {
 int modal_build(ModalPlan &p, const HostHierarchy &H, bool f64, int nb, int npre, int npost, int coarse_iters);
 void modal_free(ModalPlan &p);
 
-// u0 = T f0 for nb right-hand sides, in three parts: f0 (FP64, [rhs][z][y][x]) into mode space, the
-// cycle there, and back into u0 (elements of type `type`).  Each adds its kernel launches to
+// u0 = T f0 for nb right-hand sides, in three parts: f0 ([rhs][z][y][x], of type F64, or F32 for an FP32
+// plan) into mode space, the cycle there, and back into u0 (elements of type `type`).  Each adds its kernel launches to
 // `launches`.  Asynchronous on st.
-cudaError_t modal_transform_in(const ModalPlan &p, int nb, const double *f0, cudaStream_t st, long long &launches);
+cudaError_t modal_transform_in(const ModalPlan &p, int nb, Prec type, const void *f0, cudaStream_t st, long long &launches);
 cudaError_t modal_cycle(const ModalPlan &p, int nb, cudaStream_t st, long long &launches);
 cudaError_t modal_transform_out(const ModalPlan &p, int nb, Prec type, void *u0, cudaStream_t st, long long &launches);
 
@@ -119,7 +119,7 @@ cudaError_t modal_transform_out(const ModalPlan &p, int nb, Prec type, void *u0,
 // from lists of (system, tile) and (system, mode); systems whose active flag is not 1 are skipped.
 struct SineJob {
     SineArgs g;
-    const double *in;      // physical right-hand side
+    const float *in;       // physical right-hand side
     float *fh;             // mode-space right-hand side and result
     const float *uh;
     float *out;            // physical result
@@ -127,6 +127,10 @@ struct SineJob {
 struct SineTile {
     int sys, line_tile, mode_tile;
 };
+// FP32 transforms (sine.cu) of physical vectors with elements of type `type` (forward: F32 or F64); scratch: as
+// many values as out.
+cudaError_t sine_in_f32(const SineArgs &g, int nb, Prec type, const void *f, float *out, float *scratch, cudaStream_t st, long long &launches);
+cudaError_t sine_out_f32(const SineArgs &g, int nb, const float *a, Prec type, void *u, cudaStream_t st, long long &launches);
 int sine_line_tiles(const SineArgs &g);
 int sine_mode_tiles(const SineArgs &g);
 cudaError_t launch_sine_in_batch(const SineJob *jobs, const SineTile *tiles, int ntiles, const int *active, cudaStream_t st);
