@@ -11,8 +11,7 @@
 // 16 LT lines by 32 columns of each parity, a thread LT lines by 4 columns of each, in packed pairs of
 // lines (fma.rn.f32x2, two cycles of the FMA pipe each: at LT = 8 32 of them a step, against 6
 // shared-memory reads of 16 bytes and 8 moves that duplicate B's values).  LT = 8 while that gives every SM
-// three CTAs (12 warps; 8 warps of twice the columns reached 60% of the FMA pipe and lost a fifth of it to
-// the last wave at 1280 points), LT = 4 for smaller problems.  Operands come by cp.async three stages
+// its CTAs, LT = 4 for smaller problems.  Operands come by cp.async three stages
 // ahead.  Each stage's sum (16 terms) is formed apart and added once, which keeps the rounding error
 // of a long line that of a short sum (128 points: 0.94e-7 of the result's norm instead of 1.5e-7, 1280:
 // 1.5e-7).
@@ -114,23 +113,37 @@ template <int LT>
 __device__ __forceinline__ void stage_sum(Acc<LT> &acc, const Smem<LT> &s, int st, int ty, int tx) {
     constexpr int LD = Smem<LT>::LD;
     Acc<LT> part;
-#pragma unroll
-    for (int k = 0; k < kBK; ++k) {
+    // LT = 8, two CTAs an SM: the next term's operands are read while one is multiplied (at three CTAs, 168
+    // registers a thread, the compiler reads them when they are needed: 270 instead of 235 us at 1280 points)
+    constexpr bool kAhead = LT == 8;
+    f32x2 av[2][2][LT / 2];
+    float4 bq[2][2];
+    auto read = [&](int k, int to) {
 #pragma unroll
         for (int par = 0; par < 2; ++par) {
-            f32x2 av[LT / 2];
 #pragma unroll
             for (int h = 0; h < LT / 4; ++h) {
                 const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(&s.a[st][par][k * LD + ty * LT + 4 * h]);
-                av[2 * h] = v.x;
-                av[2 * h + 1] = v.y;
+                av[to][par][2 * h] = v.x;
+                av[to][par][2 * h + 1] = v.y;
             }
-            const float4 b = *reinterpret_cast<const float4 *>(&s.b[st][par][k * kBN + tx * 4]);
+            bq[to][par] = *reinterpret_cast<const float4 *>(&s.b[st][par][k * kBN + tx * 4]);
+        }
+    };
+    if (kAhead) read(0, 0);
+#pragma unroll
+    for (int k = 0; k < kBK; ++k) {
+        const int c = kAhead ? k & 1 : 0;
+        if (!kAhead) read(k, 0);
+        else if (k + 1 < kBK) read(k + 1, c ^ 1);
+#pragma unroll
+        for (int par = 0; par < 2; ++par) {
+            const float4 b = bq[c][par];
             const f32x2 bv[4] = {dup2(b.x), dup2(b.y), dup2(b.z), dup2(b.w)};
 #pragma unroll
             for (int j = 0; j < 4; ++j)
 #pragma unroll
-                for (int i = 0; i < LT / 2; ++i) part[par][j][i] = k == 0 ? mul2(av[i], bv[j]) : fma2(av[i], bv[j], part[par][j][i]);
+                for (int i = 0; i < LT / 2; ++i) part[par][j][i] = k == 0 ? mul2(av[c][par][i], bv[j]) : fma2(av[c][par][i], bv[j], part[par][j][i]);
         }
     }
 #pragma unroll
@@ -305,7 +318,7 @@ __global__ void __launch_bounds__(256) fold_kernel(const __grid_constant__ SineA
 }
 
 template <int LT>
-__global__ void __launch_bounds__(kNT, LT == 8 ? 3 : 4) in_kernel(const __grid_constant__ SineArgs g, const float *__restrict__ a, float *__restrict__ out) {
+__global__ void __launch_bounds__(kNT, LT == 8 ? 2 : 4) in_kernel(const __grid_constant__ SineArgs g, const float *__restrict__ a, float *__restrict__ out) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     pdl_trigger();
     pdl_wait();
@@ -371,14 +384,14 @@ __device__ __forceinline__ void out_body(const SineArgs &g, const float *__restr
     }
 }
 template <int LT, class S>
-__global__ void __launch_bounds__(kNT, LT == 8 ? 3 : 4) out_kernel(const __grid_constant__ SineArgs g, const float *__restrict__ a,
+__global__ void __launch_bounds__(kNT, LT == 8 ? 2 : 4) out_kernel(const __grid_constant__ SineArgs g, const float *__restrict__ a,
                                                             S *__restrict__ u) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     pdl_trigger();
     const long long rhs = blockIdx.z;
     out_body<LT, S>(g, a + rhs * g.nx * g.nz * g.pitch, u + rhs * g.nx * g.ny * g.nz, blockIdx.x, blockIdx.y, smem_raw);
 }
-__global__ void __launch_bounds__(kNT, 3) out_batch_kernel(const SineJob *__restrict__ jobs, const SineTile *__restrict__ tiles, const int *active) {
+__global__ void __launch_bounds__(kNT, 2) out_batch_kernel(const SineJob *__restrict__ jobs, const SineTile *__restrict__ tiles, const int *active) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const SineTile t = tiles[blockIdx.x];
     if (active[t.sys] != 1) return;
@@ -393,7 +406,7 @@ dim3 grid_of(const SineArgs &g, int nb) {
     const long long lines = static_cast<long long>(g.nz) * g.pitch;
     return dim3(static_cast<unsigned>((lines + 16 * LT - 1) / (16 * LT)), (g.nh + kBN - 1) / kBN, nb);
 }
-// Whether 128-line tiles give every SM its three CTAs.
+// Whether 128-line tiles give every SM three CTAs (two run at once; a third evens out the last wave).
 bool wide_tiles(const SineArgs &g, int nb) {
     const dim3 d = grid_of<8>(g, nb);
     return static_cast<long long>(d.x) * d.y * d.z >= 3 * 152;
