@@ -23,6 +23,7 @@
 #include "gram_tc.h"
 #include "lobpcg.h"
 #include "plane_relax.cuh"  // widen_f32 / narrow_f64 (integer-pipe conversions)
+#include "reduce.cuh"
 
 namespace smg {
 
@@ -161,54 +162,65 @@ __global__ void __launch_bounds__(256, 4) gram_partial_kernel(long long n, long 
 }
 
 // Partial Gram of a narrow product (k1, k2 <= kSmallK): thread t of CTA `chunk` accumulates all
-// k1 x k2 entries over rows chunk*rows + t, + 256, ... (coalesced loads of each column, no
-// padding work), and the CTA adds its 256 partial sums in FP64; part[] takes the tiled kernel's
-// layout (one 16 x 16 tile) so the same reduction follows.
+// k1 x k2 entries over rows chunk*rows + t, + blockDim, ... (coalesced loads of each column, no
+// padding work), and the CTA adds its partial sums in FP64; part[] takes the tiled kernel's
+// layout (one 16 x 16 tile) so the same reduction follows.  Bound by the FP32 and integer work of
+// the rows (about 190 instructions a row at k1 = k2 = 3).  One CTA of 1024 threads per SM, and its sums
+// folded on full warps: a shuffle tree in each of 32 warps an SM for all 16 entries, wanted or not,
+// took 41K cycles of FP64 issue (1.02M rows, k1 = k2 = 3: 54 us).
 constexpr int kSmallK = 4;
-__global__ void __launch_bounds__(256) gram_small_kernel(long long n, long long rows, int k1, int k2,
-                                                         const double *__restrict__ U, const double *__restrict__ V,
-                                                         double *__restrict__ part) {
-    __shared__ double red[8][kSmallK * kSmallK];
+constexpr int kSmallThreads = 1024;
+template <int K1, int K2>
+__global__ void __launch_bounds__(kSmallThreads) gram_small_kernel(long long n, long long rows, const double *__restrict__ U,
+                                                                const double *__restrict__ V, double *__restrict__ part) {
     const long long r0 = static_cast<long long>(blockIdx.x) * rows;
     const long long r1 = min(n, r0 + rows);
-    float S[kSmallK][kSmallK], sl[kSmallK][kSmallK];
+    float S[K1][K2], sl[K1][K2];
 #pragma unroll
-    for (int i = 0; i < kSmallK; ++i)
+    for (int i = 0; i < K1; ++i)
 #pragma unroll
-        for (int j = 0; j < kSmallK; ++j) S[i][j] = sl[i][j] = 0.0f;
-    for (long long r = r0 + threadIdx.x; r < r1; r += blockDim.x) {
-        float uh[kSmallK], ul[kSmallK], vh[kSmallK], vl[kSmallK];
+        for (int j = 0; j < K2; ++j) S[i][j] = sl[i][j] = 0.0f;
+    double nu[K1], nv[K2];   // the next row's values are on their way while one row is accumulated
+    auto fetch = [&](long long r) {
 #pragma unroll
-        for (int i = 0; i < kSmallK; ++i) {
-            df_split(i < k1 ? U[static_cast<long long>(i) * n + r] : 0.0, uh[i], ul[i]);
-            df_split(i < k2 ? V[static_cast<long long>(i) * n + r] : 0.0, vh[i], vl[i]);
-        }
+        for (int i = 0; i < K1; ++i) nu[i] = U[static_cast<long long>(i) * n + r];
 #pragma unroll
-        for (int i = 0; i < kSmallK; ++i)
+        for (int j = 0; j < K2; ++j) nv[j] = V[static_cast<long long>(j) * n + r];
+    };
+    long long r = r0 + threadIdx.x;
+    if (r < r1) fetch(r);
+    for (; r < r1; r += kSmallThreads) {
+        float uh[K1], ul[K1], vh[K2], vl[K2];
 #pragma unroll
-            for (int j = 0; j < kSmallK; ++j)
-                if (i < k1 && j < k2) df_mac(S[i][j], sl[i][j], uh[i], ul[i], vh[j], vl[j]);
+        for (int i = 0; i < K1; ++i) df_split(nu[i], uh[i], ul[i]);
+#pragma unroll
+        for (int j = 0; j < K2; ++j) df_split(nv[j], vh[j], vl[j]);
+        if (r + kSmallThreads < r1) fetch(r + kSmallThreads);
+#pragma unroll
+        for (int i = 0; i < K1; ++i)
+#pragma unroll
+            for (int j = 0; j < K2; ++j) df_mac(S[i][j], sl[i][j], uh[i], ul[i], vh[j], vl[j]);
     }
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
-    for (int i = 0; i < kSmallK; ++i)
+    for (int i = 0; i < K1; ++i)
 #pragma unroll
-        for (int j = 0; j < kSmallK; ++j) {
-            double v = df_value(S[i][j], sl[i][j]);
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-            if (lane == 0) red[w][i * kSmallK + j] = v;
+        for (int j = 0; j < K2; ++j) {
+            double v[1] = {df_value(S[i][j], sl[i][j])};
+            block_reduce_plain<1>(v);
+            if (threadIdx.x == 0) part[static_cast<long long>(blockIdx.x) * kGT * kGT + i * kGT + j] = v[0];
+            __syncthreads();
         }
-    __syncthreads();
-    if (threadIdx.x < kSmallK * kSmallK) {
-        const int i = threadIdx.x / kSmallK, j = threadIdx.x % kSmallK;
-        double v = 0.0;
-        for (int q = 0; q < 8; ++q) v += red[q][threadIdx.x];
-        part[static_cast<long long>(blockIdx.x) * kGT * kGT + i * kGT + j] = v;
-    }
+}
+using GramSmall = void (*)(long long, long long, const double *, const double *, double *);
+GramSmall gram_small_of(int k1, int k2) {
+#define SMG_GS(a) {gram_small_kernel<a, 1>, gram_small_kernel<a, 2>, gram_small_kernel<a, 3>, gram_small_kernel<a, 4>}
+    static const GramSmall table[kSmallK][kSmallK] = {SMG_GS(1), SMG_GS(2), SMG_GS(3), SMG_GS(4)};
+#undef SMG_GS
+    return table[k1 - 1][k2 - 1];
 }
 
 // G[i][j] (k1 x k2 row-major) = sum over chunks of the partial tiles (compensated summation), one
-// warp per entry: the lanes take every 32nd chunk, then the warp combines its 32 sums.  With
+// warp per entry: the lanes take every 32nd chunk, then the warp adds its 32 sums exactly.  With
 // sym, entries below the diagonal tiles come from the mirrored tile.
 __device__ __forceinline__ void two_sum_add(double &s, double &c, double v) {
     const double t = s + v;
@@ -231,12 +243,9 @@ __global__ void gram_reduce_kernel(int nchunks, int k1, int k2, int ntj, int nti
     const long long off = static_cast<long long>(tile) * kGT * kGT + (i - ti * kGT) * kGT + (j - tj * kGT);
     double s = 0.0, c = 0.0;
     for (int ch = lane; ch < nchunks; ch += 32) two_sum_add(s, c, part[static_cast<long long>(ch) * ntiles * kGT * kGT + off]);
-    for (int o = 16; o > 0; o >>= 1) {
-        const double so = __shfl_down_sync(0xffffffffu, s, o), co = __shfl_down_sync(0xffffffffu, c, o);
-        two_sum_add(s, c, so);
-        c += co;
-    }
-    if (lane == 0) G[idx] = s + c;
+    const double p[2] = {s, isfinite(s) ? c : 0.0};
+    const double t = warp_sum_exact<2>(p);  // the lanes' sums, rounded once
+    if (lane == 0) G[idx] = t;
 }
 
 // Y = alpha * U C + beta * Y  (U: n x k, C: k x m2 row-major, Y: n x m2, column stride n), the
@@ -290,7 +299,8 @@ __global__ void block_mul_kernel(long long n, int k, int m2, const double *U, co
         if (j < nc) {
             const double acc = df_value(S[j], sl[j]);
             double *y = Y + static_cast<long long>(j0 + j) * n + r;
-            *y = (beta == 0.0) ? alpha * acc : fma(alpha, acc, beta * *y);
+            // an FP64 operation a value is half of a narrow product's time: none for alpha = 1, beta = 0
+            *y = (beta == 0.0) ? (alpha == 1.0 ? acc : alpha * acc) : fma(alpha, acc, beta * *y);
         }
     }
 }
@@ -565,11 +575,11 @@ int gram(Ctx &c, int k1, const double *U, int k2, const double *V, std::vector<d
         return SMG_OK;
     }
     if (k1 <= kSmallK && k2 <= kSmallK) {
-        // narrow product: 4 CTAs per SM (as far as the partial buffer holds), rows a multiple of 256
-        const long long want = std::max<long long>(1, std::min<long long>(4LL * c.w.num_sms, c.w.part_tiles));
-        const long long rows = ((c.n + want - 1) / want + 255) / 256 * 256;
+        // narrow product: one CTA per SM (as far as the partial buffer holds)
+        const long long want = std::max<long long>(1, std::min<long long>(c.w.num_sms, c.w.part_tiles));
+        const long long rows = std::max<long long>((c.n + want - 1) / want, 1);
         const int nch = static_cast<int>(cdiv(c.n, rows));
-        gram_small_kernel<<<nch, 256, 0, c.st>>>(c.n, rows, k1, k2, U, V, c.w.part);
+        gram_small_of(k1, k2)<<<nch, kSmallThreads, 0, c.st>>>(c.n, rows, U, V, c.w.part);
         LCHK(cudaGetLastError());
         gram_reduce_kernel<<<cdiv(static_cast<long long>(k1) * k2 * 32, 256), 256, 0, c.st>>>(
             nch, k1, k2, 1, 1, c.w.part, c.w.gram, 0);
