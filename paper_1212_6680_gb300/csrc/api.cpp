@@ -1397,6 +1397,7 @@ int smg_destroy(smg_handle h) {
     for (auto e : h->event_pool) cudaEventDestroy(e);
     lobpcg_free(h->lw);
     net_free(h->nw);
+    net_pool_trim();
     drop_solve_graph(h);
     if (h->gs) cudaStreamDestroy(h->gs);
     if (h->gev) cudaEventDestroy(h->gev);

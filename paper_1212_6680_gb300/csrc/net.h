@@ -34,6 +34,10 @@ struct NetScal {
     int pad;
 };
 
+// Where a NetWork's memory comes from: its own allocations (it lives with a handle), or the device's pool
+// in the order of one stream (it lives for one call).
+enum class NetMem { Own, Pool };
+
 // Buffers for one grid size.  act: 0 BF16 activations, 1 FP32.
 struct NetWork {
     long long n = 0;
@@ -52,11 +56,17 @@ struct NetWork {
     float *grad = nullptr, *m = nullptr, *v = nullptr;  // training
     float *wpart = nullptr;              // per-block weight-gradient partials
     int wpart_blocks = 0;
+    void *slab = nullptr;                // the block that holds all of the above but
+    void *weights = nullptr;             // w, m and v
+    NetMem mem = NetMem::Own;
+    cudaStream_t st = nullptr;           // NetMem::Pool: the call's stream
     long long launches = 0;
 };
 
-cudaError_t net_alloc(NetWork &nw, long long n, int act, bool training);
+cudaError_t net_alloc(NetWork &nw, long long n, int act, bool training, NetMem mem = NetMem::Own, cudaStream_t st = nullptr);
 void net_free(NetWork &nw);
+// Hand the current device's idle pool memory back.
+void net_pool_trim();
 
 // delta = rms(rho) Net(rho / rms(rho)) from nw.rho (FP32) into nw.delta; keeps a1, a2.
 cudaError_t net_forward(NetWork &nw, int nx, int ny, int nz, cudaStream_t st);

@@ -63,7 +63,7 @@ extern "C" int smg_net_forward(int nx, int ny, int nz, int act_prec, const float
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const long long n = static_cast<long long>(nx) * ny * nz;
     NetWork nw;
-    NET_CUDA(net_alloc(nw, n, act, false));
+    NET_CUDA(net_alloc(nw, n, act, false, NetMem::Pool, st));
     NET_CUDA(cudaMemcpyAsync(nw.w, w, kNetWeights * sizeof(float), cudaMemcpyHostToDevice, st));
     NET_CUDA(net_to_f32(n, rho, nw.rho, st));
     NET_CUDA(net_forward(nw, nx, ny, nz, st));
@@ -82,7 +82,7 @@ extern "C" int smg_net_loss_grad(int nx, int ny, int nz, int act_prec, const flo
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const long long n = static_cast<long long>(nx) * ny * nz;
     NetWork nw;
-    NET_CUDA(net_alloc(nw, n, act, true));
+    NET_CUDA(net_alloc(nw, n, act, true, NetMem::Pool, st));
     NET_CUDA(cudaMemcpyAsync(nw.w, w, kNetWeights * sizeof(float), cudaMemcpyHostToDevice, st));
     NET_CUDA(net_to_f32(n, rho, nw.rho, st));
     NET_CUDA(net_to_f32(n, e, nw.e, st));
@@ -111,7 +111,7 @@ extern "C" int smg_net_train(int npairs, const int *dims, const float *const *rh
     }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     NetWork nw;
-    NET_CUDA(net_alloc(nw, nmax, act, true));
+    NET_CUDA(net_alloc(nw, nmax, act, true, NetMem::Pool, st));
     NET_CUDA(cudaMemcpyAsync(nw.w, w, kNetWeights * sizeof(float), cudaMemcpyHostToDevice, st));
     // the pairs are read in place: the work buffers' own input / target arrays are set aside
     float *own_rho = nw.rho, *own_e = nw.e;
