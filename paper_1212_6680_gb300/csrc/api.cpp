@@ -141,6 +141,7 @@ struct smg_ctx {
         long long gen = -1;
         const double *x = nullptr;  // the iterate the graph's kernels update
         bool ident = false;
+        Dots dots = Dots::Kernel;
         long long body_launches = 0;
     } sg;
     cudaStream_t gs = nullptr;      // capture and launch stream of the graph
@@ -735,8 +736,8 @@ void drop_solve_graph(smg_ctx *h) {
 // one iteration -- the V-cycle s = T r (unless T = I) and the four Krylov kernels -- captured from
 // the same launch code as the host loop.  Returns false when the graph cannot be built (the host
 // loop is used then).
-bool ensure_solve_graph(smg_ctx *h, void *f0, void *u0, Prec kp, void *f0k, bool ident, double *x) {
-    if (h->sg.exec && h->sg.gen == h->gen && h->sg.x == x && h->sg.ident == ident) return true;
+bool ensure_solve_graph(smg_ctx *h, void *f0, void *u0, Prec kp, void *f0k, bool ident, Dots dots, double *x) {
+    if (h->sg.exec && h->sg.gen == h->gen && h->sg.x == x && h->sg.ident == ident && h->sg.dots == dots) return true;
     drop_solve_graph(h);
     if (h->gs == nullptr && cudaStreamCreateWithFlags(&h->gs, cudaStreamNonBlocking) != cudaSuccess) return false;
     if (h->gev == nullptr && cudaEventCreateWithFlags(&h->gev, cudaEventDisableTiming) != cudaSuccess) return false;
@@ -760,8 +761,8 @@ bool ensure_solve_graph(smg_ctx *h, void *f0, void *u0, Prec kp, void *f0k, bool
         if (ok) {
             bool launched = ident || run_cycle(h, 1, f0, u0, h->gs) == SMG_OK;
             launched = launched && kry_iteration_tail(kp, h->nx, h->ny, h->nz, u0, x, h->d_r, h->d_p, h->d_q,
-                                                      f0k, h->kw, h->gs, cond, 1) == cudaSuccess;
-            h->launches += 4;
+                                                      f0k, h->kw, dots, h->gs, cond, 1) == cudaSuccess;
+            h->launches += dots == Dots::Kernel ? 4 : 3;
             cudaGraph_t out = nullptr;
             ok = (cudaStreamEndCapture(h->gs, &out) == cudaSuccess) && launched;
         }
@@ -781,6 +782,7 @@ bool ensure_solve_graph(smg_ctx *h, void *f0, void *u0, Prec kp, void *f0k, bool
     h->sg.gen = h->gen;
     h->sg.x = x;
     h->sg.ident = ident;
+    h->sg.dots = dots;
     return true;
 }
 
@@ -805,10 +807,11 @@ int krylov_device(smg_ctx *h, int variant, const double *b, double *x, double to
     const Prec kp = ident ? Prec::F64 : h->prec;                    // storage type of s
     void *f0k = (own_f0 && !ident) ? f0 : nullptr;                  // what the Krylov kernels write
     const double tol2 = tol * tol;
+    const Dots dots = ident && !h->kw.fused ? Dots::Ident : Dots::Kernel;  // the fused tail forms its own
     // the device-side loop: not with the learned correction, training-pair capture or per-launch
     // profiling (their host-side steps and events sit between the kernels of an iteration)
     const bool graph = h->use_graph && !h->learned && h->cap.count >= h->cap.max && h->profile == 0 &&
-                       ensure_solve_graph(h, f0, u0, kp, f0k, ident, x);
+                       ensure_solve_graph(h, f0, u0, kp, f0k, ident, dots, x);
     cudaStream_t ls = st;  // the stream the solve runs on
     if (graph) {
         SMG_CUDA(cudaEventRecord(h->gev, st));
@@ -882,9 +885,9 @@ int krylov_device(smg_ctx *h, int variant, const double *b, double *x, double to
         }
         {
             RegionTimer rt(h, ls, 4, 0.0);
-            SMG_CUDA(kry_iteration_tail(kp, h->nx, h->ny, h->nz, u0, x, h->d_r, h->d_p, h->d_q, f0k, h->kw, ls));
+            SMG_CUDA(kry_iteration_tail(kp, h->nx, h->ny, h->nz, u0, x, h->d_r, h->d_p, h->d_q, f0k, h->kw, dots, ls));
         }
-        h->launches += 4;
+        h->launches += dots == Dots::Kernel ? 4 : 3;
         k += 1;
         if ((rc = read_scalars(h, ls)) != SMG_OK) return rc;
     }

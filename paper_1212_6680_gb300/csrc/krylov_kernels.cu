@@ -118,6 +118,8 @@ __global__ void __launch_bounds__(kMaxThreads) k_init_residual(int nx, int ny, i
         sc->rr = tot[0];
         sc->bb = tot[1];
         sc->restart = 1;
+        sc->rho = tot[0];  // T = I: the first step's scalars
+        sc->beta = 0.0;
         if (!isfinite(tot[0]) || !isfinite(tot[1])) sc->status = -6;
     }
 }
@@ -156,28 +158,29 @@ __global__ void __launch_bounds__(kMaxThreads) k_dots_beta(long long n, const S 
     }
     double v[2] = {a0, a1};
     double tot[2];
-    if (grid_reduce<2>(v, part, counter, tot) && threadIdx.x == 0) {
-        const double rho = tot[0], sdr = -sc->alpha * tot[1];
-        double beta = 0.0;
-        if (sc->restart == 0 && variant != 2) {
-            if (sc->rho_prev == 0.0) {
-                sc->status = -4;
-            } else {
-                beta = (variant == 0) ? rho / sc->rho_prev : sdr / sc->rho_prev;
-            }
-        }
-        if (!isfinite(rho) || !isfinite(beta)) sc->status = -6;
-        sc->rho = rho;
-        sc->sdr = sdr;
-        sc->beta = beta;
-    }
+    if (grid_reduce<2>(v, part, counter, tot) && threadIdx.x == 0) finish_dots(sc, tot[0], tot[1]);
+}
+
+// T = I: after the x/r update, whose rr is the next rho and sq = (r, q) (flexible variant only), the next
+// step's beta.  It is judged when that step begins (ident_status): the solve may be over.
+__device__ __forceinline__ void ident_dots(KrylovScalars *sc, double sq) {
+    const double rho = sc->rr, sdr = -sc->alpha * sq;
+    sc->rho = rho;
+    sc->sdr = sdr;
+    sc->beta = sc->variant == 2 || sc->rho_prev == 0.0 ? 0.0 : (sc->variant == 0 ? rho : sdr) / sc->rho_prev;
+}
+__device__ __forceinline__ void ident_status(KrylovScalars *sc) {
+    if (blockIdx.x != 0 || threadIdx.x != 0) return;
+    if (sc->restart == 0 && sc->variant != 2 && sc->rho_prev == 0.0) sc->status = -4;
+    if (!isfinite(sc->rho) || !isfinite(sc->beta)) sc->status = -6;
 }
 
 // p = s + beta p
-template <class S>
-__global__ void __launch_bounds__(kMaxThreads) k_update_p(long long n, const S *__restrict__ s, double *__restrict__ p, const KrylovScalars *sc) {
+template <class S, bool IDENT>
+__global__ void __launch_bounds__(kMaxThreads) k_update_p(long long n, const S *__restrict__ s, double *__restrict__ p, KrylovScalars *sc) {
     pdl_trigger();
     pdl_wait();
+    if constexpr (IDENT) ident_status(sc);
     const double beta = sc->beta;
     const Share sh = cta_share(static_cast<int>(n));
     for (int i = sh.begin; i < sh.end; i += blockDim.x) {
@@ -214,8 +217,23 @@ __global__ void __launch_bounds__(kMaxThreads) k_spmv_alpha(int nx, int ny, int 
     }
 }
 
+// The x/r update's sums: rr, and for T = I (r, q).
+template <bool IDENT>
+__device__ __forceinline__ void finish_xr(double a0, double a1, KrylovScalars *sc, DSum *part, unsigned *counter,
+                                          cudaGraphConditionalHandle cond, int use_cond) {
+    if constexpr (IDENT) {
+        double v[2] = {a0, a1}, tot[2];
+        if (!grid_reduce<2>(v, part, counter, tot) || threadIdx.x != 0) return;
+        finish_update(sc, tot[0], cond, use_cond);
+        ident_dots(sc, tot[1]);
+    } else {
+        double v[1] = {a0}, tot[1];
+        if (grid_reduce<1>(v, part, counter, tot) && threadIdx.x == 0) finish_update(sc, tot[0], cond, use_cond);
+    }
+}
+
 // x += alpha p ; r_new = r - alpha q ; r = r_new ; f0 = (S) r_new ; rr = ||r_new||^2
-template <class S>
+template <class S, bool IDENT>
 __global__ void __launch_bounds__(kMaxThreads) k_update_xr(long long n, double *__restrict__ x, const double *__restrict__ p, double *__restrict__ r,
                             const double *__restrict__ q, S *__restrict__ f0,
                             KrylovScalars *sc, DSum *part, unsigned *counter, cudaGraphConditionalHandle cond,
@@ -223,18 +241,18 @@ __global__ void __launch_bounds__(kMaxThreads) k_update_xr(long long n, double *
     pdl_trigger();
     pdl_wait();
     const double alpha = sc->alpha;
-    double a0 = 0.0;
+    const bool sq = IDENT && sc->variant == 1;
+    double a0 = 0.0, a1 = 0.0;
     const Share sh = cta_share(static_cast<int>(n));
     for (int i = sh.begin; i < sh.end; i += blockDim.x) {
         x[i] = fma(alpha, p[i], x[i]);
-        const double rn = fma(-alpha, q[i], r[i]);
+        const double qi = q[i], rn = fma(-alpha, qi, r[i]);
         r[i] = rn;
         if (f0 != nullptr) stv<S, double>(f0 + i, rn);
         a0 = fma(rn, rn, a0);
+        if (sq) a1 = fma(rn, qi, a1);
     }
-    double v[1] = {a0};
-    double tot[1];
-    if (grid_reduce<1>(v, part, counter, tot) && threadIdx.x == 0) finish_update(sc, tot[0], cond, use_cond);
+    finish_xr<IDENT>(a0, a1, sc, part, counter, cond, use_cond);
 }
 
 // ---- the same four kernels on 4-element chunks ---------------------------------------------------
@@ -370,27 +388,14 @@ __global__ void __launch_bounds__(kMaxThreads) k_dots_beta4(int nc, const S *__r
     dots_share<S>(a0, a1, sh, s, r, q, need_sdr);
     double v[2] = {a0, a1};
     double tot[2];
-    if (grid_reduce<2>(v, part, counter, tot) && threadIdx.x == 0) {
-        const double rho = tot[0], sdr = -sc->alpha * tot[1];
-        double beta = 0.0;
-        if (sc->restart == 0 && variant != 2) {
-            if (sc->rho_prev == 0.0) {
-                sc->status = -4;
-            } else {
-                beta = (variant == 0) ? rho / sc->rho_prev : sdr / sc->rho_prev;
-            }
-        }
-        if (!isfinite(rho) || !isfinite(beta)) sc->status = -6;
-        sc->rho = rho;
-        sc->sdr = sdr;
-        sc->beta = beta;
-    }
+    if (grid_reduce<2>(v, part, counter, tot) && threadIdx.x == 0) finish_dots(sc, tot[0], tot[1]);
 }
 
-template <class S>
-__global__ void __launch_bounds__(kMaxThreads) k_update_p4(int nc, const S *__restrict__ s, double *__restrict__ p, const KrylovScalars *sc) {
+template <class S, bool IDENT>
+__global__ void __launch_bounds__(kMaxThreads) k_update_p4(int nc, const S *__restrict__ s, double *__restrict__ p, KrylovScalars *sc) {
     pdl_trigger();
     pdl_wait();
+    if constexpr (IDENT) ident_status(sc);
     const Share sh = cta_share(nc);
     const double beta = sc->beta;
     update_p_share<S>(sh, s, p, beta);
@@ -457,7 +462,7 @@ __global__ void __launch_bounds__(kMaxThreads) k_spmv_alpha4(int nx, int ny, int
     }
 }
 
-template <class S>
+template <class S, bool IDENT>
 __global__ void __launch_bounds__(kMaxThreads) k_update_xr4(int nc, double *__restrict__ x, const double *__restrict__ p, double *__restrict__ r,
                              const double *__restrict__ q, S *__restrict__ f0,
                              KrylovScalars *sc, DSum *part, unsigned *counter, cudaGraphConditionalHandle cond,
@@ -466,7 +471,8 @@ __global__ void __launch_bounds__(kMaxThreads) k_update_xr4(int nc, double *__re
     pdl_wait();
     const Share sh = cta_share(nc);
     const double alpha = sc->alpha;
-    double a0 = 0.0;
+    const bool sq = IDENT && sc->variant == 1;
+    double a0 = 0.0, a1 = 0.0;
 #pragma unroll 2
     for (int c = sh.begin; c < sh.end; c += blockDim.x) {
         const int i = 4 * c;
@@ -480,14 +486,13 @@ __global__ void __launch_bounds__(kMaxThreads) k_update_xr4(int nc, double *__re
             xv[k] = fma(alpha, pv[k], xv[k]);
             rn[k] = fma(-alpha, qv[k], ro[k]);
             a0 = fma(rn[k], rn[k], a0);
+            if (sq) a1 = fma(rn[k], qv[k], a1);
         }
         st4(x + i, xv);
         st4(r + i, rn);
         if (f0 != nullptr) sts4<S>(f0 + i, rn);
     }
-    double v[1] = {a0};
-    double tot[1];
-    if (grid_reduce<1>(v, part, counter, tot) && threadIdx.x == 0) finish_update(sc, tot[0], cond, use_cond);
+    finish_xr<IDENT>(a0, a1, sc, part, counter, cond, use_cond);
 }
 
 // ---- the four kernels above as one cooperative kernel ---------------------------------------------
@@ -533,21 +538,7 @@ __global__ void __launch_bounds__(kMaxThreads) k_tail_fused(int nx, int ny, int 
         dots_share<S>(a0, a1, sh, s, r, q, need_sdr);
         double v[2] = {a0, a1};
         double tot[2];
-        if (grid_reduce<2>(v, part, counter, tot) && threadIdx.x == 0) {
-            const double rho = tot[0], sdr = -sc->alpha * tot[1];
-            double beta = 0.0;
-            if (sc->restart == 0 && variant != 2) {
-                if (sc->rho_prev == 0.0) {
-                    sc->status = -4;
-                } else {
-                    beta = (variant == 0) ? rho / sc->rho_prev : sdr / sc->rho_prev;
-                }
-            }
-            if (!isfinite(rho) || !isfinite(beta)) sc->status = -6;
-            sc->rho = rho;
-            sc->sdr = sdr;
-            sc->beta = beta;
-        }
+        if (grid_reduce<2>(v, part, counter, tot) && threadIdx.x == 0) finish_dots(sc, tot[0], tot[1]);
     }
     if (!grid_barrier(bcount, bgen, berr, spin_limit, nblk)) {
         give_up();
@@ -710,8 +701,9 @@ cudaError_t kry_true_residual(int nx, int ny, int nz, const double *b, const dou
 }
 
 cudaError_t kry_iteration_tail(Prec st_prec, int nx, int ny, int nz, const void *s, double *x, double *r, double *p,
-                               double *q, void *f0, KrylovWork &w, cudaStream_t st,
+                               double *q, void *f0, KrylovWork &w, Dots dots, cudaStream_t st,
                                cudaGraphConditionalHandle cond, int use_cond) {
+    const bool ident = dots == Dots::Ident;
     const long long n = static_cast<long long>(nx) * ny * nz;
     const RedGrid g1 = reduction_grid(n);
     cudaError_t e = cudaSuccess;
@@ -723,7 +715,7 @@ cudaError_t kry_iteration_tail(Prec st_prec, int nx, int ny, int nz, const void 
         SMG_PREC_SWITCH(st_prec, {
             const S *sp = static_cast<const S *>(s);
             S *f0p = static_cast<S *>(f0);
-            if (w.fused && w.bar != nullptr && fused_tail_fits<S>(g4.blocks)) {
+            if (w.fused && dots == Dots::Kernel && w.bar != nullptr && fused_tail_fits<S>(g4.blocks)) {
                 // one cooperative launch: the runtime refuses it unless every CTA is resident
                 cudaLaunchConfig_t cfg = {};
                 cfg.gridDim = dim3(g4.blocks);
@@ -738,12 +730,12 @@ cudaError_t kry_iteration_tail(Prec st_prec, int nx, int ny, int nz, const void 
                                        w.bar, static_cast<long long>(kTailSpinLimit), cond, use_cond, gd4);
                 return e != cudaSuccess ? e : cudaGetLastError();
             }
-            if (e == cudaSuccess) e = launch_pdl(k_dots_beta4<S>, dim3(g4.blocks), dim3(g4.threads), 0, st, nc, sp, r, q, w.sc, w.part, w.counter);
-            if (e == cudaSuccess) e = launch_pdl(k_update_p4<S>, dim3(g4.blocks), dim3(g4.threads), 0, st, nc, sp, p, w.sc);
+            if (e == cudaSuccess && dots == Dots::Kernel) e = launch_pdl(k_dots_beta4<S>, dim3(g4.blocks), dim3(g4.threads), 0, st, nc, sp, r, q, w.sc, w.part, w.counter);
+            if (e == cudaSuccess) e = launch_pdl(ident ? k_update_p4<S, true> : k_update_p4<S, false>, dim3(g4.blocks), dim3(g4.threads), 0, st, nc, sp, p, w.sc);
             if (e == cudaSuccess)
                 e = launch_pdl(k_spmv_alpha4, dim3(g4.blocks), dim3(g4.threads), 0, st, nx, ny, nz, p, q, w.sc, w.part, w.counter, gd4);
             if (e == cudaSuccess)
-                e = launch_pdl(k_update_xr4<S>, dim3(g4.blocks), dim3(g4.threads), 0, st, nc, x, p, r, q, f0p, w.sc, w.part, w.counter,
+                e = launch_pdl(ident ? k_update_xr4<S, true> : k_update_xr4<S, false>, dim3(g4.blocks), dim3(g4.threads), 0, st, nc, x, p, r, q, f0p, w.sc, w.part, w.counter,
                                cond, use_cond);
         });
         return e != cudaSuccess ? e : cudaGetLastError();
@@ -752,12 +744,12 @@ cudaError_t kry_iteration_tail(Prec st_prec, int nx, int ny, int nz, const void 
     SMG_PREC_SWITCH(st_prec, {
         const S *sp = static_cast<const S *>(s);
         S *f0p = static_cast<S *>(f0);
-        if (e == cudaSuccess) e = launch_pdl(k_dots_beta<S>, dim3(g1.blocks), dim3(g1.threads), 0, st, n, sp, r, q, w.sc, w.part, w.counter);
-        if (e == cudaSuccess) e = launch_pdl(k_update_p<S>, dim3(g1.blocks), dim3(g1.threads), 0, st, n, sp, p, w.sc);
+        if (e == cudaSuccess && dots == Dots::Kernel) e = launch_pdl(k_dots_beta<S>, dim3(g1.blocks), dim3(g1.threads), 0, st, n, sp, r, q, w.sc, w.part, w.counter);
+        if (e == cudaSuccess) e = launch_pdl(ident ? k_update_p<S, true> : k_update_p<S, false>, dim3(g1.blocks), dim3(g1.threads), 0, st, n, sp, p, w.sc);
         if (e == cudaSuccess)
             e = launch_pdl(k_spmv_alpha, dim3(g1.blocks), dim3(g1.threads), 0, st, nx, ny, nz, p, q, w.sc, w.part, w.counter, gd);
         if (e == cudaSuccess)
-            e = launch_pdl(k_update_xr<S>, dim3(g1.blocks), dim3(g1.threads), 0, st, n, x, p, r, q, f0p, w.sc, w.part, w.counter, cond,
+            e = launch_pdl(ident ? k_update_xr<S, true> : k_update_xr<S, false>, dim3(g1.blocks), dim3(g1.threads), 0, st, n, x, p, r, q, f0p, w.sc, w.part, w.counter, cond,
                            use_cond);
     });
     return e != cudaSuccess ? e : cudaGetLastError();
