@@ -393,6 +393,68 @@ size_t plan_tail(ModalArgs<T> &a, int lt, ModalConfig cfg, const ModalKernels<T>
 
 }  // namespace
 
+// The tail's steps in order: tables of level lt; down, each level relaxed (npre sweeps of both colours) and
+// restricted; the last level solved; up, each level corrected and relaxed (npost sweeps).  A level's classes are
+// fetched while the step before its tables are spread runs.
+template <class T>
+std::vector<TailOp> tail_ops(const ModalArgs<T> &a) {
+    const int L = a.L, lt = a.lt;
+    std::vector<TailOp> ops;
+    auto add = [&](int kind, int l) -> TailOp & {
+        TailOp o{};
+        const int c = l + 1 < L ? l + 1 : L - 1;
+        o.kind = kind;
+        o.level = l;
+        o.nz = a.nz[l];
+        o.nzc = a.nz[c];
+        o.u = a.sm_u[l];
+        o.f = l == lt ? -1 : a.sm_f[l];
+        o.uc = a.sm_u[c];
+        o.fc = a.sm_f[c];
+        o.ptype = a.plane_base[l] - a.plane_base[lt];
+        ops.push_back(o);
+        return ops.back();
+    };
+    auto fetch = [&](TailOp &o, int l) {
+        if (l < lt || l >= L - 1) return;
+        o.fetch = a.cls_base[l] * a.blk;
+        o.fetch_n = a.ncls[l] * a.blk;
+    };
+    auto relax = [&](int l, int colour, int mode) -> TailOp & {
+        TailOp &o = add(OP_RELAX, l);
+        o.colour = colour;
+        o.mode = mode;
+        o.n = colour ? a.nz[l] / 2 : (a.nz[l] + 1) / 2;
+        return o;
+    };
+    TailOp &t = add(OP_TABLES, lt);
+    if (lt < L - 1) t.spread = a.ncls[lt];
+    for (int l = lt; l < L - 1; ++l) {
+        for (int s = 0; s < a.npre; ++s)
+            for (int c = 0; c < 2; ++c) {
+                TailOp &o = relax(l, c, s == 0 ? c : 2);
+                if (s == 0 && c == 0) fetch(o, l + 1);
+            }
+        TailOp &o = add(OP_RESTRICT, l);
+        if (l + 1 < L - 1) o.spread = a.ncls[l + 1];
+    }
+    TailOp &solve = add(OP_COARSEST, L - 1);
+    if (a.npost > 0) fetch(solve, L - 2);
+    for (int l = L - 2; l >= lt; --l) {
+        TailOp &o = add(OP_PROLONG, l);
+        o.out = l == lt && a.npost == 0;
+        if (a.npost > 0) o.spread = a.ncls[l];
+        for (int s = 0; s < a.npost; ++s)
+            for (int c = 1; c >= 0; --c) {
+                TailOp &r = relax(l, c, 2);
+                if (s == 0 && c == 1) fetch(r, l - 1);
+            }
+        if (l == lt && a.npost > 0) add(OP_STORE, l).out = 1;
+    }
+    add(OP_END, lt);
+    return ops;
+}
+
 template <class T>
 int modal_plan(ModalHost<T> &h, const HostHierarchy &H, ModalConfig cfg, int nb, int npre, int npost, int coarse_iters) {
     const int nx = H.nx, L = H.L, nh = (nx + 1) / 2;
@@ -477,6 +539,10 @@ int modal_plan(ModalHost<T> &h, const HostHierarchy &H, ModalConfig cfg, int nb,
     h.smem = 0;
     for (int lt = 0; lt < L && h.smem == 0; ++lt) h.smem = plan_tail(a, lt, cfg, k);
     if (h.smem == 0) return static_cast<int>(cudaErrorNotSupported);
+    const std::vector<TailOp> ops = tail_ops(a);
+    h.at[6] = h.shared.size();
+    h.shared.resize(h.at[6] + up(ops.size() * sizeof(TailOp), 256), 0);
+    std::memcpy(h.shared.data() + h.at[6], ops.data(), ops.size() * sizeof(TailOp));
     h.vec_bytes = 0;
     h.vec_off.clear();
     for (int l = 0; l <= a.lt; ++l)
@@ -496,6 +562,7 @@ void modal_place(ModalHost<T> &h, unsigned char *shared, T *coef, double *coef64
     a.ptype = reinterpret_cast<const unsigned short *>(shared + h.at[3]);
     a.pcls = reinterpret_cast<const unsigned short *>(shared + h.at[4]);
     a.ltype = reinterpret_cast<const unsigned short *>(shared + h.at[5]);
+    a.ops = reinterpret_cast<const TailOp *>(shared + h.at[6]);
     a.coef64 = coef64;
     a.coef = coef;
     for (int l = 0; l <= a.lt; ++l) {

@@ -608,16 +608,15 @@ constexpr int modal_threads() { return sizeof(T) == 8 ? 256 : 512; }
 #define SMG_MTRACE(op, l) ((void)0)
 #endif
 
-enum : int { OP_START = 0, OP_RELAX = 1, OP_RESTRICT = 2, OP_COARSEST = 3, OP_PROLONG = 4, OP_STORE = 5, OP_TABLES = 6, OP_END = 7 };
-
-// The cycle of one mode and right-hand side on the tail levels, as one loop over its steps, a CTA
+// The cycle of one mode and right-hand side on the tail levels, as one loop over planned steps, a CTA
 // barrier after each: every kind of step is compiled once (inlined at each place of the cycle it
 // appears, the kernel would not fit the instruction cache).
 template <class T, int G, int K>
 __device__ __forceinline__ void tail_body(const ModalArgs<T> &A, int mode_idx, int rhs, unsigned char *smem) {
+    __shared__ TailOp ring[2];  // the step that runs and the next
     T *sm = reinterpret_cast<T *>(smem);
     const int tid = threadIdx.x, nt = blockDim.x, ln = (tid & 31) % G;
-    const int L = A.L, lt = A.lt, sp = A.sm_pitch, npre = A.npre, npost = A.npost;
+    const int L = A.L, lt = A.lt, sp = A.sm_pitch;
     T *tab = sm + A.sm_tab, *stage = sm + A.sm_stage, *zt = sm + A.sm_zt;
     double *tab64 = reinterpret_cast<double *>(smem + A.sm_tab64);
     unsigned short *ltype = reinterpret_cast<unsigned short *>(smem + A.sm_ltype), *ptype = reinterpret_cast<unsigned short *>(smem + A.sm_ptype),
@@ -628,59 +627,62 @@ __device__ __forceinline__ void tail_body(const ModalArgs<T> &A, int mode_idx, i
     const long long vec = static_cast<long long>(rhs) * A.nmode + mode_idx;
     const Rows<T> fg{const_cast<T *>(A.f[lt]) + vec * A.nz[lt] * A.pitch, A.pitch, 0, false};
     const Rows<T> ug{A.u[lt] + vec * A.nz[lt] * A.pitch, A.pitch, 0, false};
-    auto U = [&](int l) { return Rows<T>{sm + A.sm_u[l], sp, 0, true}; };
-    auto F = [&](int l) { return l == lt ? fg : Rows<T>{sm + A.sm_f[l], sp, 0, true}; };
-    int op = OP_START, l = lt, colour = 0, sweep = 0;
-    bool down = true;
-    while (op != OP_END) {
-        const unsigned short *pt = ptype + A.plane_base[l] - pb;
+    const T *coef = A.coef + static_cast<long long>(mode_idx) * A.ncls_all * A.blk;
+    auto fetch_classes = [&](int at, int n) {
+        for (int i = tid; i < n / CH; i += nt) cp_async16(stage + i * CH, coef + at + i * CH);
+    };
+    auto fetch_op = [&](int i) {
+        if (tid < 4) cp_async16(reinterpret_cast<int4 *>(&ring[i & 1]) + tid, reinterpret_cast<const int4 *>(A.ops + i) + tid);
+    };
+    // what does not depend on the right-hand side
+    fetch_op(0);
+    if (lt < L - 1) fetch_classes(A.cls_base[lt] * A.blk, A.ncls[lt] * A.blk);
+    for (int i = tid; i < A.nptype * kCoefPerPlane; i += nt) zt[i] = A.zt[i];
+    for (int i = tid; i < A.nptype; i += nt) pcls[i] = A.pcls[i];
+    for (int i = tid; i < np; i += nt) ptype[i] = A.ptype[pb + i];
+    for (int i = tid; i < A.sum_ny; i += nt) ltype[i] = A.ltype[i];
+    cp_async_wait();
+    __syncthreads();
+    SMG_MTRACE(0, lt);
+    for (int step = 0;; ++step) {
+        const TailOp &o = ring[step & 1];
+        const int kind = o.kind;
+        if (kind == OP_END) break;
+        fetch_op(step + 1);
+        if (o.fetch_n > 0) fetch_classes(o.fetch, o.fetch_n);  // of the level relaxed after this one
+        // spread the line tables of the next level to be relaxed (nothing reads the present ones now), from
+        // the last thread on: the first ones have the restriction's planes
+        if (o.spread > 0)
+            spread_tables<T, G, K>(tab, stage, o.spread, A.blk, ltype, A.ny_m, A.line_base, A.P, A.ntype, nt - 1 - tid, nt);
+        const unsigned short *pt = ptype + o.ptype;
         auto row = [&](int z) -> const T * { return zt + pt[z] * kCoefPerPlane; };
-        // fetch the classes of the level relaxed after this one
-        int fetch = -1;
-        if (op == OP_START) fetch = lt;
-        else if (op == OP_RELAX && sweep == 0 && colour == (down ? 0 : 1)) fetch = down ? l + 1 : l - 1;
-        else if (op == OP_COARSEST && npost > 0) fetch = L - 2;
-        if (fetch >= lt && fetch < L - 1) {
-            const T *src = A.coef + (static_cast<long long>(mode_idx) * A.ncls_all + A.cls_base[fetch]) * A.blk;
-            for (int i = tid; i < A.ncls[fetch] * A.blk / CH; i += nt) cp_async16(stage + i * CH, src + i * CH);
-        }
-        // spread the line tables of the next level to be relaxed (nothing reads the present ones now)
-        int tl = -1;
-        if (op == OP_TABLES) tl = lt;
-        else if (op == OP_RESTRICT) tl = l + 1;
-        else if (op == OP_PROLONG && npost > 0) tl = l;
-        if (tl >= 0 && tl < L - 1)
-            spread_tables<T, G, K>(tab, stage, A.ncls[tl], A.blk, ltype, A.ny_m, A.line_base, A.P, A.ntype, tid, nt);
-        if (op == OP_RELAX) {
-            const int nz = A.nz[l], n = colour ? nz / 2 : (nz + 1) / 2;
-            const int mode = (down && sweep == 0) ? colour : 2;
-            const Rows<T> u = U(l), f = F(l);
-            for_planes<T, G, K>(n, colour, 2, f, [&](int z, bool act, T (&g)[K]) {
-                relax_plane<T, G, K, true>(g, u, z, nz, row(z), tab + pcls[pt[z]] * Tab<G, K>::kElems, lam, mode, l > 0, ln);
+        const Rows<T> u{sm + o.u, sp, 0, true}, f = o.f < 0 ? fg : Rows<T>{sm + o.f, sp, 0, true};
+        const bool lower = o.level > 0;
+        const int nz = o.nz;
+        if (kind == OP_RELAX) {
+            const int mode = o.mode;
+            for_planes<T, G, K>(o.n, o.colour, 2, f, [&](int z, bool act, T (&g)[K]) {
+                relax_plane<T, G, K, true>(g, u, z, nz, row(z), tab + pcls[pt[z]] * Tab<G, K>::kElems, lam, mode, lower, ln);
                 if (act) store_row<T, K, true>(u.at(z), g, ln, sp);
             });
-            cp_async_wait();
-        } else if (op == OP_RESTRICT) {
-            const Rows<T> fc = F(l + 1), u = U(l), f = F(l);
-            const int nz = A.nz[l], nch = A.pitch / CH;
-            restrict_planes<T, K>(0, A.nz[l + 1], nch, sp / CH, u, f, nz, row, lam, l > 0,
+        } else if (kind == OP_RESTRICT) {
+            const Rows<T> fc{sm + o.fc, sp, 0, true};
+            restrict_planes<T, K>(0, o.nzc, A.pitch / CH, sp / CH, u, f, nz, row, lam, lower,
                                   [&](int Z, int c, const Chunk<T, K> &g) { g.store(fc, Z, c); });
-        } else if (op == OP_COARSEST) {
+        } else if (kind == OP_COARSEST) {
             if (lt == L - 1) {  // the only level: straight to global memory
                 if (tid < 32) coarsest<T, G, K, false>(fg.p, ug.p, A.ny, A.coarse_iters, tab64, tid);
                 for (int y = A.ny + tid; y < A.pitch; y += nt) ug.p[y] = T(0);
             } else {
-                T *ul = sm + A.sm_u[L - 1];
-                if (tid < 32) coarsest<T, G, K, true>(sm + A.sm_f[L - 1], ul, A.ny, A.coarse_iters, tab64, tid);
-                for (int y = A.ny + tid; y < sp; y += nt) ul[RowMap<T, K>::elem(y)] = T(0);
+                if (tid < 32) coarsest<T, G, K, true>(f.p, u.p, A.ny, A.coarse_iters, tab64, tid);
+                for (int y = A.ny + tid; y < sp; y += nt) u.p[RowMap<T, K>::elem(y)] = T(0);
             }
-            cp_async_wait();
-        } else if (op == OP_PROLONG || op == OP_STORE) {
+        } else if (kind == OP_PROLONG || kind == OP_STORE) {
             // u_l += P u_{l+1}; on the last level, with no sweep to follow, straight to global memory
-            const bool add = op == OP_PROLONG, out = l == lt && (!add || npost == 0);
-            const int nzc = add ? A.nz[l + 1] : 1;
-            const Rows<T> u = U(l), uc = U(min(l + 1, L - 1));
-            for_chunks(A.nz[l], (out ? A.pitch : sp) / CH, [&](int z, int c) {
+            const bool add = kind == OP_PROLONG, out = o.out != 0;
+            const int nzc = add ? o.nzc : 1;
+            const Rows<T> uc{sm + o.uc, sp, 0, true};
+            for_chunks(nz, (out ? A.pitch : sp) / CH, [&](int z, int c) {
                 Chunk<T, K> g, v, w;
                 g.load(u, z, c);
                 if (add) {
@@ -694,7 +696,7 @@ __device__ __forceinline__ void tail_body(const ModalArgs<T> &A, int mode_idx, i
                 }
                 g.store(out ? ug : u, z, c);
             });
-        } else if (op == OP_TABLES) {
+        } else {  // OP_TABLES
             // the coarsest plane's table is spread over 32 lanes, from global memory
             const double *src = A.coef64 + static_cast<long long>(mode_idx) * class_values<32>(A.ntype);
             spread_tables<double, 32, K6>(tab64, src, 1, 0, ltype, A.ny_m, A.line_base, A.P, A.ntype, tid, nt);
@@ -704,48 +706,10 @@ __device__ __forceinline__ void tail_body(const ModalArgs<T> &A, int mode_idx, i
                     tab64[Tab<32, K6>::kElems + 2 * i + 1] = i < A.ny ? src[ltype[i] * kRow + 1] : 0.0;
                 }
             pdl_wait();
-        } else {  // OP_START: what does not depend on the right-hand side
-            for (int i = tid; i < A.nptype * kCoefPerPlane; i += nt) zt[i] = A.zt[i];
-            for (int i = tid; i < A.nptype; i += nt) pcls[i] = A.pcls[i];
-            for (int i = tid; i < np; i += nt) ptype[i] = A.ptype[pb + i];
-            for (int i = tid; i < A.sum_ny; i += nt) ltype[i] = A.ltype[i];
-            cp_async_wait();
         }
+        cp_async_wait();
         __syncthreads();
-        SMG_MTRACE(op, l);
-        // the next step
-        if (op == OP_START) {
-            op = OP_TABLES;
-        } else if (op == OP_TABLES) {
-            op = lt == L - 1 ? OP_COARSEST : OP_RELAX;
-        } else if (op == OP_RELAX) {
-            const int last = down ? 1 : 0;
-            if (colour != last) {
-                colour = last;
-            } else {
-                colour = 1 - last;
-                if (++sweep == (down ? npre : npost)) {
-                    sweep = 0;
-                    if (down) op = OP_RESTRICT;
-                    else if (l == lt) op = OP_STORE;
-                    else op = OP_PROLONG, --l;
-                }
-            }
-        } else if (op == OP_RESTRICT) {
-            ++l;
-            op = l == L - 1 ? OP_COARSEST : OP_RELAX;
-        } else if (op == OP_COARSEST) {
-            down = false;
-            colour = 1;
-            op = l == lt ? OP_END : OP_PROLONG;
-            --l;
-        } else if (op == OP_PROLONG) {
-            if (npost > 0) op = OP_RELAX;
-            else if (l == lt) op = OP_END;
-            else --l;
-        } else {
-            op = OP_END;
-        }
+        SMG_MTRACE(kind, o.level);
     }
 }
 

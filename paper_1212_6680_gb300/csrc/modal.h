@@ -20,6 +20,8 @@ constexpr int kMaxZLevels = 13;   // nz <= 4096
 // mode and class, modal_setup_kernel forms once the kRow multipliers of every line type and the G x G
 // matrix of the y-cycle below the levels a lane holds: `blk` values, which the kernels spread over
 // their lines.
+struct TailOp;
+
 template <class T>
 struct ModalArgs {
     int nmode, ny, pitch;      // x-modes, lines, and lines per plane in global memory (ny rounded up to 4)
@@ -46,8 +48,25 @@ struct ModalArgs {
     const T *coef;             // [mode][class][blk]
     const double *coef64;      // [mode][blk64]: the coarsest level's class in FP64, 32 lanes
     const double *lam;         // [nmode] eigenvalues of the x-line Laplacian
+    const TailOp *ops;         // the tail's steps, the last OP_END
     const double *raw;         // [class][ntype][kRawPerLine]: what the multipliers are formed from
 };
+
+// One step of the tail kernel, planned on the host (the kernel's own loop over levels, colours and sweeps spent
+// 400 of a coarse step's 1800 cycles finding out what to do next).
+enum : int { OP_RELAX = 1, OP_RESTRICT = 2, OP_COARSEST = 3, OP_PROLONG = 4, OP_STORE = 5, OP_TABLES = 6, OP_END = 7 };
+struct alignas(16) TailOp {
+    int kind;
+    int level;
+    int colour, mode, n;   // OP_RELAX: planes colour, colour + 2, ..; relax_plane's mode; how many
+    int nz, nzc;           // planes of the level and of the next
+    int u, f, uc, fc;      // shared-memory offsets of the level's vectors (f -1: in global memory) and the next's
+    int ptype;             // of the level's first plane, from the tail's first
+    int fetch, fetch_n;    // classes of the level relaxed next: first value, values (0: nothing to fetch)
+    int spread;            // classes to spread into line tables (0: none)
+    int out;               // OP_PROLONG, OP_STORE: to global memory
+};
+static_assert(sizeof(TailOp) == 64, "four 16-byte loads");
 
 constexpr int kRawPerLine = 14;  // raw_line in modal.cu
 constexpr int kRow = 8;          // multipliers of a line type
@@ -76,8 +95,8 @@ struct ModalHost {
     ModalArgs<T> a;
     ModalConfig cfg{16, 8};
     size_t smem = 0;                   // tail kernel
-    std::vector<unsigned char> shared; // raw, lam, zt, ptype, pcls, ltype
-    size_t at[6] = {0};
+    std::vector<unsigned char> shared; // raw, lam, zt, ptype, pcls, ltype, ops
+    size_t at[7] = {0};
     size_t coef_values = 0, coef64_values = 0, vec_bytes = 0;
     std::vector<size_t> vec_off;       // f and u of levels 0 .. lt
 };
