@@ -16,8 +16,8 @@
 // of a long line that of a short sum (128 points: 0.94e-7 of the result's norm instead of 1.5e-7, 1280:
 // 1.5e-7).
 //
-// Forward, lines of up to 128 points are folded on their way into shared memory (by two column tiles at
-// most); longer ones by a pass of their own.
+// Forward, lines of up to 256 points (FP64 input: 128) are folded on their way into shared memory; longer
+// ones by a pass of their own (folds_on_the_way).
 #include "modal.cuh"
 
 namespace smg {
@@ -418,10 +418,19 @@ cudaError_t launch(K kernel, dim3 grid, size_t smem, cudaStream_t st, Args... ar
     return e != cudaSuccess ? e : launch_pdl(kernel, grid, dim3(kNT), smem, st, args...);
 }
 
+// Whether lines are folded on their way into shared memory, once for every column tile, or by a pass of their
+// own first, whose result (4 bytes a point) the tiles then read: by the traffic, 4 tiles of FP32 (16 bytes a
+// point against 24; 256^3 solve: 13.46 -> 13.31 ms) but 2 of FP64 (4 tiles: 366 us for both transforms at 256^3
+// against 303).
+template <class S>
+bool folds_on_the_way(int nh) {
+    return nh <= (sizeof(S) == 4 ? 4 : 2) * kBN;
+}
+
 template <int LT, class S>
 cudaError_t in_any(const SineArgs &g, int nb, const S *f, float *out, float *scratch, cudaStream_t st, long long &launches) {
     launches += 1;
-    if (g.nh <= 2 * kBN) return launch(in_fold_kernel<LT, S>, grid_of<LT>(g, nb), sizeof(Smem<LT>), st, g, f, out);
+    if (folds_on_the_way<S>(g.nh)) return launch(in_fold_kernel<LT, S>, grid_of<LT>(g, nb), sizeof(Smem<LT>), st, g, f, out);
     launches += 1;
     const long long lines = static_cast<long long>(g.nz) * g.pitch;
     const cudaError_t e =
