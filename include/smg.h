@@ -49,27 +49,30 @@ enum {
 enum { SMG_PCG = 0, SMG_FPCG = 1, SMG_PSD = 2 };       /* eq. (1), eq. (2), beta = 0 */
 enum { SMG_FP64 = 0, SMG_FP32 = 1, SMG_BF16 = 2 };     /* V-cycle storage precision */
 
-/* Options for smg_set_option. */
+/* Options for smg_set_option.
+ *
+ * Two forms of the V-cycle exist.  In mode space (every FP32 and BF16 cycle, and FP64 ones with x-lines of at
+ * most 160 rows) it runs in the sine eigenvectors of the x-lines: the same relaxations, an exact line solve being a
+ * division per mode.  Longer FP64 x-lines run on the plane kernels, to which the options on threads, clusters, step orders,
+ * tables and restriction apply (marked "planes"); in mode space these are accepted and change nothing. */
 enum {
     SMG_OPT_COARSE_ITERS = 0, /* plane-cycle steps on the one-plane coarsest level (>= 1, default 1) */
-    SMG_OPT_THREADS = 1,      /* threads per CTA of the plane-relaxation kernels: 256 or 512
-                                 (default 512; the shortened-step kernel with FP64 compute and the
-                                 wide-line kernel with FP32 compute use at most 384, for registers) */
-    SMG_OPT_PROFILE = 2,      /* time plane-relaxation launches with CUDA events: 0 off,
-                                 1 the finest level's launches only, 2 every launch */
-    SMG_OPT_CLUSTER_MAX = 3,  /* largest thread-block cluster (CTAs per plane) for the FP64
-                                 plane relaxations: 1, 2, 4, 8 or 16 (default 16; levels other
-                                 than the one-plane coarsest use at most 8) */
-    SMG_OPT_CLUSTER_MAX32 = 4, /* the same for the FP32-compute plane relaxations of the FP32 and
-                                 BF16 cycles: 1, 2, 4, 8 or 16, or 0 (default) for 8 with x-lines
-                                 split over several warps, else 1 while a plane's 2D-cycle iterate
-                                 fits in one CTA's shared memory and 4 when it does not */
+    SMG_OPT_THREADS = 1,      /* planes: threads per CTA: 256 or 512 (default 512; the
+                                 shortened-step kernel uses at most 384, for registers) */
+    SMG_OPT_PROFILE = 2,      /* time the cycle's launches with CUDA events: 0 off, 1 the finest
+                                 level's plane launches only, 2 every launch; in mode space 1 and 2
+                                 time the transforms and the cycle between them */
+    SMG_OPT_CLUSTER_MAX = 3,  /* planes: largest thread-block cluster (CTAs per plane): 1, 2, 4, 8
+                                 or 16 (default 16; levels other than the one-plane coarsest use
+                                 at most 8) */
+    SMG_OPT_CLUSTER_MAX32 = 4, /* 0 (default), 1, 2, 4, 8 or 16: was the limit for FP32 planes, which
+                                 run in mode space; accepted and without effect */
     SMG_OPT_PRECOND = 5,      /* the preconditioner krylov_solve applies: 1 (default) the SMG cycle,
                                  0 none (T = I: plain CG by eq. (1) or (2), steepest descent for PSD;
                                  section 2, figures 1-2); lobpcg_solve always uses the cycle */
-    SMG_OPT_LEAN = 6,         /* 1 (default): plane relaxations with x-lines of at most 256 rows
-                                 whose layout keeps every 2D level's factor sets on chip (FP32 or
-                                 FP64 compute, one CTA or a cluster per plane) run the 2D cycle
+    SMG_OPT_LEAN = 6,         /* planes: 1 (default): plane relaxations with x-lines of at most 256 rows
+                                 whose layout keeps every 2D level's factor sets on chip (one CTA
+                                 or a cluster per plane) run the 2D cycle
                                  with fewer barrier-separated steps (the restriction fused with the
                                  next level's even lines; the same line solves in the same order,
                                  bit-identical), and the wide-line kernel (longer x-lines) runs its
@@ -95,38 +98,30 @@ enum {
                                  faster on GB300 (the barriers cost more than the kernel
                                  boundaries).  A barrier wait that gives up returns SMG_ERR_TIMEOUT
                                  from krylov_solve */,
-    SMG_OPT_SOLO = 10         /* T in [0, 512] (default 8): when the shortened-step plane cycle
+    SMG_OPT_SOLO = 10         /* planes: T in [0, 512] (default 8): when the shortened-step plane cycle
                                  runs on a thread-block cluster, the 2D levels of at most T lines
                                  are held whole by the cluster's first CTA, whose steps on them
                                  end in a CTA barrier instead of a cluster barrier; the same
                                  results as 0 (every level spread over the cluster) */,
-    SMG_OPT_RESTRICT_COLUMN = 11 /* 1 (default): with FP64 storage, or from 4M coarse points per
-                                 launch, each thread of the residual + restriction walks four
-                                 coarse planes, computing each fine residual (and each plane's
-                                 in-plane stencil) once; smaller FP32 / BF16 launches, and every
-                                 launch with 0, use one coarse plane per thread, recomputing the
-                                 residual of every even fine plane for both coarse planes it
-                                 feeds.  Bit-identical results */,
-    SMG_OPT_WIDE_FACTORS = 12 /* 1 (default): planes whose x-lines run on the wide-line kernel
+    SMG_OPT_RESTRICT_COLUMN = 11 /* planes: 1 (default): each thread of the residual + restriction
+                                 walks four coarse planes, computing each fine residual (and each
+                                 plane's in-plane stencil) once; 0: one coarse plane per thread,
+                                 recomputing the residual of every even fine plane for both coarse
+                                 planes it feeds.  Bit-identical results */,
+    SMG_OPT_WIDE_FACTORS = 12 /* planes: 1 (default): those whose x-lines run on the wide-line kernel
                                  (see SMG_OPT_WIDE_MIN_ROWS) read the line solver's data of every
                                  2D level's two line matrices (segment factors, the segments'
                                  responses to their end values, the reduced system's rows) from
-                                 tables formed once, in the compute precision, when the level
+                                 tables formed once when the level
                                  vectors are allocated, one per class of planes with equal
                                  coefficients (smg_plane_classes; the coarsest level always, the
                                  others while the tables take at most 512 MB); 0: formed inside the plane
                                  cycle at every change of line matrix.  Bit-identical results */,
-    SMG_OPT_WIDE_MIN_ROWS = 13 /* 257 (default) or 513: x-lines of at least this many rows (and at
+    SMG_OPT_WIDE_MIN_ROWS = 13 /* planes: 257 (default) or 513: x-lines of at least this many rows (and at
                                  most 512) are split over two warps of 8 rows per lane (the
                                  wide-line kernel, with its clusters and tables) instead of one
                                  warp of 16 (the general plane cycle); lines longer than 512 rows
-                                 always take the wide-line kernel.  The two differ by rounding */,
-    SMG_OPT_MODAL = 14        /* 1 (default): the cycle runs in the sine eigenvectors of the x-lines
-                                 where that is the faster form (every FP32 and BF16 cycle, FP64 ones
-                                 with x-lines of at most 160 rows): the same relaxations, with an
-                                 exact line solve a division per mode; 0: the plane kernels, to which
-                                 the options above on threads, clusters, step orders, tables and
-                                 restriction apply.  The two differ by rounding */
+                                 always take the wide-line kernel.  The two differ by rounding */
 };
 
 /*
@@ -135,7 +130,7 @@ enum {
  * sweeps (npost = 0 is the paper's nonsymmetric "no post-relaxation" cycle).  The hierarchy
  * is computed on the host in FP64 (z-semicoarsening, Galerkin coarse operators, per-plane
  * y-hierarchies) and copied to the current device; work vectors for one right-hand side are
- * allocated.  Sizes: 1 <= nx <= 2048, 1 <= ny <= 512, 1 <= nz <= 4096.  x-lines of up to 256
+ * allocated.  Sizes: 1 <= nx <= 2048, 1 <= ny <= 512, 1 <= nz <= 4096.  On the plane kernels x-lines of up to 256
  * rows are solved by one warp; longer ones (the paper's 16n x n x n bricks up to n = 128) are cut
  * into segments of 256 rows (lines of 257-512 rows) or 512 rows (longer lines), one warp each,
  * joined exactly through a reduced system of the segment ends (SMG_OPT_WIDE_MIN_ROWS = 513 keeps
@@ -146,7 +141,7 @@ enum {
 int smg_setup(int nx, int ny, int nz, int npre, int npost, smg_handle *out);
 
 /* smg_set_precision -- storage precision of the V-cycle: SMG_FP64, SMG_FP32 or SMG_BF16.
- * FP32 computes in FP32; BF16 stores level vectors in bfloat16 and computes in FP32.  The
+ * FP32 computes in FP32; BF16 computes in FP32 and stores its result T r in bfloat16.  The
  * one-plane coarsest level always computes in FP64.  Krylov recurrences, inner products and
  * norms stay FP64. */
 int smg_set_precision(smg_handle h, int prec);
@@ -198,7 +193,7 @@ int lobpcg_solve(smg_handle h, int m, double *X, double *lambda, double tol, int
  * (dims[3s], dims[3s+1], dims[3s+2] = nx, ny, nz of system s), solved together by Algorithm 1
  * (PCG eq. (1), flexible PCG eq. (2) or PSD) preconditioned by SMG with -v npre npost.  Per
  * iteration, one CUDA graph runs every system's V-cycle in the sine eigenvectors of its x-lines
- * (SMG_OPT_MODAL's form: one launch transforms all residuals, one CTA per system and mode runs that
+ * (one launch transforms all residuals, one CTA per system and mode runs that
  * mode's cycle, one launch transforms back) and the FP64 Krylov kernels of all systems;
  * converged systems are masked out on the device.
  *
@@ -345,12 +340,12 @@ int smg_destroy(smg_handle h);
 const char *smg_last_error(void);
 
 /*
- * smg_profile_read -- when SMG_OPT_PROFILE is on, the plane-relaxation launches timed so far
+ * smg_profile_read -- when SMG_OPT_PROFILE is on, the cycle's launches timed so far
  * on this handle: launches, total device milliseconds (CUDA events on the launch stream) and
  * algorithmic bytes (vector elements the launches must read and write), by class `which`:
- * 0 plane relaxation on the finest level, 1 plane relaxation on the other levels except the
- * coarsest, 2 the one-plane coarsest solve, 3 restriction and prolongation, 4 the Krylov
- * kernels of each iteration, 5 the learned post-correction of each iteration (its "bytes" are
+ * 0 plane relaxation on the finest level (mode space: the whole cycle of all modes), 1 plane
+ * relaxation on the other levels except the coarsest, 2 the one-plane coarsest solve, 3 restriction
+ * and prolongation (mode space: the transforms in and out), 4 the Krylov kernels of each iteration, 5 the learned post-correction of each iteration (its "bytes" are
  * the convolutions' flops, 2 x 27 x 288 per point) (classes 1-4 are timed only with
  * SMG_OPT_PROFILE = 2; classes 0 and 5 with either 1 or 2).
  * Reading resets the counters of that class.  Synchronises the device.

@@ -18,7 +18,7 @@ BUILD = os.path.join(ROOT, "_build")
 LIB = os.path.join(HERE, "libsmg.so")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-KS = (1, 2, 3, 4, 6, 8, 16)
+KS = (6, 8, 16)  # rows per lane of the FP64 plane kernels (x-lines of more than 160 rows)
 SOURCES = ["api.cpp", "hierarchy.cpp", "cycle.cu", "krylov_kernels.cu", "lobpcg.cu", "noalloc.cu", "batched.cu", "net.cu",
            "net_api.cpp", "conv_tc.cu", "gram_tc.cu", "modal.cu", "sine.cu"]
 WKS = (8, 16)  # rows per lane of the wide-line kernel's segments (plane_wide.cu, one unit each)
@@ -54,10 +54,8 @@ def _units():
         units.append((os.path.join(CSRC, "modal_inst.cu"), os.path.join(BUILD, f"modal_{t}_{g}_{k}.o"), ["-x", "cu"],
                       [f"-DSMG_MT={t}", f"-DSMG_MG={g}", f"-DSMG_MK={k}"]))
     for k in KS:
-        for prec in (0, 1, 2):
-            src = os.path.join(CSRC, "plane_relax_inst.cu")
-            obj = os.path.join(BUILD, f"plane_relax_k{k}_p{prec}.o")
-            units.append((src, obj, ["-x", "cu"], [f"-DSMG_K={k}", f"-DSMG_PREC={prec}"]))
+        units.append((os.path.join(CSRC, "plane_relax_inst.cu"), os.path.join(BUILD, f"plane_relax_k{k}.o"), ["-x", "cu"],
+                      [f"-DSMG_K={k}"]))
     return units
 
 

@@ -75,18 +75,15 @@ struct smg_ctx {
     Prec prec = Prec::F64;
     HostHierarchy H;
     double *d_zcoef = nullptr, *d_pcoef = nullptr;
-    float *d_zcoef32 = nullptr, *d_pcoef32 = nullptr;  // the same tables rounded to FP32
     // level storage (current precision) for nb_alloc right-hand sides
     int nb_alloc = 0;
     Prec alloc_prec = Prec::F64;
     std::vector<void *> d_f, d_u;   // [L]; level 0 entries used only when the caller's buffers are not
     void *d_ws = nullptr;
     size_t ws_bytes = 0;
-    PlaneLayout lay_c, lay_d;       // compute type = storage compute (float/double) and double (coarsest)
+    PlaneLayout lay_c;              // one CTA per plane
     PlaneLayout lay_cl[5];          // FP64-compute cluster layouts for R = 2, 4, 8, 16 (index log2 R)
     bool cl_ok[5] = {false, false, false, false, false};
-    PlaneLayout lay_cl32[5];        // FP32-compute cluster layouts
-    bool cl32_ok[5] = {false, false, false, false, false};
     int cluster_max = 16;           // largest cluster for FP64-compute plane relaxations (1 = none)
     int precond = 1;                // krylov_solve's preconditioner: 1 the SMG cycle, 0 none (T = I)
     int lean = 1;                   // 1: the shortened-step plane cycle where it applies
@@ -97,7 +94,7 @@ struct smg_ctx {
     int wide_min = 257;             // lines of at least this many rows run the wide-line kernel
     int wide_factors = 1;           // 1: wide-line planes read their line-solver data from tables
                                     // formed with the level vectors (d_wftab)
-    unsigned char *d_wftab = nullptr;  // those tables (each level's in its compute type)
+    unsigned char *d_wftab = nullptr;  // those tables
     std::vector<long long> wftab_off;  // [L] byte offset of level l's table in d_wftab, -1: none
     int *d_wfslot = nullptr;           // per level with a table: the slot of each plane (nz_l ints),
                                        // then the plane of each slot (one slot per plane class)
@@ -105,14 +102,9 @@ struct smg_ctx {
     std::vector<char> lean_level;   // [L] the level's line matrices allow it (lean_uniform_level)
     PlaneLayout lay_lean64[5];      // FP64-compute shortened-step layouts: one CTA, clusters of 2..16
     bool lean64_ok[5] = {false, false, false, false, false};
-    PlaneLayout lay_lean32[5];      // FP32-compute shortened-step layouts (every factor set on chip)
-    PlaneLayout lay_wcl[2][5];      // wide-line cluster layouts: [FP64 compute][log2 R]
-    bool wcl_ok[2][5] = {{false, false, false, false, false}, {false, false, false, false, false}};
-    bool lean32_ok[5] = {false, false, false, false, false};
-    int cluster_max32 = 0;          // largest cluster for FP32-compute plane relaxations; 0 = chosen
-                                    // per size (see relax)
+    PlaneLayout lay_wcl[5];         // wide-line cluster layouts: [log2 R]
+    bool wcl_ok[5] = {false, false, false, false, false};
     int num_sms = 0;
-    int modal = 1;                  // 1: the cycle in the x-lines' sine eigenvectors where use_modal holds
     bool modal_now = false;         // the level vectors in place are that cycle's
     ModalPlan mp;
     // Krylov vectors (one right-hand side)
@@ -183,8 +175,6 @@ void free_levels(smg_ctx *h) {
     h->modal_now = false;
 }
 
-size_t compute_bytes(Prec p) { return p == Prec::F64 ? 8 : 4; }
-
 int instantiated_K(int nx) {
     const int k = (nx + 31) / 32;
     if (k <= 4) return k;
@@ -222,7 +212,7 @@ PlaneLayout with_solo_levels(const HostHierarchy &H, size_t elem_bytes, int R, i
 // Whether the cycle runs in the x-lines' sine eigenvectors (modal.cuh): every FP32 and BF16 cycle; an
 // FP64 cycle up to kModalMaxNx64 points a line (its transforms are FP64 products of order nx / 2).
 constexpr int kModalMaxNx64 = 160;
-bool use_modal(const smg_ctx *h) { return h->modal && (h->prec != Prec::F64 || h->nx <= kModalMaxNx64); }
+bool use_modal(const smg_ctx *h) { return h->prec != Prec::F64 || h->nx <= kModalMaxNx64; }
 
 // Allocate level vectors for nb right-hand sides in the current precision, and the plane
 // workspace; configure the kernels' dynamic shared memory.
@@ -246,8 +236,7 @@ int ensure_levels(smg_ctx *h, int nb) {
             return SMG_OK;
         }
         modal_free(h->mp);
-        if (e != static_cast<int>(cudaErrorNotSupported))
-            return fail(SMG_ERR_CUDA, std::string("mode-space cycle: ") + cudaGetErrorString(static_cast<cudaError_t>(e)));
+        return fail(SMG_ERR_CUDA, std::string("mode-space cycle: ") + cudaGetErrorString(static_cast<cudaError_t>(e)));
     }
     h->d_f.assign(H.L, nullptr);
     h->d_u.assign(H.L, nullptr);
@@ -256,43 +245,37 @@ int ensure_levels(smg_ctx *h, int nb) {
         SMG_CUDA(cudaMalloc(&h->d_f[l], bytes));
         SMG_CUDA(cudaMalloc(&h->d_u[l], bytes));
     }
-    const bool f64c = (h->prec == Prec::F64);
+    // the plane kernels: an FP64 cycle's
     const int wk = wide_rows(h);
     const bool wide = wk > 0;
     if (wide) {
         // x-lines over several warps (plane_wide.cu): one CTA per plane, segment factors formed on
         // the fly, no cluster and no shortened-step layouts
-        h->lay_c = plan_plane_layout(H, compute_bytes(h->prec), kWideSmemBudget, wk, false, true);
-        h->lay_d = plan_plane_layout(H, 8, kWideSmemBudget, wk, false, true);
-        if (set_plane_wide_smem(wk, h->prec, f64c, false, h->lay_c.smem_bytes) != 0 ||
-            set_plane_wide_smem(wk, h->prec, true, false, h->lay_d.smem_bytes) != 0)
+        h->lay_c = plan_plane_layout(H, 8, kWideSmemBudget, wk, false, true);
+        if (set_plane_wide_smem(wk, false, h->lay_c.smem_bytes) != 0)
             return fail(SMG_ERR_CUDA, "cudaFuncSetAttribute (plane relaxation, wide lines) failed");
         // a plane spread over a cluster of R CTAs, each relaxing the lines it owns
-        for (int c64 = 0; c64 < 2; ++c64) {
-            for (int lr = 0; lr <= 4; ++lr) h->wcl_ok[c64][lr] = false;
-            if (!c64 && f64c) continue;  // an FP64 cycle has no FP32-compute planes
-            for (int lr = 1; lr <= 4; ++lr) {
-                const int R = 1 << lr;
-                PlaneLayout &ly = h->lay_wcl[c64][lr];
-                ly = plan_plane_layout_cluster(H, c64 ? 8 : 4, kWideSmemBudget, R, false, kMaxPlaneLevels, true);
-                if (ly.smem_bytes == 0 || ly.smem_bytes > kWideSmemBudget) continue;
-                if (set_plane_wide_smem(wk, h->prec, c64 != 0, true, ly.smem_bytes) != 0) {
-                    cudaGetLastError();
-                    continue;
-                }
-                h->wcl_ok[c64][lr] = wide_cluster_resident(wk, h->prec, c64 != 0, R, h->threads, ly.smem_bytes);
+        for (int lr = 0; lr <= 4; ++lr) h->wcl_ok[lr] = false;
+        for (int lr = 1; lr <= 4; ++lr) {
+            const int R = 1 << lr;
+            PlaneLayout &ly = h->lay_wcl[lr];
+            ly = plan_plane_layout_cluster(H, 8, kWideSmemBudget, R, false, kMaxPlaneLevels, true);
+            if (ly.smem_bytes == 0 || ly.smem_bytes > kWideSmemBudget) continue;
+            if (set_plane_wide_smem(wk, true, ly.smem_bytes) != 0) {
+                cudaGetLastError();
+                continue;
             }
+            h->wcl_ok[lr] = wide_cluster_resident(wk, R, h->threads, ly.smem_bytes);
         }
-        for (int lr = 0; lr <= 4; ++lr) h->cl_ok[lr] = h->cl32_ok[lr] = h->lean64_ok[lr] = h->lean32_ok[lr] = false;
+        for (int lr = 0; lr <= 4; ++lr) h->cl_ok[lr] = h->lean64_ok[lr] = false;
         if (h->num_sms == 0) {
             int dev = 0;
             SMG_CUDA(cudaGetDevice(&dev));
             SMG_CUDA(cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, dev));
         }
-        // line-solver tables, each level's in its compute type (FP64 on the coarsest level and in an
-        // FP64 cycle, else FP32), one slot per class of planes with bit-identical coefficient
-        // tables (the data depend on nothing else): the coarsest level always, the others while
-        // all tables take at most 512 MB
+        // line-solver tables, one slot per class of planes with bit-identical coefficient tables
+        // (the data depend on nothing else): the coarsest level always, the others while all tables
+        // take at most 512 MB
         h->wftab_off.assign(H.L, -1);
         h->wfslot_off.assign(H.L, -1);
         if (h->wide_factors) {
@@ -301,8 +284,7 @@ int ensure_levels(smg_ctx *h, int nb) {
             std::vector<std::vector<int>> slot(H.L), rep(H.L);
             for (int l = 0; l < H.L; ++l) plane_classes(H, l, slot[l], rep[l]);
             auto bytes_of = [&](int l) -> long long {
-                const bool c64 = f64c || l == H.L - 1;
-                return per * static_cast<long long>(rep[l].size()) * (c64 ? 8 : 4);
+                return per * static_cast<long long>(rep[l].size()) * 8;
             };
             long long all = 0;
             for (int l = 0; l < H.L; ++l) all += bytes_of(l);
@@ -332,65 +314,52 @@ int ensure_levels(smg_ctx *h, int nb) {
                 const int nc = static_cast<int>(rep[l].size());
                 SMG_CUDA(launch_wide_factor_table(wk, h->nx, W, H.P, H.sum_ny, H.ny_m.data(), H.line_base.data(), nc,
                                                   h->d_wfslot + h->wfslot_off[l] + H.nz_l[l], h->d_pcoef + pb,
-                                                  h->d_pcoef32 + pb, f64c || l == H.L - 1,
                                                   h->d_wftab + h->wftab_off[l], 0));
             }
             SMG_CUDA(cudaStreamSynchronize(0));
         }
         return alloc_plane_workspace(h, nb);
     }
-    h->lay_c = plan_plane_layout(H, compute_bytes(h->prec), kSmemBudget);
-    h->lay_d = plan_plane_layout(H, 8, kSmemBudget);
+    h->lay_c = plan_plane_layout(H, 8, kSmemBudget);
     const int K = instantiated_K(h->nx);
-    if (set_plane_relax_smem(h->prec, f64c, false, K, h->lay_c.smem_bytes) != 0)
-        return fail(SMG_ERR_CUDA, "cudaFuncSetAttribute (plane relaxation, level precision) failed");
-    if (set_plane_relax_smem(h->prec, true, false, K, h->lay_d.smem_bytes) != 0)
-        return fail(SMG_ERR_CUDA, "cudaFuncSetAttribute (plane relaxation, FP64 coarsest) failed");
-    if (h->prec != Prec::F64 && lean_supported(K) &&
-        set_plane_lean_smem(h->prec, false, false, K, h->lay_c.smem_bytes) != 0)
-        return fail(SMG_ERR_CUDA, "cudaFuncSetAttribute (plane relaxation, shortened-step cycle) failed");
+    if (set_plane_relax_smem(false, K, h->lay_c.smem_bytes) != 0)
+        return fail(SMG_ERR_CUDA, "cudaFuncSetAttribute (plane relaxation) failed");
     if (h->num_sms == 0) {
         int dev = 0;
         SMG_CUDA(cudaGetDevice(&dev));
         SMG_CUDA(cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, dev));
     }
-    // Cluster layouts (FP64 compute, and FP32 compute for the FP32/BF16 cycles): usable when
-    // they fit in shared memory and the cluster can be resident; the kernels' shared-memory
-    // limit is then set to the largest usable layout.
-    for (int pass = 0; pass < 2; ++pass) {
-        const bool cf64 = (pass == 0);
-        if (!cf64 && h->prec == Prec::F64) break;
-        PlaneLayout *lays = cf64 ? h->lay_cl : h->lay_cl32;
-        bool *ok = cf64 ? h->cl_ok : h->cl32_ok;
-        size_t cl_smem = 0;
-        for (int lr = 1; lr <= 4; ++lr) {
-            const int R = 1 << lr;
-            ok[lr] = false;
-            lays[lr] = plan_plane_layout_cluster(H, cf64 ? 8 : 4, kSmemBudget, R);
-            if (lays[lr].smem_bytes == 0) continue;
-            if (set_plane_relax_smem(h->prec, cf64, true, K, lays[lr].smem_bytes) != 0) {
-                cudaGetLastError();
-                continue;
-            }
-            ok[lr] = cluster_resident(h->prec, cf64, K, R, h->threads, lays[lr].smem_bytes);
-            if (ok[lr]) cl_smem = std::max(cl_smem, lays[lr].smem_bytes);
+    // Cluster layouts: usable when they fit in shared memory and the cluster can be resident; the
+    // kernels' shared-memory limit is then set to the largest usable layout.
+    size_t cl_smem = 0;
+    for (int lr = 1; lr <= 4; ++lr) {
+        const int R = 1 << lr;
+        h->cl_ok[lr] = false;
+        PlaneLayout &ly = h->lay_cl[lr];
+        ly = plan_plane_layout_cluster(H, 8, kSmemBudget, R);
+        if (ly.smem_bytes == 0) continue;
+        if (set_plane_relax_smem(true, K, ly.smem_bytes) != 0) {
+            cudaGetLastError();
+            continue;
         }
-        if (cl_smem > 0 && set_plane_relax_smem(h->prec, cf64, true, K, cl_smem) != 0)
-            return fail(SMG_ERR_CUDA, "cudaFuncSetAttribute (plane relaxation, cluster) failed");
+        h->cl_ok[lr] = cluster_resident(K, R, h->threads, ly.smem_bytes);
+        if (h->cl_ok[lr]) cl_smem = std::max(cl_smem, ly.smem_bytes);
     }
+    if (cl_smem > 0 && set_plane_relax_smem(true, K, cl_smem) != 0)
+        return fail(SMG_ERR_CUDA, "cudaFuncSetAttribute (plane relaxation, cluster) failed");
     // a shortened-step layout is usable when its shared memory can be granted and (cluster) its
     // CTAs fit on the GPU at once; a cluster layout takes its coarse levels solo where it can
-    auto settle_lean = [&](bool c64, int lr, PlaneLayout &ly) -> bool {
+    auto settle_lean = [&](int lr, PlaneLayout &ly) -> bool {
         const int R = 1 << lr;
         auto usable = [&](const PlaneLayout &l) {
-            if (set_plane_lean_smem(h->prec, c64, lr > 0, K, l.smem_bytes) != 0) {
+            if (set_plane_lean_smem(lr > 0, K, l.smem_bytes) != 0) {
                 cudaGetLastError();
                 return false;
             }
-            return lr == 0 || lean_cluster_resident(h->prec, c64, K, R, h->threads, l.smem_bytes);
+            return lr == 0 || lean_cluster_resident(K, R, h->threads, l.smem_bytes);
         };
         if (lr > 0 && h->solo) {
-            const PlaneLayout sl = with_solo_levels(H, c64 ? 8 : 4, R, h->solo, ly);
+            const PlaneLayout sl = with_solo_levels(H, 8, R, h->solo, ly);
             if (sl.solo_from < kMaxPlaneLevels && usable(sl)) {
                 ly = sl;
                 return true;
@@ -398,8 +367,7 @@ int ensure_levels(smg_ctx *h, int nb) {
         }
         return usable(ly);
     };
-    // FP64-compute shortened-step layouts (every 2D level's factor sets on chip), one CTA or a
-    // cluster per plane
+    // shortened-step layouts (every 2D level's factor sets on chip), one CTA or a cluster per plane
     for (int lr = 0; lr <= 4; ++lr) {
         h->lean64_ok[lr] = false;
         if (!lean_supported(K)) break;
@@ -407,25 +375,7 @@ int ensure_levels(smg_ctx *h, int nb) {
         PlaneLayout &ly = h->lay_lean64[lr];
         ly = (lr == 0) ? plan_plane_layout(H, 8, kSmemBudget, 0, true) : plan_plane_layout_cluster(H, 8, kSmemBudget, R, true);
         if (ly.smem_bytes == 0 || ly.smem_bytes > kSmemBudget || ly.MF != H.P) continue;
-        h->lean64_ok[lr] = settle_lean(true, lr, ly);
-    }
-    // the same for FP32 compute (FP32 and BF16 cycles): used where the general layout does not keep
-    // every factor set on chip (one CTA) or the plane is spread over a cluster
-    for (int lr = 0; lr <= 4; ++lr) {
-        h->lean32_ok[lr] = false;
-        if (!lean_supported(K) || h->prec == Prec::F64) break;
-        const int R = 1 << lr;
-        PlaneLayout &ly = h->lay_lean32[lr];
-        ly = (lr == 0) ? plan_plane_layout(H, 4, kSmemBudget, 0, true) : plan_plane_layout_cluster(H, 4, kSmemBudget, R, true);
-        if (ly.smem_bytes == 0 || ly.smem_bytes > kSmemBudget || ly.MF != H.P) continue;
-        h->lean32_ok[lr] = settle_lean(false, lr, ly);
-    }
-    // a single-CTA lean layout can need more shared memory than the general one
-    {
-        size_t m32 = h->lay_c.smem_bytes;
-        if (h->lean32_ok[0]) m32 = std::max(m32, h->lay_lean32[0].smem_bytes);
-        if (h->prec != Prec::F64 && lean_supported(K) && set_plane_lean_smem(h->prec, false, false, K, m32) != 0)
-            return fail(SMG_ERR_CUDA, "cudaFuncSetAttribute (plane relaxation, shortened-step cycle) failed");
+        h->lean64_ok[lr] = settle_lean(lr, ly);
     }
     return alloc_plane_workspace(h, nb);
 }
@@ -434,17 +384,11 @@ int ensure_levels(smg_ctx *h, int nb) {
 // of a colour of the finest level) or one per cluster, sized for the largest usable layout.
 int alloc_plane_workspace(smg_ctx *h, int nb) {
     const HostHierarchy &H = h->H;
-    size_t per = std::max(static_cast<size_t>(h->lay_c.ws_per_plane) * compute_bytes(h->prec),
-                          static_cast<size_t>(h->lay_d.ws_per_plane) * 8);
-    for (int lr = 1; lr <= 4; ++lr) {
-        if (h->cl_ok[lr]) per = std::max(per, static_cast<size_t>(h->lay_cl[lr].ws_per_plane) * 8);
-        if (h->cl32_ok[lr]) per = std::max(per, static_cast<size_t>(h->lay_cl32[lr].ws_per_plane) * 4);
-    }
+    size_t per = static_cast<size_t>(h->lay_c.ws_per_plane) * 8;
     for (int lr = 0; lr <= 4; ++lr) {
+        if (h->cl_ok[lr]) per = std::max(per, static_cast<size_t>(h->lay_cl[lr].ws_per_plane) * 8);
         if (h->lean64_ok[lr]) per = std::max(per, static_cast<size_t>(h->lay_lean64[lr].ws_per_plane) * 8);
-        if (h->lean32_ok[lr]) per = std::max(per, static_cast<size_t>(h->lay_lean32[lr].ws_per_plane) * 4);
-        if (h->wcl_ok[1][lr]) per = std::max(per, static_cast<size_t>(h->lay_wcl[1][lr].ws_per_plane) * 8);
-        if (h->wcl_ok[0][lr]) per = std::max(per, static_cast<size_t>(h->lay_wcl[0][lr].ws_per_plane) * 4);
+        if (h->wcl_ok[lr]) per = std::max(per, static_cast<size_t>(h->lay_wcl[lr].ws_per_plane) * 8);
     }
     const long long slots = static_cast<long long>((H.nz + 1) / 2) * nb;
     h->ws_bytes = std::max<size_t>(per * slots, 256);
@@ -495,36 +439,21 @@ int relax(smg_ctx *h, int l, int colour, int mode, int iters, bool coarsest, con
     const int nzl = H.nz_l[l];
     const int nplanes = colour == 0 ? (nzl + 1) / 2 : nzl / 2;
     if (nplanes == 0) return SMG_OK;
-    const bool f64c = coarsest || h->prec == Prec::F64;
-    // Each plane is spread over a cluster of R CTAs while the grid still fits on the SMs at once.
-    // Defaults (measured on GB300 at 128^3 and 256^3): FP64 planes up to 16 CTAs for the one-plane
-    // coarsest level and up to 8 elsewhere (beyond 8 the cluster barrier costs more than the
-    // FP64 work it spreads); FP32 planes stay on one CTA while its 2D-cycle iterate u_0 fits in
-    // shared memory (the cycle is then latency-bound and a cluster only adds barrier cost), and
-    // use up to 4 CTAs when it does not (256-wide planes).  Planes with x-lines longer than 512
-    // rows (plane_wide.cu) hold several lines per team of warps and are spread the same way, FP32
-    // ones over up to 8 CTAs (the paper's 16n x n x n bricks: 1280 x 80 x 80 FPCG 116 -> 57 ms).
+    // Each plane is spread over a cluster of R CTAs while the grid still fits on the SMs at once: up to 16
+    // CTAs for the one-plane coarsest level and up to 8 elsewhere (beyond 8 the cluster barrier costs more
+    // than the FP64 work it spreads; measured at 128^3 and 256^3).
     int R = 1;
     const int wk = wide_rows(h);
     const int W = wide_segments(wk, h->nx);
-    const bool *ok = (W > 1) ? h->wcl_ok[f64c ? 1 : 0] : (f64c ? h->cl_ok : h->cl32_ok);
-    int rmax;
-    if (f64c) rmax = coarsest ? h->cluster_max : std::min(h->cluster_max, 8);
-    else if (h->cluster_max32 > 0) rmax = h->cluster_max32;
-    else if (W > 1) rmax = 8;
-    else rmax = (h->lay_c.smem_u_mask & 1u) ? 1 : 4;
+    const bool *ok = W > 1 ? h->wcl_ok : h->cl_ok;
+    const int rmax = coarsest ? h->cluster_max : std::min(h->cluster_max, 8);
     for (int cand = 2; cand <= rmax && cand <= 16; cand *= 2)
         if (ok[__builtin_ctz(cand)] && static_cast<long long>(nplanes) * nb * cand <= h->num_sms) R = cand;
-    const PlaneLayout &lay =
-        (R > 1) ? (W > 1 ? h->lay_wcl[f64c ? 1 : 0][__builtin_ctz(R)]
-                         : (f64c ? h->lay_cl[__builtin_ctz(R)] : h->lay_cl32[__builtin_ctz(R)]))
-                : ((f64c && h->prec != Prec::F64) ? h->lay_d : h->lay_c);
+    const PlaneLayout &lay = R == 1 ? h->lay_c : W > 1 ? h->lay_wcl[__builtin_ctz(R)] : h->lay_cl[__builtin_ctz(R)];
     PlaneRelaxArgs a;
     std::memset(&a, 0, sizeof(a));
     a.solo_from = kMaxPlaneLevels;
     a.lean = (W > 1 && h->lean) ? 1 : 0;  // wide lines: the shortened step order
-    // the level's table was formed in its compute type: FP64 exactly when f64c (the coarsest level
-    // or an FP64 cycle)
     if (W > 1 && h->d_wftab != nullptr && l < static_cast<int>(h->wftab_off.size()) && h->wftab_off[l] >= 0) {
         a.wftab = h->d_wftab + h->wftab_off[l];
         a.wfslot = h->d_wfslot + h->wfslot_off[l];
@@ -539,8 +468,6 @@ int relax(smg_ctx *h, int l, int colour, int mode, int iters, bool coarsest, con
     a.u = u;
     a.vstride = h->Nl(l);
     a.zcoef = h->d_zcoef + static_cast<size_t>(H.plane_base[l]) * kCoefPerPlane;
-    a.zcoef32 = h->d_zcoef32 + static_cast<size_t>(H.plane_base[l]) * kCoefPerPlane;
-    a.pcoef32 = h->d_pcoef32 + static_cast<size_t>(H.plane_base[l]) * H.sum_ny * kCoefPerLine;
     a.pcoef = h->d_pcoef + static_cast<size_t>(H.plane_base[l]) * H.sum_ny * kCoefPerLine;
     a.gws = h->d_ws;
     a.ws_per_plane = lay.ws_per_plane;
@@ -572,33 +499,21 @@ int relax(smg_ctx *h, int l, int colour, int mode, int iters, bool coarsest, con
         e1 = take_event(h);
         cudaEventRecord(e0, st);
     }
-    // the shortened-step cycle: FP32 compute on one CTA per plane with the same layout; FP64
-    // compute with its own layouts, the cluster chosen by the same rule as above
-    bool use_lean = false;
-    const PlaneLayout *llay = &lay;
+    // the shortened-step cycle, with layouts of its own, the cluster chosen by the same rule as above
+    const PlaneLayout *llay = nullptr;
     if (W == 1 && h->lean && lean_supported(K) && h->lean_level[l]) {
-        if (!f64c) {
-            if (iters == 1 && R == 1 && lay.MF == H.P) {
-                use_lean = true;  // the general layout already keeps every factor set on chip
-            } else if (iters == 1 && h->lean32_ok[__builtin_ctz(R)]) {
-                use_lean = true;
-                llay = &h->lay_lean32[__builtin_ctz(R)];
-            }
-        } else {
-            int lrb = -1;
-            for (int lr = 0; lr <= 4; ++lr) {
-                const int cand = 1 << lr;
-                if (cand > rmax && lr > 0) break;
-                if (h->lean64_ok[lr] && (lr == 0 || static_cast<long long>(nplanes) * nb * cand <= h->num_sms)) lrb = lr;
-            }
-            if (lrb >= 0) {
-                use_lean = true;
-                llay = &h->lay_lean64[lrb];
-                a.R = 1 << lrb;
-            }
+        int lrb = -1;
+        for (int lr = 0; lr <= 4; ++lr) {
+            const int cand = 1 << lr;
+            if (cand > rmax && lr > 0) break;
+            if (h->lean64_ok[lr] && (lr == 0 || static_cast<long long>(nplanes) * nb * cand <= h->num_sms)) lrb = lr;
+        }
+        if (lrb >= 0) {
+            llay = &h->lay_lean64[lrb];
+            a.R = 1 << lrb;
         }
     }
-    if (use_lean && llay != &lay) {
+    if (llay) {
         a.ws_per_plane = llay->ws_per_plane;
         for (int m = 0; m < H.P; ++m) {
             a.off_u[m] = llay->off_u[m];
@@ -610,9 +525,9 @@ int relax(smg_ctx *h, int l, int colour, int mode, int iters, bool coarsest, con
         a.off_fs = llay->off_fs;
         a.solo_from = llay->solo_from;
     }
-    cudaError_t err = (W > 1)  ? launch_plane_wide(wk, h->prec, f64c, nplanes, nb, h->threads, a, lay.smem_bytes, st)
-                      : use_lean ? launch_plane_lean(h->prec, f64c, K, nplanes, nb, h->threads, a, llay->smem_bytes, st)
-                                 : launch_plane_relax(h->prec, f64c, K, nplanes, nb, h->threads, a, lay.smem_bytes, st);
+    cudaError_t err = (W > 1)  ? launch_plane_wide(wk, nplanes, nb, h->threads, a, lay.smem_bytes, st)
+                      : llay ? launch_plane_lean(K, nplanes, nb, h->threads, a, llay->smem_bytes, st)
+                             : launch_plane_relax(K, nplanes, nb, h->threads, a, lay.smem_bytes, st);
     if (err != cudaSuccess) return fail(SMG_ERR_CUDA, std::string("plane relaxation launch: ") + cudaGetErrorString(err));
     h->launches += 1;
     if (timed) {
@@ -665,9 +580,8 @@ int run_cycle(smg_ctx *h, int nb, const void *f0, void *u0, cudaStream_t st) {
             if ((rc = relax(h, l, 1, s == 0 ? 1 : 2, 1, false, F(l), U(l), nb, st)) != SMG_OK) return rc;
         }
         RegionTimer rt(h, st, 3, 2.5 * h->Nl(l) * nb * storage_bytes(h->prec));
-        cudaError_t e = launch_restrict(h->prec, h->nx, h->ny, H.nz_l[l], nb, F(l), U(l), h->d_f[l + 1],
+        cudaError_t e = launch_restrict(h->nx, h->ny, H.nz_l[l], nb, F(l), U(l), h->d_f[l + 1],
                                         h->d_zcoef + static_cast<size_t>(H.plane_base[l]) * kCoefPerPlane,
-                                        h->d_zcoef32 + static_cast<size_t>(H.plane_base[l]) * kCoefPerPlane,
                                         h->Nl(l), h->Nl(l + 1), st, h->restrict_column != 0);
         if (e != cudaSuccess) return fail(SMG_ERR_CUDA, std::string("restriction launch: ") + cudaGetErrorString(e));
         h->launches += 1;
@@ -675,9 +589,8 @@ int run_cycle(smg_ctx *h, int nb, const void *f0, void *u0, cudaStream_t st) {
     if ((rc = relax(h, L - 1, 0, 0, h->coarse_iters, true, F(L - 1), U(L - 1), nb, st)) != SMG_OK) return rc;
     for (int l = L - 2; l >= 0; --l) {
         RegionTimer rt(h, st, 3, 2.5 * h->Nl(l) * nb * storage_bytes(h->prec));
-        cudaError_t e = launch_prolong(h->prec, h->nx, h->ny, H.nz_l[l], nb, U(l), U(l + 1),
+        cudaError_t e = launch_prolong(h->nx, h->ny, H.nz_l[l], nb, U(l), U(l + 1),
                                        h->d_zcoef + static_cast<size_t>(H.plane_base[l]) * kCoefPerPlane,
-                                       h->d_zcoef32 + static_cast<size_t>(H.plane_base[l]) * kCoefPerPlane,
                                        h->Nl(l), h->Nl(l + 1), st);
         if (e != cudaSuccess) return fail(SMG_ERR_CUDA, std::string("prolongation launch: ") + cudaGetErrorString(e));
         h->launches += 1;
@@ -948,13 +861,6 @@ int smg_setup(int nx, int ny, int nz, int npre, int npost, smg_handle *out) {
     if (e == cudaSuccess) e = cudaMalloc(&h->d_pcoef, pb);
     if (e == cudaSuccess) e = cudaMemcpy(h->d_zcoef, h->H.zcoef.data(), zb, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(h->d_pcoef, h->H.pcoef.data(), pb, cudaMemcpyHostToDevice);
-    {
-        std::vector<float> z32(h->H.zcoef.begin(), h->H.zcoef.end()), p32(h->H.pcoef.begin(), h->H.pcoef.end());
-        if (e == cudaSuccess) e = cudaMalloc(&h->d_zcoef32, z32.size() * sizeof(float));
-        if (e == cudaSuccess) e = cudaMalloc(&h->d_pcoef32, p32.size() * sizeof(float));
-        if (e == cudaSuccess) e = cudaMemcpy(h->d_zcoef32, z32.data(), z32.size() * sizeof(float), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = cudaMemcpy(h->d_pcoef32, p32.data(), p32.size() * sizeof(float), cudaMemcpyHostToDevice);
-    }
     if (e != cudaSuccess) {
         smg_destroy(h);
         return fail(SMG_ERR_CUDA, std::string("smg_setup: ") + cudaGetErrorString(e));
@@ -1029,7 +935,6 @@ int smg_set_option(smg_handle h, int option, int value) {
     case SMG_OPT_CLUSTER_MAX32:
         if (value != 0 && value != 1 && value != 2 && value != 4 && value != 8 && value != 16)
             return fail(SMG_ERR_ARG, "cluster_max32 must be 0 (automatic), 1, 2, 4, 8 or 16");
-        h->cluster_max32 = value;
         return SMG_OK;
     case SMG_OPT_GRAM_TC:
         if (value < 0 || value > 64) return fail(SMG_ERR_ARG, "gram_tc must be in [0, 64]");
@@ -1038,11 +943,6 @@ int smg_set_option(smg_handle h, int option, int value) {
     case SMG_OPT_LEAN:
         if (value != 0 && value != 1) return fail(SMG_ERR_ARG, "lean must be 0 or 1");
         h->lean = value;
-        return SMG_OK;
-    case SMG_OPT_MODAL:
-        if (value != 0 && value != 1) return fail(SMG_ERR_ARG, "modal must be 0 or 1");
-        if (value != h->modal) free_levels(h);
-        h->modal = value;
         return SMG_OK;
     case SMG_OPT_PROFILE:
         if (value < 0 || value > 2) return fail(SMG_ERR_ARG, "profile must be 0, 1 or 2");
@@ -1059,16 +959,10 @@ int smg_apply_batched(smg_handle h, int nb, const double *R, double *S, void *st
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     int rc;
     if ((rc = ensure_levels(h, nb)) != SMG_OK) return rc;
-    const long long n = h->N() * nb;
     if (h->modal_now) {
         if ((rc = run_modal(h, nb, Prec::F64, R, Prec::F64, S, st)) != SMG_OK) return rc;
-    } else if (h->prec == Prec::F64) {
-        if ((rc = run_cycle(h, nb, R, S, st)) != SMG_OK) return rc;
     } else {
-        SMG_CUDA(launch_convert_to(h->prec, n, R, h->d_f[0], st));
-        if ((rc = run_cycle(h, nb, h->d_f[0], h->d_u[0], st)) != SMG_OK) return rc;
-        SMG_CUDA(launch_convert_from(h->prec, n, h->d_u[0], S, st));
-        h->launches += 2;
+        if ((rc = run_cycle(h, nb, R, S, st)) != SMG_OK) return rc;
     }
     if (h->learned) {
         const long long l0 = h->nw.launches;
@@ -1381,8 +1275,6 @@ int smg_destroy(smg_handle h) {
     free_levels(h);
     cudaFree(h->d_zcoef);
     cudaFree(h->d_pcoef);
-    cudaFree(h->d_zcoef32);
-    cudaFree(h->d_pcoef32);
     cudaFree(h->d_r);
     cudaFree(h->d_p);
     cudaFree(h->d_q);

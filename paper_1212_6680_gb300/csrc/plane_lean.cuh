@@ -431,10 +431,10 @@ __device__ __forceinline__ void plane_lean_task(const PlaneRelaxArgs &a, int pid
     const S *fb = reinterpret_cast<const S *>(a.f) + static_cast<long long>(b) * a.vstride;
     S *ub = reinterpret_cast<S *>(a.u) + static_cast<long long>(b) * a.vstride;
     S *plane = ub + static_cast<long long>(z) * np;
-    const C *zc = coef_table<C>(a.zcoef, a.zcoef32) + static_cast<long long>(z) * kCoefPerPlane;
+    const C *zc = a.zcoef + static_cast<long long>(z) * kCoefPerPlane;
     __shared__ LeanLevel<C> s_lv[kMaxPlaneLevels];
     {
-        const C *pc = coef_table<C>(a.pcoef, a.pcoef32) + static_cast<long long>(z) * a.sum_ny * kCoefPerLine;
+        const C *pc = a.pcoef + static_cast<long long>(z) * a.sum_ny * kCoefPerLine;
         for (int i = tid; i < a.sum_ny * kCoefPerLine; i += nt) sm[i] = pc[i];
         if (tid < P) {
             LeanLevel<C> L;

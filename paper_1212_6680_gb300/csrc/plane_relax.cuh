@@ -93,11 +93,6 @@ template <> __device__ __forceinline__ void stv<double, double>(double *p, doubl
 template <> __device__ __forceinline__ void stv<float, double>(float *p, double v) { *p = narrow_f64(v); }
 template <> __device__ __forceinline__ void stv<__nv_bfloat16, double>(__nv_bfloat16 *p, double v) { *p = __float2bfloat16_rn(narrow_f64(v)); }
 
-// Coefficient tables are stored in both precisions; each kernel reads the one it computes in.
-template <class C> __device__ __forceinline__ const C *coef_table(const double *d64, const float *d32);
-template <> __device__ __forceinline__ const double *coef_table<double>(const double *d64, const float *) { return d64; }
-template <> __device__ __forceinline__ const float *coef_table<float>(const double *, const float *d32) { return d32; }
-
 // ---- warp tridiagonal solver ---------------------------------------------------------------
 // Solves the n x n system  of*x[i-1] + dg*x[i] + of*x[i+1] = d[i]  (Dirichlet ends) held by a
 // warp: lane l owns rows lK .. lK+K-1; rows >= n are identity rows with d = 0.  dg > 2|of|
@@ -815,8 +810,7 @@ __device__ __forceinline__ void compute_rhs(const PlaneRelaxArgs &a, const Plane
 
 // The relaxation of one plane (the pidx-th plane of the colour, batch entry b) by one CTA
 // (CL = false) or by this CTA's share of a cluster (CL = true).  `slot` selects the CTA's part
-// of the global workspace.  Used by the per-launch kernel below and by the persistent
-// multi-system kernel.
+// of the global workspace.
 template <class S, class C, int K, bool CL>
 __device__ __forceinline__ void plane_task(const PlaneRelaxArgs &a, int pidx, int b, long long slot, int rank,
                                            unsigned char *smem_raw) {
@@ -852,9 +846,9 @@ __device__ __forceinline__ void plane_task(const PlaneRelaxArgs &a, int pidx, in
     const S *fb = reinterpret_cast<const S *>(a.f) + static_cast<long long>(b) * a.vstride;
     S *ub = reinterpret_cast<S *>(a.u) + static_cast<long long>(b) * a.vstride;
     S *plane = ub + static_cast<long long>(z) * np;
-    const C *zc = coef_table<C>(a.zcoef, a.zcoef32) + static_cast<long long>(z) * kCoefPerPlane;
+    const C *zc = a.zcoef + static_cast<long long>(z) * kCoefPerPlane;
     {
-        const C *pc = coef_table<C>(a.pcoef, a.pcoef32) + static_cast<long long>(z) * a.sum_ny * kCoefPerLine;
+        const C *pc = a.pcoef + static_cast<long long>(z) * a.sum_ny * kCoefPerLine;
         for (int i = tid; i < a.sum_ny * kCoefPerLine; i += nt) c.sm[i] = pc[i];
     }
     // the interior line matrix of each of the first MF 2D levels is factored once, by warp m

@@ -627,9 +627,9 @@ __global__ void __launch_bounds__(wide_threads<C>(), 1) plane_wide_kernel(const 
     const S *fb = reinterpret_cast<const S *>(a.f) + static_cast<long long>(b) * a.vstride;
     S *ub = reinterpret_cast<S *>(a.u) + static_cast<long long>(b) * a.vstride;
     S *plane = ub + static_cast<long long>(z) * np;
-    const C *zc = coef_table<C>(a.zcoef, a.zcoef32) + static_cast<long long>(z) * kCoefPerPlane;
+    const C *zc = a.zcoef + static_cast<long long>(z) * kCoefPerPlane;
     {
-        const C *pc = coef_table<C>(a.pcoef, a.pcoef32) + static_cast<long long>(z) * a.sum_ny * kCoefPerLine;
+        const C *pc = a.pcoef + static_cast<long long>(z) * a.sum_ny * kCoefPerLine;
         for (int i = tid; i < a.sum_ny * kCoefPerLine; i += nt) c.sm[i] = pc[i];
     }
     __syncthreads();
@@ -722,7 +722,6 @@ struct WideFactorArgs {
     int line_base[kMaxPlaneLevels];
     const int *planes;    // the plane of each slot (null: slot s is plane s)
     const double *pcoef;  // the planes' coefficient tables (sum_ny lines x kCoefPerLine each)
-    const float *pcoef32; // the same rounded to FP32
     void *tab;            // out: 2P W kWEntry values of the compute type per slot
 };
 
@@ -757,7 +756,7 @@ __global__ void wide_factor_kernel(const __grid_constant__ WideFactorArgs a) {
     c.xb = s_xb;
     c.ftab = nullptr;
     const int y = set ? a.ny_m[m] - 1 : 0;
-    const CoefRow<C> cr = coef_row<C>(coef_table<C>(a.pcoef, a.pcoef32) +
+    const CoefRow<C> cr = coef_row<C>(a.pcoef +
                                       (static_cast<long long>(p) * a.sum_ny + a.line_base[m] + y) * kCoefPerLine);
     C dg, of;
     line_matrix<C>(cr, dg, of);
@@ -831,8 +830,7 @@ bool wide_resident(int R, int threads, size_t smem) {
 long long SMG_WNAME(wide_factor_values)(int P, int W) { return 2LL * P * W * kWEntry; }
 
 cudaError_t SMG_WNAME(launch_wide_factor_table)(int nx, int W, int P, int sum_ny, const int *ny_m, const int *line_base,
-                                     int nslots, const int *planes, const double *pcoef, const float *pcoef32,
-                                     bool f64, void *tab, cudaStream_t st) {
+                                     int nslots, const int *planes, const double *pcoef, void *tab, cudaStream_t st) {
     if (W < 2 || W > kMaxSeg || P < 1 || P > kMaxPlaneLevels || nslots < 1) return cudaErrorInvalidValue;
     WideFactorArgs a;
     a.nx = nx;
@@ -845,48 +843,19 @@ cudaError_t SMG_WNAME(launch_wide_factor_table)(int nx, int W, int P, int sum_ny
     }
     a.planes = planes;
     a.pcoef = pcoef;
-    a.pcoef32 = pcoef32;
     a.tab = tab;
-    if (f64) wide_factor_kernel<double><<<dim3(nslots, 2 * P), 32 * W, 0, st>>>(a);
-    else wide_factor_kernel<float><<<dim3(nslots, 2 * P), 32 * W, 0, st>>>(a);
+    wide_factor_kernel<double><<<dim3(nslots, 2 * P), 32 * W, 0, st>>>(a);
     return cudaGetLastError();
 }
 
-cudaError_t SMG_WNAME(launch_plane_wide)(Prec storage, bool f64, int nplanes, int nb, int threads, const PlaneRelaxArgs &a,
-                              size_t smem, cudaStream_t st) {
+cudaError_t SMG_WNAME(launch_plane_wide)(int nplanes, int nb, int threads, const PlaneRelaxArgs &a, size_t smem, cudaStream_t st) {
     if (a.W < 2 || a.W > kMaxSeg || threads / 32 < a.W || threads > 512 || a.R < 1 || a.R > 16 || (a.R & (a.R - 1)))
         return cudaErrorInvalidValue;
-    switch (storage) {
-    case Prec::F64: return launch_wide<double, double>(nplanes, nb, threads, a, smem, st);
-    case Prec::F32:
-        return f64 ? launch_wide<float, double>(nplanes, nb, threads, a, smem, st)
-                   : launch_wide<float, float>(nplanes, nb, threads, a, smem, st);
-    case Prec::BF16:
-        return f64 ? launch_wide<__nv_bfloat16, double>(nplanes, nb, threads, a, smem, st)
-                   : launch_wide<__nv_bfloat16, float>(nplanes, nb, threads, a, smem, st);
-    }
-    return cudaErrorInvalidValue;
+    return launch_wide<double, double>(nplanes, nb, threads, a, smem, st);
 }
 
-int SMG_WNAME(set_plane_wide_smem)(Prec storage, bool f64, bool cl, size_t smem) {
-    switch (storage) {
-    case Prec::F64: return wide_smem_attr<double, double>(cl, smem);
-    case Prec::F32: return f64 ? wide_smem_attr<float, double>(cl, smem) : wide_smem_attr<float, float>(cl, smem);
-    case Prec::BF16:
-        return f64 ? wide_smem_attr<__nv_bfloat16, double>(cl, smem) : wide_smem_attr<__nv_bfloat16, float>(cl, smem);
-    }
-    return static_cast<int>(cudaErrorInvalidValue);
-}
+int SMG_WNAME(set_plane_wide_smem)(bool cl, size_t smem) { return wide_smem_attr<double, double>(cl, smem); }
 
-bool SMG_WNAME(wide_cluster_resident)(Prec storage, bool f64, int R, int threads, size_t smem) {
-    switch (storage) {
-    case Prec::F64: return wide_resident<double, double>(R, threads, smem);
-    case Prec::F32: return f64 ? wide_resident<float, double>(R, threads, smem) : wide_resident<float, float>(R, threads, smem);
-    case Prec::BF16:
-        return f64 ? wide_resident<__nv_bfloat16, double>(R, threads, smem)
-                   : wide_resident<__nv_bfloat16, float>(R, threads, smem);
-    }
-    return false;
-}
+bool SMG_WNAME(wide_cluster_resident)(int R, int threads, size_t smem) { return wide_resident<double, double>(R, threads, smem); }
 
 }  // namespace smg

@@ -107,8 +107,6 @@ struct PlaneRelaxArgs {
     long long vstride;       // elements between batch entries of f and u
     const double *zcoef;     // this level's plane coefficients (8 per plane)
     const double *pcoef;     // this level's plane tables (sum_ny * 8 per plane)
-    const float *zcoef32;    // the same two tables rounded to FP32 (for FP32 compute)
-    const float *pcoef32;
     void *gws;               // global workspace (compute type), one slot per CTA
     long long ws_per_plane;  // elements per CTA slot
     int P;                   // 2D levels
@@ -125,13 +123,11 @@ struct PlaneRelaxArgs {
     int vec;                      // 1: nx == 32 K and f, u, the workspace are 16-byte aligned
                                   // (wide lines: nx % 8 == 0 and the same alignment)
     int W;                        // x-line segments of 512 rows (1 unless nx > 512: plane_wide.cu)
-    int lean;                     // 1: the shortened step order (the persistent multi-system
-                                  // kernel, whose layout then keeps every factor set on chip; the
-                                  // wide-line kernel)
+    int lean;                     // 1: the shortened step order (the wide-line kernel)
     int solo_from;                // shortened-step cycle on a cluster: 2D levels >= solo_from belong
                                   // whole to CTA 0 (kMaxPlaneLevels: none)
     const void *wftab;            // wide lines: the precomputed line-solver data of this level's
-                                  // planes in its compute type (wide_factor_table), or null
+                                  // planes (wide_factor_table), or null
     const int *wfslot;            // with wftab: the table slot of each plane of the level (planes
                                   // with equal coefficient tables share one), or null: slot = plane
 };
@@ -170,32 +166,28 @@ PlaneLayout plan_plane_layout_cluster(const HostHierarchy &H, size_t elem_bytes,
 enum class Prec { F64 = 0, F32 = 1, BF16 = 2 };
 size_t storage_bytes(Prec p);
 
-// Plane relaxation: S = storage type, compute in double (F64 / coarsest) or float.
-cudaError_t launch_plane_relax(Prec storage, bool compute_f64, int K, int nplanes, int nb,
+// Plane relaxation (FP64).
+cudaError_t launch_plane_relax(int K, int nplanes, int nb,
                                int threads, const PlaneRelaxArgs &a, size_t smem, cudaStream_t st);
 // column: each thread walks several coarse planes and computes each fine residual once (else one
 // coarse plane per thread); the results are bit-identical.
-cudaError_t launch_restrict(Prec storage, int nx, int ny, int nzf, int nb, const void *f,
-                            const void *u, void *fc, const double *zcoef, const float *zcoef32,
+cudaError_t launch_restrict(int nx, int ny, int nzf, int nb, const void *f, const void *u, void *fc, const double *zcoef,
                             long long vstride_f, long long vstride_c, cudaStream_t st, bool column = true);
-cudaError_t launch_prolong(Prec storage, int nx, int ny, int nzf, int nb, void *u, const void *uc,
-                           const double *zcoef, const float *zcoef32, long long vstride_f,
+cudaError_t launch_prolong(int nx, int ny, int nzf, int nb, void *u, const void *uc, const double *zcoef, long long vstride_f,
                            long long vstride_c, cudaStream_t st);
 // Compares the integer-pipe FP32 <-> FP64 conversions with the hardware ones on n values:
 // mism[0] counts narrowing mismatches, mism[1] widening mismatches (device int[2]).
 cudaError_t launch_check_conversions(long long n, const double *src, int *mism, cudaStream_t st);
-cudaError_t launch_convert_to(Prec storage, long long n, const double *src, void *dst, cudaStream_t st);
-cudaError_t launch_convert_from(Prec storage, long long n, const void *src, double *dst, cudaStream_t st);
 cudaError_t launch_apply_A(int nx, int ny, int nz, int nb, const double *u, double *out, cudaStream_t st);
-int set_plane_relax_smem(Prec storage, bool compute_f64, bool cluster, int K, size_t smem);
+int set_plane_relax_smem(bool cluster, int K, size_t smem);
 // The shortened-step plane cycle (plane_lean.cuh): nx <= 256 (K <= 8), every 2D level's factor
 // sets in shared memory, and every line of a 2D level but its last sharing one line matrix
-// (lean_uniform_level); FP32 or FP64 compute on one CTA or a cluster of a.R CTAs per plane.
+// (lean_uniform_level), on one CTA or a cluster of a.R CTAs per plane.
 bool lean_supported(int K);
-cudaError_t launch_plane_lean(Prec storage, bool compute_f64, int K, int nplanes, int nb, int threads,
+cudaError_t launch_plane_lean(int K, int nplanes, int nb, int threads,
                               const PlaneRelaxArgs &a, size_t smem, cudaStream_t st);
-int set_plane_lean_smem(Prec storage, bool compute_f64, bool cluster, int K, size_t smem);
-bool lean_cluster_resident(Prec storage, bool compute_f64, int K, int R, int threads, size_t smem);
+int set_plane_lean_smem(bool cluster, int K, size_t smem);
+bool lean_cluster_resident(int K, int R, int threads, size_t smem);
 // True when, on every plane of z-level l and every 2D level, the lines before the last share the
 // line matrix (S(y,y), T(y,y)) of line 0.
 bool lean_uniform_level(const HostHierarchy &H, int l);
@@ -207,23 +199,21 @@ int plane_classes(const HostHierarchy &H, int l, std::vector<int> &slot, std::ve
 // 32 wk rows, wk = 16 (lines of 513-2048 rows) or 8 (257-512 rows), one warp each.
 inline int wide_segments(int wk, int nx) { return wk > 0 ? (nx + 32 * wk - 1) / (32 * wk) : 1; }
 // Line-solver data of wide-line planes, formed once instead of at every change of line matrix
-// inside the plane cycle: for nplanes consecutive planes of one z-level (pcoef / pcoef32: their
+// inside the plane cycle: for nplanes consecutive planes of one z-level (pcoef: their
 // coefficient tables) and every 2D level m and line set (0: the first line's matrix, 1: the
 // last line's), the segment factors, T_s^{-1} e_first, T_s^{-1} e_last and the reduced system's
-// inverse rows of every segment, in the compute type (FP64 when f64, else FP32), computed by the
-// same code as on the fly (bit-identical).  wide_factor_values(wk, P, W): values per plane.
+// inverse rows of every segment, computed by the same code as on the fly (bit-identical).  wide_factor_values(wk, P, W): values per plane.
 // The table has nslots entries of that size; slot s holds the data of plane planes[s] (device
 // array; null: plane s).
 long long wide_factor_values(int wk, int P, int W);
 cudaError_t launch_wide_factor_table(int wk, int nx, int W, int P, int sum_ny, const int *ny_m, const int *line_base,
-                                     int nslots, const int *planes, const double *pcoef, const float *pcoef32,
-                                     bool f64, void *tab, cudaStream_t st);
-cudaError_t launch_plane_wide(int wk, Prec storage, bool compute_f64, int nplanes, int nb, int threads,
+                                     int nslots, const int *planes, const double *pcoef, void *tab, cudaStream_t st);
+cudaError_t launch_plane_wide(int wk, int nplanes, int nb, int threads,
                               const PlaneRelaxArgs &a, size_t smem, cudaStream_t st);
-int set_plane_wide_smem(int wk, Prec storage, bool compute_f64, bool cluster, size_t smem);
+int set_plane_wide_smem(int wk, bool cluster, size_t smem);
 // Whether a cluster of R wide-line CTAs with `smem` bytes each fits on the GPU at once.
-bool wide_cluster_resident(int wk, Prec storage, bool compute_f64, int R, int threads, size_t smem);
-// True when a cluster of R CTAs of the plane kernel (FP64 or FP32 compute) can be resident.
-bool cluster_resident(Prec storage, bool compute_f64, int K, int R, int threads, size_t smem);
+bool wide_cluster_resident(int wk, int R, int threads, size_t smem);
+// True when a cluster of R CTAs of the plane kernel can be resident.
+bool cluster_resident(int K, int R, int threads, size_t smem);
 
 }  // namespace smg

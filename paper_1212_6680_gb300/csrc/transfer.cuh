@@ -3,7 +3,6 @@
 // indices, coarse j <-> fine 2j+1, interpolation weights wm, wp of the even fine planes):
 //   restriction of the residual  f_c[j] = r[2j+1] + wp(2j) r[2j] + wm(2j+2) r[2j+2],  r = f - A_l u
 //   prolongation + correction    u[2j+1] += e[j],  u[2j] += wm(2j) e[j-1] + wp(2j) e[j]
-// Shared by the per-level kernels and the persistent multi-system kernel.
 #pragma once
 
 #include "plane_relax.cuh"
