@@ -136,15 +136,15 @@ def source_hash():
 
     h = hashlib.sha256()
     d = os.path.join(ROOT, "paper_1212_6680_gb300", "csrc")
-    for f in ("plane_lean.cuh", "plane_relax.cuh", "plane_relax_inst.cu"):
+    for f in ("modal.cuh", "modal_inst.cu"):
         h.update(open(os.path.join(d, f), "rb").read())
     return h.hexdigest()[:16]
 
 
 def ncu_traffic():
-    """DRAM bytes per level-0 launch of the plane-relaxation kernel from the committed ncu
+    """DRAM bytes per launch of the mode-space cycle's kernel from the committed ncu
     summary, if it was captured from the current kernel source (else None)."""
-    p = os.path.join(ROOT, "profiles", "plane_lean_traffic_level0_128cube.txt")
+    p = os.path.join(ROOT, "profiles", "modal_tail_traffic_128cube.txt")
     try:
         d = json.load(open(p))
         if d.get("source_hash") == source_hash():
@@ -368,8 +368,8 @@ def run_ours(args):
     launches = smg.smg_launch_count(h32) - l0
     t_step = statistics.median(times)  # median of the timed steps
     t_max = max_over_ranks(t_step, dist, "cuda")
-    # ---- the finest level's plane-relaxation launches timed with CUDA events on the launching
-    # stream, in solves run right after the timed region (per-launch events cannot sit inside the
+    # ---- the cycle between the transforms (every mode's levels in one launch) timed with CUDA events on the
+    # launching stream, in solves run right after the timed region (per-launch events cannot sit inside the
     # graph, so these solves take the host loop) ----
     kp = max(1, min(args.steps, 3))
     smg.smg_set_option(h32, smg.SMG_OPT_PROFILE, 1)
@@ -382,7 +382,7 @@ def run_ours(args):
     thost, _, _ = timed_solves(h32, kp, 1)
     smg.smg_set_option(h32, smg.SMG_OPT_GRAPH, 1)
 
-    # ---- every plane-relaxation launch of one solve timed (all z-levels, the FP64 coarsest plane) ----
+    # ---- the transforms, the cycle and the Krylov kernels of one solve timed ----
     smg.smg_set_option(h32, smg.SMG_OPT_PROFILE, 2)
     for c in range(6):
         smg.smg_profile_read(h32, c)
@@ -412,28 +412,28 @@ def run_ours(args):
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                 "frac": (achieved / peak) if achieved else None,
                 "traffic": (tr["dram_bytes_per_launch"] if tr else None),
-                "kernel": "plane_lean_kernel<float,float,4,false> (finest level)",
+                "kernel": "modal_tail_kernel<float,16,8> (the V-cycle of every x-mode, a CTA each)",
                 "launches": pl, "avg_launch_us": (pms * 1e3 / pl) if pl else None,
                 "algorithmic_bytes_per_launch": (pbytes / pl) if pl else None,
-                "duration_source": f"CUDA events around every finest-level launch on the launching stream, in {kp} "
+                "duration_source": f"CUDA events around every launch on the launching stream, in {kp} "
                                    f"solves right after the timed region (the timed solves run as one CUDA graph, "
                                    f"which cannot hold the events)",
                 "peak_source": f"{peak_kind} (MEASURED_PEAKS.json hbm_gbs)" if peak_kind == "measured" else
                 "fallback 6.8 TB/s"}
-    # the same ratio over every plane-relaxation launch of a solve (all z-levels, FP32, and the FP64
-    # coarsest plane), and each class of the cycle (CUDA events around every launch: the profiled
-    # solve's launches lose their programmatic-dependent-launch overlap)
-    names = {0: "plane relaxation, finest level", 1: "plane relaxation, other levels", 2: "coarsest plane (FP64)",
-             3: "restriction + prolongation", 4: "Krylov kernels"}
+    # each class of the iteration (CUDA events around every launch: the profiled solve's launches lose
+    # their programmatic-dependent-launch overlap)
+    names = {0: "mode-space cycle", 3: "transforms of the x-lines", 4: "Krylov kernels"}
     classes = {}
     for c, (nl, ms, by) in prof_all.items():
+        if c not in names:
+            continue
         classes[names[c]] = {"launches": nl, "us_per_launch": (ms * 1e3 / nl) if nl else None,
                              "ms_per_solve": ms, "GB_per_s": ((by / 1e9) / (ms / 1e3)) if (ms > 0 and by > 0) else None}
-    rl_ms = sum(prof_all[c][1] for c in (0, 1, 2))
-    rl_by = sum(prof_all[c][2] for c in (0, 1, 2))
+    rl_ms = sum(prof_all[c][1] for c in (0, 3))
+    rl_by = sum(prof_all[c][2] for c in (0, 3))
     if rl_ms > 0:
-        roofline["all_levels"] = {"achieved": (rl_by / 1e9) / (rl_ms / 1e3), "frac": ((rl_by / 1e9) / (rl_ms / 1e3)) / peak,
-                                  "unit": "GB/s", "note": "every plane-relaxation launch of one solve"}
+        roofline["application"] = {"achieved": (rl_by / 1e9) / (rl_ms / 1e3), "frac": ((rl_by / 1e9) / (rl_ms / 1e3)) / peak,
+                                   "unit": "GB/s", "note": "transforms and cycle of every application of one solve"}
     cpu = None
     if not args.no_cpu_baseline:
         cpu = oracle_solve_baseline()
@@ -612,7 +612,7 @@ def run_batched(args):
     achieved = (pbytes / 1e9) / (pms / 1e3) if pms > 0 else None
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                 "frac": (achieved / peak) if achieved else None, "traffic": None,
-                "kernel": "persistent_vcycle_kernel<float,4> (every V-cycle step of every active system)",
+                "kernel": "modal_tail_batch_kernel and the batched transforms (every V-cycle of every active system)",
                 "launches": pl, "avg_launch_us": (pms * 1e3 / pl) if pl else None,
                 "algorithmic_bytes_per_launch": (pbytes / pl) if pl else None,
                 "krylov_avg_us_per_iteration": (kms * 1e3 / kl) if kl else None,
@@ -791,7 +791,7 @@ def run_lobpcg(args):
     achieved = (pbytes / 1e9) / (pms / 1e3) if pms > 0 else None
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                 "frac": (achieved / peak) if achieved else None, "traffic": None,
-                "kernel": "plane_lean_kernel<float,float,4,false> (finest level, 16 vectors per launch)",
+                "kernel": "modal_tail_kernel<float,16,8> (the V-cycle of every x-mode, a CTA each, 16 vectors per launch)",
                 "launches": pl, "avg_launch_us": (pms * 1e3 / pl) if pl else None,
                 "algorithmic_bytes_per_launch": (pbytes / pl) if pl else None,
                 "peak_source": f"{peak_kind} (MEASURED_PEAKS.json hbm_gbs)"}
@@ -935,7 +935,7 @@ def run_learned(args):
     achieved = (l0b / 1e9) / (l0ms / 1e3) if l0ms > 0 else None
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                 "frac": (achieved / peak) if achieved else None, "traffic": None,
-                "kernel": "plane_relax_kernel<float,float,8> (finest level of the 256^3 cycle)",
+                "kernel": "modal_slab_kernel, modal_tail_kernel<float,16,16> and modal_prolong_kernel (the 256^3 cycle in mode space)",
                 "launches": l0n, "avg_launch_us": (l0ms * 1e3 / l0n) if l0n else None,
                 "algorithmic_bytes_per_launch": (l0b / l0n) if l0n else None,
                 "peak_source": f"{peak_kind} (MEASURED_PEAKS.json hbm_gbs)"}

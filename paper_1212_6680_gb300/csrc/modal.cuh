@@ -5,12 +5,12 @@
 // every coupling between lines and planes is of that form too.  In the orthonormal sine basis of the
 // x-direction (Lx v_k = lambda_k v_k) an exact line solve is a division by S lambda_k + T, a coupling
 // a multiplication, and the modes k do not couple at all: the V-cycle is nx independent 2D (y, z)
-// cycles between two dense transforms of the x-lines (modal.cu).  The same linear operator as the
+// cycles between two dense transforms of the x-lines (sine.cu, FP64: modal.cu).  The same linear operator as the
 // plane kernels' in exact arithmetic, step by step the same relaxations.  What it removes is the
 // serial chain of a line solve (elimination, five rounds of cyclic reduction, back substitution) in
 // each of a plane's 4P - 3 dependent steps, and the CTA barrier between them.  One application at
-// 128^3: 672 -> 119 us (FP32), 2352 -> 1018 us (FP64); 256^3 FP32 2154 -> 829 us; 1280x80x80 FP32
-// 3802 -> 1441 us; 24x20x16 FP32 135 -> 27 us.
+// 128^3: 672 -> 75 us (FP32), 2352 -> 969 us (FP64); 256^3 FP32 2154 -> 645 us; 1280x80x80 FP32
+// 3802 -> 704 us; 24x20x16 FP32 135 -> 24 us.
 //
 // One CTA runs the whole cycle of one mode in shared memory (modal_tail); levels whose planes do
 // not fit there run as launches over global memory first (modal_slab, or the single steps).
