@@ -52,9 +52,10 @@ enum { SMG_FP64 = 0, SMG_FP32 = 1, SMG_BF16 = 2 };     /* V-cycle storage precis
 /* Options for smg_set_option.
  *
  * Two forms of the V-cycle exist.  In mode space (every FP32 and BF16 cycle, and FP64 ones with x-lines of at
- * most 160 rows) it runs in the sine eigenvectors of the x-lines: the same relaxations, an exact line solve being a
- * division per mode.  Longer FP64 x-lines run on the plane kernels, to which the options on threads, clusters, step orders,
- * tables and restriction apply (marked "planes"); in mode space these are accepted and change nothing. */
+ * most 160 rows or with nx * N * nb <= 1.5e9 for the nb vectors the handle was last sized for) it runs in the sine
+ * eigenvectors of the x-lines: the same relaxations, an exact line solve being a division per mode.  Larger FP64 cycles run
+ * on the plane kernels, to which the options on threads, clusters, step orders, tables and restriction apply (marked
+ * "planes"); in mode space these are accepted and change nothing.  The two forms differ by rounding. */
 enum {
     SMG_OPT_COARSE_ITERS = 0, /* plane-cycle steps on the one-plane coarsest level (>= 1, default 1) */
     SMG_OPT_THREADS = 1,      /* planes: threads per CTA: 256 or 512 (default 512; the

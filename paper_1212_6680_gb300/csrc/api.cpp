@@ -209,10 +209,19 @@ PlaneLayout with_solo_levels(const HostHierarchy &H, size_t elem_bytes, int R, i
     return base;
 }
 
-// Whether the cycle runs in the x-lines' sine eigenvectors (modal.cuh): every FP32 and BF16 cycle; an
-// FP64 cycle up to kModalMaxNx64 points a line (its transforms are FP64 products of order nx / 2).
+// Whether the cycle of nb right-hand sides runs in the x-lines' sine eigenvectors (modal.cuh): every FP32 and
+// BF16 cycle; an FP64 one, whose transforms are FP64 products of order nx / 2 and which the plane kernels meet
+// once their planes fill the chip, with lines of at most 160 points or while nx times the points stays below a
+// bound.  (1,0) applications in us, mode space / plane kernels: 160x80x80 979 / 2141, 256x64x64 1036 / 2492,
+// 512x64x64 2620 / 4308, 768x48x48 2977 / 4812, 200^3 (1.6e9) 6036 / 6945, 512x128x96 (3.2e9) 6914 / 6582,
+// 256^3 (4.3e9) 10475 / 9563; 8 vectors: 176x64x64 (1.0e9) 3423 / 3986, 256x64x64 (2.1e9) 5422 / 4866, 512x32x32
+// (2.1e9) 4565 / 3667.  (1,1) cycles favour mode space throughout.
 constexpr int kModalMaxNx64 = 160;
-bool use_modal(const smg_ctx *h) { return h->prec != Prec::F64 || h->nx <= kModalMaxNx64; }
+constexpr double kModalMaxWork64 = 1.5e9;
+bool use_modal(const smg_ctx *h, int nb) {
+    return h->prec != Prec::F64 || h->nx <= kModalMaxNx64 ||
+           static_cast<double>(h->N()) * nb * h->nx <= kModalMaxWork64;
+}
 
 // Allocate level vectors for nb right-hand sides in the current precision, and the plane
 // workspace; configure the kernels' dynamic shared memory.
@@ -221,7 +230,7 @@ int ensure_levels(smg_ctx *h, int nb) {
     free_levels(h);
     const HostHierarchy &H = h->H;
     const size_t sb = storage_bytes(h->prec);
-    if (use_modal(h)) {
+    if (use_modal(h, nb)) {
         const int e = modal_build(h->mp, H, h->prec == Prec::F64, nb, h->npre, h->npost, h->coarse_iters);
         if (e == 0) {
             // the Krylov kernels read T r of one right-hand side in the storage precision

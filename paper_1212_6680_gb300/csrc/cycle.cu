@@ -19,8 +19,8 @@ namespace smg {
 
 size_t storage_bytes(Prec p) { return p == Prec::F64 ? 8 : (p == Prec::F32 ? 4 : 2); }
 
-// ---- plane-relaxation dispatch over K (FP64 x-lines of more than 160 rows; shorter ones and the other
-// precisions run in mode space, modal.cuh) --------------------------------------------------------
+// ---- plane-relaxation dispatch over K (large FP64 cycles with x-lines of more than 160 rows; the others
+// run in mode space, modal.cuh) -------------------------------------------------------------------
 #define SMG_DECL_K(k)                                                                                 \
     cudaError_t launch_plane_relax_k##k(int, int, int, const PlaneRelaxArgs &, size_t, cudaStream_t); \
     int set_plane_relax_smem_k##k(bool, size_t);                                                      \

@@ -6,7 +6,8 @@
 // The scalars live on the device (KrylovScalars); the last CTA of each reduction kernel
 // combines the per-CTA partial sums and computes the scalar the next kernel needs, so one
 // iteration runs without the host.  Inner products: each thread accumulates its products
-// with FMA, then partials are combined with error-free TwoSum (compensated summation).
+// with FMA, then the CTAs' partials are added exactly (reduce.cuh).  With T = I, rho is the ||r||^2 of the step before
+// and no kernel forms it.
 // The preconditioned residual s is read straight from the V-cycle's level-0 storage
 // (FP64, FP32 or BF16): widening it to FP64 is exact, so no FP64 copy of s is made.
 #include <cuda_bf16.h>

@@ -34,7 +34,7 @@ __device__ __forceinline__ DSum shfl_down_dsum(const DSum &v, int o) {
 // themselves: a shuffle tree in every warp is 5 instructions a warp and value, a compensated sum
 // 6 a term.  So the grid is one CTA of up to 1024 threads per SM (152 partials instead of 608), a
 // block folds its partials four to one on full warps (36 instructions a value instead of 165), and
-// one warp per value adds the block partials as integers. 
+// one warp per value adds the block partials as integers.
 constexpr int kMaxThreads = 1024;
 
 template <int NV>
