@@ -568,7 +568,7 @@ int run_modal(smg_ctx *h, int nb, Prec in, const void *f0, Prec type, void *u0, 
     }
     {
         RegionTimer rt(h, st, 3, n * (cb + static_cast<double>(storage_bytes(type))));
-        const cudaError_t e = modal_transform_out(h->mp, nb, type, u0, st, h->launches);
+        const cudaError_t e = modal_transform_out(h->mp, nb, h->prec, type, u0, st, h->launches);
         if (e != cudaSuccess) return fail(SMG_ERR_CUDA, std::string("transform launch: ") + cudaGetErrorString(e));
     }
     return SMG_OK;

@@ -716,8 +716,8 @@ cudaError_t modal_cycle(const ModalPlan &p, int nb, cudaStream_t st, long long &
     return p.f64 ? cycle<double>(p, p.h64, nb, st, launches) : cycle<float>(p, p.h32, nb, st, launches);
 }
 
-cudaError_t modal_transform_out(const ModalPlan &p, int nb, Prec type, void *u0, cudaStream_t st, long long &launches) {
-    if (!p.f64) return sine_out_f32(p.sine, nb, p.h32.a.u[0], type, u0, st, launches);
+cudaError_t modal_transform_out(const ModalPlan &p, int nb, Prec value, Prec type, void *u0, cudaStream_t st, long long &launches) {
+    if (!p.f64) return sine_out_f32(p.sine, nb, p.h32.a.u[0], value, type, u0, st, launches);
     launches += 1;
     return sine_out<double, double>(p, nb, p.h64.a.u[0], u0, st);
 }

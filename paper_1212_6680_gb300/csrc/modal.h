@@ -128,11 +128,11 @@ int modal_build(ModalPlan &p, const HostHierarchy &H, bool f64, int nb, int npre
 void modal_free(ModalPlan &p);
 
 // u0 = T f0 for nb right-hand sides, in three parts: f0 ([rhs][z][y][x], of type F64, or F32 for an FP32
-// plan) into mode space, the cycle there, and back into u0 (elements of type `type`).  Each adds its kernel launches to
-// `launches`.  Asynchronous on st.
+// plan) into mode space, the cycle there, and back into u0 (elements of type `type`, values of a BF16 cycle rounded to
+// bfloat16 in either type: value = BF16).  Each adds its kernel launches to `launches`.  Asynchronous on st.
 cudaError_t modal_transform_in(const ModalPlan &p, int nb, Prec type, const void *f0, cudaStream_t st, long long &launches);
 cudaError_t modal_cycle(const ModalPlan &p, int nb, cudaStream_t st, long long &launches);
-cudaError_t modal_transform_out(const ModalPlan &p, int nb, Prec type, void *u0, cudaStream_t st, long long &launches);
+cudaError_t modal_transform_out(const ModalPlan &p, int nb, Prec value, Prec type, void *u0, cudaStream_t st, long long &launches);
 
 // Many systems at once (batched.cu), FP32: their transforms and tails as one launch each, the CTAs taken
 // from lists of (system, tile) and (system, mode); systems whose active flag is not 1 are skipped.
@@ -147,9 +147,9 @@ struct SineTile {
     int sys, line_tile, mode_tile;
 };
 // FP32 transforms (sine.cu) of physical vectors with elements of type `type` (forward: F32 or F64); scratch: as
-// many values as out.
+// many values as out.  Backward, F64 elements hold values rounded to `value` (BF16, or no further).
 cudaError_t sine_in_f32(const SineArgs &g, int nb, Prec type, const void *f, float *out, float *scratch, cudaStream_t st, long long &launches);
-cudaError_t sine_out_f32(const SineArgs &g, int nb, const float *a, Prec type, void *u, cudaStream_t st, long long &launches);
+cudaError_t sine_out_f32(const SineArgs &g, int nb, const float *a, Prec value, Prec type, void *u, cudaStream_t st, long long &launches);
 int sine_line_tiles(const SineArgs &g);
 int sine_mode_tiles(const SineArgs &g);
 cudaError_t launch_sine_in_batch(const SineJob *jobs, const SineTile *tiles, int ntiles, const int *active, cudaStream_t st);

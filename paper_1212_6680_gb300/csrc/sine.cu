@@ -337,6 +337,13 @@ template <class S> __device__ __forceinline__ S out_val(float v);
 template <> __device__ __forceinline__ float out_val<float>(float v) { return v; }
 template <> __device__ __forceinline__ double out_val<double>(float v) { return widen_f32(v); }
 template <> __device__ __forceinline__ __nv_bfloat16 out_val<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
+// A BF16 result handed out in FP64: rounded to bfloat16, then widened exactly.
+struct Bf16AsF64 {
+    double v;
+};
+template <> __device__ __forceinline__ Bf16AsF64 out_val<Bf16AsF64>(float v) {
+    return Bf16AsF64{widen_f32(__bfloat162float(__float2bfloat16_rn(v)))};
+}
 
 // u[line][x] = sum_mode s_mode(x) uhat[mode][line]: both parities' sums for BN points and their mirror images,
 // sum and difference staged in shared memory so that lines are written whole words in x order.
@@ -454,9 +461,9 @@ cudaError_t out_of(const SineArgs &g, int nb, const float *a, void *u, cudaStrea
 cudaError_t sine_in_f32(const SineArgs &g, int nb, Prec type, const void *f, float *out, float *scratch, cudaStream_t st, long long &launches) {
     return type == Prec::F32 ? in_of<float>(g, nb, f, out, scratch, st, launches) : in_of<double>(g, nb, f, out, scratch, st, launches);
 }
-cudaError_t sine_out_f32(const SineArgs &g, int nb, const float *a, Prec type, void *u, cudaStream_t st, long long &launches) {
+cudaError_t sine_out_f32(const SineArgs &g, int nb, const float *a, Prec value, Prec type, void *u, cudaStream_t st, long long &launches) {
     launches += 1;
-    if (type == Prec::F64) return out_of<double>(g, nb, a, u, st);
+    if (type == Prec::F64) return value == Prec::BF16 ? out_of<Bf16AsF64>(g, nb, a, u, st) : out_of<double>(g, nb, a, u, st);
     return type == Prec::BF16 ? out_of<__nv_bfloat16>(g, nb, a, u, st) : out_of<float>(g, nb, a, u, st);
 }
 
