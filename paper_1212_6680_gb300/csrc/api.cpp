@@ -231,7 +231,7 @@ int ensure_levels(smg_ctx *h, int nb) {
     const HostHierarchy &H = h->H;
     const size_t sb = storage_bytes(h->prec);
     if (use_modal(h, nb)) {
-        const int e = modal_build(h->mp, H, h->prec == Prec::F64, nb, h->npre, h->npost, h->coarse_iters);
+        const int e = modal_build(h->mp, H, h->prec == Prec::F64, nb, h->npre, h->npost);
         if (e == 0) {
             // the Krylov kernels read T r of one right-hand side in the storage precision
             // and, for an FP32 cycle, write r rounded to it beside r
@@ -563,7 +563,7 @@ int run_modal(smg_ctx *h, int nb, Prec in, const void *f0, Prec type, void *u0, 
     }
     {
         RegionTimer rt(h, st, 0, n * 2.0 * cb);
-        const cudaError_t e = modal_cycle(h->mp, nb, st, h->launches);
+        const cudaError_t e = modal_cycle(h->mp, nb, h->coarse_iters, st, h->launches);
         if (e != cudaSuccess) return fail(SMG_ERR_CUDA, std::string("mode-space cycle launch: ") + cudaGetErrorString(e));
     }
     {
@@ -905,7 +905,6 @@ int smg_set_option(smg_handle h, int option, int value) {
         return SMG_OK;
     case SMG_OPT_COARSE_ITERS:
         if (value < 1 || value > 64) return fail(SMG_ERR_ARG, "coarse_iters must be in [1, 64]");
-        if (value != h->coarse_iters && h->modal_now) free_levels(h);  // part of its kernels' arguments
         h->coarse_iters = value;
         return SMG_OK;
     case SMG_OPT_THREADS:

@@ -594,7 +594,7 @@ int batched_build(smg_batched_ctx &c, const int *dims, cudaStream_t st) {
         vtot += (p.N + 31) / 32 * 32;
         build_hierarchy(p.nx, p.ny, p.nz, p.H);
         p.cycle_bytes = vcycle_words(p, c.npre, c.npost) * 4.0;
-        if (modal_plan<float>(p.m, p.H, c.cfg, 1, c.npre, c.npost, 1) != 0) {
+        if (modal_plan<float>(p.m, p.H, c.cfg, 1, c.npre, c.npost) != 0) {
             set_last_error("batched solver: a system's planes do not fit the mode-space cycle");
             return SMG_ERR_CUDA;
         }

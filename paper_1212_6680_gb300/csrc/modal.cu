@@ -456,7 +456,7 @@ std::vector<TailOp> tail_ops(const ModalArgs<T> &a) {
 }
 
 template <class T>
-int modal_plan(ModalHost<T> &h, const HostHierarchy &H, ModalConfig cfg, int nb, int npre, int npost, int coarse_iters) {
+int modal_plan(ModalHost<T> &h, const HostHierarchy &H, ModalConfig cfg, int nb, int npre, int npost) {
     const int nx = H.nx, L = H.L, nh = (nx + 1) / 2;
     h.cfg = cfg;
     ModalArgs<T> &a = h.a;
@@ -469,7 +469,6 @@ int modal_plan(ModalHost<T> &h, const HostHierarchy &H, ModalConfig cfg, int nb,
     a.sum_ny = H.sum_ny;
     a.npre = npre;
     a.npost = npost;
-    a.coarse_iters = coarse_iters;
     for (int m = 0; m < H.P; ++m) a.ny_m[m] = H.ny_m[m], a.line_base[m] = H.line_base[m];
     a.sm_pitch = static_cast<int>(up(H.ny, cfg.K));
     // plane classes; plane types: planes with equal coefficients and class
@@ -601,16 +600,16 @@ int modal_tail_threads(size_t smem, long long ctas, int num_sms, int most, int p
     return std::min(most, std::max(128, (want + 31) / 32 * 32));
 }
 
-template int modal_plan<float>(ModalHost<float> &, const HostHierarchy &, ModalConfig, int, int, int, int);
+template int modal_plan<float>(ModalHost<float> &, const HostHierarchy &, ModalConfig, int, int, int);
 template void modal_place<float>(ModalHost<float> &, unsigned char *, float *, double *, unsigned char *);
 template std::vector<float> sine_matrices<float>(int);
 
 namespace {
 
 template <class T>
-int build(ModalPlan &p, ModalHost<T> &h, const HostHierarchy &H, int npre, int npost, int coarse_iters) {
+int build(ModalPlan &p, ModalHost<T> &h, const HostHierarchy &H, int npre, int npost) {
     const ModalConfig cfg = modal_config(H.ny, sizeof(T) == 8);
-    if (int e = modal_plan<T>(h, H, cfg, p.nb, npre, npost, coarse_iters)) return e;
+    if (int e = modal_plan<T>(h, H, cfg, p.nb, npre, npost)) return e;
     const ModalKernels<T> &k = modal_kernels<T>(cfg);
     const size_t b_coef = up(h.coef_values * sizeof(T), 256), b_64 = up(h.coef64_values * 8, 256);
     MCHK(cudaMalloc(&p.d_tab, h.shared.size() + b_64 + b_coef));
@@ -641,7 +640,7 @@ cudaError_t prolong(const ModalArgs<T> &a, int l, int nb, cudaStream_t st) {
 }
 
 template <class T>
-cudaError_t cycle(const ModalPlan &p, const ModalHost<T> &h, int nb, cudaStream_t st, long long &launches) {
+cudaError_t cycle(const ModalPlan &p, const ModalHost<T> &h, int nb, int coarse_iters, cudaStream_t st, long long &launches) {
     const ModalArgs<T> &a = h.a;
     const ModalKernels<T> &k = modal_kernels<T>(h.cfg);
     cudaError_t e;
@@ -660,7 +659,8 @@ cudaError_t cycle(const ModalPlan &p, const ModalHost<T> &h, int nb, cudaStream_
         launches += 1;
     }
     const int threads = modal_tail_threads(h.smem, static_cast<long long>(a.nmode) * nb, p.num_sms, k.max_threads, a.nz[a.lt], h.cfg.G);
-    if ((e = k.tail(static_cast<const ModalArgs<T> *>(p.d_args), a.nmode, nb, threads, h.smem, st)) != cudaSuccess) return e;
+    if ((e = k.tail(static_cast<const ModalArgs<T> *>(p.d_args), a.nmode, nb, coarse_iters, threads, h.smem, st)) != cudaSuccess)
+        return e;
     launches += 1;
     for (int l = a.lt - 1; l >= 0; --l) {
         if ((e = prolong(a, l, nb, st)) != cudaSuccess) return e;
@@ -698,11 +698,11 @@ cudaError_t sine_out(const ModalPlan &p, int nb, const T *uh, void *u, cudaStrea
 
 }  // namespace
 
-int modal_build(ModalPlan &p, const HostHierarchy &H, bool f64, int nb, int npre, int npost, int coarse_iters) {
+int modal_build(ModalPlan &p, const HostHierarchy &H, bool f64, int nb, int npre, int npost) {
     modal_free(p);
     p.f64 = f64;
     p.nb = nb;
-    return f64 ? build<double>(p, p.h64, H, npre, npost, coarse_iters) : build<float>(p, p.h32, H, npre, npost, coarse_iters);
+    return f64 ? build<double>(p, p.h64, H, npre, npost) : build<float>(p, p.h32, H, npre, npost);
 }
 
 cudaError_t modal_transform_in(const ModalPlan &p, int nb, Prec type, const void *f0, cudaStream_t st, long long &launches) {
@@ -712,8 +712,8 @@ cudaError_t modal_transform_in(const ModalPlan &p, int nb, Prec type, const void
     return sine_in<double>(p, nb, static_cast<const double *>(f0), p.h64.a.fw[0], st);
 }
 
-cudaError_t modal_cycle(const ModalPlan &p, int nb, cudaStream_t st, long long &launches) {
-    return p.f64 ? cycle<double>(p, p.h64, nb, st, launches) : cycle<float>(p, p.h32, nb, st, launches);
+cudaError_t modal_cycle(const ModalPlan &p, int nb, int coarse_iters, cudaStream_t st, long long &launches) {
+    return p.f64 ? cycle<double>(p, p.h64, nb, coarse_iters, st, launches) : cycle<float>(p, p.h32, nb, coarse_iters, st, launches);
 }
 
 cudaError_t modal_transform_out(const ModalPlan &p, int nb, Prec value, Prec type, void *u0, cudaStream_t st, long long &launches) {

@@ -612,7 +612,7 @@ constexpr int modal_threads() { return sizeof(T) == 8 ? 256 : 512; }
 // barrier after each: every kind of step is compiled once (inlined at each place of the cycle it
 // appears, the kernel would not fit the instruction cache).
 template <class T, int G, int K>
-__device__ __forceinline__ void tail_body(const ModalArgs<T> &A, int mode_idx, int rhs, unsigned char *smem) {
+__device__ __forceinline__ void tail_body(const ModalArgs<T> &A, int mode_idx, int rhs, int coarse_iters, unsigned char *smem) {
     __shared__ TailOp ring[2];  // the step that runs and the next
     T *sm = reinterpret_cast<T *>(smem);
     const int tid = threadIdx.x, nt = blockDim.x, ln = (tid & 31) % G;
@@ -671,10 +671,10 @@ __device__ __forceinline__ void tail_body(const ModalArgs<T> &A, int mode_idx, i
                                   [&](int Z, int c, const Chunk<T, K> &g) { g.store(fc, Z, c); });
         } else if (kind == OP_COARSEST) {
             if (lt == L - 1) {  // the only level: straight to global memory
-                if (tid < 32) coarsest<T, G, K, false>(fg.p, ug.p, A.ny, A.coarse_iters, tab64, tid);
+                if (tid < 32) coarsest<T, G, K, false>(fg.p, ug.p, A.ny, coarse_iters, tab64, tid);
                 for (int y = A.ny + tid; y < A.pitch; y += nt) ug.p[y] = T(0);
             } else {
-                if (tid < 32) coarsest<T, G, K, true>(f.p, u.p, A.ny, A.coarse_iters, tab64, tid);
+                if (tid < 32) coarsest<T, G, K, true>(f.p, u.p, A.ny, coarse_iters, tab64, tid);
                 for (int y = A.ny + tid; y < sp; y += nt) u.p[RowMap<T, K>::elem(y)] = T(0);
             }
         } else if (kind == OP_PROLONG || kind == OP_STORE) {
@@ -714,14 +714,14 @@ __device__ __forceinline__ void tail_body(const ModalArgs<T> &A, int mode_idx, i
 }
 
 template <class T, int G, int K>
-__global__ void __launch_bounds__(modal_threads<T>(), 1) modal_tail_kernel(const ModalArgs<T> *__restrict__ args) {
+__global__ void __launch_bounds__(modal_threads<T>(), 1) modal_tail_kernel(const ModalArgs<T> *__restrict__ args, int coarse_iters) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ ModalArgs<T> A;
     pdl_trigger();
     for (unsigned i = threadIdx.x; i < sizeof(ModalArgs<T>) / 4; i += blockDim.x)
         reinterpret_cast<unsigned *>(&A)[i] = reinterpret_cast<const unsigned *>(args)[i];
     __syncthreads();
-    tail_body<T, G, K>(A, blockIdx.x, blockIdx.y, smem);
+    tail_body<T, G, K>(A, blockIdx.x, blockIdx.y, coarse_iters, smem);
 }
 
 // One (system, mode) of a list per CTA; systems that are not being iterated are skipped.
@@ -735,7 +735,7 @@ __global__ void __launch_bounds__(modal_threads<T>(), 1) modal_tail_batch_kernel
     for (unsigned i = threadIdx.x; i < sizeof(ModalArgs<T>) / 4; i += blockDim.x)
         reinterpret_cast<unsigned *>(&A)[i] = reinterpret_cast<const unsigned *>(args + t.sys)[i];
     __syncthreads();
-    tail_body<T, G, K>(A, t.mode, 0, smem);
+    tail_body<T, G, K>(A, t.mode, 0, 1, smem);
 }
 
 // ---- levels above the tail, over global memory ------------------------------------------------------

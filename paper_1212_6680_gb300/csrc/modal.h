@@ -27,7 +27,7 @@ struct ModalArgs {
     int nmode, ny, pitch;      // x-modes, lines, and lines per plane in global memory (ny rounded up to 4)
     int L, lt;                 // z-levels; first tail level
     int P, sum_ny;             // 2D levels and their lines in all
-    int npre, npost, coarse_iters;
+    int npre, npost;
     int ntype, nptype, ncls_all, blk;  // line types, plane types, classes of all levels, values per class
     int ny_m[kMaxPlaneLevels], line_base[kMaxPlaneLevels];
     int nz[kMaxZLevels];       // planes of each z-level
@@ -101,7 +101,7 @@ struct ModalHost {
     std::vector<size_t> vec_off;       // f and u of levels 0 .. lt
 };
 template <class T>
-int modal_plan(ModalHost<T> &h, const HostHierarchy &H, ModalConfig cfg, int nb, int npre, int npost, int coarse_iters);
+int modal_plan(ModalHost<T> &h, const HostHierarchy &H, ModalConfig cfg, int nb, int npre, int npost);
 template <class T>
 void modal_place(ModalHost<T> &h, unsigned char *shared, T *coef, double *coef64, unsigned char *vec);
 template <class T>
@@ -124,14 +124,15 @@ struct ModalPlan {
 };
 
 // Tables and buffers for nb right-hand sides; 0, or a cudaError_t.
-int modal_build(ModalPlan &p, const HostHierarchy &H, bool f64, int nb, int npre, int npost, int coarse_iters);
+int modal_build(ModalPlan &p, const HostHierarchy &H, bool f64, int nb, int npre, int npost);
 void modal_free(ModalPlan &p);
 
 // u0 = T f0 for nb right-hand sides, in three parts: f0 ([rhs][z][y][x], of type F64, or F32 for an FP32
 // plan) into mode space, the cycle there, and back into u0 (elements of type `type`, values of a BF16 cycle rounded to
-// bfloat16 in either type: value = BF16).  Each adds its kernel launches to `launches`.  Asynchronous on st.
+// bfloat16 in either type: value = BF16).  coarse_iters: steps on the one-plane coarsest level.  Each adds its kernel
+// launches to `launches`.  Asynchronous on st.
 cudaError_t modal_transform_in(const ModalPlan &p, int nb, Prec type, const void *f0, cudaStream_t st, long long &launches);
-cudaError_t modal_cycle(const ModalPlan &p, int nb, cudaStream_t st, long long &launches);
+cudaError_t modal_cycle(const ModalPlan &p, int nb, int coarse_iters, cudaStream_t st, long long &launches);
 cudaError_t modal_transform_out(const ModalPlan &p, int nb, Prec value, Prec type, void *u0, cudaStream_t st, long long &launches);
 
 // Many systems at once (batched.cu), FP32: their transforms and tails as one launch each, the CTAs taken
@@ -163,7 +164,7 @@ cudaError_t launch_modal_prolong(const ModalArgs<float> &a, int l, int nb, cudaS
 template <class T>
 struct ModalKernels {
     cudaError_t (*setup)(const ModalArgs<T> &a, T *coef, double *coef64, cudaStream_t st);
-    cudaError_t (*tail)(const ModalArgs<T> *d_args, int nmode, int nb, int threads, size_t smem, cudaStream_t st);
+    cudaError_t (*tail)(const ModalArgs<T> *d_args, int nmode, int nb, int coarse_iters, int threads, size_t smem, cudaStream_t st);
     cudaError_t (*tail_batch)(const ModalArgs<T> *d_args, const ModalTask *tasks, int ntasks, const int *active, int threads,
                               size_t smem, cudaStream_t st);
     cudaError_t (*slab)(const ModalArgs<T> &a, int l, int nb, cudaStream_t st);

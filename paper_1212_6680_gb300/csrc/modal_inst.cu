@@ -21,10 +21,10 @@ cudaError_t setup(const ModalArgs<T> &a, T *coef, double *coef64, cudaStream_t s
     return cudaGetLastError();
 }
 
-cudaError_t tail(const ModalArgs<T> *d_args, int nmode, int nb, int threads, size_t smem, cudaStream_t st) {
+cudaError_t tail(const ModalArgs<T> *d_args, int nmode, int nb, int coarse_iters, int threads, size_t smem, cudaStream_t st) {
     cudaError_t e = raise_smem_attr(reinterpret_cast<const void *>(&modal_tail_kernel<T, G, K>), smem);
     if (e != cudaSuccess) return e;
-    return launch_pdl(modal_tail_kernel<T, G, K>, dim3(nmode, nb), dim3(threads), smem, st, d_args);
+    return launch_pdl(modal_tail_kernel<T, G, K>, dim3(nmode, nb), dim3(threads), smem, st, d_args, coarse_iters);
 }
 
 cudaError_t tail_batch(const ModalArgs<T> *d_args, const ModalTask *tasks, int ntasks, const int *active, int threads, size_t smem,
