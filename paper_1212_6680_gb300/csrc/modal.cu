@@ -681,16 +681,24 @@ dim3 sine_grid(const ModalPlan &p, int nb) {
     return dim3(static_cast<unsigned>((lines + BM - 1) / BM), (p.sine.nh + kBN - 1) / kBN, nb);
 }
 
+// Shared memory of a transform's CTAs: while there is an SM for each, so much that no two share one.  Launched
+// beside the kernel before it, they settle on the SMs that come free first, two or three together, and share an
+// FP64 unit that one of them already fills (applications at 294x11x30 923 -> 415 us, 570x13x16 1643 -> 744 us, 255x90x10
+// 829 -> 369 us; with one or two stages a transform the SM's other work can matter as much: 0.9 to 1.1 of before).
+size_t sine_smem(const ModalPlan &p, dim3 g, size_t need) {
+    return static_cast<long long>(g.x) * g.y * g.z <= p.num_sms ? std::max(need, kModalSmem / 2 + 4096) : need;
+}
+
 template <class T>
 cudaError_t sine_in(const ModalPlan &p, int nb, const double *f, T *out, cudaStream_t st) {
-    constexpr size_t smem = sizeof(SineSmem<T, tm_lines<T>()>);
+    const size_t smem = sine_smem(p, sine_grid<T>(p, nb), sizeof(SineSmem<T, tm_lines<T>()>));
     cudaError_t e = raise_smem_attr(reinterpret_cast<const void *>(&sine_in_kernel<T>), smem);
     if (e != cudaSuccess) return e;
     return launch_pdl(sine_in_kernel<T>, sine_grid<T>(p, nb), dim3(128), smem, st, p.sine, f, out);
 }
 template <class T, class S>
 cudaError_t sine_out(const ModalPlan &p, int nb, const T *uh, void *u, cudaStream_t st) {
-    constexpr size_t smem = sizeof(SineSmem<T, tm_lines<T>()>);
+    const size_t smem = sine_smem(p, sine_grid<T>(p, nb), sizeof(SineSmem<T, tm_lines<T>()>));
     cudaError_t e = raise_smem_attr(reinterpret_cast<const void *>(&sine_out_kernel<T, S>), smem);
     if (e != cudaSuccess) return e;
     return launch_pdl(sine_out_kernel<T, S>, sine_grid<T>(p, nb), dim3(128), smem, st, p.sine, uh, static_cast<S *>(u));
