@@ -681,12 +681,16 @@ dim3 sine_grid(const ModalPlan &p, int nb) {
     return dim3(static_cast<unsigned>((lines + BM - 1) / BM), (p.sine.nh + kBN - 1) / kBN, nb);
 }
 
-// Shared memory of a transform's CTAs: while there is an SM for each, so much that no two share one.  Launched
-// beside the kernel before it, they settle on the SMs that come free first, two or three together, and share an
+// Shared memory of a transform's CTAs: so much that no SM takes more of them than its share.  Launched beside the
+// kernel before it, they settle on the SMs that come free first, three or four together, and there share an
 // FP64 unit that one of them already fills (applications at 294x11x30 923 -> 415 us, 570x13x16 1643 -> 744 us, 255x90x10
-// 829 -> 369 us; with one or two stages a transform the SM's other work can matter as much: 0.9 to 1.1 of before).
+// 829 -> 369 us).  Not for few tiles of one or two stages, where it matters more that they can start
+// beside the kernel before (46x79x16 (1,1) 238 us, 261 spread).
 size_t sine_smem(const ModalPlan &p, dim3 g, size_t need) {
-    return static_cast<long long>(g.x) * g.y * g.z <= p.num_sms ? std::max(need, kModalSmem / 2 + 4096) : need;
+    constexpr size_t kPerSm = 228 * 1024, kPerCta = 1024;  // of an SM; reserved with each CTA
+    const size_t tiles = static_cast<size_t>(g.x) * g.y * g.z, sms = p.num_sms;
+    if (p.sine.nh <= 2 * kBK && 4 * tiles <= sms) return need;
+    return std::max<size_t>(need, kPerSm / ((tiles + sms - 1) / sms + 1) - kPerCta + 128);
 }
 
 template <class T>
