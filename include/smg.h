@@ -51,11 +51,11 @@ enum { SMG_FP64 = 0, SMG_FP32 = 1, SMG_BF16 = 2 };     /* V-cycle storage precis
 
 /* Options for smg_set_option.
  *
- * Two forms of the V-cycle exist.  In mode space (every FP32 and BF16 cycle, and FP64 ones with x-lines of at
- * most 160 rows or with nx * N * nb <= 1.5e9 for the nb vectors the handle was last sized for) it runs in the sine
- * eigenvectors of the x-lines: the same relaxations, an exact line solve being a division per mode.  Larger FP64 cycles run
- * on the plane kernels, to which the options on threads, clusters, step orders, tables and restriction apply (marked
- * "planes"); in mode space these are accepted and change nothing.  The two forms differ by rounding. */
+ * Two forms of the V-cycle exist.  In mode space (every FP32 and BF16 cycle, and most FP64 ones) it runs in the sine
+ * eigenvectors of the x-lines: the same relaxations, an exact line solve being a division per mode.  FP64 cycles on
+ * few lines, or on many long ones, run on the plane kernels, to which the options on threads, clusters, step orders, tables
+ * and restriction apply (marked "planes"); in mode space these are accepted and change nothing.  A call's form follows
+ * from the sizes, the cycle and its own number of vectors alone (smg_cycle_form).  The two forms differ by rounding. */
 enum {
     SMG_OPT_COARSE_ITERS = 0, /* plane-cycle steps on the one-plane coarsest level (>= 1, default 1) */
     SMG_OPT_THREADS = 1,      /* planes: threads per CTA: 256 or 512 (default 512; the
@@ -429,6 +429,15 @@ int smg_apply_A_dot_static(int nx, int ny, int nz, const double *u, double *out,
  * host allocation returns SMG_ERR_HOST): meant for inspection and tests, not for a hot loop.
  */
 int smg_setup_coefs(int nx, int ny, int nz, int l, int z, int m, double *zc, double *lines, int *nz_l, int *ny_m);
+
+/*
+ * smg_cycle_form -- which form the V-cycle of a handle on this grid takes for calls with nb right-hand sides (1 <= nb <=
+ * 64; 1 in krylov_solve), on the host only: the faster one by an estimate of both forms' times.  *form (host):
+ * SMG_FORM_MODES or SMG_FORM_PLANES (see the options above).  Returns SMG_ERR_ARG for arguments that smg_setup,
+ * smg_set_precision or smg_apply_batched refuse.
+ */
+enum { SMG_FORM_MODES = 0, SMG_FORM_PLANES = 1 };
+int smg_cycle_form(int nx, int ny, int nz, int npre, int npost, int prec, int nb, int *form);
 
 /*
  * smg_plane_classes -- the planes of z-level l that share one set of line-solver data, on the

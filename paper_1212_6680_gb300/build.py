@@ -18,9 +18,9 @@ BUILD = os.path.join(ROOT, "_build")
 LIB = os.path.join(HERE, "libsmg.so")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-KS = (6, 8, 16)  # rows per lane of the FP64 plane kernels (cycles too large for mode space)
+KS = (1, 2, 3, 4, 6, 8, 16)  # rows per lane of the FP64 plane kernels
 SOURCES = ["api.cpp", "hierarchy.cpp", "cycle.cu", "krylov_kernels.cu", "lobpcg.cu", "noalloc.cu", "batched.cu", "net.cu",
-           "net_api.cpp", "conv_tc.cu", "gram_tc.cu", "modal.cu", "sine.cu"]
+           "net_api.cpp", "conv_tc.cu", "gram_tc.cu", "modal.cu", "sine.cu", "form.cpp"]
 WKS = (8, 16)  # rows per lane of the wide-line kernel's segments (plane_wide.cu, one unit each)
 
 

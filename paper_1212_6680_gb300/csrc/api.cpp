@@ -75,10 +75,16 @@ struct smg_ctx {
     Prec prec = Prec::F64;
     HostHierarchy H;
     double *d_zcoef = nullptr, *d_pcoef = nullptr;
-    // level storage (current precision) for nb_alloc right-hand sides
-    int nb_alloc = 0;
-    Prec alloc_prec = Prec::F64;
-    std::vector<void *> d_f, d_u;   // [L]; level 0 entries used only when the caller's buffers are not
+    // Level storage in level_prec for calls of up to nb_ready right-hand sides: mode-space vectors (mp) for the counts
+    // whose cycle runs there, the plane kernels' (levels 1 .. L-1, nb_planes right-hand sides) for the others.  A call's
+    // form follows from its own count (use_modal), not from what is in place.
+    int nb_ready = 0, nb_planes = 0;
+    Prec level_prec = Prec::F64;
+    std::vector<char> modes64;      // [nb - 1] 1: the FP64 cycle of nb right-hand sides runs in mode space
+    ModalPlan mp;
+    std::vector<void *> d_f, d_u;   // [L], entry 0 unused
+    void *d_s = nullptr;            // krylov_solve: T r in level_prec
+    void *d_rf = nullptr;           // krylov_solve: r in FP32 for an FP32 cycle, written by its kernels
     void *d_ws = nullptr;
     size_t ws_bytes = 0;
     PlaneLayout lay_c;              // one CTA per plane
@@ -105,8 +111,6 @@ struct smg_ctx {
     PlaneLayout lay_wcl[5];         // wide-line cluster layouts: [log2 R]
     bool wcl_ok[5] = {false, false, false, false, false};
     int num_sms = 0;
-    bool modal_now = false;         // the level vectors in place are that cycle's
-    ModalPlan mp;
     // Krylov vectors (one right-hand side)
     double *d_r = nullptr, *d_p = nullptr, *d_q = nullptr;
     double *d_bh = nullptr, *d_xh = nullptr;  // device copies for host-pointer calls
@@ -155,7 +159,8 @@ struct smg_ctx {
 
 namespace {
 
-void free_levels(smg_ctx *h) {
+// Gives back what the plane kernels use (the options they depend on have changed, or more of it is wanted).
+void free_planes(smg_ctx *h) {
     h->gen += 1;
     cudaFree(h->d_wftab);
     h->d_wftab = nullptr;
@@ -170,9 +175,15 @@ void free_levels(smg_ctx *h) {
     cudaFree(h->d_ws);
     h->d_ws = nullptr;
     h->ws_bytes = 0;
-    h->nb_alloc = 0;
+    h->nb_planes = h->nb_ready = 0;
+}
+
+void free_levels(smg_ctx *h) {
+    free_planes(h);
     modal_free(h->mp);
-    h->modal_now = false;
+    cudaFree(h->d_s);
+    cudaFree(h->d_rf);
+    h->d_s = h->d_rf = nullptr;
 }
 
 int instantiated_K(int nx) {
@@ -210,51 +221,51 @@ PlaneLayout with_solo_levels(const HostHierarchy &H, size_t elem_bytes, int R, i
 }
 
 // Whether the cycle of nb right-hand sides runs in the x-lines' sine eigenvectors (modal.cuh): every FP32 and
-// BF16 cycle; an FP64 one, whose transforms are FP64 products of order nx / 2 and which the plane kernels meet
-// once their planes fill the chip, with lines of at most 160 points or while nx times the points stays below a
-// bound.  (1,0) applications in us, mode space / plane kernels: 160x80x80 979 / 2141, 256x64x64 1036 / 2492,
-// 512x64x64 2620 / 4308, 768x48x48 2977 / 4812, 200^3 (1.6e9) 6036 / 6945, 512x128x96 (3.2e9) 6914 / 6582,
-// 256^3 (4.3e9) 10475 / 9563; 8 vectors: 176x64x64 (1.0e9) 3423 / 3986, 256x64x64 (2.1e9) 5422 / 4866, 512x32x32
-// (2.1e9) 4565 / 3667.  (1,1) cycles favour mode space throughout.
-constexpr int kModalMaxNx64 = 160;
-constexpr double kModalMaxWork64 = 1.5e9;
-bool use_modal(const smg_ctx *h, int nb) {
-    return h->prec != Prec::F64 || h->nx <= kModalMaxNx64 ||
-           static_cast<double>(h->N()) * nb * h->nx <= kModalMaxWork64;
+// BF16 cycle, and an FP64 one where that is the faster form (form.cpp).
+bool use_modal(const smg_ctx *h, int nb) { return h->prec != Prec::F64 || h->modes64[nb - 1] != 0; }
+
+int alloc_planes(smg_ctx *h, int nb);
+
+// Everything that calls with 1 .. nb right-hand sides need in the current precision.
+int ensure_levels(smg_ctx *h, int nb) {
+    if (h->nb_ready >= nb && h->level_prec == h->prec) return SMG_OK;
+    if (h->level_prec != h->prec) free_levels(h);
+    h->level_prec = h->prec;
+    h->nb_ready = 0;  // until all of it is there
+    h->gen += 1;
+    for (int c = static_cast<int>(h->modes64.size()) + 1; c <= nb; ++c)
+        h->modes64.push_back(mode_space_faster(h->nx, h->ny, h->nz, c, h->npre, h->npost) ? 1 : 0);
+    int modes = 0, planes = 0;
+    for (int c = 1; c <= nb; ++c) (use_modal(h, c) ? modes : planes) = c;
+    const size_t one = static_cast<size_t>(h->N()) * storage_bytes(h->prec);
+    if (h->d_s == nullptr) SMG_CUDA(cudaMalloc(&h->d_s, one));
+    if (h->d_rf == nullptr && h->prec == Prec::F32) SMG_CUDA(cudaMalloc(&h->d_rf, one));
+    if (modes > h->mp.nb) {
+        const int e = modal_build(h->mp, h->H, h->prec == Prec::F64, modes, h->npre, h->npost);
+        if (e != 0) {
+            modal_free(h->mp);
+            return fail(SMG_ERR_CUDA, std::string("mode-space cycle: ") + cudaGetErrorString(static_cast<cudaError_t>(e)));
+        }
+    }
+    if (planes > h->nb_planes) {
+        free_planes(h);
+        if (int rc = alloc_planes(h, planes)) return rc;
+    }
+    h->nb_ready = nb;
+    return SMG_OK;
 }
 
-// Allocate level vectors for nb right-hand sides in the current precision, and the plane
-// workspace; configure the kernels' dynamic shared memory.
-int ensure_levels(smg_ctx *h, int nb) {
-    if (h->nb_alloc >= nb && h->alloc_prec == h->prec) return SMG_OK;
-    free_levels(h);
+// The plane kernels' level vectors for nb right-hand sides and their workspace; configures the kernels'
+// dynamic shared memory.
+int alloc_planes(smg_ctx *h, int nb) {
     const HostHierarchy &H = h->H;
-    const size_t sb = storage_bytes(h->prec);
-    if (use_modal(h, nb)) {
-        const int e = modal_build(h->mp, H, h->prec == Prec::F64, nb, h->npre, h->npost);
-        if (e == 0) {
-            // the Krylov kernels read T r of one right-hand side in the storage precision
-            // and, for an FP32 cycle, write r rounded to it beside r
-            h->d_f.assign(1, nullptr);
-            h->d_u.assign(1, nullptr);
-            if (h->prec == Prec::F32) SMG_CUDA(cudaMalloc(&h->d_f[0], static_cast<size_t>(h->N()) * sb));
-            SMG_CUDA(cudaMalloc(&h->d_u[0], static_cast<size_t>(h->N()) * sb));
-            h->modal_now = true;
-            h->nb_alloc = nb;
-            h->alloc_prec = h->prec;
-            return SMG_OK;
-        }
-        modal_free(h->mp);
-        return fail(SMG_ERR_CUDA, std::string("mode-space cycle: ") + cudaGetErrorString(static_cast<cudaError_t>(e)));
-    }
     h->d_f.assign(H.L, nullptr);
     h->d_u.assign(H.L, nullptr);
-    for (int l = 0; l < H.L; ++l) {
-        const size_t bytes = static_cast<size_t>(h->Nl(l)) * nb * sb;
+    for (int l = 1; l < H.L; ++l) {
+        const size_t bytes = static_cast<size_t>(h->Nl(l)) * nb * sizeof(double);
         SMG_CUDA(cudaMalloc(&h->d_f[l], bytes));
         SMG_CUDA(cudaMalloc(&h->d_u[l], bytes));
     }
-    // the plane kernels: an FP64 cycle's
     const int wk = wide_rows(h);
     const bool wide = wk > 0;
     if (wide) {
@@ -402,8 +413,7 @@ int alloc_plane_workspace(smg_ctx *h, int nb) {
     const long long slots = static_cast<long long>((H.nz + 1) / 2) * nb;
     h->ws_bytes = std::max<size_t>(per * slots, 256);
     SMG_CUDA(cudaMalloc(&h->d_ws, h->ws_bytes));
-    h->nb_alloc = nb;
-    h->alloc_prec = h->prec;
+    h->nb_planes = nb;
     return SMG_OK;
 }
 
@@ -577,7 +587,7 @@ int run_modal(smg_ctx *h, int nb, Prec in, const void *f0, Prec type, void *u0, 
 // u0 = T f0 for nb right-hand sides; f0, u0 in storage precision, level-0 layout (in mode space a BF16
 // cycle's f0 is in FP64).
 int run_cycle(smg_ctx *h, int nb, const void *f0, void *u0, cudaStream_t st) {
-    if (h->modal_now) return run_modal(h, nb, h->prec == Prec::F32 ? Prec::F32 : Prec::F64, f0, h->prec, u0, st);
+    if (use_modal(h, nb)) return run_modal(h, nb, h->prec == Prec::F32 ? Prec::F32 : Prec::F64, f0, h->prec, u0, st);
     const HostHierarchy &H = h->H;
     const int L = H.L;
     int rc;
@@ -720,12 +730,11 @@ int krylov_device(smg_ctx *h, int variant, const double *b, double *x, double to
         SMG_CUDA(cudaMalloc(&h->d_hist, sizeof(double) * (maxit + 2)));
         h->hist_cap = maxit + 2;
     }
-    const bool f64 = (h->prec == Prec::F64);
     const bool ident = (h->precond == 0);                           // T = I: s is r itself
-    // cycle input: (S) r, written by the Krylov kernels, or r itself (FP64 cycles, and BF16 in mode space)
-    const bool own_f0 = !f64 && !(h->modal_now && h->prec == Prec::BF16);
-    void *f0 = own_f0 ? h->d_f[0] : static_cast<void *>(h->d_r);
-    void *u0 = ident ? static_cast<void *>(h->d_r) : h->d_u[0];   // s = T r
+    // cycle input: r in FP32, written by the Krylov kernels, or r itself (FP64 and BF16 cycles)
+    const bool own_f0 = h->prec == Prec::F32;
+    void *f0 = own_f0 ? h->d_rf : static_cast<void *>(h->d_r);
+    void *u0 = ident ? static_cast<void *>(h->d_r) : h->d_s;        // s = T r
     const Prec kp = ident ? Prec::F64 : h->prec;                    // storage type of s
     void *f0k = (own_f0 && !ident) ? f0 : nullptr;                  // what the Krylov kernels write
     const double tol2 = tol * tol;
@@ -909,17 +918,17 @@ int smg_set_option(smg_handle h, int option, int value) {
         return SMG_OK;
     case SMG_OPT_THREADS:
         if (value != 256 && value != 512) return fail(SMG_ERR_ARG, "threads must be 256 or 512");
-        if (value != h->threads) free_levels(h);  // the layouts and residency checks depend on it
+        if (value != h->threads) free_planes(h);  // the layouts and residency checks depend on it
         h->threads = value;
         return SMG_OK;
     case SMG_OPT_WIDE_MIN_ROWS:
         if (value != 257 && value != 513) return fail(SMG_ERR_ARG, "wide_min_rows must be 257 or 513");
-        if (value != h->wide_min) free_levels(h);
+        if (value != h->wide_min) free_planes(h);
         h->wide_min = value;
         return SMG_OK;
     case SMG_OPT_WIDE_FACTORS:
         if (value != 0 && value != 1) return fail(SMG_ERR_ARG, "wide_factors must be 0 or 1");
-        if (value != h->wide_factors) free_levels(h);
+        if (value != h->wide_factors) free_planes(h);
         h->wide_factors = value;
         return SMG_OK;
     case SMG_OPT_RESTRICT_COLUMN:
@@ -928,7 +937,7 @@ int smg_set_option(smg_handle h, int option, int value) {
         return SMG_OK;
     case SMG_OPT_SOLO:
         if (value < 0 || value > kMaxNy) return fail(SMG_ERR_ARG, "solo must be in [0, 512]");
-        if (value != h->solo) free_levels(h);
+        if (value != h->solo) free_planes(h);
         h->solo = value;
         return SMG_OK;
     case SMG_OPT_CLUSTER_MAX:
@@ -967,7 +976,7 @@ int smg_apply_batched(smg_handle h, int nb, const double *R, double *S, void *st
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     int rc;
     if ((rc = ensure_levels(h, nb)) != SMG_OK) return rc;
-    if (h->modal_now) {
+    if (use_modal(h, nb)) {
         if ((rc = run_modal(h, nb, Prec::F64, R, Prec::F64, S, st)) != SMG_OK) return rc;
     } else {
         if ((rc = run_cycle(h, nb, R, S, st)) != SMG_OK) return rc;
@@ -1181,6 +1190,17 @@ int smg_setup_coefs(int nx, int ny, int nz, int l, int z, int m, double *zc, dou
             lines[static_cast<size_t>(y) * kCoefPerLine + k] = pc[static_cast<size_t>(H.line_base[m] + y) * kCoefPerLine + k];
     if (nz_l) *nz_l = H.nz_l[l];
     if (ny_m) *ny_m = H.ny_m[m];
+    return SMG_OK;
+}
+
+int smg_cycle_form(int nx, int ny, int nz, int npre, int npost, int prec, int nb, int *form) {
+    using namespace smg;
+    if (const char *e = grid_size_error(nx, ny, nz)) return fail(SMG_ERR_ARG, e);
+    if (npre < 1 || npost < 0) return fail(SMG_ERR_ARG, "npre >= 1 and npost >= 0 required");
+    if (prec != SMG_FP64 && prec != SMG_FP32 && prec != SMG_BF16) return fail(SMG_ERR_ARG, "unknown precision");
+    if (nb < 1 || nb > 64) return fail(SMG_ERR_ARG, "nb must be in [1, 64]");
+    if (form == nullptr) return fail(SMG_ERR_ARG, "null pointer");
+    *form = prec != SMG_FP64 || mode_space_faster(nx, ny, nz, nb, npre, npost) ? SMG_FORM_MODES : SMG_FORM_PLANES;
     return SMG_OK;
 }
 

@@ -19,8 +19,7 @@ namespace smg {
 
 size_t storage_bytes(Prec p) { return p == Prec::F64 ? 8 : (p == Prec::F32 ? 4 : 2); }
 
-// ---- plane-relaxation dispatch over K (large FP64 cycles with x-lines of more than 160 rows; the others
-// run in mode space, modal.cuh) -------------------------------------------------------------------
+// ---- plane-relaxation dispatch over K (FP64 cycles that are faster on the planes than in mode space, form.cpp)
 #define SMG_DECL_K(k)                                                                                 \
     cudaError_t launch_plane_relax_k##k(int, int, int, const PlaneRelaxArgs &, size_t, cudaStream_t); \
     int set_plane_relax_smem_k##k(bool, size_t);                                                      \
@@ -29,20 +28,36 @@ size_t storage_bytes(Prec p) { return p == Prec::F64 ? 8 : (p == Prec::F32 ? 4 :
     cudaError_t launch_plane_lean_k##k(int, int, int, const PlaneRelaxArgs &, size_t, cudaStream_t);  \
     int set_plane_lean_smem_k##k(bool, size_t);                                                       \
     bool lean_cluster_resident_k##k(int, int, size_t);
+SMG_DECL_K(1)
+SMG_DECL_K(2)
+SMG_DECL_K(3)
+SMG_DECL_K(4)
 SMG_DECL_K(6)
 SMG_DECL_K(8)
 SMG_DECL_K(16)
+SMG_DECL_LEAN_K(1)
+SMG_DECL_LEAN_K(2)
+SMG_DECL_LEAN_K(3)
+SMG_DECL_LEAN_K(4)
 SMG_DECL_LEAN_K(6)
 SMG_DECL_LEAN_K(8)
 
 #define SMG_SWITCH_K(K, CALL)   \
     switch (K) {                \
+    case 1: return CALL(1);     \
+    case 2: return CALL(2);     \
+    case 3: return CALL(3);     \
+    case 4: return CALL(4);     \
     case 6: return CALL(6);     \
     case 8: return CALL(8);     \
     case 16: return CALL(16);   \
     }
 #define SMG_LEAN_SWITCH(K, CALL) \
     switch (K) {                 \
+    case 1: return CALL(1);      \
+    case 2: return CALL(2);      \
+    case 3: return CALL(3);      \
+    case 4: return CALL(4);      \
     case 6: return CALL(6);      \
     case 8: return CALL(8);      \
     }

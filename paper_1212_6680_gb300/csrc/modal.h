@@ -135,6 +135,9 @@ cudaError_t modal_transform_in(const ModalPlan &p, int nb, Prec type, const void
 cudaError_t modal_cycle(const ModalPlan &p, int nb, int coarse_iters, cudaStream_t st, long long &launches);
 cudaError_t modal_transform_out(const ModalPlan &p, int nb, Prec value, Prec type, void *u0, cudaStream_t st, long long &launches);
 
+// Whether the FP64 cycle of nb right-hand sides is faster in mode space than on the plane kernels (form.cpp).
+bool mode_space_faster(int nx, int ny, int nz, int nb, int npre, int npost);
+
 // Many systems at once (batched.cu), FP32: their transforms and tails as one launch each, the CTAs taken
 // from lists of (system, tile) and (system, mode); systems whose active flag is not 1 are skipped.
 struct SineJob {

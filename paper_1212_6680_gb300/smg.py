@@ -20,6 +20,7 @@ SMG_OK, SMG_ERR_ARG, SMG_ERR_CUDA, SMG_ERR_NOCONV, SMG_ERR_BREAKDOWN, SMG_ERR_TI
 SMG_ERR_HOST = -7
 SMG_PCG, SMG_FPCG, SMG_PSD = 0, 1, 2
 SMG_FP64, SMG_FP32, SMG_BF16 = 0, 1, 2
+SMG_FORM_MODES, SMG_FORM_PLANES = 0, 1
 SMG_OPT_COARSE_ITERS, SMG_OPT_THREADS, SMG_OPT_PROFILE, SMG_OPT_CLUSTER_MAX, SMG_OPT_CLUSTER_MAX32 = 0, 1, 2, 3, 4
 SMG_OPT_PRECOND = 5
 SMG_OPT_LEAN = 6
@@ -42,7 +43,8 @@ EXPORTS = ("smg_setup", "smg_set_precision", "smg_set_option", "smg_apply", "smg
            "smg_batched_destroy", "smg_batched_apply", "smg_batched_info", "smg_batched_set_profile", "smg_batched_profile_read",
            "smg_set_learned", "smg_learned_stats", "smg_collect_pairs", "smg_net_forward", "smg_net_loss_grad",
            "smg_net_train", "smg_net_set_tensor_cores", "smg_net_tc_status", "smg_setup_coefs",
-           "smg_plane_layout", "smg_plane_layout_kind", "smg_gram", "smg_krylov_history", "smg_plane_classes")
+           "smg_plane_layout", "smg_plane_layout_kind", "smg_gram", "smg_krylov_history", "smg_plane_classes",
+           "smg_cycle_form")
 NET_WEIGHTS = 7776
 
 
@@ -68,6 +70,7 @@ def _load():
     L.smg_destroy.argtypes = [vp]
     L.smg_setup_coefs.argtypes = [i, i, i, i, i, i, dp, dp, ip, ip]
     L.smg_plane_classes.argtypes = [i, i, i, i, ip]
+    L.smg_cycle_form.argtypes = [i, i, i, i, i, i, i, ip]
     L.smg_plane_layout.argtypes = [i, i, i, i, ctypes.POINTER(ctypes.c_longlong)]
     L.smg_plane_layout_kind.argtypes = [i, i, i, i, i, i, ctypes.POINTER(ctypes.c_longlong)]
     L.smg_last_error.restype = ctypes.c_char_p
@@ -227,6 +230,13 @@ def smg_plane_classes(nx: int, ny: int, nz: int, l: int):
     for _ in range(l):
         nzl //= 2
     return rc, cls[:nzl].copy()
+
+
+def smg_cycle_form(nx: int, ny: int, nz: int, npre: int, npost: int, precision: str, nb: int = 1) -> int:
+    """SMG_FORM_MODES or SMG_FORM_PLANES: the form the V-cycle takes for nb right-hand sides (host only)."""
+    form = ctypes.c_int(-1)
+    _check(_lib.smg_cycle_form(nx, ny, nz, npre, npost, PRECISIONS[precision], nb, ctypes.byref(form)))
+    return form.value
 
 
 def smg_plane_layout(nx: int, ny: int, elem_bytes: int, R: int = 1) -> dict:
