@@ -55,15 +55,31 @@ __device__ __forceinline__ bool grid_reduce(double (&v)[NV], DSum *part, unsigne
 
 // This CTA's share of n items: contiguous (a grid-wide stride leaves some CTAs a whole trip more than
 // others: 4 against 3 at 128^3, and takes a CTA's rows apart), walked with the CTA's threads.
+// A grid may have 2^32 points: the share's place in the vectors is a 64-bit base, and its items are counted from
+// there in 32 bits (64-bit counts in the loops: solve-101x75x53 855 -> 867 us).
 struct Share {
+    long long base;
     int begin, end;
 };
-__device__ __forceinline__ Share cta_share(int n) {
-    return Share{static_cast<int>(static_cast<long long>(n) * blockIdx.x / gridDim.x) + static_cast<int>(threadIdx.x),
-                 static_cast<int>(static_cast<long long>(n) * (blockIdx.x + 1) / gridDim.x)};
+__device__ __forceinline__ Share cta_share(long long n) {
+    const long long base = n * blockIdx.x / gridDim.x;
+    return Share{base, static_cast<int>(threadIdx.x), static_cast<int>(n * (blockIdx.x + 1) / gridDim.x - base)};
 }
 struct GridDiv {  // rows of nx values (or nx / 4 chunks), ny rows a plane
     FastDiv row, plane;
+};
+// The row of the share's item i and its place in that row of `len` items.
+struct RowOf {
+    int row0, x0;
+    __device__ __forceinline__ RowOf(const Share &sh, int len, const FastDiv &by) {
+        row0 = div_by_wide(static_cast<unsigned>(sh.base), by);
+        x0 = static_cast<int>(sh.base - static_cast<long long>(row0) * len);
+    }
+    __device__ __forceinline__ void at(int i, int len, const FastDiv &by, int &row, int &x) const {
+        const int t = x0 + i, dr = div_by(t, by);
+        row = row0 + dr;
+        x = t - dr * len;
+    }
 };
 
 __device__ __forceinline__ double stencil7(const double *__restrict__ u, long long i, int x, int y, int z, int nx,
@@ -103,9 +119,16 @@ __global__ void __launch_bounds__(kMaxThreads) k_init_residual(int nx, int ny, i
                                 unsigned *counter, GridDiv gd) {
     const long long np = static_cast<long long>(nx) * ny;
     double a0 = 0.0, a1 = 0.0;
-    const Share sh = cta_share(nx * ny * nz);
+    const Share sh = cta_share(np * nz);
+    const RowOf rows(sh, nx, gd.row);
+    b += sh.base;
+    x += sh.base;
+    r += sh.base;
+    if (f0 != nullptr) f0 += sh.base;
     for (int i = sh.begin; i < sh.end; i += blockDim.x) {
-        const int row = div_by(i, gd.row), xx = i - row * nx, zz = div_by(row, gd.plane), yy = row - zz * ny;
+        int row, xx;
+        rows.at(i, nx, gd.row, row, xx);
+        const int zz = div_by(row, gd.plane), yy = row - zz * ny;
         const double bi = b[i];
         const double ri = bi - stencil7(x, i, xx, yy, zz, nx, ny, nz, np);
         r[i] = ri;
@@ -130,9 +153,14 @@ __global__ void __launch_bounds__(kMaxThreads) k_true_residual(int nx, int ny, i
                                 KrylovScalars *sc, DSum *part, unsigned *counter, GridDiv gd) {
     const long long np = static_cast<long long>(nx) * ny;
     double a0 = 0.0;
-    const Share sh = cta_share(nx * ny * nz);
+    const Share sh = cta_share(np * nz);
+    const RowOf rows(sh, nx, gd.row);
+    b += sh.base;
+    x += sh.base;
     for (int i = sh.begin; i < sh.end; i += blockDim.x) {
-        const int row = div_by(i, gd.row), xx = i - row * nx, zz = div_by(row, gd.plane), yy = row - zz * ny;
+        int row, xx;
+        rows.at(i, nx, gd.row, row, xx);
+        const int zz = div_by(row, gd.plane), yy = row - zz * ny;
         const double ri = b[i] - stencil7(x, i, xx, yy, zz, nx, ny, nz, np);
         a0 = fma(ri, ri, a0);
     }
@@ -151,7 +179,10 @@ __global__ void __launch_bounds__(kMaxThreads) k_dots_beta(long long n, const S 
     const int variant = sc->variant;
     const bool need_sdr = (variant == 1) && (sc->restart == 0);
     double a0 = 0.0, a1 = 0.0;
-    const Share sh = cta_share(static_cast<int>(n));
+    const Share sh = cta_share(n);
+    s += sh.base;
+    r += sh.base;
+    q += sh.base;
     for (int i = sh.begin; i < sh.end; i += blockDim.x) {
         const double si = ldv<double>(s + i);
         a0 = fma(si, r[i], a0);
@@ -183,7 +214,9 @@ __global__ void __launch_bounds__(kMaxThreads) k_update_p(long long n, const S *
     pdl_wait();
     if constexpr (IDENT) ident_status(sc);
     const double beta = sc->beta;
-    const Share sh = cta_share(static_cast<int>(n));
+    const Share sh = cta_share(n);
+    s += sh.base;
+    p += sh.base;
     for (int i = sh.begin; i < sh.end; i += blockDim.x) {
         const double si = ldv<double>(s + i);
         p[i] = (beta == 0.0) ? si : fma(beta, p[i], si);
@@ -197,9 +230,14 @@ __global__ void __launch_bounds__(kMaxThreads) k_spmv_alpha(int nx, int ny, int 
     pdl_wait();
     const long long np = static_cast<long long>(nx) * ny;
     double a0 = 0.0;
-    const Share sh = cta_share(nx * ny * nz);
+    const Share sh = cta_share(np * nz);
+    const RowOf rows(sh, nx, gd.row);
+    p += sh.base;
+    q += sh.base;
     for (int i = sh.begin; i < sh.end; i += blockDim.x) {
-        const int row = div_by(i, gd.row), xx = i - row * nx, zz = div_by(row, gd.plane), yy = row - zz * ny;
+        int row, xx;
+        rows.at(i, nx, gd.row, row, xx);
+        const int zz = div_by(row, gd.plane), yy = row - zz * ny;
         const double qi = stencil7(p, i, xx, yy, zz, nx, ny, nz, np);
         q[i] = qi;
         a0 = fma(p[i], qi, a0);
@@ -244,7 +282,12 @@ __global__ void __launch_bounds__(kMaxThreads) k_update_xr(long long n, double *
     const double alpha = sc->alpha;
     const bool sq = IDENT && sc->variant == 1;
     double a0 = 0.0, a1 = 0.0;
-    const Share sh = cta_share(static_cast<int>(n));
+    const Share sh = cta_share(n);
+    x += sh.base;
+    p += sh.base;
+    r += sh.base;
+    q += sh.base;
+    if (f0 != nullptr) f0 += sh.base;
     for (int i = sh.begin; i < sh.end; i += blockDim.x) {
         x[i] = fma(alpha, p[i], x[i]);
         const double qi = q[i], rn = fma(-alpha, qi, r[i]);
@@ -325,6 +368,9 @@ template <class S>
 __device__ __forceinline__ void dots_share(double &a0, double &a1, const Share &sh, const S *s, const double *r, const double *q,
                                            bool with_q) {
     if (sh.begin >= sh.end) return;
+    s += 4 * sh.base;
+    r += 4 * sh.base;
+    q += 4 * sh.base;
     RawChunk<S> ns = raw4<S>(s + 4 * sh.begin);
     RawChunk<double> nr = raw4<double>(r + 4 * sh.begin), nq;
     if (with_q) nq = raw4<double>(q + 4 * sh.begin);
@@ -355,6 +401,8 @@ template <class S>
 __device__ __forceinline__ void update_p_share(const Share &sh, const S *s, double *p, double beta) {
     if (sh.begin >= sh.end) return;
     const bool keep = beta != 0.0;
+    s += 4 * sh.base;
+    p += 4 * sh.base;
     RawChunk<S> ns = raw4<S>(s + 4 * sh.begin);
     RawChunk<double> np;
     if (keep) np = raw4<double>(p + 4 * sh.begin);
@@ -410,10 +458,14 @@ __global__ void __launch_bounds__(kMaxThreads) k_spmv_alpha4(int nx, int ny, int
     pdl_wait();
     const int nq = nx >> 2, npi = nx * ny, nc = (npi >> 2) * nz;
     const Share sh = cta_share(nc);
+    const RowOf rows(sh, nq, gd.row);
+    p += 4 * sh.base;
+    q += 4 * sh.base;
     double a0 = 0.0;
 #pragma unroll 2
     for (int c = sh.begin; c < sh.end; c += blockDim.x) {
-        const int row = div_by(c, gd.row), xq = c - row * nq;
+        int row, xq;
+        rows.at(c, nq, gd.row, row, xq);
         const int zz = div_by(row, gd.plane), yy = row - zz * ny, xx = 4 * xq;
         const int i = 4 * c;
         double pc[4];
@@ -471,6 +523,11 @@ __global__ void __launch_bounds__(kMaxThreads) k_update_xr4(int nc, double *__re
     pdl_trigger();
     pdl_wait();
     const Share sh = cta_share(nc);
+    x += 4 * sh.base;
+    p += 4 * sh.base;
+    r += 4 * sh.base;
+    q += 4 * sh.base;
+    if (f0 != nullptr) f0 += 4 * sh.base;
     const double alpha = sc->alpha;
     const bool sq = IDENT && sc->variant == 1;
     double a0 = 0.0, a1 = 0.0;
@@ -556,12 +613,15 @@ __global__ void __launch_bounds__(kMaxThreads) k_tail_fused(int nx, int ny, int 
     }
     // ---- q = A p, pq = (p, q), alpha ----
     {
+        const RowOf rows(sh, nq, gd.row);
+        const long long to = 4 * sh.base;
         double a0 = 0.0;
 #pragma unroll 2
         for (int c = sh.begin; c < sh.end; c += blockDim.x) {
-            const int row = div_by(c, gd.row), xq = c - row * nq;
+            int row, xq;
+            rows.at(c, nq, gd.row, row, xq);
             const int zz = div_by(row, gd.plane), yy = row - zz * ny, xx = 4 * xq;
-            const int i = 4 * c;
+            const long long i = to + 4 * c;
             double pc[4];
             ld4cg(pc, p + i);
             const double pl = (xx > 0) ? __ldcg(p + i - 1) : 0.0, pr = (xx + 4 < nx) ? __ldcg(p + i + 4) : 0.0;
@@ -615,10 +675,11 @@ __global__ void __launch_bounds__(kMaxThreads) k_tail_fused(int nx, int ny, int 
     // ---- x += alpha p, r_new = r - alpha q, f0 = (S) r_new, rr ----
     {
         const double alpha = __ldcg(&sc->alpha);
-            double a0 = 0.0;
+        const long long to = 4 * sh.base;
+        double a0 = 0.0;
 #pragma unroll 2
         for (int c = sh.begin; c < sh.end; c += blockDim.x) {
-            const int i = 4 * c;
+            const long long i = to + 4 * c;
             double xv[4], pv[4], ro[4], qv[4], rn[4];
             ld4(xv, x + i);
             ld4(pv, p + i);

@@ -129,5 +129,9 @@ inline FastDiv fast_div(int d) {
 __device__ __forceinline__ int div_by(int n, const FastDiv &f) {
     return static_cast<int>((__umulhi(static_cast<unsigned>(n), f.mul) + static_cast<unsigned>(n)) >> f.shift);
 }
+// The same for 0 <= n < 2^32 (the sum may need a 33rd bit).
+__device__ __forceinline__ int div_by_wide(unsigned n, const FastDiv &f) {
+    return static_cast<int>((static_cast<unsigned long long>(__umulhi(n, f.mul)) + n) >> f.shift);
+}
 
 }  // namespace smg
