@@ -582,8 +582,9 @@ int batched_build(smg_batched_ctx &c, const int *dims, cudaStream_t st) {
     auto up = [](size_t v) { return (v + 255) / 256 * 256; };
     size_t b_shared = 0, b_coef = 0, b_c64 = 0, b_vec = 0;
     long long vtot = 0;
-    std::map<int, size_t> sines;  // transform matrices by nx: offset
-    std::vector<float> mats;
+    std::map<int, std::pair<size_t, size_t>> sines;  // by nx: offsets of its sines and of its matrices
+    std::vector<double> tables;
+    size_t n_mats = 0;
     for (int s = 0; s < nsys; ++s) {
         SysPlan &p = sys[s];
         p.nx = dims[3 * s];
@@ -602,10 +603,10 @@ int batched_build(smg_batched_ctx &c, const int *dims, cudaStream_t st) {
         b_coef += up(p.m.coef_values * sizeof(float));
         b_c64 += up(p.m.coef64_values * sizeof(double));
         b_vec += p.m.vec_bytes;
-        if (sines.emplace(p.nx, mats.size()).second) {
-            const std::vector<float> m = sine_matrices<float>(p.nx);
-            mats.insert(mats.end(), m.begin(), m.end());
-            mats.resize((mats.size() + 63) / 64 * 64);
+        if (sines.emplace(p.nx, std::make_pair(tables.size(), n_mats)).second) {
+            const std::vector<double> t = sine_table(p.nx);
+            tables.insert(tables.end(), t.begin(), t.end());
+            n_mats += 4 * static_cast<size_t>(sine_order(p.nx)) * sine_order(p.nx);
         }
     }
     unsigned char *d_shared, *d_coef, *d_c64, *d_vec;
@@ -614,7 +615,9 @@ int batched_build(smg_batched_ctx &c, const int *dims, cudaStream_t st) {
     BCHK(buf.alloc(&d_coef, b_coef));
     BCHK(buf.alloc(&d_c64, b_c64));
     BCHK(buf.alloc(&d_vec, b_vec));
-    BCHK(buf.alloc(&d_mats, mats.size()));
+    BCHK(buf.alloc(&d_mats, n_mats));
+    double *d_tables;
+    BCHK(buf.alloc(&d_tables, tables.size()));
     BCHK(buf.alloc(&c.kk.r, vtot));
     BCHK(buf.alloc(&c.kk.p, vtot));
     BCHK(buf.alloc(&c.kk.q, vtot));
@@ -622,7 +625,8 @@ int batched_build(smg_batched_ctx &c, const int *dims, cudaStream_t st) {
     BCHK(buf.alloc(&c.kk.s, vtot));
     BCHK(cudaMemsetAsync(c.kk.p, 0, vtot * sizeof(double), st));
     BCHK(cudaMemsetAsync(c.kk.q, 0, vtot * sizeof(double), st));
-    BCHK(cudaMemcpyAsync(d_mats, mats.data(), mats.size() * sizeof(float), cudaMemcpyHostToDevice, st));
+    BCHK(cudaMemcpyAsync(d_tables, tables.data(), tables.size() * sizeof(double), cudaMemcpyHostToDevice, st));
+    for (const auto &e : sines) BCHK(launch_sine_matrices<float>(e.first, d_tables + e.second.first, d_mats + e.second.second, st));
     std::vector<unsigned char> shared;
     shared.reserve(b_shared);
     {
@@ -654,7 +658,7 @@ int batched_build(smg_batched_ctx &c, const int *dims, cudaStream_t st) {
     for (int s : by_size) {
         SysPlan &p = sys[s];
         args[s] = p.m.a;
-        SineArgs g{p.nx, p.ny, p.nz, p.m.a.pitch, (p.nx + 1) / 2, ((p.nx + 1) / 2 + 63) / 64 * 64, d_mats + sines[p.nx]};
+        SineArgs g{p.nx, p.ny, p.nz, p.m.a.pitch, (p.nx + 1) / 2, sine_order(p.nx), d_mats + sines[p.nx].second};
         jobs[s] = SineJob{g, c.kk.rf + p.off, p.m.a.fw[0], p.m.a.u[0], c.kk.s + p.off};
         for (int m = 0; m < sine_mode_tiles(g); ++m)
             for (int t = 0; t < sine_line_tiles(g); ++t) tiles.push_back(SineTile{s, t, m});

@@ -571,24 +571,30 @@ void modal_place(ModalHost<T> &h, unsigned char *shared, T *coef, double *coef64
     }
 }
 
-template <class T>
-std::vector<T> sine_matrices(int nx) {
-    const int nh = (nx + 1) / 2;
-    const size_t hp = up(nh, 64);
+std::vector<double> sine_table(int nx) {
     const double pi = 3.14159265358979323846, sc = std::sqrt(2.0 / (nx + 1));
-    std::vector<T> mat(4 * hp * hp, T(0));
     std::vector<double> sines(2 * (nx + 1));
     for (int i = 0; i < 2 * (nx + 1); ++i) sines[i] = sc * std::sin(pi * i / (nx + 1));
-    for (int x = 0; x < nh; ++x)
-        for (int q = 0; q < nh; ++q)
-            for (int par = 0; par < 2; ++par) {
-                if (par == 1 && (q >= nx / 2 || x >= nx / 2)) continue;
-                const long long ph = static_cast<long long>(x + 1) * (2 * q + 1 + par) % (2 * (nx + 1));
-                const T v = static_cast<T>(sines[ph]);
-                mat[par * hp * hp + x * hp + q] = v;
-                mat[(2 + par) * hp * hp + q * hp + x] = v;
-            }
-    return mat;
+    return sines;
+}
+
+// The four matrices from the sines of one period, zero in the padding.  HBM: writes them once (on the host they took
+// 6.5 ms at 2048 points, and their copy as long again).
+template <class T>
+__global__ void __launch_bounds__(256) sine_matrices_kernel(int nx, int nh, int hp, const double *__restrict__ sines, T *__restrict__ mat) {
+    const int c = blockIdx.x * blockDim.x + threadIdx.x, r = blockIdx.y, par = blockIdx.z & 1;
+    if (c >= hp) return;
+    const int x = blockIdx.z < 2 ? r : c, q = blockIdx.z < 2 ? c : r;  // by point, then by mode
+    const int n = par ? nx / 2 : nh;
+    T v = T(0);
+    if (x < n && q < n) v = static_cast<T>(sines[(x + 1) * (2 * q + 1 + par) % (2 * (nx + 1))]);
+    mat[(static_cast<long long>(blockIdx.z) * hp + r) * hp + c] = v;
+}
+template <class T>
+cudaError_t launch_sine_matrices(int nx, const double *sines, T *mat, cudaStream_t st) {
+    const int nh = (nx + 1) / 2, hp = sine_order(nx);
+    sine_matrices_kernel<T><<<dim3((hp + 255) / 256, hp, 4), 256, 0, st>>>(nx, nh, hp, sines, mat);
+    return cudaGetLastError();
 }
 
 int modal_tail_threads(size_t smem, long long ctas, int num_sms, int most, int planes, int G) {
@@ -602,7 +608,7 @@ int modal_tail_threads(size_t smem, long long ctas, int num_sms, int most, int p
 
 template int modal_plan<float>(ModalHost<float> &, const HostHierarchy &, ModalConfig, int, int, int);
 template void modal_place<float>(ModalHost<float> &, unsigned char *, float *, double *, unsigned char *);
-template std::vector<float> sine_matrices<float>(int);
+template cudaError_t launch_sine_matrices<float>(int, const double *, float *, cudaStream_t);
 
 namespace {
 
@@ -620,10 +626,14 @@ int build(ModalPlan &p, ModalHost<T> &h, const HostHierarchy &H, int npre, int n
     T *coef = reinterpret_cast<T *>(d + h.shared.size() + b_64);
     modal_place<T>(h, d, coef, c64, static_cast<unsigned char *>(p.d_buf));
     MCHK(k.setup(h.a, coef, c64, 0));
-    const std::vector<T> mat = sine_matrices<T>(H.nx);
-    MCHK(cudaMalloc(&p.d_sin, mat.size() * sizeof(T)));
-    MCHK(cudaMemcpy(p.d_sin, mat.data(), mat.size() * sizeof(T), cudaMemcpyHostToDevice));
-    p.sine = SineArgs{H.nx, H.ny, H.nz, h.a.pitch, (H.nx + 1) / 2, static_cast<int>(up((H.nx + 1) / 2, 64)), p.d_sin};
+    const std::vector<double> sines = sine_table(H.nx);
+    const size_t b_sines = up(sines.size() * sizeof(double), 256);
+    const int hp = sine_order(H.nx);
+    MCHK(cudaMalloc(&p.d_sin, b_sines + 4 * sizeof(T) * hp * hp));
+    MCHK(cudaMemcpy(p.d_sin, sines.data(), sines.size() * sizeof(double), cudaMemcpyHostToDevice));
+    T *const mat = reinterpret_cast<T *>(static_cast<unsigned char *>(p.d_sin) + b_sines);
+    MCHK(launch_sine_matrices<T>(H.nx, static_cast<const double *>(p.d_sin), mat, 0));
+    p.sine = SineArgs{H.nx, H.ny, H.nz, h.a.pitch, (H.nx + 1) / 2, hp, mat};
     MCHK(cudaMalloc(&p.d_args, sizeof(h.a)));
     MCHK(cudaMemcpy(p.d_args, &h.a, sizeof(h.a), cudaMemcpyHostToDevice));
     int dev = 0;

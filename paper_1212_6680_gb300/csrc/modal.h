@@ -104,8 +104,12 @@ template <class T>
 int modal_plan(ModalHost<T> &h, const HostHierarchy &H, ModalConfig cfg, int nb, int npre, int npost);
 template <class T>
 void modal_place(ModalHost<T> &h, unsigned char *shared, T *coef, double *coef64, unsigned char *vec);
+// The transforms' matrices of lines of nx points: their order as stored, the sines they are made of (host), and the
+// four of them, 4 sine_order^2 values at mat, from those sines on the device.
+inline int sine_order(int nx) { return ((nx + 1) / 2 + 63) / 64 * 64; }
+std::vector<double> sine_table(int nx);
 template <class T>
-std::vector<T> sine_matrices(int nx);
+cudaError_t launch_sine_matrices(int nx, const double *sines, T *mat, cudaStream_t st);
 // Threads of the tail kernel for systems that need smem bytes when ctas of them are to run: the kernel
 // takes 128 registers a thread, so 512 threads fill an SM; with more CTAs than SMs the SM is shared by as
 // many as the shared memory allows, else one CTA takes it whole (as far as its planes fill it).
