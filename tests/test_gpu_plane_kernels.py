@@ -52,16 +52,16 @@ def check(orc, shape, cycle, r, s, what=""):
 
 CASES = [
     # rows a lane 1, 2, 3, 4: a line, a plane, and planes of several lines and levels
-    ((8, 1, 1), (1, 0), 1), ((32, 1, 4), (1, 1), 1), ((30, 3, 1), (2, 1), 1), ((40, 5, 4), (1, 0), 16), ((64, 5, 4), (1, 1), 32),
-    ((60, 200, 1), (1, 0), 1), ((75, 5, 7), (1, 0), 8), ((96, 5, 4), (2, 1), 32), ((96, 100, 1), (1, 0), 1),
-    ((100, 1, 100), (1, 0), 1), ((101, 5, 4), (1, 1), 16), ((128, 5, 4), (2, 1), 16), ((128, 60, 12), (1, 0), 64),
+    ((8, 1, 1), (1, 0), 1), ((32, 1, 4), (1, 1), 1), ((30, 3, 1), (2, 1), 1), ((32, 5, 4), (1, 1), 64), ((40, 5, 4), (1, 0), 64),
+    ((64, 5, 4), (2, 1), 48), ((75, 5, 4), (1, 0), 48), ((96, 5, 4), (2, 1), 32), ((96, 100, 1), (1, 0), 1),
+    ((100, 1, 100), (1, 0), 1), ((101, 5, 4), (1, 1), 32), ((128, 5, 4), (2, 1), 24), ((128, 60, 12), (1, 0), 64),
     # 6 and 8
-    ((160, 200, 1), (1, 0), 1), ((161, 5, 4), (2, 1), 16), ((192, 9, 5), (1, 0), 16), ((192, 60, 12), (1, 0), 32),
-    ((200, 5, 4), (1, 1), 16), ((256, 5, 4), (2, 1), 16), ((256, 128, 3), (1, 0), 16), ((256, 60, 12), (1, 1), 32),
+    ((161, 5, 4), (2, 1), 32), ((192, 5, 4), (1, 1), 24), ((192, 60, 12), (1, 0), 32),
+    ((200, 5, 4), (1, 1), 32), ((256, 5, 4), (2, 1), 24), ((256, 128, 3), (1, 0), 24), ((256, 60, 12), (1, 0), 32),
     # two warps of 8; two, three and four warps of 16
-    ((300, 1, 64), (2, 0), 1), ((300, 5, 4), (1, 1), 16), ((512, 5, 4), (2, 1), 8), ((512, 32, 32), (1, 0), 8), ((512, 512, 1), (1, 0), 1),
-    ((777, 1, 6), (1, 1), 1), ((777, 5, 4), (1, 1), 8), ((777, 60, 50), (1, 0), 1), ((1024, 5, 4), (1, 1), 1),
-    ((1290, 5, 4), (2, 1), 3), ((1536, 5, 4), (2, 1), 1), ((2047, 5, 4), (2, 1), 1), ((2048, 512, 1), (1, 0), 1),
+    ((300, 1, 64), (2, 0), 1), ((300, 5, 4), (1, 1), 32), ((512, 5, 4), (2, 1), 12), ((512, 32, 32), (1, 0), 8), ((500, 300, 1), (1, 0), 1),
+    ((777, 1, 6), (1, 1), 1), ((777, 5, 4), (1, 1), 12), ((777, 60, 50), (1, 0), 2), ((1024, 5, 4), (2, 1), 12),
+    ((1290, 5, 4), (2, 1), 8), ((1536, 5, 4), (1, 1), 1), ((2047, 5, 4), (2, 1), 2), ((2048, 512, 1), (1, 0), 1),
 ]
 
 
@@ -81,14 +81,14 @@ def test_bit_identical_options(smg, shape, cycle, nb):
         assert np.array_equal(s, apply(smg, shape, cycle, r, options)), options
 
 
-@pytest.mark.parametrize("shape,cycle,nb", [((96, 100, 1), (1, 0), 1), ((101, 5, 4), (1, 1), 16), ((256, 60, 12), (1, 1), 32),
-                                            ((512, 512, 1), (1, 0), 1), ((1290, 5, 4), (2, 1), 3)])
+@pytest.mark.parametrize("shape,cycle,nb", [((96, 100, 1), (1, 0), 1), ((101, 5, 4), (1, 1), 32), ((256, 60, 12), (1, 0), 32),
+                                            ((500, 300, 1), (1, 0), 1), ((1290, 5, 4), (2, 1), 8)])
 def test_cta_size(smg, orc, shape, cycle, nb):
     r = rhs(shape, nb)
     check(orc, shape, cycle, r, apply(smg, shape, cycle, r, [(smg.SMG_OPT_THREADS, 256)]), "256 threads")
 
 
-@pytest.mark.parametrize("shape,cycle,nb", [((300, 1, 64), (2, 0), 1), ((300, 5, 4), (1, 1), 16), ((512, 5, 4), (2, 1), 8),
+@pytest.mark.parametrize("shape,cycle,nb", [((300, 1, 64), (2, 0), 1), ((300, 5, 4), (1, 1), 32), ((512, 5, 4), (2, 1), 12),
                                             ((512, 32, 32), (1, 0), 8), ((511, 300, 1), (1, 0), 1)])
 def test_sixteen_rows_a_lane_in_one_warp(smg, orc, shape, cycle, nb):
     """Lines of 257 to 512 rows on one warp (SMG_OPT_WIDE_MIN_ROWS = 513): the general plane cycle."""
@@ -98,7 +98,7 @@ def test_sixteen_rows_a_lane_in_one_warp(smg, orc, shape, cycle, nb):
 
 @pytest.mark.parametrize("iters", [2, 5])
 def test_coarsest_steps_on_planes(smg, orc, iters):
-    shape, cycle, nb = (101, 5, 4), (1, 1), 16
+    shape, cycle, nb = (101, 5, 4), (1, 1), 32
     r = rhs(shape, nb)
     s = apply(smg, shape, cycle, r, [(smg.SMG_OPT_COARSE_ITERS, iters)])
     ref = orc.SMG(*shape, *cycle, iters).apply(r[nb - 1].reshape(shape[::-1])).ravel()
@@ -119,7 +119,7 @@ def test_solves_on_planes_follow_the_oracle(smg, orc, shape):
     assert np.all(np.abs(hist - ref["hist"]) <= 1e-6 * ref["hist"])
 
 
-@pytest.mark.parametrize("shape,block", [((96, 5, 4), 16), ((512, 32, 12), 4)])
+@pytest.mark.parametrize("shape,block", [((96, 5, 4), 32), ((512, 32, 12), 12)])
 def test_form_follows_from_the_call_alone(smg, shape, block):
     """One vector runs in mode space and a block on the planes: neither call changes the other's result, in either
     order, and the single one can be captured after the block (its vectors are there)."""
@@ -161,7 +161,7 @@ def test_form_follows_from_the_call_alone(smg, shape, block):
 def test_eigenpairs_across_the_line(smg):
     """A block whose applications start on the planes and go to mode space as columns converge: eigenvalues
     within 1e-10 of the closed form, as test_gpu_parity.py's."""
-    shape, m = (75, 5, 7), 8
+    shape, m = (128, 5, 4), 12
     assert smg.smg_cycle_form(*shape, 1, 0, "fp64", m) == smg.SMG_FORM_PLANES
     assert smg.smg_cycle_form(*shape, 1, 0, "fp64", 2) == smg.SMG_FORM_MODES
     w = [4 * np.sin(np.pi * np.arange(1, n + 1) / (2 * (n + 1))) ** 2 for n in shape]
