@@ -82,9 +82,11 @@ struct smg_ctx {
     Prec level_prec = Prec::F64;
     std::vector<char> modes64;      // [nb - 1] 1: the FP64 cycle of nb right-hand sides runs in mode space
     ModalPlan mp;
+    ModalShape shape;               // formed when mode space is first used
     std::vector<void *> d_f, d_u;   // [L], entry 0 unused
-    void *d_s = nullptr;            // krylov_solve: T r in level_prec
-    void *d_rf = nullptr;           // krylov_solve: r in FP32 for an FP32 cycle, written by its kernels
+    // krylov_solve's T r in level_prec and, for an FP32 cycle, behind it r in FP32, which its kernels write: N doubles,
+    // allocated once (with a small grid's tables they keep the driver's block in place over a change of precision)
+    void *d_s = nullptr;
     void *d_ws = nullptr;
     size_t ws_bytes = 0;
     PlaneLayout lay_c;              // one CTA per plane
@@ -181,9 +183,6 @@ void free_planes(smg_ctx *h) {
 void free_levels(smg_ctx *h) {
     free_planes(h);
     modal_free(h->mp);
-    cudaFree(h->d_s);
-    cudaFree(h->d_rf);
-    h->d_s = h->d_rf = nullptr;
 }
 
 int instantiated_K(int nx) {
@@ -237,11 +236,10 @@ int ensure_levels(smg_ctx *h, int nb) {
         h->modes64.push_back(mode_space_faster(h->nx, h->ny, h->nz, c, h->npre, h->npost) ? 1 : 0);
     int modes = 0, planes = 0;
     for (int c = 1; c <= nb; ++c) (use_modal(h, c) ? modes : planes) = c;
-    const size_t one = static_cast<size_t>(h->N()) * storage_bytes(h->prec);
-    if (h->d_s == nullptr) SMG_CUDA(cudaMalloc(&h->d_s, one));
-    if (h->d_rf == nullptr && h->prec == Prec::F32) SMG_CUDA(cudaMalloc(&h->d_rf, one));
+    if (h->d_s == nullptr) SMG_CUDA(cudaMalloc(&h->d_s, static_cast<size_t>(h->N()) * sizeof(double)));
     if (modes > h->mp.nb) {
-        const int e = modal_build(h->mp, h->H, h->prec == Prec::F64, modes, h->npre, h->npost);
+        if (h->shape.lam.empty()) h->shape = modal_shape(h->H);
+        const int e = modal_build(h->mp, h->H, h->shape, h->prec == Prec::F64, modes, h->npre, h->npost);
         if (e != 0) {
             modal_free(h->mp);
             return fail(SMG_ERR_CUDA, std::string("mode-space cycle: ") + cudaGetErrorString(static_cast<cudaError_t>(e)));
@@ -259,6 +257,17 @@ int ensure_levels(smg_ctx *h, int nb) {
 // dynamic shared memory.
 int alloc_planes(smg_ctx *h, int nb) {
     const HostHierarchy &H = h->H;
+    if (h->d_pcoef == nullptr) {  // their coefficients, kept from then on
+        const size_t zb = H.zcoef.size() * sizeof(double), pb = H.pcoef.size() * sizeof(double);
+        if (h->d_zcoef == nullptr) SMG_CUDA(cudaMalloc(&h->d_zcoef, zb));
+        SMG_CUDA(cudaMemcpy(h->d_zcoef, H.zcoef.data(), zb, cudaMemcpyHostToDevice));
+        double *d = nullptr;
+        SMG_CUDA(cudaMalloc(&d, pb));
+        const cudaError_t e = cudaMemcpy(d, H.pcoef.data(), pb, cudaMemcpyHostToDevice);
+        if (e != cudaSuccess) cudaFree(d);
+        SMG_CUDA(e);
+        h->d_pcoef = d;
+    }
     h->d_f.assign(H.L, nullptr);
     h->d_u.assign(H.L, nullptr);
     for (int l = 1; l < H.L; ++l) {
@@ -733,7 +742,7 @@ int krylov_device(smg_ctx *h, int variant, const double *b, double *x, double to
     const bool ident = (h->precond == 0);                           // T = I: s is r itself
     // cycle input: r in FP32, written by the Krylov kernels, or r itself (FP64 and BF16 cycles)
     const bool own_f0 = h->prec == Prec::F32;
-    void *f0 = own_f0 ? h->d_rf : static_cast<void *>(h->d_r);
+    void *f0 = own_f0 ? static_cast<void *>(static_cast<float *>(h->d_s) + h->N()) : static_cast<void *>(h->d_r);
     void *u0 = ident ? static_cast<void *>(h->d_r) : h->d_s;        // s = T r
     const Prec kp = ident ? Prec::F64 : h->prec;                    // storage type of s
     void *f0k = (own_f0 && !ident) ? f0 : nullptr;                  // what the Krylov kernels write
@@ -874,15 +883,6 @@ int smg_setup(int nx, int ny, int nz, int npre, int npost, smg_handle *out) {
     build_hierarchy(nx, ny, nz, h->H);
     h->lean_level.assign(h->H.L, 0);
     for (int l = 0; l < h->H.L; ++l) h->lean_level[l] = lean_uniform_level(h->H, l) ? 1 : 0;
-    const size_t zb = h->H.zcoef.size() * sizeof(double), pb = h->H.pcoef.size() * sizeof(double);
-    cudaError_t e = cudaMalloc(&h->d_zcoef, zb);
-    if (e == cudaSuccess) e = cudaMalloc(&h->d_pcoef, pb);
-    if (e == cudaSuccess) e = cudaMemcpy(h->d_zcoef, h->H.zcoef.data(), zb, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(h->d_pcoef, h->H.pcoef.data(), pb, cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) {
-        smg_destroy(h);
-        return fail(SMG_ERR_CUDA, std::string("smg_setup: ") + cudaGetErrorString(e));
-    }
     int rc = ensure_levels(h, 1);
     if (rc != SMG_OK) {
         smg_destroy(h);
@@ -1301,6 +1301,7 @@ int smg_plane_layout_kind(int nx, int ny, int elem_bytes, int R, int kind, int s
 int smg_destroy(smg_handle h) {
     if (h == nullptr) return SMG_OK;
     free_levels(h);
+    cudaFree(h->d_s);
     cudaFree(h->d_zcoef);
     cudaFree(h->d_pcoef);
     cudaFree(h->d_r);

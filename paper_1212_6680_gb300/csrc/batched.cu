@@ -595,10 +595,11 @@ int batched_build(smg_batched_ctx &c, const int *dims, cudaStream_t st) {
         vtot += (p.N + 31) / 32 * 32;
         build_hierarchy(p.nx, p.ny, p.nz, p.H);
         p.cycle_bytes = vcycle_words(p, c.npre, c.npost) * 4.0;
-        if (modal_plan<float>(p.m, p.H, c.cfg, 1, c.npre, c.npost) != 0) {
+        if (modal_plan<float>(p.m, p.H, modal_shape(p.H), c.cfg, c.npre, c.npost) != 0) {
             set_last_error("batched solver: a system's planes do not fit the mode-space cycle");
             return SMG_ERR_CUDA;
         }
+        modal_vectors<float>(p.m, 1);
         b_shared += p.m.shared.size();
         b_coef += up(p.m.coef_values * sizeof(float));
         b_c64 += up(p.m.coef64_values * sizeof(double));

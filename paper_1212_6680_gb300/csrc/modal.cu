@@ -339,10 +339,8 @@ static void raw_line(const HostHierarchy &H, const double *pc, int m, int y, dou
 }
 
 void modal_free(ModalPlan &p) {
-    cudaFree(p.d_args);
     cudaFree(p.d_buf);
     cudaFree(p.d_tab);
-    cudaFree(p.d_sin);
     p = ModalPlan();
 }
 
@@ -455,49 +453,32 @@ std::vector<TailOp> tail_ops(const ModalArgs<T> &a) {
     return ops;
 }
 
-template <class T>
-int modal_plan(ModalHost<T> &h, const HostHierarchy &H, ModalConfig cfg, int nb, int npre, int npost) {
-    const int nx = H.nx, L = H.L, nh = (nx + 1) / 2;
-    h.cfg = cfg;
-    ModalArgs<T> &a = h.a;
-    std::memset(&a, 0, sizeof(a));
-    a.nmode = nx;
-    a.ny = H.ny;
-    a.pitch = static_cast<int>(up(H.ny, 4));
-    a.L = L;
-    a.P = H.P;
-    a.sum_ny = H.sum_ny;
-    a.npre = npre;
-    a.npost = npost;
-    for (int m = 0; m < H.P; ++m) a.ny_m[m] = H.ny_m[m], a.line_base[m] = H.line_base[m];
-    a.sm_pitch = static_cast<int>(up(H.ny, cfg.K));
+ModalShape modal_shape(const HostHierarchy &H) {
+    ModalShape s;
     // plane classes; plane types: planes with equal coefficients and class
-    std::vector<unsigned short> ptype(H.nplanes_total), pcls, ltype(H.sum_ny);
-    std::vector<T> zt;
+    s.ptype.resize(H.nplanes_total);
     std::vector<const double *> reps;  // each class's plane table
     std::map<std::string, int> seen;
-    for (int l = 0; l < L; ++l) {
+    for (int l = 0; l < H.L; ++l) {
         std::vector<int> slot, rep;
-        a.nz[l] = H.nz_l[l];
-        a.plane_base[l] = H.plane_base[l];
-        a.cls_base[l] = static_cast<int>(reps.size());
-        a.ncls[l] = plane_classes(H, l, slot, rep);
-        for (int z = 0; z < a.nz[l]; ++z) {
+        s.cls_base[l] = static_cast<int>(reps.size());
+        s.ncls[l] = plane_classes(H, l, slot, rep);
+        for (int z = 0; z < H.nz_l[l]; ++z) {
             const double *zc = &H.zcoef[static_cast<size_t>(H.plane_base[l] + z) * kCoefPerPlane];
             std::string key(reinterpret_cast<const char *>(zc), sizeof(double) * kCoefPerPlane);
             key.append(reinterpret_cast<const char *>(&slot[z]), sizeof(int));
             const auto it = seen.emplace(key, static_cast<int>(seen.size()));
             if (it.second) {
-                for (int i = 0; i < kCoefPerPlane; ++i) zt.push_back(static_cast<T>(zc[i]));
-                pcls.push_back(static_cast<unsigned short>(slot[z]));
+                s.zt.insert(s.zt.end(), zc, zc + kCoefPerPlane);
+                s.pcls.push_back(static_cast<unsigned short>(slot[z]));
             }
-            ptype[H.plane_base[l] + z] = static_cast<unsigned short>(it.first->second);
+            s.ptype[H.plane_base[l] + z] = static_cast<unsigned short>(it.first->second);
         }
         for (int z : rep) reps.push_back(&H.pcoef[static_cast<size_t>(H.plane_base[l] + z) * H.sum_ny * kCoefPerLine]);
     }
-    a.ncls_all = static_cast<int>(reps.size());
-    a.nptype = static_cast<int>(pcls.size());
+    s.ncls_all = static_cast<int>(reps.size());
     // line types: lines with equal coefficients in every class
+    s.ltype.resize(H.sum_ny);
     std::vector<std::vector<double>> rows;  // [type][class][kRawPerLine]
     seen.clear();
     for (int m = 0; m < H.P; ++m)
@@ -507,23 +488,66 @@ int modal_plan(ModalHost<T> &h, const HostHierarchy &H, ModalConfig cfg, int nb,
             const auto it = seen.emplace(std::string(reinterpret_cast<const char *>(r.data()), r.size() * sizeof(double)),
                                          static_cast<int>(rows.size()));
             if (it.second) rows.push_back(std::move(r));
-            ltype[H.line_base[m] + y] = static_cast<unsigned short>(it.first->second);
+            s.ltype[H.line_base[m] + y] = static_cast<unsigned short>(it.first->second);
         }
-    a.ntype = static_cast<int>(rows.size());
-    a.blk = a.ntype * kRow + cfg.G * cfg.G;
-    std::vector<double> raw(static_cast<size_t>(a.ncls_all) * a.ntype * kRawPerLine), lam(nx);
-    for (int t = 0; t < a.ntype; ++t)
-        for (int c = 0; c < a.ncls_all; ++c)
-            std::memcpy(&raw[(static_cast<size_t>(c) * a.ntype + t) * kRawPerLine], &rows[t][static_cast<size_t>(c) * kRawPerLine],
+    s.ntype = static_cast<int>(rows.size());
+    s.raw.resize(static_cast<size_t>(s.ncls_all) * s.ntype * kRawPerLine);
+    for (int t = 0; t < s.ntype; ++t)
+        for (int c = 0; c < s.ncls_all; ++c)
+            std::memcpy(&s.raw[(static_cast<size_t>(c) * s.ntype + t) * kRawPerLine], &rows[t][static_cast<size_t>(c) * kRawPerLine],
                         kRawPerLine * sizeof(double));
     const double pi = 3.14159265358979323846;
-    for (int q = 0; q < nx; ++q) {
+    const int nh = (H.nx + 1) / 2;
+    s.lam.resize(H.nx);
+    for (int q = 0; q < H.nx; ++q) {
         const int kk = q < nh ? 2 * q + 1 : 2 * (q - nh) + 2;
-        const double s = std::sin(pi * kk / (2.0 * (nx + 1)));
-        lam[q] = 4.0 * s * s;
+        const double v = std::sin(pi * kk / (2.0 * (H.nx + 1)));
+        s.lam[q] = 4.0 * v * v;
     }
-    const size_t sizes[] = {raw.size() * 8, lam.size() * 8, zt.size() * sizeof(T), ptype.size() * 2, pcls.size() * 2, ltype.size() * 2};
-    const void *const src[] = {raw.data(), lam.data(), zt.data(), ptype.data(), pcls.data(), ltype.data()};
+    return s;
+}
+
+template <class T>
+void modal_vectors(ModalHost<T> &h, int nb) {
+    const ModalArgs<T> &a = h.a;
+    h.vec_bytes = 0;
+    h.vec_off.clear();
+    for (int l = 0; l <= a.lt; ++l)
+        for (int t = 0; t < 2; ++t) {
+            h.vec_off.push_back(h.vec_bytes);
+            h.vec_bytes += up(static_cast<size_t>(nb) * a.nmode * a.nz[l] * a.pitch * sizeof(T), 256);
+        }
+}
+
+template <class T>
+int modal_plan(ModalHost<T> &h, const HostHierarchy &H, const ModalShape &s, ModalConfig cfg, int npre, int npost) {
+    const int L = H.L;
+    h.cfg = cfg;
+    ModalArgs<T> &a = h.a;
+    std::memset(&a, 0, sizeof(a));
+    a.nmode = H.nx;
+    a.ny = H.ny;
+    a.pitch = static_cast<int>(up(H.ny, 4));
+    a.L = L;
+    a.P = H.P;
+    a.sum_ny = H.sum_ny;
+    a.npre = npre;
+    a.npost = npost;
+    for (int m = 0; m < H.P; ++m) a.ny_m[m] = H.ny_m[m], a.line_base[m] = H.line_base[m];
+    a.sm_pitch = static_cast<int>(up(H.ny, cfg.K));
+    for (int l = 0; l < L; ++l) {
+        a.nz[l] = H.nz_l[l];
+        a.plane_base[l] = H.plane_base[l];
+        a.cls_base[l] = s.cls_base[l];
+        a.ncls[l] = s.ncls[l];
+    }
+    a.ncls_all = s.ncls_all;
+    a.nptype = static_cast<int>(s.pcls.size());
+    a.ntype = s.ntype;
+    a.blk = a.ntype * kRow + cfg.G * cfg.G;
+    const std::vector<T> zt(s.zt.begin(), s.zt.end());
+    const size_t sizes[] = {s.raw.size() * 8, s.lam.size() * 8, zt.size() * sizeof(T), s.ptype.size() * 2, s.pcls.size() * 2, s.ltype.size() * 2};
+    const void *const src[] = {s.raw.data(), s.lam.data(), zt.data(), s.ptype.data(), s.pcls.data(), s.ltype.data()};
     size_t o = 0;
     for (int i = 0; i < 6; ++i) {
         h.at[i] = o;
@@ -531,8 +555,8 @@ int modal_plan(ModalHost<T> &h, const HostHierarchy &H, ModalConfig cfg, int nb,
     }
     h.shared.assign(o, 0);
     for (int i = 0; i < 6; ++i) std::memcpy(h.shared.data() + h.at[i], src[i], sizes[i]);
-    h.coef_values = static_cast<size_t>(nx) * a.ncls_all * a.blk;
-    h.coef64_values = static_cast<size_t>(nx) * (a.ntype * kRow + 1024);
+    h.coef_values = static_cast<size_t>(a.nmode) * a.ncls_all * a.blk;
+    h.coef64_values = static_cast<size_t>(a.nmode) * (a.ntype * kRow + 1024);
     // the first level whose coarser levels all fit in one CTA's shared memory
     const ModalKernels<T> &k = modal_kernels<T>(cfg);
     h.smem = 0;
@@ -542,13 +566,6 @@ int modal_plan(ModalHost<T> &h, const HostHierarchy &H, ModalConfig cfg, int nb,
     h.at[6] = h.shared.size();
     h.shared.resize(h.at[6] + up(ops.size() * sizeof(TailOp), 256), 0);
     std::memcpy(h.shared.data() + h.at[6], ops.data(), ops.size() * sizeof(TailOp));
-    h.vec_bytes = 0;
-    h.vec_off.clear();
-    for (int l = 0; l <= a.lt; ++l)
-        for (int t = 0; t < 2; ++t) {
-            h.vec_off.push_back(h.vec_bytes);
-            h.vec_bytes += up(static_cast<size_t>(nb) * nx * a.nz[l] * a.pitch * sizeof(T), 256);
-        }
     return 0;
 }
 
@@ -606,40 +623,55 @@ int modal_tail_threads(size_t smem, long long ctas, int num_sms, int most, int p
     return std::min(most, std::max(128, (want + 31) / 32 * 32));
 }
 
-template int modal_plan<float>(ModalHost<float> &, const HostHierarchy &, ModalConfig, int, int, int);
+template int modal_plan<float>(ModalHost<float> &, const HostHierarchy &, const ModalShape &, ModalConfig, int, int);
+template void modal_vectors<float>(ModalHost<float> &, int);
 template void modal_place<float>(ModalHost<float> &, unsigned char *, float *, double *, unsigned char *);
 template cudaError_t launch_sine_matrices<float>(int, const double *, float *, cudaStream_t);
 
 namespace {
 
+// Vectors for nb right-hand sides in place of those there are, and the tables unless they are there: one block with
+// what is copied (shared data, arguments, sines) first, then what is formed there (coefficients, transform matrices).
 template <class T>
-int build(ModalPlan &p, ModalHost<T> &h, const HostHierarchy &H, int npre, int npost) {
-    const ModalConfig cfg = modal_config(H.ny, sizeof(T) == 8);
-    if (int e = modal_plan<T>(h, H, cfg, p.nb, npre, npost)) return e;
-    const ModalKernels<T> &k = modal_kernels<T>(cfg);
-    const size_t b_coef = up(h.coef_values * sizeof(T), 256), b_64 = up(h.coef64_values * 8, 256);
-    MCHK(cudaMalloc(&p.d_tab, h.shared.size() + b_64 + b_coef));
+int build(ModalPlan &p, ModalHost<T> &h, const HostHierarchy &H, const ModalShape &s, int nb, int npre, int npost) {
+    const bool fresh = p.d_tab == nullptr;
+    if (fresh)
+        if (int e = modal_plan<T>(h, H, s, modal_config(H.ny, sizeof(T) == 8), npre, npost)) return e;
+    p.nb = 0;
+    cudaFree(p.d_buf);
+    p.d_buf = nullptr;
+    modal_vectors<T>(h, nb);
     MCHK(cudaMalloc(&p.d_buf, h.vec_bytes));
-    unsigned char *d = static_cast<unsigned char *>(p.d_tab);
-    MCHK(cudaMemcpy(d, h.shared.data(), h.shared.size(), cudaMemcpyHostToDevice));
-    double *c64 = reinterpret_cast<double *>(d + h.shared.size());
-    T *coef = reinterpret_cast<T *>(d + h.shared.size() + b_64);
-    modal_place<T>(h, d, coef, c64, static_cast<unsigned char *>(p.d_buf));
-    MCHK(k.setup(h.a, coef, c64, 0));
-    const std::vector<double> sines = sine_table(H.nx);
-    const size_t b_sines = up(sines.size() * sizeof(double), 256);
-    const int hp = sine_order(H.nx);
-    MCHK(cudaMalloc(&p.d_sin, b_sines + 4 * sizeof(T) * hp * hp));
-    MCHK(cudaMemcpy(p.d_sin, sines.data(), sines.size() * sizeof(double), cudaMemcpyHostToDevice));
-    T *const mat = reinterpret_cast<T *>(static_cast<unsigned char *>(p.d_sin) + b_sines);
-    MCHK(launch_sine_matrices<T>(H.nx, static_cast<const double *>(p.d_sin), mat, 0));
-    p.sine = SineArgs{H.nx, H.ny, H.nz, h.a.pitch, (H.nx + 1) / 2, hp, mat};
-    MCHK(cudaMalloc(&p.d_args, sizeof(h.a)));
-    MCHK(cudaMemcpy(p.d_args, &h.a, sizeof(h.a), cudaMemcpyHostToDevice));
-    int dev = 0;
-    MCHK(cudaGetDevice(&dev));
-    MCHK(cudaDeviceGetAttribute(&p.num_sms, cudaDevAttrMultiProcessorCount, dev));
-    MCHK(cudaStreamSynchronize(0));  // the set-up kernel: callers' streams need not wait for the default one
+    unsigned char *const vec = static_cast<unsigned char *>(p.d_buf);
+    if (fresh) {
+        const std::vector<double> sines = sine_table(H.nx);
+        const int hp = sine_order(H.nx);
+        p.at_args = h.shared.size();
+        const size_t at_sines = p.at_args + up(sizeof(h.a), 256), at_64 = at_sines + up(sines.size() * sizeof(double), 256);
+        const size_t at_coef = at_64 + up(h.coef64_values * 8, 256), at_mat = at_coef + up(h.coef_values * sizeof(T), 256);
+        MCHK(cudaMalloc(&p.d_tab, at_mat + 4 * sizeof(T) * hp * hp));
+        unsigned char *const d = static_cast<unsigned char *>(p.d_tab);
+        double *const c64 = reinterpret_cast<double *>(d + at_64);
+        T *const coef = reinterpret_cast<T *>(d + at_coef), *const mat = reinterpret_cast<T *>(d + at_mat);
+        modal_place<T>(h, d, coef, c64, vec);
+        h.shared.resize(at_64, 0);
+        std::memcpy(h.shared.data() + p.at_args, &h.a, sizeof(h.a));
+        std::memcpy(h.shared.data() + at_sines, sines.data(), sines.size() * sizeof(double));
+        MCHK(cudaMemcpy(d, h.shared.data(), h.shared.size(), cudaMemcpyHostToDevice));
+        MCHK(launch_sine_matrices<T>(H.nx, reinterpret_cast<const double *>(d + at_sines), mat, 0));
+        const ModalKernels<T> &k = modal_kernels<T>(h.cfg);
+        MCHK(k.setup(h.a, coef, c64, 0));
+        p.sine = SineArgs{H.nx, H.ny, H.nz, h.a.pitch, (H.nx + 1) / 2, hp, mat};
+        int dev = 0;
+        MCHK(cudaGetDevice(&dev));
+        MCHK(cudaDeviceGetAttribute(&p.num_sms, cudaDevAttrMultiProcessorCount, dev));
+    } else {
+        unsigned char *const d = static_cast<unsigned char *>(p.d_tab);
+        modal_place<T>(h, d, const_cast<T *>(h.a.coef), const_cast<double *>(h.a.coef64), vec);
+        MCHK(cudaMemcpy(d + p.at_args, &h.a, sizeof(h.a), cudaMemcpyHostToDevice));
+    }
+    MCHK(cudaStreamSynchronize(0));  // the set-up kernels: callers' streams need not wait for the default one
+    p.nb = nb;
     return 0;
 }
 
@@ -669,7 +701,7 @@ cudaError_t cycle(const ModalPlan &p, const ModalHost<T> &h, int nb, int coarse_
         launches += 1;
     }
     const int threads = modal_tail_threads(h.smem, static_cast<long long>(a.nmode) * nb, p.num_sms, k.max_threads, a.nz[a.lt], h.cfg.G);
-    if ((e = k.tail(static_cast<const ModalArgs<T> *>(p.d_args), a.nmode, nb, coarse_iters, threads, h.smem, st)) != cudaSuccess)
+    if ((e = k.tail(reinterpret_cast<const ModalArgs<T> *>(static_cast<const unsigned char *>(p.d_tab) + p.at_args), a.nmode, nb, coarse_iters, threads, h.smem, st)) != cudaSuccess)
         return e;
     launches += 1;
     for (int l = a.lt - 1; l >= 0; --l) {
@@ -720,11 +752,10 @@ cudaError_t sine_out(const ModalPlan &p, int nb, const T *uh, void *u, cudaStrea
 
 }  // namespace
 
-int modal_build(ModalPlan &p, const HostHierarchy &H, bool f64, int nb, int npre, int npost) {
-    modal_free(p);
+int modal_build(ModalPlan &p, const HostHierarchy &H, const ModalShape &s, bool f64, int nb, int npre, int npost) {
+    if (p.d_tab != nullptr && p.f64 != f64) modal_free(p);
     p.f64 = f64;
-    p.nb = nb;
-    return f64 ? build<double>(p, p.h64, H, npre, npost) : build<float>(p, p.h32, H, npre, npost);
+    return f64 ? build<double>(p, p.h64, H, s, nb, npre, npost) : build<float>(p, p.h32, H, s, nb, npre, npost);
 }
 
 cudaError_t modal_transform_in(const ModalPlan &p, int nb, Prec type, const void *f0, cudaStream_t st, long long &launches) {

@@ -100,8 +100,20 @@ struct ModalHost {
     size_t coef_values = 0, coef64_values = 0, vec_bytes = 0;
     std::vector<size_t> vec_off;       // f and u of levels 0 .. lt
 };
+// What a hierarchy's plans of either type and any lane configuration are made of: the types and classes of its planes and
+// lines.  Reads every plane's table (3 x 512 x 4096 points: 24 ms), so a handle keeps it.
+struct ModalShape {
+    int ntype = 0, ncls_all = 0;
+    int cls_base[kMaxZLevels] = {0}, ncls[kMaxZLevels] = {0};
+    std::vector<unsigned short> ptype, pcls, ltype;
+    std::vector<double> zt, raw, lam;
+};
+ModalShape modal_shape(const HostHierarchy &H);
 template <class T>
-int modal_plan(ModalHost<T> &h, const HostHierarchy &H, ModalConfig cfg, int nb, int npre, int npost);
+int modal_plan(ModalHost<T> &h, const HostHierarchy &H, const ModalShape &s, ModalConfig cfg, int npre, int npost);
+// The vectors' sizes for nb right-hand sides (vec_off, vec_bytes).
+template <class T>
+void modal_vectors(ModalHost<T> &h, int nb);
 template <class T>
 void modal_place(ModalHost<T> &h, unsigned char *shared, T *coef, double *coef64, unsigned char *vec);
 // The transforms' matrices of lines of nx points: their order as stored, the sines they are made of (host), and the
@@ -117,18 +129,17 @@ int modal_tail_threads(size_t smem, long long ctas, int num_sms, int most, int p
 
 struct ModalPlan {
     bool f64 = false;
-    int nb = 0, threads = 0, num_sms = 0;
+    int nb = 0, num_sms = 0;
     ModalHost<float> h32;
     ModalHost<double> h64;
     SineArgs sine{};
-    void *d_args = nullptr;
     void *d_buf = nullptr;        // mode-space vectors
-    void *d_tab = nullptr;        // coefficients
-    void *d_sin = nullptr;        // transform matrices
+    void *d_tab = nullptr;        // coefficients and transform matrices, the kernels' arguments at at_args
+    size_t at_args = 0;
 };
 
-// Tables and buffers for nb right-hand sides; 0, or a cudaError_t.
-int modal_build(ModalPlan &p, const HostHierarchy &H, bool f64, int nb, int npre, int npost);
+// Tables, unless they are there, and vectors for nb right-hand sides; 0, or a cudaError_t (give the plan back then).
+int modal_build(ModalPlan &p, const HostHierarchy &H, const ModalShape &s, bool f64, int nb, int npre, int npost);
 void modal_free(ModalPlan &p);
 
 // u0 = T f0 for nb right-hand sides, in three parts: f0 ([rhs][z][y][x], of type F64, or F32 for an FP32
