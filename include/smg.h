@@ -324,6 +324,11 @@ int smg_net_loss_grad(int nx, int ny, int nz, int act_prec, const float *w, cons
 int smg_net_train(int npairs, const int *dims, const float *const *rho, const float *const *e, int epochs, double lr,
                   unsigned long long seed, int act_prec, float *w, double *loss_hist, void *stream);
 
+/* smg_net_release -- the three calls above take their work buffers from a pool of the library's own on the current
+ * device, which keeps up to 1 GB of them between calls; this gives back what is idle (so does smg_destroy).
+ * Synchronises the device; safe beside calls on other threads. */
+int smg_net_release(void);
+
 /* smg_net_set_tensor_cores -- process-wide choice for the BF16 16 -> 16 channel layer: 1 (the
  * default) runs it on the tcgen05 tensor cores, 0 on the CUDA cores (FP32 FMAs, the same BF16
  * inputs and rounding).  Takes effect at the next launch; not for concurrent use with solves. */

@@ -984,6 +984,7 @@ cudaError_t net_alloc(NetWork &nw, long long n, int act, bool training, NetMem m
     const int count = training ? 13 : 7;
     size_t total = 0;
     for (int i = 0; i < count; ++i) total += (parts[i].bytes + 255) / 256 * 256;
+    nw.slab_bytes = total;
     cudaError_t e = get(&nw.slab, total);
     if (e == cudaSuccess) {
         unsigned char *at = static_cast<unsigned char *>(nw.slab);
@@ -1007,6 +1008,8 @@ cudaError_t net_alloc(NetWork &nw, long long n, int act, bool training, NetMem m
 }
 
 void net_free(NetWork &nw) {
+    const cudaStream_t st = nw.st;
+    const bool large = nw.mem == NetMem::Pool && nw.slab_bytes > kNetPoolKeep;
     for (void *p : {nw.slab, nw.weights}) {
         if (p == nullptr) continue;
         if (nw.mem == NetMem::Own) cudaFree(p);
@@ -1015,6 +1018,8 @@ void net_free(NetWork &nw) {
     const long long launches = nw.launches;
     nw = NetWork();
     nw.launches = launches;
+    // the pool looks at what it keeps when a stream is synchronised
+    if (large) cudaStreamSynchronize(st);
 }
 
 cudaError_t net_forward(NetWork &nw, int nx, int ny, int nz, cudaStream_t st) {

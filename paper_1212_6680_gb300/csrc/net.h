@@ -58,6 +58,7 @@ struct NetWork {
     int wpart_blocks = 0;
     void *slab = nullptr;                // the block that holds all of the above but
     void *weights = nullptr;             // w, m and v
+    size_t slab_bytes = 0;
     NetMem mem = NetMem::Own;
     cudaStream_t st = nullptr;           // NetMem::Pool: the call's stream
     long long launches = 0;

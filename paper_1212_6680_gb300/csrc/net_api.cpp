@@ -149,6 +149,13 @@ extern "C" int smg_net_train(int npairs, const int *dims, const float *const *rh
     return SMG_OK;
 }
 
+extern "C" int smg_net_release(void) {
+    const cudaError_t e = cudaDeviceSynchronize();  // blocks freed in a stream's order are idle only then
+    if (e != cudaSuccess) return nfail(SMG_ERR_CUDA, std::string("smg_net_release: ") + cudaGetErrorString(e));
+    net_pool_trim();
+    return SMG_OK;
+}
+
 extern "C" int smg_net_set_tensor_cores(int on) {
     if (on != 0 && on != 1) return nfail(SMG_ERR_ARG, "on must be 0 or 1");
     net_tensor_cores() = (on == 1);

@@ -42,7 +42,7 @@ EXPORTS = ("smg_setup", "smg_set_precision", "smg_set_option", "smg_apply", "smg
            "krylov_solve_batched", "smg_barrier_selftest", "smg_batched_setup", "smg_batched_solve",
            "smg_batched_destroy", "smg_batched_apply", "smg_batched_info", "smg_batched_set_profile", "smg_batched_profile_read",
            "smg_set_learned", "smg_learned_stats", "smg_collect_pairs", "smg_net_forward", "smg_net_loss_grad",
-           "smg_net_train", "smg_net_set_tensor_cores", "smg_net_tc_status", "smg_setup_coefs",
+           "smg_net_train", "smg_net_release", "smg_net_set_tensor_cores", "smg_net_tc_status", "smg_setup_coefs",
            "smg_plane_layout", "smg_plane_layout_kind", "smg_gram", "smg_krylov_history", "smg_plane_classes",
            "smg_cycle_form")
 NET_WEIGHTS = 7776
@@ -94,6 +94,7 @@ def _load():
     L.smg_net_forward.argtypes = [i, i, i, i, vp, vp, vp, vp]
     L.smg_net_loss_grad.argtypes = [i, i, i, i, vp, vp, vp, dp, vp, vp]
     L.smg_net_train.argtypes = [i, vp, vp, vp, i, d, ctypes.c_ulonglong, i, vp, vp, vp]
+    L.smg_net_release.argtypes = []
     L.smg_net_set_tensor_cores.argtypes = [i]
     L.smg_net_tc_status.argtypes = [ip]
     L.smg_gram.argtypes = [ctypes.c_longlong, i, vp, i, vp, vp, vp]
@@ -408,6 +409,11 @@ def smg_net_train(dims_list, rho_list, e_list, w, epochs=3, lr=1e-3, seed=0, act
                               epochs, lr, seed, PRECISIONS.get(act, act), w.ctypes.data, hist.ctypes.data,
                               _stream(stream)))
     return w, hist
+
+
+def smg_net_release() -> None:
+    """Give back the device memory the training calls keep between calls (up to 1 GB)."""
+    _check(_lib.smg_net_release())
 
 
 def smg_net_set_tensor_cores(on: bool) -> None:
