@@ -247,9 +247,10 @@ int smg_batched_info(smg_batched_handle h, int *threads, int *order, int *blocks
  * smg_batched_set_profile / smg_batched_profile_read -- with profiling on, each iteration's
  * graph replay is timed by its event nodes: class 0 the V-cycles' kernels, class 1 the
  * Krylov kernels.  Read returns replays, total device milliseconds and, for class 0, the
- * algorithmic bytes of the V-cycles performed (storage words each active system's cycle must
- * read and write: 2.5 words per point per relaxation sweep, 5 per point for residual +
- * restriction + prolongation, 2 per point on the coarsest plane); reading resets the class.
+ * bytes of the vectors that the V-cycles performed have to move (each active system's: 6 words of 4
+ * bytes a point where all of a mode's levels fit in one CTA's shared memory, else also those of the
+ * levels above: 4 words a point, 2 a point of the next level and 3 a point for each sweep beyond the
+ * first pre-sweep); reading resets the class.
  */
 int smg_batched_set_profile(smg_batched_handle h, int on);
 int smg_batched_profile_read(smg_batched_handle h, int which, long long *launches, double *ms, double *bytes);

@@ -5,7 +5,7 @@
 // Per iteration, one CUDA graph:
 //   1. the V-cycles of all systems in the sine eigenvectors of their x-lines (modal.cuh): one launch
 //      transforms every system's residuals, one CTA per (system, mode) runs that mode's whole cycle
-//      in shared memory (largest systems first; up to three launches side by side, by how many CTAs
+//      in shared memory (largest systems first; up to two launches side by side, by how many CTAs
 //      share an SM), one launch transforms back.  Systems with planes too many for that run their
 //      finest levels through the slab kernels first;
 //   2. the FP64 Krylov kernels over all systems at once: vectors are concatenated, every CTA
@@ -402,28 +402,19 @@ struct SysPlan {
     long long N, off;                  // unknowns; offset into the concatenated vectors
     HostHierarchy H;
     ModalHost<float> m;                // the mode-space cycle
-    double cycle_bytes;                // algorithmic bytes of one V-cycle of this system
+    double cycle_bytes;                // bytes of its vectors that one V-cycle has to move
 };
 
-// Algorithmic traffic of one V-cycle (npre pre-sweeps, npost post-sweeps) of one system, in
-// storage words: a relaxation of a colour reads f and writes u of its planes (and reads u in
-// correction form, mode 2), and reads each opposite-colour plane once when it can be nonzero;
-// residual + restriction and prolongation + correction move 2.5 words per fine point each.
+// Vectors' words that one V-cycle of a system has to move.  The transforms read r and write f, read u and write s; the
+// levels one CTA runs in shared memory read the first one's f and write its u; a level above them reads f and writes u and the
+// next f, and on the way up reads the next u, and reads and writes its own; each further sweep there reads f and u
+// and writes u.
 double vcycle_words(const SysPlan &p, int npre, int npost) {
     const double np = static_cast<double>(p.nx) * p.ny;
-    double w = 0.0;
-    auto colour = [&](int nzl, int col, int mode) {
-        const int nplanes = col == 0 ? (nzl + 1) / 2 : nzl / 2;
-        const int nother = nzl - nplanes;
-        return (nplanes * (2.0 + (mode == 2 ? 1.0 : 0.0)) + (mode >= 1 ? nother : 0)) * np;
-    };
-    for (int l = 0; l + 1 < p.H.L; ++l) {
-        const int nzl = p.H.nz_l[l];
-        for (int sw = 0; sw < npre; ++sw) w += colour(nzl, 0, sw == 0 ? 0 : 2) + colour(nzl, 1, sw == 0 ? 1 : 2);
-        for (int sw = 0; sw < npost; ++sw) w += colour(nzl, 1, 2) + colour(nzl, 0, 2);
-        w += 5.0 * nzl * np;
-    }
-    w += 2.0 * np;  // the coarsest plane: read f, write u
+    const int lt = p.m.a.lt;
+    double w = 4.0 * np * p.nz + 2.0 * np * p.H.nz_l[lt];
+    for (int l = 0; l < lt; ++l)
+        w += np * ((2.0 + 2.0 + 3.0 * (npre - 1 + npost)) * p.H.nz_l[l] + 2.0 * p.H.nz_l[l + 1]);
     return w;
 }
 
@@ -594,12 +585,12 @@ int batched_build(smg_batched_ctx &c, const int *dims, cudaStream_t st) {
         p.off = vtot;
         vtot += (p.N + 31) / 32 * 32;
         build_hierarchy(p.nx, p.ny, p.nz, p.H);
-        p.cycle_bytes = vcycle_words(p, c.npre, c.npost) * 4.0;
         if (modal_plan<float>(p.m, p.H, modal_shape(p.H), c.cfg, c.npre, c.npost) != 0) {
             set_last_error("batched solver: a system's planes do not fit the mode-space cycle");
             return SMG_ERR_CUDA;
         }
         modal_vectors<float>(p.m, 1);
+        p.cycle_bytes = vcycle_words(p, c.npre, c.npost) * sizeof(float);
         b_shared += p.m.shared.size();
         b_coef += up(p.m.coef_values * sizeof(float));
         b_c64 += up(p.m.coef64_values * sizeof(double));

@@ -600,14 +600,6 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_al
 template <class T>
 constexpr int modal_threads() { return sizeof(T) == 8 ? 256 : 512; }
 
-// Phase-trace hook for latency studies: compiled out unless SMG_MODAL_TRACE names a device function
-// `void f(int op, int level)` called after each step.
-#ifdef SMG_MODAL_TRACE
-#define SMG_MTRACE(op, l) SMG_MODAL_TRACE((op), (l))
-#else
-#define SMG_MTRACE(op, l) ((void)0)
-#endif
-
 // The cycle of one mode and right-hand side on the tail levels, as one loop over planned steps, a CTA
 // barrier after each: every kind of step is compiled once (inlined at each place of the cycle it
 // appears, the kernel would not fit the instruction cache).
@@ -643,7 +635,6 @@ __device__ __forceinline__ void tail_body(const ModalArgs<T> &A, int mode_idx, i
     for (int i = tid; i < A.sum_ny; i += nt) ltype[i] = A.ltype[i];
     cp_async_wait();
     __syncthreads();
-    SMG_MTRACE(0, lt);
     for (int step = 0;; ++step) {
         const TailOp &o = ring[step & 1];
         const int kind = o.kind;
@@ -709,7 +700,6 @@ __device__ __forceinline__ void tail_body(const ModalArgs<T> &A, int mode_idx, i
         }
         cp_async_wait();
         __syncthreads();
-        SMG_MTRACE(kind, o.level);
     }
 }
 
