@@ -47,7 +47,7 @@ enum {
 };
 
 enum { SMG_PCG = 0, SMG_FPCG = 1, SMG_PSD = 2 };       /* eq. (1), eq. (2), beta = 0 */
-enum { SMG_FP64 = 0, SMG_FP32 = 1, SMG_BF16 = 2 };     /* V-cycle storage precision */
+enum { SMG_FP64 = 0, SMG_FP32 = 1, SMG_BF16 = 2 };     /* V-cycle precision (smg_set_precision) */
 
 /* Options for smg_set_option.
  *
@@ -141,8 +141,9 @@ enum {
  */
 int smg_setup(int nx, int ny, int nz, int npre, int npost, smg_handle *out);
 
-/* smg_set_precision -- storage precision of the V-cycle: SMG_FP64, SMG_FP32 or SMG_BF16.
- * FP32 computes in FP32; BF16 computes in FP32 and stores its result T r in bfloat16.  The
+/* smg_set_precision -- precision of the V-cycle: SMG_FP64, SMG_FP32 or SMG_BF16.
+ * FP32 computes and stores its vectors in FP32; BF16 is the FP32 cycle with its result T r rounded to bfloat16
+ * (krylov_solve stores it so, smg_apply widens it exactly): the same memory and time.  The
  * one-plane coarsest level always computes in FP64.  Krylov recurrences, inner products and
  * norms stay FP64. */
 int smg_set_precision(smg_handle h, int prec);

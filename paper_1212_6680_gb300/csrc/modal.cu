@@ -289,6 +289,10 @@ SMG_MODAL_CFG(1, 16, 8);
 SMG_MODAL_CFG(1, 32, 8);
 SMG_MODAL_CFG(1, 32, 16);
 
+// Few lanes a plane leave more planes to a warp and fewer shuffles, few lines a lane a shorter chain and fewer
+// registers: up to 128 lines 8 and 16 lanes.  The two splits of 129 to 256 lines, applications in us: FP32 16 x 16 / 32 x 8
+// 256^3 645 / 669, 64x160x100 77 / 78, 64x256x64 71 / 70, 128x200x64 (1,1) 113 / 108; FP64 32 x 8 / 16 x 16 64x256x64 455 /
+// 500, 100x256x200 2562 / 2485, 64x160x100 552 / 513, 128x200x64 (1,1) 1296 / 1218.
 ModalConfig modal_config(int ny, bool f64) {
     if (ny <= 32) return {8, 4};
     if (ny <= 64) return {8, 8};

@@ -40,7 +40,8 @@ cudaError_t tail_batch(const ModalArgs<T> *d_args, const ModalTask *tasks, int n
 }
 
 // The slab's coarse planes: as many as its red planes (the slab's share + 3) fit in one pass over the
-// groups, in at most half of an SM's shared memory (two CTAs per SM) where that holds a useful slab.
+// groups, in at most half of an SM's shared memory (two CTAs per SM) where that holds a useful slab: four coarse planes,
+// 13 rows (256^3 and 384^3 with two coarse planes, or one CTA an SM always: within 1 %).
 int slab_count(const ModalArgs<T> &a, int l, size_t *smem) {
     const int groups = modal_threads<T>() / G, nzc = a.nz[l + 1];
     const size_t row = static_cast<size_t>(a.sm_pitch) * sizeof(T), tabs = static_cast<size_t>(a.ncls[l]) * Tab<G, K>::kElems * sizeof(T);

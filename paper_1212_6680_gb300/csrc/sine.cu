@@ -413,7 +413,9 @@ dim3 grid_of(const SineArgs &g, int nb) {
     const long long lines = static_cast<long long>(g.nz) * g.pitch;
     return dim3(static_cast<unsigned>((lines + 16 * LT - 1) / (16 * LT)), (g.nh + kBN - 1) / kBN, nb);
 }
-// Whether 128-line tiles give every SM three CTAs (two run at once; a third evens out the last wave).
+// Whether 128-line tiles give every SM three CTAs (two run at once; a third evens out the last wave).  Applications with
+// 64-line tiles / 128-line tiles, us: below the line 24x20x16 23 / 29, 101x75x53 55 / 63, 128^3 74 / 80; above it 200x128x128
+// 166 / 170, 8 vectors at 96^3 305 / 322, 512x512x64 964 / 943, 384^3 2550 / 2496, 1280x80x80 757 / 703.
 bool wide_tiles(const SineArgs &g, int nb) {
     const dim3 d = grid_of<8>(g, nb);
     return static_cast<long long>(d.x) * d.y * d.z >= 3 * 152;
