@@ -85,7 +85,7 @@ struct smg_ctx {
     ModalShape shape;               // formed when mode space is first used
     std::vector<void *> d_f, d_u;   // [L], entry 0 unused
     // krylov_solve's T r in level_prec and, for an FP32 cycle, behind it r in FP32, which its kernels write: N doubles,
-    // allocated once (with a small grid's tables they keep the driver's block in place over a change of precision)
+    // allocated once (with a small grid's tables they keep the CUDA allocator's block in place over a change of precision)
     void *d_s = nullptr;
     void *d_ws = nullptr;
     size_t ws_bytes = 0;

@@ -24,7 +24,7 @@ def free_bytes():
     return torch.cuda.mem_get_info()[0]
 
 
-SLACK = 64 << 20  # code and driver blocks that a first launch brings with it
+SLACK = 64 << 20  # code and allocator blocks that a first launch brings with it
 
 
 @pytest.mark.parametrize("call", ["forward", "loss_grad", "train"])
